@@ -424,6 +424,23 @@ m1_status Engine<R>::rebuild()
     return M1_OK;
 }
 
+// Constants of the fixed-point form of the FP64 strips (m1_fx.cuh), and whether
+// a level may take it: its blocks hold E in 2^-500 .. 2^500, so c and b = dt / (2 h)
+// of ordinary size keep every product inside FP64's range.  Unequal cell sides
+// scale one axis' pair of neighbours by the ratio of the two b.
+template <typename R>
+static void set_fx(Level<R>& q, double c, double bx, double by)
+{
+    const double b = std::max(bx, by), s = std::min(bx, q.dim == 2 ? by : bx);
+    q.cb = c * b;
+    q.cbF = c * c * b;
+    q.ic = 1.0 / c;
+    q.rho = 0;
+    const bool ok = c > 1e-60 && c < 1e60 && s > 1e-60 && b < 1e60;
+    q.fx = !ok ? 0 : (s == b ? 1 : (bx < by ? 2 : 3));
+    if (q.fx > 1) q.rho = std::llrint(std::ldexp(s / b, 62));
+}
+
 template <typename R>
 m1_status Engine<R>::set_dt(int i, double dt)
 {
@@ -434,8 +451,9 @@ m1_status Engine<R>::set_dt(int i, double dt)
         const double hx = g.lx / g.nx * (double)(1 << l);
         const double hy = g.dim == 2 ? g.ly / g.ny * (double)(1 << l) : 1.0;
         const double ax = g.c * dt / hx, ay = g.dim == 2 ? g.c * dt / hy : 0.0;
-        q.ax = (R)ax; q.ay = (R)ay;
-        q.bx = (R)(dt / (2.0 * hx)); q.by = g.dim == 2 ? (R)(dt / (2.0 * hy)) : R(0);
+        const double bx = dt / (2.0 * hx), by = g.dim == 2 ? dt / (2.0 * hy) : 0.0;
+        q.bx = (R)bx; q.by = (R)by;
+        set_fx(q, g.c, bx, by);
         q.diag = (R)(1.0 + ax + ay);
         q.cdt = (R)(g.c * dt);
         M1_CK(cudaMemcpyAsync(d + (size_t)l * cap + i, &q, sizeof(Level<R>), cudaMemcpyHostToDevice,

@@ -51,12 +51,16 @@ struct Level {
     int prof_len;                 // stride of the inflow profile table
     int sx, sh, strips;           // warp strips: count along x, rows each, total
     int ring;                     // FP32 correction form: stage strip rows by cp.async
+    int fx;                       // FP64: the strips may take the fixed-point form (m1_fx.cuh):
+                                  // 1 square cells (or 1D), 2 scale the x pair by rho, 3 the y pair
     R c, a_r, c_v;
     R ic2;                        // 1 / c^2
-    R ax, ay, bx, by;             // c dt / h and dt / (2 h) per axis (y: 0 in 1D)
-    R diag;                       // 1 + ax + ay
+    R bx, by;                     // dt / (2 h) per axis (y: 0 in 1D)
+    R diag;                       // 1 + c dt / hx + c dt / hy
     R cdt;                        // c dt
     double vol;                   // cell volume h^d (norm weight)
+    double cb, cbF, ic;           // fixed-point form: c b and c^2 b, b the larger of bx, by; 1 / c
+    long long rho;                // ... and the smaller over the larger, times 2^62
     Cell4<R>* v;                  // restricted iterate v_l
     Cell4<R>* u[2];               // ping-pong iterate u_l
     Cell4<R>* f;                  // right-hand side (b at level 0, FAS rhs above)

@@ -1,0 +1,217 @@
+// FP64 work on the integer pipe: the M1 closure and the neighbour sums of a cell
+// in 64-bit fixed point.
+//
+// GB300 issues one FP64 warp instruction per 64 clocks and SM partition, a
+// 32 x 32 + 64-bit multiply-add per 2.6 and a 64-bit add per 4 (measured).  The
+// stencil kernels were bound by the FP64 pipe with nearly 90% of their issue
+// slots idle.  A cell's closure and its contribution to its neighbours need no
+// exponents of their own: with |F| <= c E every quantity (F / c, the tensor
+// P) is at most E in size, so the six numbers of a cell fit one block: an
+// exponent, E's, and 64-bit significands relative to it.  Products keep 62 bits,
+// sums are exact, so the results carry 57 bits or more relative to E where FP64
+// carried 53 with a rounding per operation: no precision is lost.
+//
+// Blocks are formed for regular cells only (fx_regular below: E a normal number
+// of ordinary size, |F| <= c E up to a slack); a warp that meets another cell
+// takes the FP64 form of its strip instead, which is the one that handles
+// infinities, NaN and inadmissible states.
+//
+// The functions are host code too, so that their arithmetic can be checked
+// without a GPU (the host takes IEEE results where the device takes the
+// hardware's approximate reciprocals; both are seeds of the same iterations).
+#pragma once
+#include <cmath>
+#include <cuda_runtime.h>
+
+#include "m1_device.cuh"
+
+namespace m1 {
+
+typedef long long i64;
+typedef unsigned long long u64;
+
+__host__ __device__ __forceinline__ u64 bits_of_double(double x)
+{
+#ifdef __CUDA_ARCH__
+    return (u64)__double_as_longlong(x);
+#else
+    u64 b;
+    memcpy(&b, &x, sizeof b);
+    return b;
+#endif
+}
+
+__host__ __device__ __forceinline__ double double_of_bits(u64 b)
+{
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double((i64)b);
+#else
+    double x;
+    memcpy(&x, &b, sizeof x);
+    return x;
+#endif
+}
+
+// seeds: about 2^-22 relative
+__host__ __device__ __forceinline__ float seed_rcp(float x)
+{
+#ifdef __CUDA_ARCH__
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+#else
+    return 1.0f / x;
+#endif
+}
+
+__host__ __device__ __forceinline__ float seed_rsqrt(float x)
+{
+#ifdef __CUDA_ARCH__
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+#else
+    return 1.0f / sqrtf(x);
+#endif
+}
+
+// a * b + c of 32-bit a, b and 64-bit c (one instruction)
+__host__ __device__ __forceinline__ i64 madw(int a, int b, i64 c) { return (i64)a * b + c; }
+
+// A number |x| < 2^62 split at bit 31 (h signed, 0 <= l < 2^31), so that the
+// partial products are signed 32 x 32 bits.
+struct Split {
+    int h, l;
+};
+__host__ __device__ __forceinline__ Split split62(i64 x)
+{
+    return Split{ (int)(x >> 31), (int)((unsigned)x & 0x7fffffffu) };
+}
+
+// a b / 2^62 (+ c), |a|, |b| < 2^62, within 2 units
+__host__ __device__ __forceinline__ i64 mul62(Split a, Split b, i64 c = 0)
+{
+    const i64 mid = madw(a.h, b.l, madw(a.l, b.h, 0));
+    return madw(a.h, b.h, mid >> 31) + c;
+}
+
+__host__ __device__ __forceinline__ i64 sqr62(Split a)
+{
+    const i64 mid = madw(a.h, a.l, 0);
+    return madw(a.h, a.h, mid >> 30);
+}
+
+// a cell's block: values v = m 2^(e - 60), F over c
+struct FxCell {
+    int e;
+    i64 E, Fx, Fy, Pxx, Pxy, Pyy;
+};
+
+// exponents (biased) of the E a block can hold: 2^-500 .. 2^500
+constexpr unsigned kFxMinExp = 1023 - 500, kFxMaxExp = 1023 + 500;
+
+// The significand of x relative to 2^(be - 1023) at scale 2^61, truncated; the
+// biased exponent of x is at most be (d >= 0), subnormals and zero give 0.
+__host__ __device__ __forceinline__ i64 fx_align(u64 bits, int d)
+{
+    const u64 m = ((bits & 0xfffffffffffffull) | 0x10000000000000ull) << 9;
+    const i64 v = (i64)(d > 63 ? 0 : m >> d);
+    const i64 s = (i64)bits >> 63;
+    return (v ^ s) - s;
+}
+
+// The closure of Eq. (5) and the cell's block, from E and F / c.  With x = E and
+// sigma = sqrt(x^2 - 3/4 |F/c|^2) >= x/2 it reads
+//   P = (2 sigma - x)/3 I + 3/2 (F/c)(F/c)^T / (x + sigma),
+// the form of closure() multiplied through by E: one square root and one
+// reciprocal, no division by E, smooth at F = 0.  Returns false when the cell is
+// not regular (the block is then meaningless).
+__host__ __device__ __forceinline__ bool fx_stage(double E, double Fx, double Fy, FxCell& o)
+{
+    const u64 be = bits_of_double(E), bx = bits_of_double(Fx), by = bits_of_double(Fy);
+    const unsigned te = (unsigned)(be >> 52);                  // sign included
+    const int dx = (int)te - (int)((unsigned)(bx >> 52) & 0x7ffu);
+    const int dy = (int)te - (int)((unsigned)(by >> 52) & 0x7ffu);
+    bool ok = te - kFxMinExp <= kFxMaxExp - kFxMinExp && dx >= 0 && dy >= 0;
+    // scale 2^61: x in [1, 2), |F / c| < 2
+    const i64 xE = (i64)(((be & 0xfffffffffffffull) | 0x10000000000000ull) << 9);
+    const i64 xF = fx_align(bx, dx), yF = fx_align(by, dy);
+    const Split sE = split62(xE), sX = split62(xF), sY = split62(yF);
+    // scale 2^60: x^2 and |F/c|^2
+    const i64 E2 = sqr62(sE);
+    const i64 midF = madw(sX.h, sX.l, madw(sY.h, sY.l, 0));
+    const i64 F2 = madw(sX.h, sX.h, madw(sY.h, sY.h, midF >> 30));
+    ok = ok && F2 <= E2 + (E2 >> 10);
+    // xi = x^2 - 3/4 |F/c|^2 in [x^2/4, x^2], scale 2^60
+    i64 xi = E2 - F2 + (F2 >> 2);
+    const i64 q2 = E2 >> 2;
+    xi = xi > q2 ? xi : q2;
+    // sigma = sqrt(xi): a 30-bit start s0 from the seed y of 1/sqrt(xi), then two
+    // Newton corrections sigma += (xi - sigma^2) y / 2, exact residuals
+    const float xif = (float)(int)(xi >> 32) * 0x1p-28f;
+    const float yf = seed_rsqrt(xif);
+    const int Y = (int)(yf * 0x1p29f);                         // y <= 2
+    const float sf = xif * yf;
+    const int s0 = (int)(sf * 0x1.fffffcp29f);                  // < 2^31 (sigma < 2 up to rounding)
+    const i64 t0 = xi - madw(s0, s0, 0);                       // scale 2^60, |t0| < 2^42
+    const i64 d0 = madw((int)(t0 >> 12), Y, 0) >> 18;          // t0 y / 2, scale 2^60
+    i64 sg = ((i64)s0 << 30) + d0;
+    const i64 t1 = xi - sqr62(split62(sg << 1));
+    sg += madw((int)t1, Y, 0) >> 30;
+    const i64 hx = xE >> 2;                                    // x / 2 at scale 2^60
+    sg = sg > hx ? sg : hx;
+    // D = 1 / (x + sigma), scale 2^62, from the seed r: D = r (1 + d + d^2),
+    // d = 1 - (x + sigma) r, less 2^-57 so that 3/2 D stays below 2^62
+    const i64 w = (xE >> 1) + sg;                              // scale 2^60, in [1.5, 4)
+    const float rf = seed_rcp((float)(int)(w >> 32) * 0x1p-28f);
+    const int Rr = (int)(rf * 0x1p31f);                        // r <= 2/3
+    const Split sw = split62(w);
+    const i64 d = ((1ll << 60) - 8) - madw(sw.h, Rr, madw(sw.l, Rr, 0) >> 31);
+    const Split sd = split62(d);                               // |d| < 2^39
+    const i64 rd = madw(sd.h, Rr, madw(sd.l, Rr, 0) >> 31);    // r d, scale 2^60
+    const i64 rdd = madw((int)(d >> 22), (int)(rd >> 22), 0) >> 16;
+    const i64 D = ((i64)Rr << 31) + ((rd + rdd) << 2);
+    const Split sD = split62(D + (D >> 1));                    // 3/2 D, scale 2^62
+    // (2 sigma - x) / 3, scale 2^60: the factor is 2^61 / 3
+    constexpr i64 third = 768614336404564651ll;
+    const i64 iso = mul62(split62((sg << 2) - xE), split62(third));
+    // 3/2 D F/c at scale 2^61, the tensor at scale 2^60
+    const Split gx = split62(mul62(sX, sD)), gy = split62(mul62(sY, sD));
+    o.Pxx = mul62(gx, sX, iso);
+    o.Pxy = mul62(gx, sY);
+    o.Pyy = mul62(gy, sY, iso);
+    o.E = xE >> 1;
+    o.Fx = xF >> 1;
+    o.Fy = yF >> 1;
+    o.e = (int)te - 1023;
+    return ok;
+}
+
+// The double nearest s 2^(e - 58) up to one unit in its last place (rounded half
+// up in magnitude); e within the blocks' exponents, |s| < 2^63.
+__host__ __device__ __forceinline__ double fx_double(i64 s, int e)
+{
+    const u64 sign = (u64)s & 0x8000000000000000ull;
+    u64 m = (u64)(s < 0 ? -s : s);
+    if (m == 0) return 0.0;
+#ifdef __CUDA_ARCH__
+    const int z = __clzll((i64)m);
+#else
+    const int z = __builtin_clzll(m);
+#endif
+    m <<= z;                                                   // bit 63 set: value m 2^(e - 58 - z)
+    m = (m >> 11) + ((m >> 10) & 1);                           // 53 bits (2^53 carries into the exponent)
+    return double_of_bits(sign | (m + ((u64)(1023 + 63 - 58 - 1 - z + e) << 52)));
+}
+
+// Arithmetic right shift by n >= 0 (63 and more: the sign).
+__host__ __device__ __forceinline__ i64 fx_sar(i64 x, int n) { return x >> (n < 63 ? n : 63); }
+
+// What a cell adds to its neighbour's sums across one face (Eq. (9) with F over
+// c and a common factor c dt / (2 h) taken out): E +- F_d, F_x +- P_xd, F_y +- P_yd.
+struct FxFlux {
+    int e;
+    i64 E, Fx, Fy;
+};
+
+}  // namespace m1

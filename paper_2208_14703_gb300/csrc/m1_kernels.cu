@@ -1,6 +1,6 @@
 // Kernels of the implicit M1 multigrid step (arXiv:2208.14703), FP64 and FP32.
 //
-//   k_sweep     one Jacobi sweep (Algorithm 1 / Eq. (10)); PSEUDO = true fuses
+//   k_sweep64, k_sweep   one Jacobi sweep (Algorithm 1 / Eq. (10)); PSEUDO = true fuses
 //               the explicit and implicit halves of the pseudo-time step
 //               (Eq. (30), Algorithm 3) into the same sweep
 //   k_apply     A(u) for the residual r = f - A(u) (Eq. (13)) with per-strip norm
@@ -22,6 +22,7 @@
 
 #include "m1_dw.cuh"
 #include "m1_kernels.cuh"
+#include "m1_strip64.cuh"
 
 namespace m1 {
 
@@ -338,18 +339,11 @@ __device__ __forceinline__ bool enter_item(Level<R>& L, const Level<R>* src, con
     return true;
 }
 
-// Persistent sweep over every listed (instance, strip): one warp per item.
-// FP64 instances are held to 128 registers (8 blocks per SM): one register
-// more (the pseudo-time variant) cost 4% of the FP64 step on GB300.
-// NORM: the fine Jacobi sweep that also writes each strip's weighted residual
-// norm partial of its input state (the stop test of the cycle that left it).
-// FAS: the first pseudo-time step of a fresh coarse visit, which also forms the
-// FAS right-hand side.
-template <typename R, bool PSEUDO, bool DELTA = false, bool NORM = false, bool FAS = false>
-__global__ void __launch_bounds__(kStripWarps * 32, (sizeof(R) == 8 ? 8 : 10)) k_sweep(const Level<R>* __restrict__ lv,
-                                                            WorkList wl, Ctl* __restrict__ ctls,
-                                                            int in_buf, int out_buf,
-                                                            double* __restrict__ partials)
+// Persistent FP32 sweep over every listed (instance, strip): one warp per item.
+template <typename R, bool PSEUDO, bool DELTA>
+__global__ void __launch_bounds__(kStripWarps * 32, 10) k_sweep(const Level<R>* __restrict__ lv,
+                                                                WorkList wl, Ctl* __restrict__ ctls,
+                                                                int in_buf, int out_buf)
 {
     __shared__ Level<R> Ls[kStripWarps];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -361,8 +355,111 @@ __global__ void __launch_bounds__(kStripWarps * 32, (sizeof(R) == 8 ? 8 : 10)) k
         const int2 it = nx;
         if (!enter_item(L, lv + it.x, ctls, it.x, lane)) continue;
         const Cell4<R>* __restrict__ src = in_buf < 0 ? L.v : L.u[in_buf];
-        const double nrm =
-            strip_regs<R, PSEUDO, DELTA, NORM, FAS>(L, ctls + it.x, it, lane, src, out_buf);
+        strip_regs<R, PSEUDO, DELTA>(L, ctls + it.x, it, lane, src, out_buf);
+        __syncwarp();
+    }
+}
+
+// ---------------------------------------------------------------------------
+// The FP64 sweep: a strip in fixed point (m1_strip64.cuh), or, where a cell of it
+// is not regular, in FP64 throughout (strip_regs, out of line).
+template <bool PSEUDO, bool NORM, bool FAS>
+__device__ __noinline__ double strip_general64(const Level<double>& L, Ctl* ctl, int2 it, int lane,
+                                               const Cell4<double>* __restrict__ src, int out_buf)
+{
+    return strip_regs<double, PSEUDO, false, NORM, FAS>(L, ctl, it, lane, src, out_buf);
+}
+
+// One fine Jacobi sweep, or one fused pseudo-time step, of an (instance, strip)
+// item: what update_cell does, with N from the fixed-point sums.
+template <bool PSEUDO, bool NORM, bool FAS>
+__device__ __forceinline__ double strip_sweep64(const Level<double>& L, Ctl* ctl, int2 it, int lane,
+                                                const Cell4<double>* __restrict__ src, int out_buf)
+{
+    struct Pre {
+        Cell4<double> b, u;
+        Sig2<double> sg;
+    };
+    double nrm = 0.0;
+    unsigned fails = 0;
+    if (L.fx) {
+        const Pseudo<double> ps = PSEUDO ? pseudo_of<double>(ctl) : Pseudo<double>{};
+        const double cbE = PSEUDO ? ps.dtau * L.cb : L.cb, cbF = PSEUDO ? ps.dtau * L.cbF : L.cbF;
+        auto pre = [&](size_t k) {
+            Pre p;
+            p.b = FAS ? L.r[k] : L.f[k];
+            p.sg = L.sig[k];
+            if (PSEUDO || NORM) p.u = src[k];
+            return p;
+        };
+        const bool regular = strip_march_fx(L, it, lane, src, pre, [&](size_t k, const Pre& p,
+                                                                       const FxFlux& s) {
+            const double NE = fx_double(s.E, s.e), NFx = fx_double(s.Fx, s.e),
+                         NFy = fx_double(s.Fy, s.e);
+            const double ka = L.cdt * p.sg.sa, kt = L.cdt * (p.sg.sa + p.sg.ss);
+            Cell4<double> b = p.b;
+            bool ok;
+            Cell4<double> o;
+            if (NORM || FAS) {
+                // the local part of A(u): r = (b + N) - D(u), or f = D(u) - N + r
+                const Cell4<double>& u = p.u;
+                const double T2 = u.T * u.T, src_e = ka * fma(-L.a_r, T2 * T2, u.E);
+                const double dF = L.diag + kt;
+                if (FAS) {
+                    b.E = fma(-L.cb, NE, fma(L.diag, u.E, src_e)) + b.E;
+                    b.Fx = fma(-L.cbF, NFx, dF * u.Fx) + b.Fx;
+                    b.Fy = fma(-L.cbF, NFy, dF * u.Fy) + b.Fy;
+                    b.T = fma(L.c_v, u.T, -src_e) + b.T;
+                    L.f[k] = b;
+                } else {
+                    const double rE = b.E - fma(-L.cb, NE, fma(L.diag, u.E, src_e));
+                    const double rFx = b.Fx - fma(-L.cbF, NFx, dF * u.Fx);
+                    const double rFy = b.Fy - fma(-L.cbF, NFy, dF * u.Fy);
+                    const double rT = b.T - fma(L.c_v, u.T, -src_e);
+                    nrm += fma(fma(rFy, rFy, rFx * rFx), L.ic2, fma(rE, rE, rT * rT));
+                }
+            }
+            if (!PSEUDO) {
+                o = local_solve64(0.0, 1.0, L.diag, ka, kt, L.c_v, L.a_r, fma(cbE, NE, b.E),
+                                  fma(cbF, NFx, b.Fx), fma(cbF, NFy, b.Fy), b.T, ok);
+            } else {
+                const double tau = limited_step(p.u, b, ps.dtau, ps.theta, ps.s, L.c);
+                o = local_solve64(1.0, ps.dtau, L.diag, ka, kt, L.c_v, L.a_r,
+                                  fma(cbE, NE, fma(tau, b.E, p.u.E)),
+                                  fma(cbF, NFx, fma(tau, b.Fx, p.u.Fx)),
+                                  fma(cbF, NFy, fma(tau, b.Fy, p.u.Fy)), fma(tau, b.T, p.u.T), ok);
+            }
+            if (!ok) ++fails;
+            L.u[out_buf][k] = o;
+        });
+        if (regular) {
+            if (fails) atomicAdd(&ctl->newton_fail, fails);
+            return nrm;
+        }
+    }
+    return strip_general64<PSEUDO, NORM, FAS>(L, ctl, it, lane, src, out_buf);
+}
+
+// Persistent FP64 sweep (the item loop of k_sweep), held to 128 registers (8 blocks
+// per SM).  Bound by the FP64 pipe, now at 36 of its operations a fine update and
+// not 109: 0.37 ms a sweep at 2048^2 where the FP64 form took 0.88 ms.
+template <bool PSEUDO, bool NORM = false, bool FAS = false>
+__global__ void __launch_bounds__(kStripWarps * 32, 8) k_sweep64(const Level<double>* __restrict__ lv,
+                                                                 WorkList wl, Ctl* __restrict__ ctls,
+                                                                 int in_buf, int out_buf,
+                                                                 double* __restrict__ partials)
+{
+    __shared__ Level<double> Ls[kStripWarps];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    Level<double>& L = Ls[wib];
+    const int w0 = blockIdx.x * kStripWarps + wib, ws = gridDim.x * kStripWarps;
+    int2 nx = item_at(wl, w0);
+    const int nw = *wl.count;
+    for (int w = w0; w < nw; w += ws, nx = item_at(wl, w)) {
+        const int2 it = nx;
+        if (!enter_item(L, lv + it.x, ctls, it.x, lane)) continue;
+        const Cell4<double>* __restrict__ src = in_buf < 0 ? L.v : L.u[in_buf];
+        const double nrm = strip_sweep64<PSEUDO, NORM, FAS>(L, ctls + it.x, it, lane, src, out_buf);
         if (NORM) {
             const double sum = warp_sum(nrm);
             if (lane == 0) partials[L.part_off + it.y] = sum * L.vol;
@@ -627,6 +724,58 @@ __device__ __forceinline__ double apply_item(const Level<R>& L, int2 it, int lan
     return nrm;
 }
 
+template <int MODE>
+__device__ __noinline__ double apply_general64(const Level<double>& L, int2 it, int lane,
+                                               int state_buf, int write_r)
+{
+    return apply_item<double, MODE, false>(L, it, lane, state_buf, write_r);
+}
+
+// apply_item in FP64 with the neighbour sums in fixed point (state_buf >= -1: the
+// FP64 levels carry no base state).
+template <int MODE>
+__device__ __forceinline__ double apply_item64(const Level<double>& L, int2 it, int lane,
+                                               int state_buf, int write_r)
+{
+    struct Pre {
+        Cell4<double> u, f;
+        Sig2<double> sg;
+    };
+    if (L.fx) {
+        const Cell4<double>* __restrict__ src = state_buf < 0 ? L.v : L.u[state_buf];
+        double nrm = 0.0;
+        auto pre = [&](size_t k) {
+            Pre p;
+            p.u = src[k];
+            if (MODE == APPLY_RESID) p.f = L.f[k];
+            if (MODE == APPLY_FAS) p.f = L.r[k];
+            p.sg = L.sig[k];
+            return p;
+        };
+        const bool regular = strip_march_fx(L, it, lane, src, pre, [&](size_t k, const Pre& p,
+                                                                       const FxFlux& s) {
+            const double ka = L.cdt * p.sg.sa, dF = L.diag + L.cdt * (p.sg.sa + p.sg.ss);
+            const Cell4<double>& u = p.u;
+            const double T2 = u.T * u.T, src_e = ka * fma(-L.a_r, T2 * T2, u.E);
+            const Cell4<double> a = {
+                fma(-L.cb, fx_double(s.E, s.e), fma(L.diag, u.E, src_e)),
+                fma(-L.cbF, fx_double(s.Fx, s.e), dF * u.Fx),
+                fma(-L.cbF, fx_double(s.Fy, s.e), dF * u.Fy), fma(L.c_v, u.T, -src_e) };
+            if (MODE == APPLY_RESID) {
+                const Cell4<double> r = { p.f.E - a.E, p.f.Fx - a.Fx, p.f.Fy - a.Fy, p.f.T - a.T };
+                if (write_r) L.r[k] = r;
+                nrm += fma(fma(r.Fy, r.Fy, r.Fx * r.Fx), L.ic2, fma(r.E, r.E, r.T * r.T));
+            } else if (MODE == APPLY_FAS) {
+                L.f[k] = Cell4<double>{ a.E + p.f.E, a.Fx + p.f.Fx, a.Fy + p.f.Fy, a.T + p.f.T };
+            } else {
+                L.r[k] = a;
+            }
+        });
+        if (regular) return nrm;
+    }
+    return apply_general64<MODE>(L, it, lane, state_buf, write_r);
+}
+
 // A(u) of Eq. (12) (+ sources) at one level, per (instance, strip) item:
 //   APPLY_RESID  r = f - A(u) (Eq. (13)), written to L.r if write_r, and the
 //                weighted norm partial of the strip (partials != null)
@@ -650,7 +799,11 @@ __global__ void __launch_bounds__(kStripWarps * 32) k_apply(const Level<R>* __re
     for (int w = w0; w < nw; w += ws, nx = item_at(wl, w)) {
         const int2 it = nx;
         if (!enter_item(L, lv + it.x, ctls, it.x, lane)) continue;
-        const double nrm = apply_item<R, MODE, DELTA>(L, it, lane, state_buf, write_r);
+        double nrm;
+        if constexpr (std::is_same<R, double>::value)
+            nrm = apply_item64<MODE>(L, it, lane, state_buf, write_r);
+        else
+            nrm = apply_item<R, MODE, DELTA>(L, it, lane, state_buf, write_r);
         if (MODE == APPLY_RESID && partials) {
             const double sum = warp_sum(nrm);
             if (lane == 0) partials[L.part_off + it.y] = sum * L.vol;
@@ -1615,28 +1768,27 @@ void launch_sweep(const Level<R>* lv, WorkList wl, Ctl* ctls, bool pseudo, int i
                   int out_buf, cudaStream_t s, bool delta, bool ring, double* partials, bool fas)
 {
     const int g = pgrid_warps(wl), t = kStripWarps * 32;
-    if (fas && pseudo && !delta) {
-        k_sweep<R, true, false, false, true><<<g, t, 0, s>>>(lv, wl, ctls, in_buf, out_buf, nullptr);
-        return;
-    }
-    if (partials && !pseudo && !delta) {
-        k_sweep<R, false, false, true><<<g, t, 0, s>>>(lv, wl, ctls, in_buf, out_buf, partials);
-        return;
-    }
-    if constexpr (std::is_same<R, float>::value) {
+    if constexpr (std::is_same<R, double>::value) {
+        if (pseudo && fas)
+            k_sweep64<true, false, true><<<g, t, 0, s>>>(lv, wl, ctls, in_buf, out_buf, nullptr);
+        else if (pseudo)
+            k_sweep64<true><<<g, t, 0, s>>>(lv, wl, ctls, in_buf, out_buf, nullptr);
+        else if (partials)
+            k_sweep64<false, true><<<g, t, 0, s>>>(lv, wl, ctls, in_buf, out_buf, partials);
+        else
+            k_sweep64<false><<<g, t, 0, s>>>(lv, wl, ctls, in_buf, out_buf, nullptr);
+    } else {
         if (delta && ring) {
             if (pseudo) k_sweep_ring32<true><<<g, t, 0, s>>>(lv, wl, ctls, in_buf, out_buf);
             else k_sweep_ring32<false><<<g, t, 0, s>>>(lv, wl, ctls, in_buf, out_buf);
-            return;
+        } else if (delta) {
+            if (pseudo) k_sweep<R, true, true><<<g, t, 0, s>>>(lv, wl, ctls, in_buf, out_buf);
+            else k_sweep<R, false, true><<<g, t, 0, s>>>(lv, wl, ctls, in_buf, out_buf);
+        } else {
+            if (pseudo) k_sweep<R, true, false><<<g, t, 0, s>>>(lv, wl, ctls, in_buf, out_buf);
+            else k_sweep<R, false, false><<<g, t, 0, s>>>(lv, wl, ctls, in_buf, out_buf);
         }
     }
-    if (delta) {
-        if (pseudo) k_sweep<R, true, true><<<g, t, 0, s>>>(lv, wl, ctls, in_buf, out_buf, nullptr);
-        else k_sweep<R, false, true><<<g, t, 0, s>>>(lv, wl, ctls, in_buf, out_buf, nullptr);
-        return;
-    }
-    if (pseudo) k_sweep<R, true><<<g, t, 0, s>>>(lv, wl, ctls, in_buf, out_buf, nullptr);
-    else k_sweep<R, false><<<g, t, 0, s>>>(lv, wl, ctls, in_buf, out_buf, nullptr);
 }
 
 template <typename R>

@@ -221,9 +221,9 @@ extern "C" m1_status m1_residual_norm_noalloc(const m1_grid_desc* desc, double d
     L.prof_len = L.nx > L.ny ? L.nx : L.ny;
     const double hx = desc->lx / desc->nx, hy = desc->dim == 2 ? desc->ly / desc->ny : 1.0;
     L.c = desc->c; L.a_r = desc->a_r; L.c_v = desc->c_v;
-    L.ax = desc->c * dt / hx; L.ay = desc->dim == 2 ? desc->c * dt / hy : 0.0;
+    const double ax = desc->c * dt / hx, ay = desc->dim == 2 ? desc->c * dt / hy : 0.0;
     L.bx = dt / (2.0 * hx); L.by = desc->dim == 2 ? dt / (2.0 * hy) : 0.0;
-    L.diag = 1.0 + L.ax + L.ay;
+    L.diag = 1.0 + ax + ay;
     L.cdt = desc->c * dt;
     L.vol = desc->dim == 2 ? hx * hy : hx;
 
