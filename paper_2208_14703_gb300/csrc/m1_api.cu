@@ -588,6 +588,12 @@ m1_status Engine<R>::get_state(int i, double* E, double* Fx, double* Fy, double*
 
 // ---- the V-cycle ----------------------------------------------------------------
 template <typename R>
+void Engine<R>::coefs(WorkList wl)
+{
+    if constexpr (std::is_same<R, double>::value) launch_coef64(d, wl, stream);
+}
+
+template <typename R>
 void Engine<R>::sweeps_fine(int& cur, int count, cudaStream_t s)
 {
     for (int k = 0; k < count; ++k) {
@@ -818,6 +824,7 @@ m1_status Engine<R>::step(const double* dts, const m1_solve_params& sp, m1_step_
     M1_CK(cudaEventRecord(ev0, stream));
     const WorkList t0 = strips[0].view(), c0 = chunks[0].view();
     launch_make_rhs<R>(d, c0, ctl, 0, stream);
+    coefs(c0);
     launch_apply<R>(d, t0, ctl, APPLY_RESID, 0, part, 0, stream);
     launch_norm_state<R>(d, t0, ctl, partb, stream);
     launch_finalize<R>(ctl, d, cap, part, partb, FIN_INIT, 0, bctl, stream);
@@ -854,7 +861,7 @@ m1_status Engine<R>::step(const double* dts, const m1_solve_params& sp, m1_step_
             s.status = c.status;
             s.newton_fail = c.newton_fail;
             s.damped = c.damped;
-            s.launches = 4 + launched * (kernels_per_cycle(p) + 1);   // + deferred finalize
+            s.launches = 5 + launched * (kernels_per_cycle(p) + 1);   // + deferred finalize
         }
         ++k;
     }
@@ -916,6 +923,7 @@ m1_status Engine<R>::jacobi(int i, double dt, int sweeps)
     M1_TRY(set_dt(0, dt));
     M1_TRY(set_ctl_simple(0, 0.0, 0.5, 0.5));
     launch_make_rhs<R>(d, chunks[0].view(), ctl, 0, stream);
+    coefs(chunks[0].view());
     int cur = 0;
     sweeps_fine(cur, sweeps, stream);
     M1_CK(cudaGetLastError());
@@ -1007,6 +1015,7 @@ m1_status Engine<R>::op_level(double dt, const double* sig, const double* state,
     case M1_OP_PSEUDO:
         M1_TRY(pack_planar(q.u[0], n, state));
         M1_TRY(pack_planar(q.f, n, rhs));
+        if (mode == M1_OP_JACOBI) coefs(chunks[0].view());
         launch_sweep<R>(d, strips[0].view(), ctl, mode == M1_OP_PSEUDO, 0, 1, stream);
         M1_CK(cudaGetLastError());
         M1_TRY(unpack_planar(q.u[1], n, out));
@@ -1172,6 +1181,7 @@ m1_status PlainModel::sv_begin(const std::vector<int>& slots, const std::vector<
     }
     M1_TRY(e.set_init_lists(slots));
     launch_make_rhs<double>(e.d, e.init_chunks.view(), e.ctl, 0, e.stream);
+    e.coefs(e.init_chunks.view());
     launch_apply<double>(e.d, e.init_strips.view(), e.ctl, APPLY_RESID, 0, e.part, 0, e.stream);
     launch_norm_state<double>(e.d, e.init_strips.view(), e.ctl, e.partb, e.stream);
     launch_finalize<double>(e.ctl, e.d, (int)slots.size(), e.part, e.partb, FIN_INIT, 0, e.bctl,

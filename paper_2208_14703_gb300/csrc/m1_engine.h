@@ -137,6 +137,8 @@ struct Engine {
                         const double* sa, const double* ss, int dev);
     m1_status set_inflow(int i, int side, const double* E, const double* Fx, const double* Fy);
     m1_status get_state(int i, double* E, double* Fx, double* Fy, double* T, int dev);
+    // the FP64 fine sweeps' coefficients for the slots of a chunk list (FP32: nothing)
+    void coefs(WorkList wl);
     void sweeps_fine(int& cur, int count, cudaStream_t s);
     void fas_rhs(int l, cudaStream_t s);
     void pseudo(int l, int& cur, int m, bool from_v, cudaStream_t s, bool fas = false);

@@ -75,6 +75,17 @@ __host__ __device__ __forceinline__ float seed_rsqrt(float x)
 #endif
 }
 
+__host__ __device__ __forceinline__ float seed_sqrt(float x)
+{
+#ifdef __CUDA_ARCH__
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+#else
+    return sqrtf(x);
+#endif
+}
+
 // a * b + c of 32-bit a, b and 64-bit c (one instruction)
 __host__ __device__ __forceinline__ i64 madw(int a, int b, i64 c) { return (i64)a * b + c; }
 
@@ -206,6 +217,93 @@ __host__ __device__ __forceinline__ double fx_double(i64 s, int e)
 
 // Arithmetic right shift by n >= 0 (63 and more: the sign).
 __host__ __device__ __forceinline__ i64 fx_sar(i64 x, int n) { return x >> (n < 63 ? n : 63); }
+
+// x rounded toward zero to FP32: values below its normal range give 0, above it
+// (and NaN) infinity.  For seeds, corrections and decisions with a margin.
+__host__ __device__ __forceinline__ float narrow_rz(double x)
+{
+    const u64 b = bits_of_double(x);
+    const unsigned mag = (unsigned)(b >> 32) & 0x7fffffffu;
+    unsigned f = (unsigned)((b & 0x7fffffffffffffffull) >> 29) - (896u << 23);
+    f = mag < (897u << 20) ? 0u : (mag >= (1151u << 20) ? 0x7f800000u : f);
+    return float_of_bits(f | ((unsigned)(b >> 32) & 0x80000000u));
+}
+
+// The significand of a positive normal x at scale 2^61, and its exponent.
+__host__ __device__ __forceinline__ i64 fx_significand(double x, int& e)
+{
+    const u64 b = bits_of_double(x);
+    e = (int)(b >> 52) - 1023;
+    return (i64)(((b & 0xfffffffffffffull) | 0x10000000000000ull) << 9);
+}
+
+// The root T of C T + K T^4 = R (C, K, R > 0) and T^4: Newton in FP32 to about
+// 2e-7, then two corrections whose residuals are formed in fixed point relative
+// to R (both terms are positive and sum to R) and whose quotients are FP32 (each
+// needs only the digits it adds).  With t = T 2^(61 - eT) the powers are
+// t^2 = T2 2^62, T2^2 = T4 2^62.  The residual is good to 2^-55 R, hence T to
+// about 2^-55 and T^4 to 2^-53.  False where FP32 cannot hold or seed the problem.
+__host__ __device__ __forceinline__ bool fx_quartic(double C, double K, double R, double& Tout,
+                                                    double& T4out)
+{
+    const float Cf = narrow_rz(C), Kf = narrow_rz(K), Rf = narrow_rz(R);
+    const float K4 = 4.0f * Kf;
+    float T = fminf(Rf * seed_rcp(Cf), seed_sqrt(seed_sqrt(Rf * seed_rcp(Kf))));
+    bool ok = false;
+    for (int it = 0; it < 40; ++it) {
+        const float T3 = T * T * T;
+        const float g = fmaf(Kf, T3 * T, Cf * T) - Rf;
+        const float dT = g * seed_rcp(fmaf(K4, T3, Cf));
+        T -= dT;
+        // Newton's error is at most 1.5 dT^2 / T here (g'' T <= 3 g')
+        if (fabsf(dT) <= 3e-4f * T) { ok = true; break; }
+    }
+    const unsigned bt = bits_of_float(T);
+    const int eT = (int)(bt >> 23) - 127;                      // sign set: out of range below
+    int eC, eK, eR;
+    const i64 mC = fx_significand(C, eC), mR = fx_significand(R, eR);
+    const Split sC = split62(mC), sK = split62(fx_significand(K, eK));
+    const float dg = fmaf(K4, T * T * T, Cf);
+    // 2^(eR - eT) / g' <= 4; the significand of T away from its upper end, so that
+    // the corrections (below 2^-18 T) keep it under 2^62
+    ok = ok && eT > -60 && eT < 60 && eR > -120 && eR < 120 && eR - eT > -120 && eR - eT < 120 &&
+         dg > 1e-35f && dg < 1e35f && (bt & 0x7fffffu) < 0x7fff00u;
+    const float q = float_of_bits((unsigned)((ok ? eR - eT : 0) + 127) << 23) * seed_rcp(dg);
+    const int nC = eR - eC - eT + 4, nK = eR - eK - 4 * eT + 1;
+    ok = ok && nC >= 0 && nK >= 0;
+    i64 m = (i64)((bt & 0x7fffffu) | 0x800000u) << 38, T4 = 0;
+    float d = 0.0f;
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int pass = 0; pass < 2; ++pass) {
+        const Split sm = split62(m);
+        T4 = sqr62(split62(sqr62(sm)));
+        const i64 g = fx_sar(mul62(sC, sm), nC) + fx_sar(mul62(sK, split62(T4)), nK) - (mR >> 5);
+        if (pass == 0) {                                       // |g| < 2^38, in units 2^(eR - 56)
+            const i64 gs = g >> 8;
+            ok = ok && gs < 0x7fffffffll && gs > -0x7fffffffll;
+            d = (float)(int)gs * q * 2.0f;                     // in units 2^12 of m
+            ok = ok && fabsf(d) < 0x1p30f;
+            m -= (i64)(int)(ok ? d : 0.0f) << 12;
+        } else {
+            ok = ok && g < 0x7fffffffll && g > -0x7fffffffll;
+            d = (float)(int)g * q * 32.0f;
+            ok = ok && fabsf(d) < 0x1p30f;
+            d = ok ? d : 0.0f;
+        }
+    }
+    // T^4 at the corrected root: T4 (1 - 4 d / m), with 4 T4 / m = t^3 / 2, t in [1, 2)
+    const float t = float_of_bits((bt & 0x7fffffu) | 0x3f800000u);
+    T4 -= (i64)(int)(d * t * t * t * 0.5f);
+    m -= (i64)(int)d;
+    T4out = fx_double(T4, ok ? 4 * eT : 0);
+    // m in [2^60, 2^62) at exponent eT
+    const int z = m < (1ll << 61) ? 1 : 0;
+    const u64 r = ((u64)(m << z) >> 9) + (((u64)(m << z) >> 8) & 1);
+    Tout = double_of_bits(r + ((u64)(1022 + (ok ? eT : 0) - z) << 52));
+    return ok;
+}
 
 // What a cell adds to its neighbour's sums across one face (Eq. (9) with F over
 // c and a common factor c dt / (2 h) taken out): E +- F_d, F_x +- P_xd, F_y +- P_yd.

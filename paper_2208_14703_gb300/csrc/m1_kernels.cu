@@ -379,24 +379,30 @@ __device__ __forceinline__ double strip_sweep64(const Level<double>& L, Ctl* ctl
     struct Pre {
         Cell4<double> b, u;
         Sig2<double> sg;
+        Coef q;
     };
     double nrm = 0.0;
     unsigned fails = 0;
     if (L.fx) {
         const Pseudo<double> ps = PSEUDO ? pseudo_of<double>(ctl) : Pseudo<double>{};
         const double cbE = PSEUDO ? ps.dtau * L.cb : L.cb, cbF = PSEUDO ? ps.dtau * L.cbF : L.cbF;
+        // the pseudo-time step's A and C, and the FP32 values of its admissibility check
+        const double Ap = PSEUDO ? fma(ps.dtau, L.diag, 1.0) : 0.0;
+        const double Cp = PSEUDO ? fma(ps.dtau, L.c_v, 1.0) : 0.0;
+        const float s32 = (float)ps.s, c32 = (float)L.c;
         auto pre = [&](size_t k) {
             Pre p;
             p.b = FAS ? L.r[k] : L.f[k];
-            p.sg = L.sig[k];
-            if (PSEUDO || NORM) p.u = src[k];
+            if (PSEUDO || NORM) { p.sg = L.sig[k]; p.u = src[k]; }
+            if (!PSEUDO) p.q = reinterpret_cast<const Coef*>(L.v)[k];
             return p;
         };
         const bool regular = strip_march_fx(L, it, lane, src, pre, [&](size_t k, const Pre& p,
                                                                        const FxFlux& s) {
             const double NE = fx_double(s.E, s.e), NFx = fx_double(s.Fx, s.e),
                          NFy = fx_double(s.Fy, s.e);
-            const double ka = L.cdt * p.sg.sa, kt = L.cdt * (p.sg.sa + p.sg.ss);
+            double ka = 0.0, kt = 0.0;
+            if (PSEUDO || NORM) { ka = L.cdt * p.sg.sa; kt = L.cdt * (p.sg.sa + p.sg.ss); }
             Cell4<double> b = p.b;
             bool ok;
             Cell4<double> o;
@@ -420,11 +426,13 @@ __device__ __forceinline__ double strip_sweep64(const Level<double>& L, Ctl* ctl
                 }
             }
             if (!PSEUDO) {
-                o = local_solve64(0.0, 1.0, L.diag, ka, kt, L.c_v, L.a_r, fma(cbE, NE, b.E),
-                                  fma(cbF, NFx, b.Fx), fma(cbF, NFy, b.Fy), b.T, ok);
+                o = local_solve64(p.q, L.diag, L.c_v, L.a_r, fma(cbE, NE, b.E), fma(cbF, NFx, b.Fx),
+                                  fma(cbF, NFy, b.Fy), b.T, ok);
             } else {
-                const double tau = limited_step(p.u, b, ps.dtau, ps.theta, ps.s, L.c);
-                o = local_solve64(1.0, ps.dtau, L.diag, ka, kt, L.c_v, L.a_r,
+                const double tau = surely_admissible(p.u, b, s32, c32)
+                                       ? ps.dtau
+                                       : limited_step(p.u, b, ps.dtau, ps.theta, ps.s, L.c);
+                o = local_solve64(make_coef(1.0, ps.dtau, L.diag, ka, kt, L.a_r), Ap, Cp, L.a_r,
                                   fma(cbE, NE, fma(tau, b.E, p.u.E)),
                                   fma(cbF, NFx, fma(tau, b.Fx, p.u.Fx)),
                                   fma(cbF, NFy, fma(tau, b.Fy, p.u.Fy)), fma(tau, b.T, p.u.T), ok);
@@ -438,6 +446,33 @@ __device__ __forceinline__ double strip_sweep64(const Level<double>& L, Ctl* ctl
         }
     }
     return strip_general64<PSEUDO, NORM, FAS>(L, ctl, it, lane, src, out_buf);
+}
+
+// The local solve's coefficients of the fine Jacobi sweeps, formed once per step
+// (they depend on the opacities and dt): kept in the fine level's array v, which
+// no FP64 hierarchy uses there.
+__global__ void __launch_bounds__(kThreads) k_coef64(const Level<double>* __restrict__ lv, WorkList wl)
+{
+    __shared__ Level<double> L;
+    const int w0 = blockIdx.x, ws = gridDim.x;
+    int2 nx = item_at(wl, w0);
+    const int nw = *wl.count;
+    int inst = -1;
+    for (int w = w0; w < nw; w += ws, nx = item_at(wl, w)) {
+        const int2 it = nx;
+        if (it.x != inst) {
+            __syncthreads();
+            load_level(L, lv + it.x);
+            __syncthreads();
+            inst = it.x;
+        }
+        const int k = it.y * kThreads + threadIdx.x;
+        if (k < L.n) {
+            const Sig2<double> g = L.sig[k];
+            reinterpret_cast<Coef*>(L.v)[k] =
+                make_coef(0.0, 1.0, L.diag, L.cdt * g.sa, L.cdt * (g.sa + g.ss), L.a_r);
+        }
+    }
 }
 
 // Persistent FP64 sweep (the item loop of k_sweep), held to 128 registers (8 blocks
@@ -1811,6 +1846,11 @@ void launch_apply(const Level<R>* lv, WorkList wl, Ctl* ctls, int mode, int stat
         k_apply<R, APPLY_FAS><<<g, kThreads, 0, s>>>(lv, wl, ctls, state_buf, partials, write_r);
     else
         k_apply<R, APPLY_A><<<g, kThreads, 0, s>>>(lv, wl, ctls, state_buf, partials, write_r);
+}
+
+void launch_coef64(const Level<double>* lv, WorkList wl, cudaStream_t s)
+{
+    k_coef64<<<pgrid(wl), kThreads, 0, s>>>(lv, wl);
 }
 
 void launch_fas_aw32(const Level<float>* lv, WorkList wl, Ctl* ctls, cudaStream_t s)

@@ -50,6 +50,10 @@ template <typename R>
 void launch_check_state(const Cell4<R>* st, const Sig2<R>* sig, int n, double c, unsigned int* bad,
                         cudaStream_t s);
 
+// The local solve's coefficients of the fine FP64 Jacobi sweeps (into level 0's v),
+// before the first of them for a new dt or new opacities.
+void launch_coef64(const Level<double>* lv, WorkList wl, cudaStream_t s);
+
 // FP32 correction form, coarse level: A(w) -> aw and f = [A(w + v) - A(w)] + r.
 void launch_fas_aw32(const Level<float>* lv, WorkList wl, Ctl* ctls, cudaStream_t s);
 // The FP64 defect and the next FP32 cycle's problem (w = fl32(v), g = fl32(r));

@@ -5,7 +5,9 @@
 // What bounds them: the FP64 pipe (64 clocks a warp instruction and SM partition).
 // A fine Jacobi update in FP64 alone issues 109 of them; here the closure (about 27,
 // evaluated 1.2 times a cell) and the neighbour sums (26) take none, and the local
-// solve 31 instead of 42.
+// solve seven instead of 42: its coefficients depend on the opacities and the time
+// step alone (kept per cell over a step on the fine level), and its quartic is
+// solved in fixed point.
 #pragma once
 #include "m1_fx.cuh"
 
@@ -138,96 +140,72 @@ __device__ __forceinline__ bool strip_march_fx(const Level<double>& L, int2 it, 
     return __all_sync(0xffffffffu, ok);
 }
 
-// x rounded toward zero to FP32: values below its normal range give 0, above it
-// (and NaN) infinity.  For corrections that need a few digits.
-__device__ __forceinline__ float narrow_rz(double x, int eshift = 0)
+// The coefficients of one cell's local solve D^{-1} (local_solve in m1_device.cuh):
+// with A = w0 + w1 diag and k = w1 ka, 1 / (w0 + w1 (diag + kt)), k / (A + k),
+// 1 / (A + k) and K = a_r A k / (A + k).  (w0, w1) as there: (0, 1) for a Jacobi
+// sweep, (1, dtau) for a pseudo-time step.
+struct Coef {
+    double iF, kk, iAk, K;
+};
+
+__device__ __forceinline__ Coef make_coef(double w0, double w1, double diag, double ka, double kt,
+                                          double a_r)
 {
-    const int hi = __double2hiint(x);
-    const int mag = (hi & 0x7fffffff) - (eshift << 20);        // x 2^-eshift
-    unsigned f = __funnelshift_l((unsigned)__double2loint(x), (unsigned)mag, 3) - (896u << 23);
-    f = mag < (897 << 20) ? 0u : (mag >= (1151 << 20) ? 0x7f800000u : f);
-    return __uint_as_float(f | ((unsigned)hi & 0x80000000u));
+    const double A = fma(w1, diag, w0), k = w1 * ka;
+    const double dF = fma(w1, diag + kt, w0), dE = A + k;
+    // one reciprocal serves both denominators: 1/a = b / (a b), 1/b = a / (a b)
+    const double ip = Fm<double>::rcp(dF * dE);
+    const double iAk = dF * ip, kk = k * iAk;
+    return Coef{ dE * ip, kk, iAk, A * (a_r * kk) };
 }
 
-// (double)x for a normal FP32 x; zero gives a number below 2^-126.
-__device__ __forceinline__ double widen_normal(float x)
-{
-    const unsigned u = __float_as_uint(x);
-    return __hiloint2double((int)((((u & 0x7fffffffu) >> 3) + (896u << 20)) | (u & 0x80000000u)),
-                            (int)(u << 29));
-}
-
-// The root of C T + K T^4 = R in FP64: Newton in FP32 to about 2e-7, then two
-// Newton corrections whose residuals are formed in FP64 and whose quotients in
-// FP32 (each correction needs only the digits it adds: the first leaves an error
-// near 1e-13, the second FP64 rounding).  Ten FP64 operations; a Halley step with
-// an FP64 quotient took 17.  Where FP32 cannot seed the root, Quartic<double>
-// takes the cell.
-__device__ __forceinline__ double quartic64(double C, double K, double R, bool& ok)
-{
-    const float Cf = narrow_rz(C), Kf = narrow_rz(K), Rf = narrow_rz(R);
-    const float K4 = 4.0f * Kf;
-    float T = fminf(Rf * seed_rcp(Cf), Fm<float>::sqrt(Fm<float>::sqrt(Rf * seed_rcp(Kf))));
-    bool conv = false;
-    for (int it = 0; it < 40; ++it) {
-        const float T3 = T * T * T;
-        const float g = fmaf(Kf, T3 * T, Cf * T) - Rf;
-        const float dT = g * seed_rcp(fmaf(K4, T3, Cf));
-        T -= dT;
-        // Newton's error is at most 1.5 dT^2 / T here (g'' T <= 3 g')
-        if (fabsf(dT) <= 3e-4f * T) { conv = true; break; }
-    }
-    const int eR = (int)((__float_as_uint(Rf) >> 23) & 0xffu) - 127;
-    // 1 / g' in units of 1 / R: at most about 2 T, so the quotients below stay in range
-    const float q = seed_rcp(fmaf(K4, T * T * T, Cf)) * __uint_as_float((unsigned)(eR + 127) << 23);
-    if (conv && T > 1e-18f && T < 1e18f && q > 1e-18f * T && eR > -126) {
-        double Td = widen_normal(T);
-        double T2 = Td * Td, KT2 = K * T2;
-        const float d1 = narrow_rz(fma(KT2, T2, fma(C, Td, -R)), eR) * q;
-        Td -= widen_normal(d1);
-        T2 = Td * Td;
-        KT2 = K * T2;
-        const float d2 = narrow_rz(fma(KT2, T2, fma(C, Td, -R)), eR) * q;
-        if (fabsf(d1) <= 1e-5f * T && fabsf(d2) <= 1e-9f * T) {
-            ok = true;
-            return Td - widen_normal(d2);
-        }
-    }
-    return Quartic<double>::solve(C, K, R, ok);
-}
-
-// local_solve in FP64 for the strips: quartic64, and without absorption the
-// quotients by one shared reciprocal (each followed by its remainder's
-// correction) instead of FP64 divisions.
-__device__ __forceinline__ Cell4<double> local_solve64(double w0, double w1, double diag, double ka,
-                                                       double kt, double c_v, double a_r, double bE,
-                                                       double bFx, double bFy, double bT, bool& ok)
+// The local solve with its coefficients given: seven FP64 operations, the quartic
+// in fixed point (fx_quartic) or, where that cannot hold it, by Quartic<double>.
+// A is used without absorption only: E = bE / A with the quotient's remainder added.
+__device__ __forceinline__ Cell4<double> local_solve64(const Coef& q, double A, double C, double a_r,
+                                                       double bE, double bFx, double bFy, double bT,
+                                                       bool& ok)
 {
     Cell4<double> o;
-    const double A = fma(w1, diag, w0), k = w1 * ka, C = fma(w1, c_v, w0);
-    const double dF = fma(w1, diag + kt, w0);
     ok = true;
-    if (is_zero_f64(k)) {
-        const double ip = Fm<double>::rcp(dF * A), iF = A * ip, iA = dF * ip;
-        o.Fx = bFx * iF;
-        o.Fy = bFy * iF;
-        const double q = bE * iA;
-        o.E = fma(fma(-A, q, bE), iA, q);
+    o.Fx = bFx * q.iF;
+    o.Fy = bFy * q.iF;
+    if (is_zero_f64(q.kk)) {
+        const double e = bE * q.iAk;
+        o.E = fma(fma(-A, e, bE), q.iAk, e);
         o.T = bT;
         if (C != 1.0) o.T = bT / C;
         return o;
     }
-    const double dE = A + k;
-    const double ip = Fm<double>::rcp(dF * dE);
-    const double iF = dE * ip, iAk = dF * ip;
-    o.Fx = bFx * iF;
-    o.Fy = bFy * iF;
-    const double ark = a_r * (k * iAk);
-    const double T = quartic64(C, A * ark, fma(k * iAk, bE, bT), ok);
-    const double T2 = T * T;
-    o.T = T;
-    o.E = fma(ark, T2 * T2, bE * iAk);
+    const double R = fma(q.kk, bE, bT);
+    double T4;
+    if (!fx_quartic(C, q.K, R, o.T, T4)) {
+        o.T = Quartic<double>::solve(C, q.K, R, ok);
+        const double T2 = o.T * o.T;
+        T4 = T2 * T2;
+    }
+    double ark = q.kk;
+    if (a_r != 1.0) ark *= a_r;
+    o.E = fma(ark, T4, bE * q.iAk);
     return o;
+}
+
+// Whether u + s f is admissible beyond doubt in FP32 (values rounded toward zero, a
+// margin of 1e-6 of the terms' sizes where the roundings leave at most 5e-7): the
+// explicit pseudo-time step is then not limited.  c, s in FP32.
+__device__ __forceinline__ bool surely_admissible(const Cell4<double>& u, const Cell4<double>& f,
+                                                  float s, float c)
+{
+    const float m = 1e-6f;
+    const float uE = narrow_rz(u.E), fE = s * narrow_rz(f.E);
+    const float uT = narrow_rz(u.T), fT = s * narrow_rz(f.T);
+    const float ux = narrow_rz(u.Fx), fx = s * narrow_rz(f.Fx);
+    const float uy = narrow_rz(u.Fy), fy = s * narrow_rz(f.Fy);
+    const float pE = c * ((uE + fE) - m * (uE + fabsf(fE)));
+    const float px = fabsf(ux + fx) + m * (fabsf(ux) + fabsf(fx));
+    const float py = fabsf(uy + fy) + m * (fabsf(uy) + fabsf(fy));
+    return uT + fT > m * (uT + fabsf(fT)) && uE > 1e-30f && uT > 1e-30f && pE > 1e-15f * c &&
+           fmaf(px, px, py * py) <= 0.99999f * pE * pE;
 }
 
 }  // namespace m1

@@ -107,6 +107,7 @@ m1_status time_level(int n, bool delta, cudaStream_t stream, std::vector<double>
         e.h[0].ring = ring;
         M1_TRY(e.rebuild());
         int cur = 0;
+        e.coefs(e.chunks[0].view());
         e.sweeps_fine(cur, 2, e.stream);              // warm-up
         M1_CK(cudaEventRecord(e.ev0, e.stream));
         e.sweeps_fine(cur, reps, e.stream);
