@@ -15,6 +15,7 @@
 #include <type_traits>
 
 #include "m1_engine.h"
+#include "m1_tail.h"
 
 namespace m1 {
 
@@ -151,6 +152,8 @@ std::vector<DevList*> Engine<R>::all_lists()
     std::vector<DevList*> v;
     for (auto& l : chunks) v.push_back(&l);
     for (auto& l : strips) v.push_back(&l);
+    for (auto& l : tails) v.push_back(&l);
+    v.push_back(&tail_all);
     v.push_back(&init_strips);
     v.push_back(&init_chunks);
     return v;
@@ -189,6 +192,9 @@ m1_status Engine<R>::init(int capacity, int levels, bool correction_form, cudaSt
     last_cycles.assign(cap, 0);
     chunks.assign(L, DevList{});
     strips.assign(L, DevList{});
+    tails.assign(L, DevList{});
+    tail_first.assign(cap, L);
+    if (sizeof(R) == 8) M1_CK(tail_prepare());
     M1_TRY(calloc_common((void**)&d, sizeof(Level<R>) * L * cap));
     M1_TRY(calloc_common((void**)&ctl, sizeof(Ctl) * cap));
     M1_TRY(calloc_common((void**)&bctl, sizeof(BatchCtl)));
@@ -282,6 +288,17 @@ m1_status Engine<R>::add_slot(const m1_grid_desc& dsc, int* out)
         }
         nx /= 2; if (g.dim == 2) ny /= 2;
         hx *= 2; if (g.dim == 2) hy *= 2;
+    }
+    // the tail: from the first coarse level that is small enough and whose levels
+    // fit a block's shared memory (a rule on the instance alone, so that its result
+    // does not depend on the batch)
+    tail_first[i] = L;
+    for (int l = L - 1; l >= 1 && sizeof(R) == 8; --l) {
+        const int n = h[(size_t)l * cap + i].n;
+        if (L - l > kTailLevels || n > kTailCells ||
+            tail_smem(n, kTailBlocks, g.dim, L - l) > (size_t)kTailSmem)
+            break;
+        tail_first[i] = l;
     }
     used[i] = 1;
     dt_set[i] = NAN;
@@ -392,18 +409,38 @@ m1_status Engine<R>::rebuild()
         for (int i = 0; i < cap; ++i) {
             if (!used[i]) continue;
             const Level<R>& q = h[(size_t)l * cap + i];
-            for (int t = 0; t < q.strips; ++t) strips[l].host.push_back(make_int2(i, t));
-            for (int c = 0; c < q.chunks; ++c) chunks[l].host.push_back(make_int2(i, c));
+            // the tail's levels have no launches of their own but the transfers to and
+            // from its first one
+            if (l < tail_first[i])
+                for (int t = 0; t < q.strips; ++t) strips[l].host.push_back(make_int2(i, t));
+            if (l <= tail_first[i])
+                for (int c = 0; c < q.chunks; ++c) chunks[l].host.push_back(make_int2(i, c));
         }
         M1_TRY(upload_list(strips[l]));
         M1_TRY(upload_list(chunks[l]));
     }
+    tail_all.host.clear();
+    size_t bytes = 0;
+    for (int l = 0; l < L; ++l) {
+        tails[l].host.clear();
+        for (int i = 0; i < cap; ++i)
+            if (used[i] && tail_first[i] == l) {
+                tails[l].host.push_back(make_int2(i, l));
+                tail_all.host.push_back(make_int2(i, l));
+                bytes = std::max(bytes, tail_smem(h[(size_t)l * cap + i].n, kTailBlocks,
+                                                  desc[i].dim, L - l));
+            }
+        M1_TRY(upload_list(tails[l]));
+    }
+    M1_TRY(upload_list(tail_all));
+    if (bytes != tail_bytes) { tail_bytes = bytes; graph_dirty = true; }
     // a captured cycle launches nothing for an empty list: re-capture when a
     // list becomes empty or stops being empty
     std::vector<char> sig;
     for (int l = 0; l < L; ++l) {
         sig.push_back(strips[l].n > 0);
         sig.push_back(chunks[l].n > 0);
+        sig.push_back(tails[l].n > 0);
     }
     if (sig != list_sig) { list_sig = sig; graph_dirty = true; }
     // the sweeps of a level share one launch for all slots: the cp.async kernel
@@ -650,6 +687,11 @@ void Engine<R>::fas_rhs(int l, cudaStream_t s)
 template <typename R>
 void Engine<R>::corrections(const Params& p, int l, int shape, std::vector<int>& cur, cudaStream_t s)
 {
+    // the instances whose tail begins at level l + 1 take all of it in one launch; in a
+    // V-cycle one launch at the bottom serves the tails of every level
+    if (p.cycle != M1_CYCLE_V) tail(tails[l + 1], shape, s);
+    else if (strips[l + 1].n == 0 || l + 1 == L - 1) tail(tail_all, shape, s);
+    if (strips[l + 1].n == 0) return;
     if (l + 1 == L - 1 || shape == M1_CYCLE_V) {
         visit(p, l + 1, true, shape, cur, s);
     } else if (shape == M1_CYCLE_W) {
@@ -659,6 +701,89 @@ void Engine<R>::corrections(const Params& p, int l, int shape, std::vector<int>&
         visit(p, l + 1, true, M1_CYCLE_F, cur, s);
         visit(p, l + 1, false, M1_CYCLE_V, cur, s);
     }
+}
+
+template <typename R>
+void Engine<R>::tail(const DevList& list, int shape, cudaStream_t s)
+{
+    if constexpr (std::is_same<R, double>::value) {
+        if (list.n)
+            launch_tail(d, cap, L, list.view(), ctl, prog, progs + (size_t)shape * L, tail_bytes, s);
+    }
+}
+
+namespace {
+
+// The operations of the coarse-grid corrections of level l, as the tail of an
+// instance walks them (levels counted from `first`): the recursion of
+// Engine::corrections and Engine::visit.
+void program(const Params& p, int L, int first, int l, int shape, std::vector<unsigned char>& out)
+{
+    auto put = [&](int op, int level) { out.push_back((unsigned char)(op + 8 * (level - first))); };
+    auto visit = [&](int v, bool fresh, int sh) {
+        const int steps = v == L - 1 ? p.mc : p.m;
+        for (int k = 0; k < steps; ++k) put(k == 0 && fresh ? TAIL_FIRST : TAIL_PSEUDO, v);
+        if (v == L - 1) return;
+        put(TAIL_RESID, v);
+        put(TAIL_RESTRICT, v + 1);
+        program(p, L, first, v, sh, out);
+        put(TAIL_PROLONG, v);
+        for (int k = 0; k < p.m; ++k) put(TAIL_PSEUDO, v);
+    };
+    if (l + 1 == L - 1 || shape == M1_CYCLE_V) {
+        visit(l + 1, true, shape);
+    } else if (shape == M1_CYCLE_W) {
+        visit(l + 1, true, M1_CYCLE_W);
+        visit(l + 1, false, M1_CYCLE_W);
+    } else {
+        visit(l + 1, true, M1_CYCLE_F);
+        visit(l + 1, false, M1_CYCLE_V);
+    }
+}
+
+// Kernel nodes of a graph.
+long long graph_nodes(cudaGraph_t g)
+{
+    size_t n = 0;
+    return cudaGraphGetNodes(g, nullptr, &n) == cudaSuccess ? (long long)n : 0;
+}
+
+}  // namespace
+
+// The tails' programs for the parameters, on the device: a shape's for every first
+// level in use.  Before a capture (the graph holds their addresses).
+template <typename R>
+m1_status Engine<R>::write_programs(const Params& p)
+{
+    if (prog && pparams == p && !graph_dirty) return M1_OK;
+    std::vector<unsigned char> ops;
+    std::vector<int2> at((size_t)3 * L, make_int2(0, 0));
+    for (int shape = 0; shape < 3; ++shape)
+        for (int f = 1; f < L; ++f) {
+            // shapes a cycle reaches: its own, and V below an F-cycle
+            const bool reached = shape == p.cycle || (p.cycle == M1_CYCLE_F && shape == M1_CYCLE_V);
+            if (!reached || tails[f].n == 0) continue;
+            const int off = (int)ops.size();
+            program(p, L, f, f - 1, shape, ops);
+            at[(size_t)shape * L + f] = make_int2(off, (int)ops.size() - off);
+        }
+    M1_CK(cudaStreamSynchronize(stream));
+    auto drop = [this](void* q) {
+        if (!q) return;
+        cudaFree(q);
+        common.erase(std::find(common.begin(), common.end(), q));
+    };
+    drop(prog);
+    drop(progs);
+    prog = nullptr;
+    progs = nullptr;
+    M1_TRY(calloc_common((void**)&prog, ops.size()));
+    M1_TRY(calloc_common((void**)&progs, sizeof(int2) * at.size()));
+    if (!ops.empty()) M1_CK(cudaMemcpyAsync(prog, ops.data(), ops.size(), cudaMemcpyHostToDevice, stream));
+    M1_CK(cudaMemcpyAsync(progs, at.data(), sizeof(int2) * at.size(), cudaMemcpyHostToDevice, stream));
+    M1_CK(cudaStreamSynchronize(stream));
+    pparams = p;
+    return M1_OK;
 }
 
 // One visit of coarse level l >= 1: FAS right-hand side (Eq. (24)) when fresh,
@@ -729,48 +854,12 @@ void Engine<R>::record_cycle(const Params& p, int& cur0, cudaStream_t s, bool ta
     cur0 = cur[0];
 }
 
-namespace {
-
-// Fresh and repeated visits of each level in one cycle of the given shape.
-void count_visits(int L, int l, bool fresh, int shape, std::vector<long long>& fr,
-                  std::vector<long long>& rep)
-{
-    (fresh ? fr : rep)[l] += 1;
-    if (l == L - 1) return;
-    if (l + 1 == L - 1 || shape == M1_CYCLE_V) {
-        count_visits(L, l + 1, true, shape, fr, rep);
-    } else if (shape == M1_CYCLE_W) {
-        count_visits(L, l + 1, true, M1_CYCLE_W, fr, rep);
-        count_visits(L, l + 1, false, M1_CYCLE_W, fr, rep);
-    } else {
-        count_visits(L, l + 1, true, M1_CYCLE_F, fr, rep);
-        count_visits(L, l + 1, false, M1_CYCLE_V, fr, rep);
-    }
-}
-
-}  // namespace
-
-template <typename R>
-long long Engine<R>::kernels_per_cycle(const Params& p) const
-{
-    if (L == 1) return p.nu0;
-    // a fresh visit's FAS right-hand side: fused into the first pseudo-time step
-    // in the plain form, its own kernel in the correction form
-    const int aw = delta ? 1 : 0;
-    std::vector<long long> fr(L, 0), rep(L, 0);
-    count_visits(L, 0, true, p.cycle, fr, rep);
-    long long k = 2 * p.nu0 + 3;                       // fine smoothing, residual, restrict, prolong
-    for (int l = 1; l < L - 1; ++l)                    // pseudo x 2, residual, restrict, prolong
-        k += fr[l] * (aw + 2 * p.m + 3) + rep[l] * (2 * p.m + 3);
-    k += fr[L - 1] * (aw + p.mc);                      // coarsest
-    return k;
-}
-
 template <typename R>
 m1_status Engine<R>::build_graph(const Params& p)
 {
     if (graph && gparams == p && !graph_dirty) return M1_OK;
     if (graph) { cudaGraphExecDestroy(graph); graph = nullptr; }
+    M1_TRY(write_programs(p));
     // a captured graph must return the fine iterate to buffer 0
     const int per_cycle = L == 1 ? p.nu0 : 2 * p.nu0;
     graph_cycles = (per_cycle % 2) ? 2 : 1;
@@ -781,6 +870,7 @@ m1_status Engine<R>::build_graph(const Params& p)
     cudaError_t e = cudaStreamEndCapture(cap_stream, &g);
     if (e != cudaSuccess) { set_err(e, "cudaStreamEndCapture"); return M1_ERR_CUDA; }
     if (cur0 != 0) { cudaGraphDestroy(g); return M1_ERR_INVALID_ARG; }
+    kernels_per_launch = graph_nodes(g);
     e = cudaGraphInstantiate(&graph, g, 0);
     cudaGraphDestroy(g);
     if (e != cudaSuccess) { set_err(e, "cudaGraphInstantiate"); graph = nullptr; return M1_ERR_CUDA; }
@@ -861,7 +951,7 @@ m1_status Engine<R>::step(const double* dts, const m1_solve_params& sp, m1_step_
             s.status = c.status;
             s.newton_fail = c.newton_fail;
             s.damped = c.damped;
-            s.launches = 5 + launched * (kernels_per_cycle(p) + 1);   // + deferred finalize
+            s.launches = 5 + launched / graph_cycles * kernels_per_launch;
         }
         ++k;
     }
@@ -1355,11 +1445,13 @@ m1_status MixedModel::build_graph(const Params& p)
 {
     if (graph && gparams == p && !hi.graph_dirty && !lo.graph_dirty) return M1_OK;
     if (graph) { cudaGraphExecDestroy(graph); graph = nullptr; }
+    M1_TRY(lo.write_programs(p));
     cudaGraph_t g = nullptr;
     M1_CK(cudaStreamBeginCapture(lo.cap_stream, cudaStreamCaptureModeThreadLocal));
     record_cycle(p, lo.cap_stream);
     cudaError_t e = cudaStreamEndCapture(lo.cap_stream, &g);
     if (e != cudaSuccess) { set_err(e, "cudaStreamEndCapture"); return M1_ERR_CUDA; }
+    kernels_per_launch = graph_nodes(g);
     e = cudaGraphInstantiate(&graph, g, 0);
     cudaGraphDestroy(g);
     if (e != cudaSuccess) { set_err(e, "cudaGraphInstantiate"); graph = nullptr; return M1_ERR_CUDA; }
@@ -1414,8 +1506,7 @@ m1_status MixedModel::step(const double* dts, const m1_solve_params& sp, m1_step
             o.status = c.status;
             o.newton_fail = c.newton_fail;
             o.damped = c.damped;
-            // accumulate, defects, finalize; the first fine sweep is the defects'
-            o.launches = 4 + launched * (lo.kernels_per_cycle(p) + 4 - (p.nu0 > 0 ? 1 : 0));
+            o.launches = 5 + launched * kernels_per_launch;
         }
         ++k;
     }

@@ -109,6 +109,16 @@ struct Engine {
     Params gparams{};
     int graph_cycles = 1;
     bool graph_dirty = true;
+    // the coarse end in one launch per cycle (m1_tail.h): each slot's first tail
+    // level (L: none), the lists of (slot, first level) by first level and of all
+    // slots, the programs by cycle shape and first level, the largest slot's memory
+    std::vector<int> tail_first;
+    std::vector<DevList> tails;
+    DevList tail_all;
+    unsigned char* prog = nullptr;
+    int2* progs = nullptr;                  // [shape][first level]: (offset, length) in prog
+    Params pparams{};                       // the parameters the programs were written for
+    size_t tail_bytes = 0;
     std::vector<char> ring;                 // per level: the sweeps take the cp.async kernel
     std::vector<char> list_sig;             // which work lists were non-empty at capture
     // double-word copies of each slot's level-0 iterate, right-hand side and
@@ -148,7 +158,9 @@ struct Engine {
                       bool first_done = false);
     void visit(const Params& p, int l, bool fresh, int shape, std::vector<int>& cur, cudaStream_t s);
     void corrections(const Params& p, int l, int shape, std::vector<int>& cur, cudaStream_t s);
-    long long kernels_per_cycle(const Params& p) const;
+    void tail(const DevList& list, int shape, cudaStream_t s);
+    m1_status write_programs(const Params& p);
+    long long kernels_per_launch = 0;       // kernel nodes of the captured graph
     m1_status build_graph(const Params& p);
     m1_status begin_step(const double* dts, const m1_solve_params& sp);
     m1_status step(const double* dts, const m1_solve_params& sp, m1_step_stats* st);
@@ -256,6 +268,7 @@ struct MixedModel : Model {
     Engine<float> lo;    // FP32 hierarchy in correction form
     cudaGraphExec_t graph = nullptr;
     Params gparams{};
+    long long kernels_per_launch = 0;
     ~MixedModel() override;
     m1_status create(const std::vector<m1_grid_desc>& descs, cudaStream_t s);
     m1_status set_state(int i, const double* E, const double* Fx, const double* Fy, const double* T,

@@ -1,0 +1,428 @@
+// The coarse end of a cycle in one launch.
+//
+// The FP64 levels of a few thousand cells and fewer take as long as their launches:
+// a cycle runs about ten dependent kernels on each, 5 to 9 us apiece whatever their
+// size (launch, work list, descriptor, rows from L2, one pass, drain), with the chip
+// idle.  Here a cluster of thread blocks holds all levels of one instance from the
+// first of at most kTailCells cells down in its shared memory, one thread per cell,
+// and walks the whole sequence of coarse visits (Algorithm 4, V, W or F) with a
+// cluster barrier (0.2 us) between operations.
+//
+// The FP32 levels of the mixed path keep their launches: their roundings would
+// change, and small mixed problems carry FP32 roundings into the ninth digit.
+//
+// Layout: a level's cells are split into equal ranges of consecutive cells, one
+// range per block (small levels: fewer blocks).  What a cell's neighbours need,
+// its iterate and closure, is stored by the thread that forms the iterate, so
+// each closure is evaluated once; neighbours in another block's range are read
+// through distributed shared memory.
+#include <cooperative_groups.h>
+
+#include "m1_cell.cuh"
+#include "m1_strip64.cuh"
+#include "m1_tail.h"
+
+namespace cg = cooperative_groups;
+
+namespace m1 {
+
+namespace {
+
+constexpr int kTailThreads = 512;
+
+// One level in the cluster's shared memory: `blocks` ranges of `per` cells, the
+// arrays of a range at byte offset `off` of its block, one after another.
+struct TailGeo {
+    int nx, n, per, blocks, off;
+    unsigned mx, mper;             // ceil(2^32 / nx), ceil(2^32 / per): k / nx = k mx >> 32 for k < 2^16
+};
+
+__device__ __forceinline__ int row_of(const TailGeo& g, int k)
+{
+    return g.mx ? (int)__umulhi((unsigned)k, g.mx) : k;
+}
+
+// Arrays of a range of `per` cells: the iterates e0, e1, v and f (which first holds
+// the restricted residual), 32 bytes a cell each; the blocks of e0 (first of v) and
+// e1, 56 each; sigma.
+enum { ARR_E = 0, ARR_V = 2, ARR_F = 3, ARR_P = 4 };
+constexpr int kTailBytes = 4 * 32 + 2 * 56 + 16;
+
+__device__ __forceinline__ int arr_at(int a, int per)
+{
+    return a < 4 ? a * 32 * per : 4 * 32 * per + (a - 4) * 56 * per;
+}
+
+// A cell's block that could not be formed (m1_fx.cuh: not regular): its
+// neighbours and itself take the FP64 form.
+constexpr int kIrregular = 1 << 20;
+
+struct Tail {
+    const Level<double>* L;             // descriptors, [0] = the tail's first level
+    const TailGeo* geo;
+    unsigned char* smem;           // this block's arrays
+    int rank;
+    cg::cluster_group cl;
+
+    // cell k of array a of level l, wherever it lies
+    template <typename T>
+    __device__ const T* at(int l, int a, int k) const
+    {
+        const TailGeo& g = geo[l];
+        const int b = (int)__umulhi((unsigned)k, g.mper);
+        const T* p = reinterpret_cast<const T*>(smem + g.off + arr_at(a, g.per)) +
+                     (k - b * g.per);
+        return b == rank ? p : cl.map_shared_rank(p, b);
+    }
+    // this block's own cell q of its range
+    template <typename T>
+    __device__ T* own(int l, int a, int q) const
+    {
+        const TailGeo& g = geo[l];
+        return reinterpret_cast<T*>(smem + g.off + arr_at(a, g.per)) + q;
+    }
+    __device__ Sig2<double>* sig(int l, int q) const
+    {
+        const TailGeo& g = geo[l];
+        return reinterpret_cast<Sig2<double>*>(smem + g.off + arr_at(6, g.per)) + q;
+    }
+    // a cell of array a with the wall rules of fetch()
+    __device__ Cell4<double> fetch(int l, int a, int i, int j, int kind) const
+    {
+        const Ghost g = ghost_map(L[l], i, j);
+        return ghost_apply(L[l], *at<Cell4<double>>(l, a, (int)g.k), g, kind);
+    }
+};
+
+// The four faces of a cell: the neighbour's index and the wall rule there (-1:
+// inside or periodic).
+struct Faces {
+    int k[4], rule[4];
+};
+
+__device__ __forceinline__ Faces faces_of(const Level<double>& L, int k, int i, int j, bool two_d)
+{
+    Faces f;
+    auto face = [&](int w, bool inside, int kin, int kwrap) {
+        f.rule[w] = -1;
+        f.k[w] = kin;
+        if (!inside) {
+            const int bc = L.bc[w];
+            f.k[w] = bc == BC_PERIODIC ? kwrap : k;
+            if (bc != BC_PERIODIC) f.rule[w] = bc;
+        }
+    };
+    face(WALL_W, i > 0, k - 1, k + L.nx - 1);
+    face(WALL_E, i + 1 < L.nx, k + 1, k - L.nx + 1);
+    if (two_d) {
+        face(WALL_S, j > 0, k - L.nx, k + L.n - L.nx);
+        face(WALL_N, j + 1 < L.ny, k + L.nx, k - L.n + L.nx);
+    }
+    return f;
+}
+
+__device__ __forceinline__ void put_block(const Tail& t, int l, int buf, int q,
+                                          const Cell4<double>& u)
+{
+    FxCell c;
+    if (!(t.L[l].fx && fx_stage_cell(t.L[l], u, c))) c.e = kIrregular;
+    *t.own<FxCell>(l, ARR_P + buf, q) = c;
+}
+
+// What the neighbour across `wall` gives (its flux towards this cell).
+__device__ __forceinline__ FxFlux side64(const Tail& t, int l, int buf, const Faces& f,
+                                         int wall, int i, int j)
+{
+    const Level<double>& L = t.L[l];
+    FxCell c;
+    if (f.rule[wall] == BC_INFLOW) {
+        const int q = wall < 2 ? j : i;
+        const double* p = L.inflow + (size_t)(wall * 3) * L.prof_len;
+        const Cell4<double> u = { p[q], p[L.prof_len + q], p[2 * L.prof_len + q], 0.0 };
+        if (!fx_stage_cell(L, u, c)) c.e = kIrregular;
+    } else {
+        c = *t.at<FxCell>(l, ARR_P + buf, f.k[wall]);
+        if (f.rule[wall] == BC_REFLECT) {
+            if (wall < 2) c.Fx = -c.Fx;
+            else c.Fy = -c.Fy;
+            c.Pxy = -c.Pxy;
+        }
+    }
+    return wall == WALL_W ? fx_east(c) : wall == WALL_E ? fx_west(c)
+         : wall == WALL_S ? fx_north(c) : fx_south(c);
+}
+
+// The cell's neighbour sums in FP64 throughout (a block nearby is irregular).
+__device__ __noinline__ void general_sums64(const Tail& t, int l, int arr, int i, int j,
+                                            bool two_d, double& NE, double& NFx, double& NFy)
+{
+    const Level<double>& L = t.L[l];
+    Staged<double> s[4];
+    for (int w = 0; w < (two_d ? 4 : 2); ++w) {
+        const Cell4<double> c = t.fetch(l, arr, i + (w == 0 ? -1 : w == 1 ? 1 : 0),
+                                        j + (w == 2 ? -1 : w == 3 ? 1 : 0), KIND_STATE);
+        s[w].E = c.E; s[w].Fx = c.Fx; s[w].Fy = c.Fy; s[w].T = c.T;
+        closure(c.E, c.Fx, c.Fy, L.ic2, s[w].Pxx, s[w].Pxy, s[w].Pyy);
+    }
+    if (!two_d) s[2] = s[3] = s[0];
+    strip_neighbours(L, s[0], s[1], s[2], s[3], two_d, NE, NFx, NFy);
+}
+
+// The neighbour sums of Eq. (9) over the factors fE (E) and fF (F): cb, cbF, or 1
+// where they were formed in FP64 throughout.
+__device__ __forceinline__ void sums64(const Tail& t, int l, int arr, int buf, const Faces& f,
+                                       int i, int j, bool two_d, double& NE, double& NFx, double& NFy,
+                                       double& fE, double& fF)
+{
+    const Level<double>& L = t.L[l];
+    const FxFlux w = side64(t, l, buf, f, WALL_W, i, j), e = side64(t, l, buf, f, WALL_E, i, j);
+    int em = max(w.e, e.e);
+    FxFlux s;
+    if (two_d) {
+        const FxFlux b = side64(t, l, buf, f, WALL_S, i, j), n = side64(t, l, buf, f, WALL_N, i, j);
+        em = max(em, max(b.e, n.e));
+        s = fx_add(fx_to(w, em), fx_to(e, em));
+        FxFlux sy = fx_add(fx_to(b, em), fx_to(n, em));
+        if (L.fx == 2) s = fx_scale(s, split62(L.rho));
+        if (L.fx == 3) sy = fx_scale(sy, split62(L.rho));
+        s = fx_add(s, sy);
+    } else {
+        s = fx_add(fx_to(w, em), fx_to(e, em));
+    }
+    if (em == kIrregular) {
+        general_sums64(t, l, arr, i, j, two_d, NE, NFx, NFy);
+        fE = fF = 1.0;
+        return;
+    }
+    fE = L.cb;
+    fF = L.cbF;
+    NE = fx_double(s.E, s.e);
+    NFx = fx_double(s.Fx, s.e);
+    NFy = fx_double(s.Fy, s.e);
+}
+
+__device__ __forceinline__ void arrive64(const Tail& t, int l, int q, const Cell4<double>& v,
+                                         const Cell4<double>& r)
+{
+    *t.own<Cell4<double>>(l, ARR_V, q) = v;
+    *t.own<Cell4<double>>(l, ARR_F, q) = r;
+    put_block(t, l, 0, q, v);
+}
+
+__device__ __forceinline__ void op_cell(const Tail& t, int op, int l, int cur, int ccur,
+                                        int k, int q, const Pseudo<double>& ps, double theta_c,
+                                        unsigned& fails, unsigned& damped)
+{
+    typedef Cell4<double> C;
+    const Level<double>& L = t.L[l];
+    const bool two_d = L.dim == 2;
+    const int j = two_d ? row_of(t.geo[l], k) : 0, i = k - j * L.nx;
+    if (op == TAIL_PROLONG) {
+        const int ic = i >> 1, jc = two_d ? j >> 1 : 0, ox = i & 1, oy = two_d ? j & 1 : 0;
+        const double wt = pow2_neg<double>(ox + oy);
+        C pe = { 0, 0, 0, 0 };
+        for (int b = 0; b <= oy; ++b)
+            for (int a = 0; a <= ox; ++a) {
+                const C cu = t.fetch(l + 1, ARR_E + ccur, ic + a, jc + b, KIND_DIFF);
+                const C cv = t.fetch(l + 1, ARR_V, ic + a, jc + b, KIND_DIFF);
+                pe.E += wt * (cu.E - cv.E); pe.Fx += wt * (cu.Fx - cv.Fx);
+                pe.Fy += wt * (cu.Fy - cv.Fy); pe.T += wt * (cu.T - cv.T);
+            }
+        const C u = *t.own<C>(l, ARR_E + cur, q);
+        C tg = { u.E + pe.E, u.Fx + pe.Fx, u.Fy + pe.Fy, u.T + pe.T };
+        if (!admissible(tg, L.c)) {
+            const double th = theta_c * fmin(1.0, max_admissible_step(u, pe, L.c));
+            tg = C{ u.E + th * pe.E, u.Fx + th * pe.Fx, u.Fy + th * pe.Fy, u.T + th * pe.T };
+            ++damped;
+        }
+        *t.own<C>(l, ARR_E + cur, q) = tg;
+        put_block(t, l, cur, q, tg);
+        return;
+    }
+    if (op == TAIL_RESTRICT) {
+        C av = { 0, 0, 0, 0 }, ar = { 0, 0, 0, 0 };
+        const int b0 = two_d ? -1 : 0, b1 = two_d ? 1 : 0;
+        for (int b = b0; b <= b1; ++b) {
+            const int eb = two_d ? (b == 0 ? 1 : 2) : 0;
+            for (int a = -1; a <= 1; ++a) {
+                const double wt = pow2_neg<double>(eb + (a == 0 ? 1 : 2));
+                const Ghost g = ghost_map(t.L[l - 1], 2 * i + a, two_d ? 2 * j + b : 0);
+                const C s = ghost_apply(t.L[l - 1], *t.at<C>(l - 1, ARR_E + ccur, (int)g.k), g, KIND_STATE);
+                const C r = ghost_apply(t.L[l - 1], *t.at<C>(l - 1, ARR_E + 1 - ccur, (int)g.k), g,
+                                        KIND_DIFF);
+                av.E += wt * s.E; av.Fx += wt * s.Fx; av.Fy += wt * s.Fy; av.T += wt * s.T;
+                ar.E += wt * r.E; ar.Fx += wt * r.Fx; ar.Fy += wt * r.Fy; ar.T += wt * r.T;
+            }
+        }
+        arrive64(t, l, q, av, ar);
+        return;
+    }
+    const Faces f = faces_of(L, k, i, j, two_d);
+    const Sig2<double> sg = *t.sig(l, q);
+    const double ka = L.cdt * sg.sa, kt = L.cdt * (sg.sa + sg.ss);
+    double NE, NFx, NFy, fE, fF;
+    const int arr = op == TAIL_FIRST ? ARR_V : ARR_E + cur, buf = op == TAIL_FIRST ? 0 : cur;
+    sums64(t, l, arr, buf, f, i, j, two_d, NE, NFx, NFy, fE, fF);
+    const C u = *t.own<C>(l, arr, q);
+    C b = *t.own<C>(l, ARR_F, q);
+    if (op != TAIL_PSEUDO) {
+        const double T2 = u.T * u.T, src_e = ka * fma(-L.a_r, T2 * T2, u.E), dF = L.diag + kt;
+        const C a = { fma(-fE, NE, fma(L.diag, u.E, src_e)), fma(-fF, NFx, dF * u.Fx),
+                      fma(-fF, NFy, dF * u.Fy), fma(L.c_v, u.T, -src_e) };
+        if (op == TAIL_RESID) {
+            *t.own<C>(l, ARR_E + 1 - cur, q) = C{ b.E - a.E, b.Fx - a.Fx, b.Fy - a.Fy, b.T - a.T };
+            return;
+        }
+        b = C{ a.E + b.E, a.Fx + b.Fx, a.Fy + b.Fy, a.T + b.T };
+        *t.own<C>(l, ARR_F, q) = b;
+    }
+    const double cbE = ps.dtau * fE, cbF = ps.dtau * fF;
+    const double tau = surely_admissible(u, b, (float)ps.s, (float)L.c)
+                           ? ps.dtau
+                           : limited_step(u, b, ps.dtau, ps.theta, ps.s, L.c);
+    bool ok;
+    const C o = local_solve64(make_coef(1.0, ps.dtau, L.diag, ka, kt, L.a_r),
+                              fma(ps.dtau, L.diag, 1.0), fma(ps.dtau, L.c_v, 1.0), L.a_r,
+                              fma(cbE, NE, fma(tau, b.E, u.E)), fma(cbF, NFx, fma(tau, b.Fx, u.Fx)),
+                              fma(cbF, NFy, fma(tau, b.Fy, u.Fy)), fma(tau, b.T, u.T), ok);
+    if (!ok) ++fails;
+    const int out = op == TAIL_FIRST ? 1 : 1 - cur;
+    *t.own<C>(l, ARR_E + out, q) = o;
+    put_block(t, l, out, q, o);
+}
+
+// Items are (instance, first tail level), one cluster each.
+__global__ void __launch_bounds__(kTailThreads, 1) k_tail(const Level<double>* __restrict__ lv,
+                                                          int cap, int nlev, WorkList wl,
+                                                          Ctl* __restrict__ ctls,
+                                                          const unsigned char* __restrict__ prog,
+                                                          const int2* __restrict__ progs)
+{
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ Level<double> Ls[kTailLevels];
+    __shared__ TailGeo geo[kTailLevels];
+    cg::cluster_group cl = cg::this_cluster();
+    const int nb = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+    const int w0 = blockIdx.x / nb, ws = gridDim.x / nb;
+    const int nw = *wl.count;
+    Tail t{ Ls, geo, smem, rank, cl };
+    for (int w = w0; w < nw; w += ws) {
+        const int2 it = wl.items[w];
+        if (skip(ctls, it.x)) continue;            // the same for the whole cluster
+        Ctl* ctl = ctls + it.x;
+        const int first = it.y, nl = nlev - first;
+        const Level<double>* src = lv + (size_t)first * cap + it.x;
+        for (int l = threadIdx.x / 32; l < nl; l += kTailThreads / 32) {
+            const unsigned long long* s =
+                reinterpret_cast<const unsigned long long*>(src + (size_t)l * cap);
+            if ((threadIdx.x & 31) < sizeof(Level<double>) / 8)
+                reinterpret_cast<unsigned long long*>(&Ls[l])[threadIdx.x & 31] =
+                    s[threadIdx.x & 31];
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            int off = 0;
+            for (int l = 0; l < nl; ++l) {
+                TailGeo g;
+                g.nx = Ls[l].nx;
+                g.n = Ls[l].n;
+                g.per = tail_per(g.n, nb);
+                g.blocks = (g.n + g.per - 1) / g.per;
+                g.off = off;
+                g.mx = g.nx > 1 ? (unsigned)((0x100000000ull + g.nx - 1) / g.nx) : 0u;
+                g.mper = (unsigned)((0x100000000ull + g.per - 1) / g.per);
+                geo[l] = g;
+                off += kTailBytes * g.per;
+            }
+        }
+        __syncthreads();
+        const Pseudo<double> ps = pseudo_of<double>(ctl);
+        const double theta_c = ctl->theta_c;
+        unsigned fails = 0, damped = 0;
+        for (int l = 0; l < nl; ++l)
+            for (int q = threadIdx.x; q < geo[l].per; q += kTailThreads) {
+                const int k = rank * geo[l].per + q;
+                if (k >= geo[l].n) break;
+                *t.sig(l, q) = Ls[l].sig[k];
+                if (l == 0) arrive64(t, 0, q, Ls[0].v[k], Ls[0].r[k]);
+            }
+        unsigned curs = 0;                          // bit l: the buffer of level l's iterate
+        const int2 pr = progs[first];
+        bool was_multi = true;
+        for (int p = 0; p <= pr.y; ++p) {
+            const int code = p < pr.y ? prog[pr.x + p] : 0;
+            const int op = code & 7, l = code >> 3;
+            // the levels the operation reads or writes: l, and (restriction, prolongation)
+            // one more; a single block works while all of them lie in block 0
+            const int lo = p == pr.y ? 0 : (op == TAIL_RESTRICT ? l - 1 : l);
+            const bool multi = geo[lo].blocks > 1;
+            if (multi || was_multi) cl.sync();
+            else if (rank == 0) __syncthreads();
+            was_multi = multi;
+            if (p == pr.y) break;
+            const int cur = (curs >> l) & 1;
+            const int ccur = op == TAIL_RESTRICT ? (curs >> (l - 1)) & 1
+                           : op == TAIL_PROLONG ? (curs >> (l + 1)) & 1 : 0;
+            const int base = rank * geo[l].per, end = min(geo[l].per, geo[l].n - base);
+            for (int q = threadIdx.x; q < end; q += kTailThreads)
+                op_cell(t, op, l, cur, ccur, base + q, q, ps, theta_c, fails, damped);
+            if (op == TAIL_FIRST) curs |= 1u << l;
+            else if (op == TAIL_PSEUDO) curs ^= 1u << l;
+        }
+        // the result to global memory, into both buffers of the tail's first level (the
+        // other instances of the level decide which one the prolongation reads)
+        for (int q = threadIdx.x; q < geo[0].per; q += kTailThreads) {
+            const int k = rank * geo[0].per + q;
+            if (k >= geo[0].n) break;
+            const Cell4<double> o = *t.own<Cell4<double>>(0, ARR_E + (curs & 1), q);
+            Ls[0].u[0][k] = o;
+            Ls[0].u[1][k] = o;
+        }
+        if (fails) atomicAdd(&ctl->newton_fail, fails);
+        if (damped) atomicAdd(&ctl->damped, damped);
+        cl.sync();                                  // before the next item's arrays
+    }
+    cl.sync();                                      // no block leaves while another reads it
+}
+
+}  // namespace
+
+size_t tail_smem(int n0, int nb, int dim, int nlev)
+{
+    size_t s = 0;
+    for (int l = 0; l < nlev; ++l) {
+        s += (size_t)kTailBytes * tail_per(n0, nb);
+        n0 /= dim == 2 ? 4 : 2;
+    }
+    return s;
+}
+
+cudaError_t tail_prepare()
+{
+    const cudaError_t e =
+        cudaFuncSetAttribute(k_tail, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(k_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, kTailSmem);
+}
+
+cudaError_t launch_tail(const Level<double>* lv, int cap, int nlev, WorkList wl, Ctl* ctls,
+                        const unsigned char* prog, const int2* progs, size_t smem, cudaStream_t s)
+{
+    const int clusters = wl.capacity < kTailClusters ? (wl.capacity > 0 ? wl.capacity : 1)
+                                                     : kTailClusters;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(clusters * kTailBlocks);
+    cfg.blockDim = dim3(kTailThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = kTailBlocks;
+    at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_tail, lv, cap, nlev, wl, ctls, prog, progs);
+}
+
+}  // namespace m1

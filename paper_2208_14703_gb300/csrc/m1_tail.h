@@ -1,0 +1,47 @@
+// The coarse end of a cycle in one launch (m1_tail.cu): its interface, and the rule
+// for where it begins.
+#pragma once
+#include <cstddef>
+#include <cuda_runtime.h>
+
+#include "m1_device.cuh"
+
+namespace m1 {
+
+// Blocks of a cluster, clusters of a launch, levels, and the dynamic shared memory
+// a block may take.
+constexpr int kTailBlocks = 16, kTailClusters = 36, kTailLevels = 20;
+constexpr int kTailSmem = 216 * 1024;
+// The tail begins at the first coarse FP64 level of at most this many cells.
+constexpr int kTailCells = 8192;
+
+// Operations of a tail's program, one byte each: the operation + 8 x the level
+// counted from the tail's first.  FIRST: the FAS right-hand side and the first
+// pseudo-time step of a fresh visit; PSEUDO: one more step; RESID: the residual;
+// RESTRICT: from the level above into this one; PROLONG: from the level below onto
+// this one.
+enum TailOp { TAIL_FIRST = 0, TAIL_PSEUDO = 1, TAIL_RESID = 2, TAIL_RESTRICT = 3, TAIL_PROLONG = 4 };
+
+// Cells per block of a level of n cells over nb blocks: equal shares, but no
+// fewer than make a block's work worth a cluster barrier.
+__host__ __device__ inline int tail_per(int n, int nb)
+{
+    int p = (n + nb - 1) / nb;
+    const int least = 64;
+    const int cap = n < least ? n : least;
+    p = p < cap ? cap : p;
+    return (p + 3) & ~3;
+}
+
+// Dynamic shared memory of a block for a tail of nlev levels, the first of n0 cells.
+size_t tail_smem(int n0, int nb, int dim, int nlev);
+
+// The kernel's attributes on the current device (once per engine).
+cudaError_t tail_prepare();
+
+// items of wl: (instance, first tail level); progs[first level]: (offset, length)
+// in prog.
+cudaError_t launch_tail(const Level<double>* lv, int cap, int nlev, WorkList wl, Ctl* ctls,
+                        const unsigned char* prog, const int2* progs, size_t smem, cudaStream_t s);
+
+}  // namespace m1
