@@ -131,6 +131,38 @@ __host__ __device__ __forceinline__ i64 fx_align(u64 bits, int d)
     return (v ^ s) - s;
 }
 
+// sigma = sqrt(xi) (scale 2^60; xi at 2^60, in [x^2/4, x^2]) and, returned, 3/2 D =
+// 3/2 / (x + sigma) at scale 2^62, x at 2^61.
+__host__ __device__ __forceinline__ i64 fx_sigma_d(i64 xE, i64 xi, i64& sg)
+{
+    // sigma = sqrt(xi): a 30-bit start s0 from the seed y of 1/sqrt(xi), then two
+    // Newton corrections sigma += (xi - sigma^2) y / 2, exact residuals
+    const float xif = (float)(int)(xi >> 32) * 0x1p-28f;
+    const float yf = seed_rsqrt(xif);
+    const int Y = (int)(yf * 0x1p29f);                         // y <= 2
+    const float sf = xif * yf;
+    const int s0 = (int)(sf * 0x1.fffffcp29f);                  // < 2^31 (sigma < 2 up to rounding)
+    const i64 t0 = xi - madw(s0, s0, 0);                       // scale 2^60, |t0| < 2^42
+    const i64 d0 = madw((int)(t0 >> 12), Y, 0) >> 18;          // t0 y / 2, scale 2^60
+    sg = ((i64)s0 << 30) + d0;
+    const i64 t1 = xi - sqr62(split62(sg << 1));
+    sg += madw((int)t1, Y, 0) >> 30;
+    const i64 hx = xE >> 2;                                    // x / 2 at scale 2^60
+    sg = sg > hx ? sg : hx;
+    // D = 1 / (x + sigma), scale 2^62, from the seed r: D = r (1 + d + d^2),
+    // d = 1 - (x + sigma) r, less 2^-57 so that 3/2 D stays below 2^62
+    const i64 w = (xE >> 1) + sg;                              // scale 2^60, in [1.5, 4)
+    const float rf = seed_rcp((float)(int)(w >> 32) * 0x1p-28f);
+    const int Rr = (int)(rf * 0x1p31f);                        // r <= 2/3
+    const Split sw = split62(w);
+    const i64 d = ((1ll << 60) - 8) - madw(sw.h, Rr, madw(sw.l, Rr, 0) >> 31);
+    const Split sd = split62(d);                               // |d| < 2^39
+    const i64 rd = madw(sd.h, Rr, madw(sd.l, Rr, 0) >> 31);    // r d, scale 2^60
+    const i64 rdd = madw((int)(d >> 22), (int)(rd >> 22), 0) >> 16;
+    const i64 D = ((i64)Rr << 31) + ((rd + rdd) << 2);
+    return D + (D >> 1);
+}
+
 // The closure of Eq. (5) and the cell's block, from E and F / c.  With x = E and
 // sigma = sqrt(x^2 - 3/4 |F/c|^2) >= x/2 it reads
 //   P = (2 sigma - x)/3 I + 3/2 (F/c)(F/c)^T / (x + sigma),
@@ -157,32 +189,8 @@ __host__ __device__ __forceinline__ bool fx_stage(double E, double Fx, double Fy
     i64 xi = E2 - F2 + (F2 >> 2);
     const i64 q2 = E2 >> 2;
     xi = xi > q2 ? xi : q2;
-    // sigma = sqrt(xi): a 30-bit start s0 from the seed y of 1/sqrt(xi), then two
-    // Newton corrections sigma += (xi - sigma^2) y / 2, exact residuals
-    const float xif = (float)(int)(xi >> 32) * 0x1p-28f;
-    const float yf = seed_rsqrt(xif);
-    const int Y = (int)(yf * 0x1p29f);                         // y <= 2
-    const float sf = xif * yf;
-    const int s0 = (int)(sf * 0x1.fffffcp29f);                  // < 2^31 (sigma < 2 up to rounding)
-    const i64 t0 = xi - madw(s0, s0, 0);                       // scale 2^60, |t0| < 2^42
-    const i64 d0 = madw((int)(t0 >> 12), Y, 0) >> 18;          // t0 y / 2, scale 2^60
-    i64 sg = ((i64)s0 << 30) + d0;
-    const i64 t1 = xi - sqr62(split62(sg << 1));
-    sg += madw((int)t1, Y, 0) >> 30;
-    const i64 hx = xE >> 2;                                    // x / 2 at scale 2^60
-    sg = sg > hx ? sg : hx;
-    // D = 1 / (x + sigma), scale 2^62, from the seed r: D = r (1 + d + d^2),
-    // d = 1 - (x + sigma) r, less 2^-57 so that 3/2 D stays below 2^62
-    const i64 w = (xE >> 1) + sg;                              // scale 2^60, in [1.5, 4)
-    const float rf = seed_rcp((float)(int)(w >> 32) * 0x1p-28f);
-    const int Rr = (int)(rf * 0x1p31f);                        // r <= 2/3
-    const Split sw = split62(w);
-    const i64 d = ((1ll << 60) - 8) - madw(sw.h, Rr, madw(sw.l, Rr, 0) >> 31);
-    const Split sd = split62(d);                               // |d| < 2^39
-    const i64 rd = madw(sd.h, Rr, madw(sd.l, Rr, 0) >> 31);    // r d, scale 2^60
-    const i64 rdd = madw((int)(d >> 22), (int)(rd >> 22), 0) >> 16;
-    const i64 D = ((i64)Rr << 31) + ((rd + rdd) << 2);
-    const Split sD = split62(D + (D >> 1));                    // 3/2 D, scale 2^62
+    i64 sg;
+    const Split sD = split62(fx_sigma_d(xE, xi, sg));          // 3/2 D, scale 2^62
     // (2 sigma - x) / 3, scale 2^60: the factor is 2^61 / 3
     constexpr i64 third = 768614336404564651ll;
     const i64 iso = mul62(split62((sg << 2) - xE), split62(third));
@@ -238,25 +246,32 @@ __host__ __device__ __forceinline__ i64 fx_significand(double x, int& e)
 }
 
 // The root T of C T + K T^4 = R (C, K, R > 0) and T^4: Newton in FP32 to about
-// 2e-7, then two corrections whose residuals are formed in fixed point relative
+// 2e-7 (from `seed` when that is positive and a quarter
+// or less off), then two
+// corrections whose residuals are formed in fixed point relative
 // to R (both terms are positive and sum to R) and whose quotients are FP32 (each
 // needs only the digits it adds).  With t = T 2^(61 - eT) the powers are
 // t^2 = T2 2^62, T2^2 = T4 2^62.  The residual is good to 2^-55 R, hence T to
 // about 2^-55 and T^4 to 2^-53.  False where FP32 cannot hold or seed the problem.
 __host__ __device__ __forceinline__ bool fx_quartic(double C, double K, double R, double& Tout,
-                                                    double& T4out)
+                                                    double& T4out, float seed = 0.0f)
 {
     const float Cf = narrow_rz(C), Kf = narrow_rz(K), Rf = narrow_rz(R);
     const float K4 = 4.0f * Kf;
-    float T = fminf(Rf * seed_rcp(Cf), seed_sqrt(seed_sqrt(Rf * seed_rcp(Kf))));
-    bool ok = false;
-    for (int it = 0; it < 40; ++it) {
+    // one Newton step; the root then lies within 1.5 dT^2 / T (g'' T <= 3 g')
+    auto newton = [&](float T, float& dT) {
         const float T3 = T * T * T;
         const float g = fmaf(Kf, T3 * T, Cf * T) - Rf;
-        const float dT = g * seed_rcp(fmaf(K4, T3, Cf));
-        T -= dT;
-        // Newton's error is at most 1.5 dT^2 / T here (g'' T <= 3 g')
-        if (fabsf(dT) <= 3e-4f * T) { ok = true; break; }
+        dT = g * seed_rcp(fmaf(K4, T3, Cf));
+        return T - dT;
+    };
+    float dT = 0.0f, T = seed > 0.0f ? newton(seed, dT) : 0.0f;
+    bool ok = seed > 0.0f && fabsf(dT) <= 3e-4f * T;
+    if (!(seed > 0.0f && fabsf(dT) <= 0.25f * seed))
+        T = fminf(Rf * seed_rcp(Cf), seed_sqrt(seed_sqrt(Rf * seed_rcp(Kf))));
+    for (int it = 0; it < 40 && !ok; ++it) {
+        T = newton(T, dT);
+        ok = fabsf(dT) <= 3e-4f * T;
     }
     const unsigned bt = bits_of_float(T);
     const int eT = (int)(bt >> 23) - 127;                      // sign set: out of range below

@@ -335,10 +335,9 @@ __device__ __forceinline__ double strip_sweep64(const Level<double>& L, Ctl* ctl
     if (L.fx) {
         const Pseudo<double> ps = PSEUDO ? pseudo_of<double>(ctl) : Pseudo<double>{};
         const double cbE = PSEUDO ? ps.dtau * L.cb : L.cb, cbF = PSEUDO ? ps.dtau * L.cbF : L.cbF;
-        // the pseudo-time step's A and C, and the FP32 values of its admissibility check
+        // the pseudo-time step's A and C
         const double Ap = PSEUDO ? fma(ps.dtau, L.diag, 1.0) : 0.0;
         const double Cp = PSEUDO ? fma(ps.dtau, L.c_v, 1.0) : 0.0;
-        const float s32 = (float)ps.s, c32 = (float)L.c;
         auto pre = [&](size_t k) {
             Pre p;
             p.b = FAS ? L.r[k] : L.f[k];
@@ -378,9 +377,7 @@ __device__ __forceinline__ double strip_sweep64(const Level<double>& L, Ctl* ctl
                 o = local_solve64(p.q, L.diag, L.c_v, L.a_r, fma(cbE, NE, b.E), fma(cbF, NFx, b.Fx),
                                   fma(cbF, NFy, b.Fy), b.T, ok);
             } else {
-                const double tau = surely_admissible(p.u, b, s32, c32)
-                                       ? ps.dtau
-                                       : limited_step(p.u, b, ps.dtau, ps.theta, ps.s, L.c);
+                const double tau = limited_step64(p.u, b, ps.dtau, ps.theta, ps.s, L.c);
                 o = local_solve64(make_coef(1.0, ps.dtau, L.diag, ka, kt, L.a_r), Ap, Cp, L.a_r,
                                   fma(cbE, NE, fma(tau, b.E, p.u.E)),
                                   fma(cbF, NFx, fma(tau, b.Fx, p.u.Fx)),

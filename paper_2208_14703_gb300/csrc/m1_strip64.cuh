@@ -162,9 +162,10 @@ __device__ __forceinline__ Coef make_coef(double w0, double w1, double diag, dou
 // The local solve with its coefficients given: seven FP64 operations, the quartic
 // in fixed point (fx_quartic) or, where that cannot hold it, by Quartic<double>.
 // A is used without absorption only: E = bE / A with the quotient's remainder added.
+// Tseed: a temperature near the solution (0: none).
 __device__ __forceinline__ Cell4<double> local_solve64(const Coef& q, double A, double C, double a_r,
                                                        double bE, double bFx, double bFy, double bT,
-                                                       bool& ok)
+                                                       bool& ok, double Tseed = 0.0)
 {
     Cell4<double> o;
     ok = true;
@@ -179,7 +180,7 @@ __device__ __forceinline__ Cell4<double> local_solve64(const Coef& q, double A, 
     }
     const double R = fma(q.kk, bE, bT);
     double T4;
-    if (!fx_quartic(C, q.K, R, o.T, T4)) {
+    if (!fx_quartic(C, q.K, R, o.T, T4, narrow_rz(Tseed))) {
         o.T = Quartic<double>::solve(C, q.K, R, ok);
         const double T2 = o.T * o.T;
         T4 = T2 * T2;
@@ -190,22 +191,93 @@ __device__ __forceinline__ Cell4<double> local_solve64(const Coef& q, double A, 
     return o;
 }
 
-// Whether u + s f is admissible beyond doubt in FP32 (values rounded toward zero, a
-// margin of 1e-6 of the terms' sizes where the roundings leave at most 5e-7): the
-// explicit pseudo-time step is then not limited.  c, s in FP32.
-__device__ __forceinline__ bool surely_admissible(const Cell4<double>& u, const Cell4<double>& f,
-                                                  float s, float c)
+// x / y and sqrt(x) for the limited step, by the refined estimates of Fm<double>
+// where both arguments are of ordinary size, else IEEE.
+__device__ __forceinline__ bool ordinary(double x)
+{
+    return ((unsigned)(__double2hiint(x) >> 20) & 0x7ffu) - 200u < 1647u;
+}
+__device__ __forceinline__ double quotient(double x, double y)
+{
+    if (!ordinary(y)) return x / y;
+    const double r = Fm<double>::rcp(y), q = x * r;
+    return fma(fma(-y, q, x), r, q);
+}
+
+// max_admissible_step in two (the bound that binds alone) to thirty FP64 operations
+// where the IEEE divisions and square root took sixty-five; the same bounds, each
+// within an ulp or two.  
+__device__ __forceinline__ double cone_step(double a, double b, double c0)
+{
+    c0 = c0 > 0.0 ? 0.0 : c0;
+    const double disc = fma(b, b, -(a * c0));
+    const double sd = disc > 0.0 && ordinary(disc) ? Fm<double>::sqrt(disc) : sqrt(disc);
+    if (a > 0.0) return b <= 0.0 ? quotient(sd - b, a) : quotient(-c0, b + sd);
+    if (a < 0.0) return b > 0.0 && disc >= 0.0 ? quotient(-c0, b + sd) : (double)INFINITY;
+    return b > 0.0 ? quotient(-c0, 2.0 * b) : (double)INFINITY;
+}
+
+// A bound u / (-d) on tau where d < 0.
+__device__ __forceinline__ double plane_step(double u, double d)
+{
+    return d < 0.0 ? quotient(-u, d) : (double)INFINITY;
+}
+
+__device__ __forceinline__ double max_admissible_step64(const Cell4<double>& u,
+                                                        const Cell4<double>& d, double c)
+{
+    const double c2 = c * c, cd = c2 * d.E, cu = c2 * u.E;
+    const double a = fma(-cd, d.E, fma(d.Fy, d.Fy, d.Fx * d.Fx));
+    const double b = fma(-cu, d.E, fma(u.Fy, d.Fy, u.Fx * d.Fx));
+    const double c0 = fma(-cu, u.E, fma(u.Fy, u.Fy, u.Fx * u.Fx));
+    return fmin(fmin(plane_step(u.E, d.E), plane_step(u.T, d.T)), cone_step(a, b, c0));
+}
+
+// Whether u + s f is admissible, decided in FP32 where that is beyond doubt (values
+// rounded toward zero, a margin of 1e-6 of the terms' sizes where the roundings
+// leave at most 5e-7): 1 yes, -1 no, 0 unknown.  c, s in FP32; F2 the squared length
+// of u_F + s f_F and its margin are the caller's (two or three components).
+struct FluxSum {
+    float hi = 0.f, lo = 0.f;      // squared length with the margins added, taken off
+    __device__ __forceinline__ void add(float u, float f)
+    {
+        const float p = fabsf(u + f), m = 1e-6f * (fabsf(u) + fabsf(f));
+        hi = fmaf(p + m, p + m, hi);
+        lo = fmaf(fmaxf(p - m, 0.f), fmaxf(p - m, 0.f), lo);
+    }
+};
+
+__device__ __forceinline__ int admissible_sure(float uE, float fE, float uT, float fT, float c,
+                                               const FluxSum& F)
 {
     const float m = 1e-6f;
-    const float uE = narrow_rz(u.E), fE = s * narrow_rz(f.E);
-    const float uT = narrow_rz(u.T), fT = s * narrow_rz(f.T);
-    const float ux = narrow_rz(u.Fx), fx = s * narrow_rz(f.Fx);
-    const float uy = narrow_rz(u.Fy), fy = s * narrow_rz(f.Fy);
-    const float pE = c * ((uE + fE) - m * (uE + fabsf(fE)));
-    const float px = fabsf(ux + fx) + m * (fabsf(ux) + fabsf(fx));
-    const float py = fabsf(uy + fy) + m * (fabsf(uy) + fabsf(fy));
-    return uT + fT > m * (uT + fabsf(fT)) && uE > 1e-30f && uT > 1e-30f && pE > 1e-15f * c &&
-           fmaf(px, px, py * py) <= 0.99999f * pE * pE;
+    if (!(uE > 1e-15f && uT > 1e-30f && uE < 1e15f)) return 0;
+    const float mE = m * (uE + fabsf(fE)), mT = m * (uT + fabsf(fT));
+    const float pE = uE + fE, pT = uT + fT;
+    if (pE < -mE || pT < -mT) return -1;
+    const float lo = c * (pE - mE), hi = c * (pE + mE);
+    if (pT > mT && lo > 1e-15f * c && F.hi <= 0.99999f * lo * lo) return 1;
+    if (F.lo >= 1.00001f * hi * hi && F.lo < 1e30f) return -1;
+    return 0;
+}
+
+// limited_step with the question whether it binds put in FP32 first.
+__device__ __forceinline__ double limited_step64(const Cell4<double>& u, const Cell4<double>& f,
+                                                 double dtau, double theta, double s, double c)
+{
+    const float s32 = (float)s;
+    FluxSum F;
+    F.add(narrow_rz(u.Fx), s32 * narrow_rz(f.Fx));
+    F.add(narrow_rz(u.Fy), s32 * narrow_rz(f.Fy));
+    const int sure = admissible_sure(narrow_rz(u.E), s32 * narrow_rz(f.E), narrow_rz(u.T),
+                                     s32 * narrow_rz(f.T), (float)c, F);
+    if (sure > 0) return dtau;
+    if (sure == 0) {
+        const Cell4<double> p = { fma(s, f.E, u.E), fma(s, f.Fx, u.Fx), fma(s, f.Fy, u.Fy),
+                                  fma(s, f.T, u.T) };
+        if (admissible_c2<double, false>(p, c * c)) return dtau;
+    }
+    return fmin(dtau, theta * max_admissible_step64(u, f, c));
 }
 
 }  // namespace m1

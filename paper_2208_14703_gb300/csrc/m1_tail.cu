@@ -43,15 +43,23 @@ __device__ __forceinline__ int row_of(const TailGeo& g, int k)
 }
 
 // Arrays of a range of `per` cells: the iterates e0, e1, v and f (which first holds
-// the restricted residual), 32 bytes a cell each; the blocks of e0 (first of v) and
-// e1, 56 each; sigma.
-enum { ARR_E = 0, ARR_V = 2, ARR_F = 3, ARR_P = 4 };
-constexpr int kTailBytes = 4 * 32 + 2 * 56 + 16;
+// the restricted residual) and the local solve's coefficients (formed by the first
+// step of a fresh visit), 32 bytes a cell each; the blocks of e0 (first of v) and e1,
+// 56 each; sigma; the four neighbours (side_code).
+enum { ARR_E = 0, ARR_V = 2, ARR_F = 3, ARR_Q = 4, ARR_P = 5, ARR_SIG = 7, ARR_NB = 8 };
+constexpr int kTailBytes = 5 * 32 + 2 * 56 + 16 + 16;
 
 __device__ __forceinline__ int arr_at(int a, int per)
 {
-    return a < 4 ? a * 32 * per : 4 * 32 * per + (a - 4) * 56 * per;
+    return (a < ARR_P ? a * 32 : a < ARR_SIG ? 5 * 32 + (a - ARR_P) * 56
+                                             : 5 * 32 + 2 * 56 + (a - ARR_SIG) * 16) * per;
 }
+
+// What a level's pseudo-time steps share: dtau c b, dtau c^2 b (the sums' factors),
+// A = 1 + dtau diag, C = 1 + dtau C_v.
+struct TailStep {
+    double cbE, cbF, A, C;
+};
 
 // A cell's block that could not be formed (m1_fx.cuh: not regular): its
 // neighbours and itself take the FP64 form.
@@ -60,6 +68,7 @@ constexpr int kIrregular = 1 << 20;
 struct Tail {
     const Level<double>* L;             // descriptors, [0] = the tail's first level
     const TailGeo* geo;
+    const TailStep* step;
     unsigned char* smem;           // this block's arrays
     int rank;
     cg::cluster_group cl;
@@ -84,7 +93,7 @@ struct Tail {
     __device__ Sig2<double>* sig(int l, int q) const
     {
         const TailGeo& g = geo[l];
-        return reinterpret_cast<Sig2<double>*>(smem + g.off + arr_at(6, g.per)) + q;
+        return reinterpret_cast<Sig2<double>*>(smem + g.off + arr_at(ARR_SIG, g.per)) + q;
     }
     // a cell of array a with the wall rules of fetch()
     __device__ Cell4<double> fetch(int l, int a, int i, int j, int kind) const
@@ -94,31 +103,25 @@ struct Tail {
     }
 };
 
-// The four faces of a cell: the neighbour's index and the wall rule there (-1:
-// inside or periodic).
-struct Faces {
-    int k[4], rule[4];
-};
-
-__device__ __forceinline__ Faces faces_of(const Level<double>& L, int k, int i, int j, bool two_d)
+// A cell's neighbour across a wall of the stencil, packed: its index in its range
+// (16 bits), the range's block (8), and the wall rule there + 1 (0: none).
+__device__ __forceinline__ unsigned side_code(const Tail& t, int l, int k, int i, int j, int wall)
 {
-    Faces f;
-    auto face = [&](int w, bool inside, int kin, int kwrap) {
-        f.rule[w] = -1;
-        f.k[w] = kin;
-        if (!inside) {
-            const int bc = L.bc[w];
-            f.k[w] = bc == BC_PERIODIC ? kwrap : k;
-            if (bc != BC_PERIODIC) f.rule[w] = bc;
-        }
-    };
-    face(WALL_W, i > 0, k - 1, k + L.nx - 1);
-    face(WALL_E, i + 1 < L.nx, k + 1, k - L.nx + 1);
-    if (two_d) {
-        face(WALL_S, j > 0, k - L.nx, k + L.n - L.nx);
-        face(WALL_N, j + 1 < L.ny, k + L.nx, k - L.n + L.nx);
+    const Level<double>& L = t.L[l];
+    int kn, rule = -1;
+    const bool inside = wall == WALL_W ? i > 0 : wall == WALL_E ? i + 1 < L.nx
+                      : wall == WALL_S ? j > 0 : j + 1 < L.ny;
+    if (inside) {
+        kn = wall == WALL_W ? k - 1 : wall == WALL_E ? k + 1 : wall == WALL_S ? k - L.nx : k + L.nx;
+    } else if (L.bc[wall] == BC_PERIODIC) {
+        kn = wall == WALL_W ? k + L.nx - 1 : wall == WALL_E ? k - L.nx + 1
+           : wall == WALL_S ? k + L.n - L.nx : k - L.n + L.nx;
+    } else {
+        kn = k;
+        rule = L.bc[wall];
     }
-    return f;
+    const int b = (int)__umulhi((unsigned)kn, t.geo[l].mper);
+    return (unsigned)(kn - b * t.geo[l].per) | (unsigned)b << 16 | (unsigned)(rule + 1) << 24;
 }
 
 __device__ __forceinline__ void put_block(const Tail& t, int l, int buf, int q,
@@ -130,19 +133,23 @@ __device__ __forceinline__ void put_block(const Tail& t, int l, int buf, int q,
 }
 
 // What the neighbour across `wall` gives (its flux towards this cell).
-__device__ __forceinline__ FxFlux side64(const Tail& t, int l, int buf, const Faces& f,
-                                         int wall, int i, int j)
+__device__ __forceinline__ FxFlux side64(const Tail& t, int l, int buf, unsigned code, int wall,
+                                         int k)
 {
     const Level<double>& L = t.L[l];
+    const int rule = (int)(code >> 24) - 1;
     FxCell c;
-    if (f.rule[wall] == BC_INFLOW) {
-        const int q = wall < 2 ? j : i;
+    if (rule == BC_INFLOW) {
+        const int j = L.dim == 2 ? row_of(t.geo[l], k) : 0, q = wall < 2 ? j : k - j * L.nx;
         const double* p = L.inflow + (size_t)(wall * 3) * L.prof_len;
         const Cell4<double> u = { p[q], p[L.prof_len + q], p[2 * L.prof_len + q], 0.0 };
         if (!fx_stage_cell(L, u, c)) c.e = kIrregular;
     } else {
-        c = *t.at<FxCell>(l, ARR_P + buf, f.k[wall]);
-        if (f.rule[wall] == BC_REFLECT) {
+        const FxCell* p = t.own<FxCell>(l, ARR_P + buf, (int)(code & 0xffffu));
+        const int b = (int)(code >> 16) & 0xff;
+        if (b != t.rank) p = t.cl.map_shared_rank(p, b);
+        c = *p;
+        if (rule == BC_REFLECT) {
             if (wall < 2) c.Fx = -c.Fx;
             else c.Fy = -c.Fy;
             c.Pxy = -c.Pxy;
@@ -153,10 +160,11 @@ __device__ __forceinline__ FxFlux side64(const Tail& t, int l, int buf, const Fa
 }
 
 // The cell's neighbour sums in FP64 throughout (a block nearby is irregular).
-__device__ __noinline__ void general_sums64(const Tail& t, int l, int arr, int i, int j,
-                                            bool two_d, double& NE, double& NFx, double& NFy)
+__device__ __noinline__ void general_sums64(const Tail& t, int l, int arr, int k, bool two_d,
+                                            double& NE, double& NFx, double& NFy)
 {
     const Level<double>& L = t.L[l];
+    const int j = two_d ? row_of(t.geo[l], k) : 0, i = k - j * L.nx;
     Staged<double> s[4];
     for (int w = 0; w < (two_d ? 4 : 2); ++w) {
         const Cell4<double> c = t.fetch(l, arr, i + (w == 0 ? -1 : w == 1 ? 1 : 0),
@@ -168,18 +176,18 @@ __device__ __noinline__ void general_sums64(const Tail& t, int l, int arr, int i
     strip_neighbours(L, s[0], s[1], s[2], s[3], two_d, NE, NFx, NFy);
 }
 
-// The neighbour sums of Eq. (9) over the factors fE (E) and fF (F): cb, cbF, or 1
-// where they were formed in FP64 throughout.
-__device__ __forceinline__ void sums64(const Tail& t, int l, int arr, int buf, const Faces& f,
-                                       int i, int j, bool two_d, double& NE, double& NFx, double& NFy,
-                                       double& fE, double& fF)
+// The neighbour sums of Eq. (9): over the factors cb (E) and cbF (F) when fx, else
+// whole, formed in FP64 throughout.
+__device__ __forceinline__ void sums64(const Tail& t, int l, int arr, int buf, int k, int q,
+                                       bool two_d, double& NE, double& NFx, double& NFy, bool& fx)
 {
     const Level<double>& L = t.L[l];
-    const FxFlux w = side64(t, l, buf, f, WALL_W, i, j), e = side64(t, l, buf, f, WALL_E, i, j);
+    const uint4 nb = *t.own<uint4>(l, ARR_NB, q);
+    const FxFlux w = side64(t, l, buf, nb.x, WALL_W, k), e = side64(t, l, buf, nb.y, WALL_E, k);
     int em = max(w.e, e.e);
     FxFlux s;
     if (two_d) {
-        const FxFlux b = side64(t, l, buf, f, WALL_S, i, j), n = side64(t, l, buf, f, WALL_N, i, j);
+        const FxFlux b = side64(t, l, buf, nb.z, WALL_S, k), n = side64(t, l, buf, nb.w, WALL_N, k);
         em = max(em, max(b.e, n.e));
         s = fx_add(fx_to(w, em), fx_to(e, em));
         FxFlux sy = fx_add(fx_to(b, em), fx_to(n, em));
@@ -190,12 +198,11 @@ __device__ __forceinline__ void sums64(const Tail& t, int l, int arr, int buf, c
         s = fx_add(fx_to(w, em), fx_to(e, em));
     }
     if (em == kIrregular) {
-        general_sums64(t, l, arr, i, j, two_d, NE, NFx, NFy);
-        fE = fF = 1.0;
+        general_sums64(t, l, arr, k, two_d, NE, NFx, NFy);
+        fx = false;
         return;
     }
-    fE = L.cb;
-    fF = L.cbF;
+    fx = true;
     NE = fx_double(s.E, s.e);
     NFx = fx_double(s.Fx, s.e);
     NFy = fx_double(s.Fy, s.e);
@@ -216,8 +223,8 @@ __device__ __forceinline__ void op_cell(const Tail& t, int op, int l, int cur, i
     typedef Cell4<double> C;
     const Level<double>& L = t.L[l];
     const bool two_d = L.dim == 2;
-    const int j = two_d ? row_of(t.geo[l], k) : 0, i = k - j * L.nx;
     if (op == TAIL_PROLONG) {
+        const int j = two_d ? row_of(t.geo[l], k) : 0, i = k - j * L.nx;
         const int ic = i >> 1, jc = two_d ? j >> 1 : 0, ox = i & 1, oy = two_d ? j & 1 : 0;
         const double wt = pow2_neg<double>(ox + oy);
         C pe = { 0, 0, 0, 0 };
@@ -231,7 +238,7 @@ __device__ __forceinline__ void op_cell(const Tail& t, int op, int l, int cur, i
         const C u = *t.own<C>(l, ARR_E + cur, q);
         C tg = { u.E + pe.E, u.Fx + pe.Fx, u.Fy + pe.Fy, u.T + pe.T };
         if (!admissible(tg, L.c)) {
-            const double th = theta_c * fmin(1.0, max_admissible_step(u, pe, L.c));
+            const double th = theta_c * fmin(1.0, max_admissible_step64(u, pe, L.c));
             tg = C{ u.E + th * pe.E, u.Fx + th * pe.Fx, u.Fy + th * pe.Fy, u.T + th * pe.T };
             ++damped;
         }
@@ -239,7 +246,8 @@ __device__ __forceinline__ void op_cell(const Tail& t, int op, int l, int cur, i
         put_block(t, l, cur, q, tg);
         return;
     }
-    if (op == TAIL_RESTRICT) {
+    if (op == TAIL_RESTRICT) {             // cell k of level l from level l - 1; ccur: its buffer
+        const int j = two_d ? row_of(t.geo[l], k) : 0, i = k - j * L.nx;
         C av = { 0, 0, 0, 0 }, ar = { 0, 0, 0, 0 };
         const int b0 = two_d ? -1 : 0, b1 = two_d ? 1 : 0;
         for (int b = b0; b <= b1; ++b) {
@@ -257,15 +265,19 @@ __device__ __forceinline__ void op_cell(const Tail& t, int op, int l, int cur, i
         arrive64(t, l, q, av, ar);
         return;
     }
-    const Faces f = faces_of(L, k, i, j, two_d);
-    const Sig2<double> sg = *t.sig(l, q);
-    const double ka = L.cdt * sg.sa, kt = L.cdt * (sg.sa + sg.ss);
-    double NE, NFx, NFy, fE, fF;
+    double NE, NFx, NFy;
+    bool fx;
     const int arr = op == TAIL_FIRST ? ARR_V : ARR_E + cur, buf = op == TAIL_FIRST ? 0 : cur;
-    sums64(t, l, arr, buf, f, i, j, two_d, NE, NFx, NFy, fE, fF);
+    sums64(t, l, arr, buf, k, q, two_d, NE, NFx, NFy, fx);
     const C u = *t.own<C>(l, arr, q);
     C b = *t.own<C>(l, ARR_F, q);
-    if (op != TAIL_PSEUDO) {
+    Coef co;
+    if (op == TAIL_PSEUDO) {
+        co = *t.own<Coef>(l, ARR_Q, q);
+    } else {
+        const Sig2<double> sg = *t.sig(l, q);
+        const double ka = L.cdt * sg.sa, kt = L.cdt * (sg.sa + sg.ss);
+        const double fE = fx ? L.cb : 1.0, fF = fx ? L.cbF : 1.0;
         const double T2 = u.T * u.T, src_e = ka * fma(-L.a_r, T2 * T2, u.E), dF = L.diag + kt;
         const C a = { fma(-fE, NE, fma(L.diag, u.E, src_e)), fma(-fF, NFx, dF * u.Fx),
                       fma(-fF, NFy, dF * u.Fy), fma(L.c_v, u.T, -src_e) };
@@ -275,16 +287,16 @@ __device__ __forceinline__ void op_cell(const Tail& t, int op, int l, int cur, i
         }
         b = C{ a.E + b.E, a.Fx + b.Fx, a.Fy + b.Fy, a.T + b.T };
         *t.own<C>(l, ARR_F, q) = b;
+        co = make_coef(1.0, ps.dtau, L.diag, ka, kt, L.a_r);
+        *t.own<Coef>(l, ARR_Q, q) = co;
     }
-    const double cbE = ps.dtau * fE, cbF = ps.dtau * fF;
-    const double tau = surely_admissible(u, b, (float)ps.s, (float)L.c)
-                           ? ps.dtau
-                           : limited_step(u, b, ps.dtau, ps.theta, ps.s, L.c);
+    const TailStep& ts = t.step[l];
+    const double cbE = fx ? ts.cbE : ps.dtau, cbF = fx ? ts.cbF : ps.dtau;
+    const double tau = limited_step64(u, b, ps.dtau, ps.theta, ps.s, L.c);
     bool ok;
-    const C o = local_solve64(make_coef(1.0, ps.dtau, L.diag, ka, kt, L.a_r),
-                              fma(ps.dtau, L.diag, 1.0), fma(ps.dtau, L.c_v, 1.0), L.a_r,
-                              fma(cbE, NE, fma(tau, b.E, u.E)), fma(cbF, NFx, fma(tau, b.Fx, u.Fx)),
-                              fma(cbF, NFy, fma(tau, b.Fy, u.Fy)), fma(tau, b.T, u.T), ok);
+    const C o = local_solve64(co, ts.A, ts.C, L.a_r, fma(cbE, NE, fma(tau, b.E, u.E)),
+                              fma(cbF, NFx, fma(tau, b.Fx, u.Fx)),
+                              fma(cbF, NFy, fma(tau, b.Fy, u.Fy)), fma(tau, b.T, u.T), ok, u.T);
     if (!ok) ++fails;
     const int out = op == TAIL_FIRST ? 1 : 1 - cur;
     *t.own<C>(l, ARR_E + out, q) = o;
@@ -301,11 +313,12 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const Level<double>* _
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ Level<double> Ls[kTailLevels];
     __shared__ TailGeo geo[kTailLevels];
+    __shared__ TailStep steps[kTailLevels];
     cg::cluster_group cl = cg::this_cluster();
     const int nb = (int)cl.num_blocks(), rank = (int)cl.block_rank();
     const int w0 = blockIdx.x / nb, ws = gridDim.x / nb;
     const int nw = *wl.count;
-    Tail t{ Ls, geo, smem, rank, cl };
+    Tail t{ Ls, geo, steps, smem, rank, cl };
     for (int w = w0; w < nw; w += ws) {
         const int2 it = wl.items[w];
         if (skip(ctls, it.x)) continue;            // the same for the whole cluster
@@ -337,6 +350,11 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const Level<double>* _
         }
         __syncthreads();
         const Pseudo<double> ps = pseudo_of<double>(ctl);
+        if (threadIdx.x < nl) {
+            const Level<double>& L = Ls[threadIdx.x];
+            steps[threadIdx.x] = TailStep{ ps.dtau * L.cb, ps.dtau * L.cbF, fma(ps.dtau, L.diag, 1.0),
+                                           fma(ps.dtau, L.c_v, 1.0) };
+        }
         const double theta_c = ctl->theta_c;
         unsigned fails = 0, damped = 0;
         for (int l = 0; l < nl; ++l)
@@ -344,6 +362,14 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const Level<double>* _
                 const int k = rank * geo[l].per + q;
                 if (k >= geo[l].n) break;
                 *t.sig(l, q) = Ls[l].sig[k];
+                const int j = Ls[l].dim == 2 ? row_of(geo[l], k) : 0, i = k - j * Ls[l].nx;
+                uint4 nb = make_uint4(side_code(t, l, k, i, j, WALL_W), side_code(t, l, k, i, j, WALL_E),
+                                      0u, 0u);
+                if (Ls[l].dim == 2) {
+                    nb.z = side_code(t, l, k, i, j, WALL_S);
+                    nb.w = side_code(t, l, k, i, j, WALL_N);
+                }
+                *t.own<uint4>(l, ARR_NB, q) = nb;
                 if (l == 0) arrive64(t, 0, q, Ls[0].v[k], Ls[0].r[k]);
             }
         unsigned curs = 0;                          // bit l: the buffer of level l's iterate
