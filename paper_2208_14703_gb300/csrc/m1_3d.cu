@@ -13,7 +13,7 @@
 
 #include <cstdio>
 
-#include "m1_3d.cuh"
+#include "m1_3fx.cuh"
 
 namespace m1 {
 void set_err(cudaError_t e, const char* what);
@@ -343,7 +343,7 @@ __global__ void __launch_bounds__(kThreads3) k_finalize3(Ctl* __restrict__ ctl,
                                                          BatchCtl* __restrict__ bctl,
                                                          const double* __restrict__ part,
                                                          const double* __restrict__ partb, int np,
-                                                         int mode)
+                                                         int npb, int mode)
 {
     __shared__ double red[kThreads3];
     if (mode != FIN3_INIT && ctl->done) return;
@@ -361,7 +361,7 @@ __global__ void __launch_bounds__(kThreads3) k_finalize3(Ctl* __restrict__ ctl,
     __syncthreads();
     double sb = 0.0;
     if (mode == FIN3_INIT) {
-        for (int k = threadIdx.x; k < np; k += blockDim.x) b += partb[k];
+        for (int k = threadIdx.x; k < npb; k += blockDim.x) b += partb[k];
         sb = block_sum3(b, red);
     }
     if (threadIdx.x != 0) return;
@@ -522,10 +522,10 @@ void launch3_norm_state(const G3& g, const EF* x, const double* xT, double* part
     k_norm_state3<<<blocks3(n), kThreads3, 0, s>>>(g, x, xT, part, n);
 }
 
-void launch3_finalize(Ctl* ctl, BatchCtl* bctl, const double* part, const double* partb, int np,
-                      int mode, cudaStream_t s)
+void launch3_finalize(Ctl* ctl, BatchCtl* bctl, const double* part, int np, const double* partb,
+                      int npb, int mode, cudaStream_t s)
 {
-    k_finalize3<<<1, kThreads3, 0, s>>>(ctl, bctl, part, partb, np, mode);
+    k_finalize3<<<1, kThreads3, 0, s>>>(ctl, bctl, part, partb, np, npb, mode);
 }
 
 void launch3_pack(const double* planes, EF* ef, double* T, size_t n, cudaStream_t s)
@@ -558,23 +558,26 @@ using m1::G3;
 using m1::P6;
 using m1::Sig2;
 
-// Device buffers of one call, freed on every return path.
-struct Buffers {
-    void* p[12] = {};
-    int count = 0;
-    ~Buffers()
+// The device memory of one call: one allocation, its arrays at 256-byte offsets,
+// freed on every return path.
+struct Arena {
+    unsigned char* base = nullptr;
+    size_t size = 0;
+    ~Arena()
     {
-        for (int k = 0; k < count; ++k)
-            if (p[k]) cudaFree(p[k]);
+        if (base) cudaFree(base);
     }
-    template <typename T>
-    cudaError_t get(T** out, size_t bytes)
+    size_t take(size_t bytes)
     {
-        void* q = nullptr;
-        const cudaError_t e = cudaMalloc(&q, bytes);
-        if (e == cudaSuccess) p[count++] = q;
-        *out = static_cast<T*>(q);
-        return e;
+        const size_t at = size;
+        size += (bytes + 255) & ~(size_t)255;
+        return at;
+    }
+    cudaError_t get() { return cudaMalloc(&base, size); }
+    template <typename T>
+    T* at(size_t off) const
+    {
+        return reinterpret_cast<T*>(base + off);
     }
 };
 
@@ -627,23 +630,41 @@ extern "C" m1_status m1_op_level3(const m1_grid3_desc* d, double dt, const doubl
     for (int a = 0; a < 3; ++a) g.beta[a] = dt / (2.0 * h[a]);
     g.vol = h[0] * h[1] * h[2];
 
+    m1::set_fx3(g);
+
+    // the fixed-point passes where their arrays fit the device, else the FP64 form (48
+    // bytes a cell of closures in place of 84 to 200 of blocks and coefficients)
     const cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    Buffers buf;
-    EF *u0 = nullptr, *u1 = nullptr, *b = nullptr;
-    double *T0 = nullptr, *T1 = nullptr, *bT = nullptr, *stage = nullptr;
-    P6* P = nullptr;
-    Sig2<double>* sg = nullptr;
-    M1_CK3(buf.get(&u0, n * sizeof(EF)));
-    M1_CK3(buf.get(&u1, n * sizeof(EF)));
-    M1_CK3(buf.get(&T0, n * sizeof(double)));
-    M1_CK3(buf.get(&T1, n * sizeof(double)));
-    M1_CK3(buf.get(&P, n * sizeof(P6)));
-    M1_CK3(buf.get(&sg, n * sizeof(Sig2<double>)));
-    if (rhs) {
-        M1_CK3(buf.get(&b, n * sizeof(EF)));
-        M1_CK3(buf.get(&bT, n * sizeof(double)));
+    const bool jac = mode == M1_OP3_JACOBI;
+    Arena mem;
+    size_t ou[2], oT[2], ob = 0, obT = 0, osg, ost = 0, oB[2] = { 0, 0 }, oQ = 0, oP = 0;
+    bool fx = g.fx != 0;
+    for (;;) {
+        mem.size = 0;
+        for (int k = 0; k < 2; ++k) {
+            ou[k] = mem.take(n * sizeof(EF));
+            oT[k] = mem.take(n * sizeof(double));
+            if (fx && (k == 0 || (jac && sweeps > 1))) oB[k] = mem.take(m1::blocks3_bytes(n));
+        }
+        osg = mem.take(n * sizeof(Sig2<double>));
+        if (rhs) {
+            ob = mem.take(n * sizeof(EF));
+            obT = mem.take(n * sizeof(double));
+        }
+        if (!on_device) ost = mem.take(5 * n * sizeof(double));
+        if (fx && jac) oQ = mem.take(n * sizeof(m1::Coef));
+        if (!fx) oP = mem.take(n * sizeof(P6));
+        const cudaError_t e = mem.get();
+        if (e == cudaSuccess) break;
+        mem.base = nullptr;
+        if (!fx || e != cudaErrorMemoryAllocation) M1_CK3(e);
+        cudaGetLastError();
+        fx = false;
     }
-    if (!on_device) M1_CK3(buf.get(&stage, 5 * n * sizeof(double)));
+    EF *u0 = mem.at<EF>(ou[0]), *u1 = mem.at<EF>(ou[1]), *b = rhs ? mem.at<EF>(ob) : nullptr;
+    double *T0 = mem.at<double>(oT[0]), *T1 = mem.at<double>(oT[1]);
+    double *bT = rhs ? mem.at<double>(obT) : nullptr, *stage = mem.at<double>(ost);
+    Sig2<double>* sg = mem.at<Sig2<double>>(osg);
 
     // caller planes -> device layout
     auto pack = [&](const double* src, EF* ef, double* T) -> cudaError_t {
@@ -679,12 +700,27 @@ extern "C" m1_status m1_op_level3(const m1_grid3_desc* d, double dt, const doubl
     double* curT = T0;
     EF* nxt = u1;
     double* nxtT = T1;
-    const int passes = mode == M1_OP3_JACOBI ? sweeps : 1;
+    const int passes = jac ? sweeps : 1;
     const int kmode = mode == M1_OP3_APPLY ? m1::OP3K_APPLY
                     : mode == M1_OP3_RESIDUAL ? m1::OP3K_RESID : m1::OP3K_JACOBI;
+    const int xmode = mode == M1_OP3_APPLY ? m1::OPX3_APPLY
+                    : mode == M1_OP3_RESIDUAL ? m1::OPX3_RESID : m1::OPX3_JACOBI;
+    if (fx) {
+        m1::launchx3_block(g, cur, m1::blocks3_at(mem.at<void>(oB[0]), n), n, nullptr, s);
+        if (jac) m1::launchx3_coef(g, sg, mem.at<m1::Coef>(oQ), n, s);
+    }
     for (int it = 0; it < passes; ++it) {
-        m1::launch3_closure(g, cur, P, n, nullptr, s);
-        m1::launch3_op(kmode, g, cur, curT, P, sg, b, bT, nxt, nxtT, n, nullptr, nullptr, s);
+        if (fx) {
+            m1::Blocks3 next{ nullptr, nullptr };
+            if (it + 1 < passes) next = m1::blocks3_at(mem.at<void>(oB[(it + 1) & 1]), n);
+            m1::launchx3_op(xmode, g, cur, curT, m1::blocks3_at(mem.at<void>(oB[it & 1]), n),
+                            mem.at<m1::Coef>(oQ), sg, b, bT, nullptr, nullptr, nxt, nxtT, next, n,
+                            nullptr, nullptr, s);
+        } else {
+            m1::launch3_closure(g, cur, mem.at<P6>(oP), n, nullptr, s);
+            m1::launch3_op(kmode, g, cur, curT, mem.at<P6>(oP), sg, b, bT, nxt, nxtT, n, nullptr,
+                           nullptr, s);
+        }
         M1_CK3(cudaGetLastError());
         EF* t = cur; cur = nxt; nxt = t;
         double* tt = curT; curT = nxtT; nxtT = tt;

@@ -30,7 +30,28 @@ struct G3 {
     double vol;                                                  // hx hy hz (norm weight)
     const double* in[6];                                         // inflow profiles, or null
     int fstride;
+    // the fixed-point form (m1_3fx.cuh): c b and c^2 b with b the largest beta, 1 / c,
+    // each axis' beta / b times 2^62 (0: equal), and whether a level may take it
+    double cb, cbF, ic;
+    long long rho[3];
+    int fx;
 };
+
+// Those constants from c and beta (the rule of the 2D levels).
+inline void set_fx3(G3& g)
+{
+    double b = g.beta[0], s = g.beta[0];
+    for (int a = 1; a < 3; ++a) {
+        b = g.beta[a] > b ? g.beta[a] : b;
+        s = g.beta[a] < s ? g.beta[a] : s;
+    }
+    g.cb = g.c * b;
+    g.cbF = g.c * g.c * b;
+    g.ic = 1.0 / g.c;
+    g.fx = g.c > 1e-60 && g.c < 1e60 && s > 1e-60 && b < 1e60;
+    for (int a = 0; a < 3; ++a)
+        g.rho[a] = g.fx && g.beta[a] < b ? (long long)(g.beta[a] / b * 4611686018427387904.0) : 0;
+}
 
 constexpr int kThreads3 = 256;
 constexpr int kMaxBlocks3 = 152 * 8;
@@ -279,6 +300,28 @@ void launch3_restrict_sig(const G3& gf, const G3& gc, const Sig2<double>* sf, Si
                           cudaStream_t s);
 void launch3_prolong(const G3& gc, const G3& gf, const EF* uc, const double* ucT, const EF* vc,
                      const double* vcT, EF* uf, double* ufT, Ctl* ctl, cudaStream_t s);
+// ---- the same passes in fixed point (m1_3fx.cuh): blocks of the states read and
+// written (B: of u; Bo: of out, its planes null when not wanted), the local solve's
+// coefficients Q.
+struct Blocks3;
+struct Coef;
+enum OpX3 { OPX3_APPLY = 0, OPX3_RESID = 1, OPX3_JACOBI = 2, OPX3_JACOBI_NORM = 3, OPX3_FIRST = 4,
+            OPX3_PSEUDO = 5 };
+void launchx3_block(const G3& g, const EF* u, const Blocks3& B, size_t n, const Ctl* ctl,
+                    cudaStream_t s);
+void launchx3_coef(const G3& g, const Sig2<double>* sig, Coef* Q, size_t n, cudaStream_t s);
+// FIRST: the first pseudo-time step of a fresh visit, from u = v with b = r: also the
+// FAS right-hand side (into f, fT) and the coefficients (into Q).
+void launchx3_op(int mode, const G3& g, const EF* u, const double* uT, const Blocks3& B, Coef* Q,
+                 const Sig2<double>* sig, const EF* b, const double* bT, EF* f, double* fT, EF* out,
+                 double* outT, const Blocks3& Bo, size_t n, Ctl* ctl, double* part, cudaStream_t s);
+void launchx3_restrict(const G3& gf, const G3& gc, const EF* u, const double* uT, const EF* r,
+                       const double* rT, EF* vc, double* vcT, EF* rc, double* rcT, const Blocks3& Bo,
+                       const Ctl* ctl, cudaStream_t s);
+void launchx3_prolong(const G3& gc, const G3& gf, const EF* uc, const double* ucT, const EF* vc,
+                      const double* vcT, EF* uf, double* ufT, const Blocks3& Bo, Ctl* ctl,
+                      cudaStream_t s);
+int blocksx3(size_t n);                                          // blocks (norm partials) of an operator pass
 void launch3_copy(const EF* src, const double* srcT, EF* dst, double* dstT, size_t n,
                   const Ctl* ctl, cudaStream_t s);
 void launch3_rhs(const G3& g, const EF* u, const double* uT, EF* b, double* bT, size_t n,
@@ -286,8 +329,9 @@ void launch3_rhs(const G3& g, const EF* u, const double* uT, EF* b, double* bT, 
 void launch3_norm_state(const G3& g, const EF* x, const double* xT, double* part, size_t n,
                         cudaStream_t s);
 enum { FIN3_INIT = 0, FIN3_CYCLE = 1, FIN3_DEFER = 2 };
-void launch3_finalize(Ctl* ctl, BatchCtl* bctl, const double* part, const double* partb, int np,
-                      int mode, cudaStream_t s);
+// np, npb: entries of part and of partb (INIT)
+void launch3_finalize(Ctl* ctl, BatchCtl* bctl, const double* part, int np, const double* partb,
+                      int npb, int mode, cudaStream_t s);
 void launch3_pack(const double* planes, EF* ef, double* T, size_t n, cudaStream_t s);
 void launch3_unpack(const EF* ef, const double* T, double* planes, size_t n, cudaStream_t s);
 void launch3_pack_sig(const double* planes, Sig2<double>* sig, size_t n, cudaStream_t s);

@@ -29,7 +29,7 @@
 #include <memory>
 #include <vector>
 
-#include "m1_3d.cuh"
+#include "m1_3fx.cuh"
 #include "m1_engine.h"
 
 namespace m1 {
@@ -41,7 +41,10 @@ struct Lev3 {
     size_t n = 0;
     EF *v = nullptr, *u[2] = { nullptr, nullptr }, *f = nullptr, *r = nullptr;
     double *vT = nullptr, *uT[2] = { nullptr, nullptr }, *fT = nullptr, *rT = nullptr;
-    P6* P = nullptr;
+    P6* P = nullptr;                        // FP64 form only
+    Blocks3 B[2] = {};                      // fixed point: blocks of u[0], u[1] (u[1]'s first of v;
+                                            // level 0: of v and u[0])
+    Coef* Q = nullptr;                      // ... and the local solve's coefficients
     Sig2<double>* sig = nullptr;
     double* prof = nullptr;                 // [6][4][fstride] inflow profiles (inflow walls only)
 };
@@ -55,6 +58,7 @@ size_t face_max3(const int n[3])
 struct Grid3 {
     m1_grid3_desc desc{};
     int L = 0;
+    bool fx = true;                         // the fixed-point passes; false: their arrays did not fit
     cudaStream_t stream = nullptr, cap_stream = nullptr;
     bool own_stream = false;
     std::vector<Lev3> lv;
@@ -103,11 +107,15 @@ struct Grid3 {
     }
 
     m1_status init(const m1_grid3_desc& d, int lmax, cudaStream_t s);
+    m1_status alloc_levels();
+    void emit_sweeps_fx(int nsweeps, bool deferred, cudaStream_t s);
     void set_dt(double dt);
     void emit_sweeps_fine(int nsweeps, cudaStream_t s);
     void emit_pseudo(int l, int steps, cudaStream_t s);
     void emit_visit(int l, bool fresh, int shape, const Params& p, cudaStream_t s);
     void emit_corrections(int l, int shape, const Params& p, cudaStream_t s);
+    void emit_down(int l, EF* u, double* uT, int a, cudaStream_t s);
+    void emit_up(int l, EF* u, double* uT, int a, cudaStream_t s);
     void emit_cycle(const Params& p, cudaStream_t s);
     m1_status build_graph(const Params& p, double dt);
     m1_status set_state(const double* state, const double* sig, int on_device);
@@ -144,22 +152,17 @@ m1_status Grid3::init(const m1_grid3_desc& d, int lmax, cudaStream_t s)
         q.g.ic2 = 1.0 / (d.c * d.c);
         q.g.vol = q.h[0] * q.h[1] * q.h[2];
         q.n = (size_t)q.g.n[0] * q.g.n[1] * q.g.n[2];
-        M1_TRY(alloc(&q.v, q.n)); M1_TRY(alloc(&q.vT, q.n));
-        for (int b = 0; b < 2; ++b) { M1_TRY(alloc(&q.u[b], q.n)); M1_TRY(alloc(&q.uT[b], q.n)); }
-        M1_TRY(alloc(&q.f, q.n)); M1_TRY(alloc(&q.fT, q.n));
-        M1_TRY(alloc(&q.r, q.n)); M1_TRY(alloc(&q.rT, q.n));
-        M1_TRY(alloc(&q.P, q.n));
-        M1_TRY(alloc(&q.sig, q.n));
-        if (has_inflow) {
-            q.g.fstride = (int)face_max3(q.g.n);
-            M1_TRY(alloc(&q.prof, (size_t)6 * 4 * q.g.fstride));
-            M1_CK(cudaMemsetAsync(q.prof, 0, sizeof(double) * 6 * 4 * q.g.fstride, stream));
-            for (int w = 0; w < 6; ++w)
-                q.g.in[w] = d.bc[w] == M1_BC_INFLOW ? q.prof + (size_t)w * 4 * q.g.fstride : nullptr;
-        }
     }
-    M1_TRY(alloc(&stage, 5 * lv[0].n));
-    M1_TRY(alloc(&part, kMaxBlocks3));
+    m1_status st = alloc_levels();
+    if (st == M1_ERR_OOM) {                 // without the blocks (the FP64 form)
+        for (void* p : mem) cudaFree(p);
+        mem.clear();
+        cudaGetLastError();
+        fx = false;
+        st = alloc_levels();
+    }
+    M1_TRY(st);
+    M1_TRY(alloc(&part, blocksx3((size_t)1 << 31)));
     M1_TRY(alloc(&partb, kMaxBlocks3));
     M1_TRY(alloc(&ctl, 1));
     M1_TRY(alloc(&bctl, 1));
@@ -175,6 +178,42 @@ m1_status Grid3::init(const m1_grid3_desc& d, int lmax, cudaStream_t s)
     return M1_OK;
 }
 
+// The levels' arrays.  Level 0 in fixed point sweeps between v and u[0] (v is free
+// once the first sweep of a cycle has read it and the stop test is taken).
+m1_status Grid3::alloc_levels()
+{
+    M1_TRY(alloc(&stage, 5 * lv[0].n));
+    for (int l = 0; l < L; ++l) {
+        Lev3& q = lv[l];
+        M1_TRY(alloc(&q.v, q.n)); M1_TRY(alloc(&q.vT, q.n));
+        for (int b = 0; b < (fx && l == 0 ? 1 : 2); ++b) {
+            M1_TRY(alloc(&q.u[b], q.n));
+            M1_TRY(alloc(&q.uT[b], q.n));
+        }
+        M1_TRY(alloc(&q.f, q.n)); M1_TRY(alloc(&q.fT, q.n));
+        M1_TRY(alloc(&q.r, q.n)); M1_TRY(alloc(&q.rT, q.n));
+        M1_TRY(alloc(&q.sig, q.n));
+        if (fx) {
+            for (auto& B : q.B) {
+                unsigned char* p = nullptr;
+                M1_TRY(alloc(&p, blocks3_bytes(q.n)));
+                B = blocks3_at(p, q.n);
+            }
+            M1_TRY(alloc(&q.Q, q.n));
+        } else {
+            M1_TRY(alloc(&q.P, q.n));
+        }
+        if (has_inflow) {
+            q.g.fstride = (int)face_max3(q.g.n);
+            M1_TRY(alloc(&q.prof, (size_t)6 * 4 * q.g.fstride));
+            M1_CK(cudaMemsetAsync(q.prof, 0, sizeof(double) * 6 * 4 * q.g.fstride, stream));
+            for (int w = 0; w < 6; ++w)
+                q.g.in[w] = desc.bc[w] == M1_BC_INFLOW ? q.prof + (size_t)w * 4 * q.g.fstride : nullptr;
+        }
+    }
+    return M1_OK;
+}
+
 // The constants of every level that depend on the time step.
 void Grid3::set_dt(double dt)
 {
@@ -185,6 +224,7 @@ void Grid3::set_dt(double dt)
             q.g.diag += q.g.c * dt / q.h[a];
             q.g.beta[a] = dt / (2.0 * q.h[a]);
         }
+        set_fx3(q.g);
     }
 }
 
@@ -205,16 +245,47 @@ void Grid3::emit_sweeps_fine(int nsweeps, cudaStream_t s)
                    q.u[dst], q.uT[dst], q.n, ctl, first ? part : nullptr, s);
         kernels_per_cycle += 2;
         if (first) {
-            launch3_finalize(ctl, bctl, part, nullptr, blocks3(q.n), FIN3_DEFER, s);
+            launch3_finalize(ctl, bctl, part, blocks3(q.n), nullptr, 0, FIN3_DEFER, s);
             kernels_per_cycle += 1;
         }
         cur[0] = dst;
     }
 }
 
+// The same in fixed point, between v (buffer 0) and u[0] (buffer 1) of level 0;
+// deferred: the first sweep also takes the stop test of the cycle before.
+void Grid3::emit_sweeps_fx(int nsweeps, bool deferred, cudaStream_t s)
+{
+    Lev3& q = lv[0];
+    EF* x[2] = { q.v, q.u[0] };
+    double* xT[2] = { q.vT, q.uT[0] };
+    for (int k = 0; k < nsweeps; ++k) {
+        const int a = cur[0], b = 1 - a;
+        const bool first = deferred && k == 0;
+        launchx3_op(first ? OPX3_JACOBI_NORM : OPX3_JACOBI, q.g, x[a], xT[a], q.B[a], q.Q, q.sig, q.f,
+                    q.fT, nullptr, nullptr, x[b], xT[b], q.B[b], q.n, ctl, first ? part : nullptr, s);
+        kernels_per_cycle += 1;
+        if (first) {
+            launch3_finalize(ctl, bctl, part, blocksx3(q.n), nullptr, 0, FIN3_DEFER, s);
+            kernels_per_cycle += 1;
+        }
+        cur[0] = b;
+    }
+}
+
 void Grid3::emit_pseudo(int l, int steps, cudaStream_t s)
 {
     Lev3& q = lv[l];
+    if (fx) {
+        for (int k = 0; k < steps; ++k) {
+            const int a = cur[l], b = a ^ 1;
+            launchx3_op(OPX3_PSEUDO, q.g, q.u[a], q.uT[a], q.B[a], q.Q, q.sig, q.f, q.fT, nullptr,
+                        nullptr, q.u[b], q.uT[b], q.B[b], q.n, ctl, nullptr, s);
+            kernels_per_cycle += 1;
+            cur[l] = b;
+        }
+        return;
+    }
     for (int k = 0; k < steps; ++k) {
         const int a = cur[l], b = a ^ 1;
         launch3_closure(q.g, q.u[a], q.P, q.n, ctl, s);
@@ -241,47 +312,86 @@ void Grid3::emit_corrections(int l, int shape, const Params& p, cudaStream_t s)
 void Grid3::emit_visit(int l, bool fresh, int shape, const Params& p, cudaStream_t s)
 {
     Lev3& q = lv[l];
-    if (fresh) {
+    int steps = l == L - 1 ? p.mc : p.m;
+    if (fresh && fx) {
+        launchx3_op(OPX3_FIRST, q.g, q.v, q.vT, q.B[1], q.Q, q.sig, q.r, q.rT, q.f, q.fT, q.u[0],
+                    q.uT[0], q.B[0], q.n, ctl, nullptr, s);
+        kernels_per_cycle += 1;
+        cur[l] = 0;
+        --steps;
+    } else if (fresh) {
         launch3_closure(q.g, q.v, q.P, q.n, ctl, s);
         launch3_op(OP3K_FAS, q.g, q.v, q.vT, q.P, q.sig, q.r, q.rT, q.f, q.fT, q.n, ctl, nullptr, s);
         launch3_copy(q.v, q.vT, q.u[0], q.uT[0], q.n, ctl, s);
         kernels_per_cycle += 3;
         cur[l] = 0;
     }
-    if (l == L - 1) {
-        emit_pseudo(l, p.mc, s);
+    emit_pseudo(l, steps, s);
+    if (l == L - 1) return;
+    const int a = cur[l];
+    emit_down(l, q.u[a], q.uT[a], a, s);
+    emit_corrections(l, shape, p, s);
+    emit_up(l, q.u[a], q.uT[a], a, s);
+    emit_pseudo(l, p.m, s);
+}
+
+// The residual of the iterate u (blocks B[a]) of level l and its restriction to the
+// next level.
+void Grid3::emit_down(int l, EF* u, double* uT, int a, cudaStream_t s)
+{
+    Lev3 &q = lv[l], &c = lv[l + 1];
+    if (fx) {
+        launchx3_op(OPX3_RESID, q.g, u, uT, q.B[a], q.Q, q.sig, q.f, q.fT, nullptr, nullptr, q.r, q.rT,
+                    Blocks3{}, q.n, ctl, nullptr, s);
+        launchx3_restrict(q.g, c.g, u, uT, q.r, q.rT, c.v, c.vT, c.r, c.rT, c.B[1], ctl, s);
+        kernels_per_cycle += 2;
         return;
     }
-    emit_pseudo(l, p.m, s);
-    Lev3& c = lv[l + 1];
-    const int a = cur[l];
-    launch3_closure(q.g, q.u[a], q.P, q.n, ctl, s);
-    launch3_op(OP3K_RESID, q.g, q.u[a], q.uT[a], q.P, q.sig, q.f, q.fT, q.r, q.rT, q.n, ctl,
-               nullptr, s);
-    launch3_restrict(q.g, c.g, q.u[a], q.uT[a], q.r, q.rT, c.v, c.vT, c.r, c.rT, ctl, s);
+    launch3_closure(q.g, u, q.P, q.n, ctl, s);
+    launch3_op(OP3K_RESID, q.g, u, uT, q.P, q.sig, q.f, q.fT, q.r, q.rT, q.n, ctl, nullptr, s);
+    launch3_restrict(q.g, c.g, u, uT, q.r, q.rT, c.v, c.vT, c.r, c.rT, ctl, s);
     kernels_per_cycle += 3;
-    emit_corrections(l, shape, p, s);
-    launch3_prolong(c.g, q.g, c.u[cur[l + 1]], c.uT[cur[l + 1]], c.v, c.vT, q.u[a], q.uT[a], ctl, s);
+}
+
+// The prolongation of the next level's correction onto the iterate u of level l.
+void Grid3::emit_up(int l, EF* u, double* uT, int a, cudaStream_t s)
+{
+    Lev3 &q = lv[l], &c = lv[l + 1];
+    const int b = cur[l + 1];
+    if (fx) launchx3_prolong(c.g, q.g, c.u[b], c.uT[b], c.v, c.vT, u, uT, q.B[a], ctl, s);
+    else launch3_prolong(c.g, q.g, c.u[b], c.uT[b], c.v, c.vT, u, uT, ctl, s);
     kernels_per_cycle += 1;
-    emit_pseudo(l, p.m, s);
 }
 
 void Grid3::emit_cycle(const Params& p, cudaStream_t s)
 {
     Lev3& q = lv[0];
+    if (fx) {
+        cur[0] = 0;                                 // v
+        emit_sweeps_fx(p.nu0, true, s);
+        if (L > 1) {
+            const int a = cur[0];
+            EF* u = a ? q.u[0] : q.v;
+            double* uT = a ? q.uT[0] : q.vT;
+            emit_down(0, u, uT, a, s);
+            emit_corrections(0, p.cycle, p, s);
+            emit_up(0, u, uT, a, s);
+            emit_sweeps_fx(p.nu0, false, s);
+        }
+        if (cur[0] == 1) {                          // an odd count: back to v
+            launch3_copy(q.u[0], q.uT[0], q.v, q.vT, q.n, ctl, s);
+            launchx3_block(q.g, q.v, q.B[0], q.n, ctl, s);
+            kernels_per_cycle += 2;
+        }
+        return;
+    }
     cur[0] = -1;                                    // the first sweep reads v
     emit_sweeps_fine(p.nu0, s);
     if (L > 1) {
-        Lev3& c = lv[1];
         const int a = cur[0];
-        launch3_closure(q.g, q.u[a], q.P, q.n, ctl, s);
-        launch3_op(OP3K_RESID, q.g, q.u[a], q.uT[a], q.P, q.sig, q.f, q.fT, q.r, q.rT, q.n, ctl,
-                   nullptr, s);
-        launch3_restrict(q.g, c.g, q.u[a], q.uT[a], q.r, q.rT, c.v, c.vT, c.r, c.rT, ctl, s);
-        kernels_per_cycle += 3;
+        emit_down(0, q.u[a], q.uT[a], a, s);
         emit_corrections(0, p.cycle, p, s);
-        launch3_prolong(c.g, q.g, c.u[cur[1]], c.uT[cur[1]], c.v, c.vT, q.u[a], q.uT[a], ctl, s);
-        kernels_per_cycle += 1;
+        emit_up(0, q.u[a], q.uT[a], a, s);
         emit_sweeps_fine(p.nu0, s);
     }
     // end of the cycle: v <- u; its residual norm, stop test and dtau_im update
@@ -415,10 +525,17 @@ m1_status Grid3::step(double dt, const m1_solve_params& sp, m1_step_stats* st)
     Lev3& q = lv[0];
     const int np = blocks3(q.n);
     launch3_rhs(q.g, q.v, q.vT, q.f, q.fT, q.n, stream);
-    launch3_closure(q.g, q.v, q.P, q.n, ctl, stream);
-    launch3_op(OP3K_RESID, q.g, q.v, q.vT, q.P, q.sig, q.f, q.fT, q.r, q.rT, q.n, ctl, part, stream);
+    if (fx) {
+        launchx3_block(q.g, q.v, q.B[0], q.n, nullptr, stream);
+        launchx3_coef(q.g, q.sig, q.Q, q.n, stream);
+        launchx3_op(OPX3_RESID, q.g, q.v, q.vT, q.B[0], q.Q, q.sig, q.f, q.fT, nullptr, nullptr, q.r,
+                    q.rT, Blocks3{}, q.n, ctl, part, stream);
+    } else {
+        launch3_closure(q.g, q.v, q.P, q.n, ctl, stream);
+        launch3_op(OP3K_RESID, q.g, q.v, q.vT, q.P, q.sig, q.f, q.fT, q.r, q.rT, q.n, ctl, part, stream);
+    }
     launch3_norm_state(q.g, q.f, q.fT, partb, q.n, stream);
-    launch3_finalize(ctl, bctl, part, partb, np, FIN3_INIT, stream);
+    launch3_finalize(ctl, bctl, part, fx ? blocksx3(q.n) : np, partb, np, FIN3_INIT, stream);
     M1_CK(cudaGetLastError());
     long long launched = 0;
     M1_TRY(run_until_done(graph, 1, sp.max_cycles, stream, bctl, done_h, poll, &launched));
@@ -439,7 +556,7 @@ m1_status Grid3::step(double dt, const m1_solve_params& sp, m1_step_stats* st)
         st->status = r.status;
         st->newton_fail = r.newton_fail;
         st->damped = r.damped;
-        st->launches = 5 + launched * kernels_per_cycle;
+        st->launches = (fx ? 6 : 5) + launched * kernels_per_cycle;
     }
     return r.status == CTL_OK ? M1_OK : M1_ERR_NOT_CONVERGED;
 }

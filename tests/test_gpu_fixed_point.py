@@ -11,7 +11,9 @@ import numpy as np
 import pytest
 
 from oracle import oracle as O
+from oracle import oracle3d as O3
 from paper_2208_14703_gb300 import inputs
+from tests.test_oracle3d import opacities, random_state3
 
 pytestmark = pytest.mark.gpu
 
@@ -51,6 +53,7 @@ CASES = [
                          bc=("inflow", "reflect", "neumann", "inflow"))),
     ("out-of-range", dict(nx=70, ny=40, ly=40 / 70, c=1.0, spread=1, bc=("reflect",) * 4, seed=6,
                           tiny=5)),
+    ("no-blocks", dict(nx=40, ny=18, ly=0.5, c=1e61, spread=1, bc=("reflect",) * 4, seed=8)),
 ]
 
 
@@ -105,3 +108,56 @@ def test_strips_with_nan_stay_local():
     assert np.isfinite(got[:, far]).all()
     big = np.abs(clean).max()
     assert np.max(np.abs(got[:, far] - clean[:, far])) <= 1e-12 * big
+
+
+def _local3(x, bc):
+    p = np.pad(np.abs(x), 1, mode="wrap" if bc[0] == "periodic" else "edge")
+    c = slice(1, -1)
+    return np.max([p[c, c, c], p[:-2, c, c], p[2:, c, c], p[c, :-2, c], p[c, 2:, c], p[c, c, :-2],
+                   p[c, c, 2:]], axis=0)
+
+
+@pytest.mark.parametrize("name,dims,lengths,c,spread,bc,tiny", [
+    ("equal", (33, 5, 4), (33.0, 5.0, 4.0), 1.0, 0, ("reflect",) * 6, 0),
+    ("unequal-cells", (9, 31, 3), (1.0, 0.7, 2.0), 1.0, 2, ("periodic",) * 6, 0),
+    ("unequal-states", (16, 8, 8), (16.0, 8.0, 8.0), 1.0, 40, ("neumann",) * 6, 0),
+    ("light-speed", (7, 6, 20), (1.0, 1.0, 1.0), 2.9979e3, 1, ("reflect",) * 6, 0),
+    ("out-of-range", (12, 11, 9), (1.2, 1.1, 0.9), 1.0, 1, ("reflect",) * 6, 6),
+    ("no-blocks", (12, 6, 5), (1.0, 1.0, 1.0), 1e61, 1, ("reflect",) * 6, 0),
+])
+def test_fixed_point_3d_matches_oracle(name, dims, lengths, c, spread, bc, tiny):
+    """A(u) and two Jacobi sweeps in 3D, on the scale of each cell's stencil."""
+    nx, ny, nz = dims
+    h = [lengths[a] / dims[a] for a in range(3)]
+    dt = 3.0 * min(h) / c
+    g = O3.Grid3(nx, ny, nz, *h, bc, c)
+    d = m1.make_desc3(nx, ny, nz, *lengths, bc, c)
+    rng = np.random.default_rng(11)
+    s, b = random_state3(nx, ny, nz, 50, fmax=1.0), random_state3(nx, ny, nz, 51, fmax=0.95)
+    if spread:
+        s[:4] *= 10.0 ** rng.uniform(-spread, spread, (nz, ny, nx))
+    if tiny:
+        k, j, i = (rng.integers(0, n, tiny) for n in (nz, ny, nx))
+        s[0][k, j, i], s[1:4, k, j, i] = 1e-170, 0.0
+    s[1:4] *= c
+    b[1:4] *= c
+    sa, ss = opacities((nz, ny, nx), 52)
+    sa, ss = sa / c, ss / c
+    sig = np.stack([sa, ss])
+    stiff = 1.0 + 3.0 * sum(min(h) / x for x in h) + c * dt * (sa + ss)
+    got, _ = m1.m1_op_level3(d, dt, sig, s, mode=m1.OP3_APPLY)
+    ref = O3.apply_A(g, dt, sa, ss, s)
+    big = stiff * (_local3(s[0], bc) + s[4] ** 4 + s[4])
+    for f, unit in enumerate((1.0, c, c, c, 1.0)):
+        assert np.max(np.abs(got[f] - ref[f]) / (big * unit)) <= 1e-12, (name, f)
+    # two sweeps: the second takes the blocks the first one wrote; E and F on the scale
+    # of the stencil of the first one's result, T by its row
+    got, _ = m1.m1_op_level3(d, dt, sig, s, rhs=b, mode=m1.OP3_JACOBI, sweeps=2)
+    one, _ = O3.jacobi_sweep(g, dt, sa, ss, b, s)
+    ref, _ = O3.jacobi_sweep(g, dt, sa, ss, b, one)
+    big = _local3(_local3(s[0], bc) + b[0] + b[4], bc) + ref[4] ** 4
+    for f, unit in enumerate((1.0, c, c, c)):
+        assert np.max(np.abs(got[f] - ref[f]) / (big * unit)) <= 1e-12, (name, f)
+    ka, T = c * dt * sa, got[4]
+    row = T - ka * (got[0] - T ** 4) - b[4]
+    assert np.max(np.abs(row) / (T + ka * (big + T ** 4) + b[4])) <= 1e-12
