@@ -601,6 +601,99 @@ struct Events {
         }                                                                                          \
     } while (0)
 
+namespace {
+
+// Whether the two ranges of doubles share memory.
+bool overlap(const double* a, size_t na, const double* b, size_t nb)
+{
+    return a && b && a < b + nb && b < a + na;
+}
+
+// m1_op_level3 in fixed point, on the caller's planes themselves (host callers':
+// staged): blocks of the state, then one pass a sweep, 84 or 168 bytes a cell of
+// device memory where packed copies and closures took 250 to 290 (the allocation is a
+// good part of such a call).  done is left false where the FP64 form has to take the
+// call: the output shares memory with an input, the blocks do not fit, or a cell has
+// no block.
+m1_status op3_fx(const G3& g, size_t n, const double* sig, const double* state, const double* rhs,
+                 int mode, int sweeps, double* out, int on_device, cudaStream_t s, double* ms, bool& done)
+{
+    const bool jac = mode == M1_OP3_JACOBI;
+    if (on_device && (overlap(out, 5 * n, state, 5 * n) || overlap(out, 5 * n, rhs, 5 * n) ||
+                      overlap(out, 5 * n, sig, 2 * n)))
+        return M1_OK;
+    Arena mem;
+    size_t oB[2] = { mem.take(m1::blocks3_bytes(n)), 0 };
+    if (jac && sweeps > 1) oB[1] = mem.take(m1::blocks3_bytes(n));
+    const size_t oflag = mem.take(sizeof(int));
+    const size_t ost = on_device ? 0 : mem.take(5 * n * sizeof(double));
+    const size_t osg = on_device ? 0 : mem.take(2 * n * sizeof(double));
+    const size_t ob = on_device || !rhs ? 0 : mem.take(5 * n * sizeof(double));
+    const size_t oo = on_device ? 0 : mem.take(5 * n * sizeof(double));
+    const cudaError_t e = mem.get();
+    if (e == cudaErrorMemoryAllocation) {
+        mem.base = nullptr;
+        cudaGetLastError();
+        return M1_OK;
+    }
+    done = true;                                 // from here every error is the call's
+    M1_CK3(e);
+    const double *du = state, *dsig = sig, *db = rhs;
+    double* dout = out;
+    if (!on_device) {
+        M1_CK3(cudaMemcpyAsync(mem.at<double>(ost), state, 5 * n * sizeof(double),
+                               cudaMemcpyHostToDevice, s));
+        M1_CK3(cudaMemcpyAsync(mem.at<double>(osg), sig, 2 * n * sizeof(double),
+                               cudaMemcpyHostToDevice, s));
+        if (rhs)
+            M1_CK3(cudaMemcpyAsync(mem.at<double>(ob), rhs, 5 * n * sizeof(double),
+                                   cudaMemcpyHostToDevice, s));
+        du = mem.at<double>(ost);
+        dsig = mem.at<double>(osg);
+        db = rhs ? mem.at<double>(ob) : nullptr;
+        dout = mem.at<double>(oo);
+    }
+    int* flag = mem.at<int>(oflag);
+    M1_CK3(cudaMemsetAsync(flag, 0, sizeof(int), s));
+    Events ev;
+    if (ms) {
+        M1_CK3(cudaEventCreate(&ev.e[0]));
+        M1_CK3(cudaEventCreate(&ev.e[1]));
+        M1_CK3(cudaEventRecord(ev.e[0], s));
+    }
+    m1::Blocks3 B[2] = { m1::blocks3_at(mem.at<void>(oB[0]), n), m1::blocks3_at(mem.at<void>(oB[1]), n) };
+    m1::launchx3_block_planar(g, du, B[0], n, s);
+    const int passes = jac ? sweeps : 1;
+    const int xmode = mode == M1_OP3_APPLY ? m1::OPX3_APPLY
+                    : mode == M1_OP3_RESIDUAL ? m1::OPX3_RESID : m1::OPX3_JACOBI;
+    for (int it = 0; it < passes; ++it) {
+        const bool last = it + 1 == passes;
+        m1::launchx3_planar(xmode, g, du, B[it & 1], dsig, db, last ? dout : nullptr,
+                            last ? m1::Blocks3{} : B[(it + 1) & 1], n, flag, s);
+    }
+    M1_CK3(cudaGetLastError());
+    if (ms) M1_CK3(cudaEventRecord(ev.e[1], s));
+    int irregular = 0;
+    M1_CK3(cudaMemcpyAsync(&irregular, flag, sizeof(int), cudaMemcpyDeviceToHost, s));
+    M1_CK3(cudaStreamSynchronize(s));
+    if (irregular) {
+        done = false;
+        return M1_OK;
+    }
+    if (!on_device) {
+        M1_CK3(cudaMemcpyAsync(out, dout, 5 * n * sizeof(double), cudaMemcpyDeviceToHost, s));
+        M1_CK3(cudaStreamSynchronize(s));
+    }
+    if (ms) {
+        float t = 0.f;
+        M1_CK3(cudaEventElapsedTime(&t, ev.e[0], ev.e[1]));
+        *ms = t;
+    }
+    return M1_OK;
+}
+
+}  // namespace
+
 extern "C" m1_status m1_op_level3(const m1_grid3_desc* d, double dt, const double* sig,
                                   const double* state, const double* rhs, int mode, int sweeps,
                                   double* out, int on_device, void* cuda_stream, double* ms)
@@ -631,39 +724,25 @@ extern "C" m1_status m1_op_level3(const m1_grid3_desc* d, double dt, const doubl
     g.vol = h[0] * h[1] * h[2];
 
     m1::set_fx3(g);
-
-    // the fixed-point passes where their arrays fit the device, else the FP64 form (48
-    // bytes a cell of closures in place of 84 to 200 of blocks and coefficients)
     const cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    const bool jac = mode == M1_OP3_JACOBI;
-    Arena mem;
-    size_t ou[2], oT[2], ob = 0, obT = 0, osg, ost = 0, oB[2] = { 0, 0 }, oQ = 0, oP = 0;
-    bool fx = g.fx != 0;
-    for (;;) {
-        mem.size = 0;
-        for (int k = 0; k < 2; ++k) {
-            ou[k] = mem.take(n * sizeof(EF));
-            oT[k] = mem.take(n * sizeof(double));
-            if (fx && (k == 0 || (jac && sweeps > 1))) oB[k] = mem.take(m1::blocks3_bytes(n));
-        }
-        osg = mem.take(n * sizeof(Sig2<double>));
-        if (rhs) {
-            ob = mem.take(n * sizeof(EF));
-            obT = mem.take(n * sizeof(double));
-        }
-        if (!on_device) ost = mem.take(5 * n * sizeof(double));
-        if (fx && jac) oQ = mem.take(n * sizeof(m1::Coef));
-        if (!fx) oP = mem.take(n * sizeof(P6));
-        const cudaError_t e = mem.get();
-        if (e == cudaSuccess) break;
-        mem.base = nullptr;
-        if (!fx || e != cudaErrorMemoryAllocation) M1_CK3(e);
-        cudaGetLastError();
-        fx = false;
+    if (g.fx) {
+        bool done = false;
+        const m1_status st = op3_fx(g, n, sig, state, rhs, mode, sweeps, out, on_device, s, ms, done);
+        if (done) return st;
     }
-    EF *u0 = mem.at<EF>(ou[0]), *u1 = mem.at<EF>(ou[1]), *b = rhs ? mem.at<EF>(ob) : nullptr;
-    double *T0 = mem.at<double>(oT[0]), *T1 = mem.at<double>(oT[1]);
+
+    // the FP64 form
+    Arena mem;
+    const size_t ou0 = mem.take(n * sizeof(EF)), ou1 = mem.take(n * sizeof(EF));
+    const size_t oT0 = mem.take(n * sizeof(double)), oT1 = mem.take(n * sizeof(double));
+    const size_t oP = mem.take(n * sizeof(P6)), osg = mem.take(n * sizeof(Sig2<double>));
+    const size_t ob = rhs ? mem.take(n * sizeof(EF)) : 0, obT = rhs ? mem.take(n * sizeof(double)) : 0;
+    const size_t ost = on_device ? 0 : mem.take(5 * n * sizeof(double));
+    M1_CK3(mem.get());
+    EF *u0 = mem.at<EF>(ou0), *u1 = mem.at<EF>(ou1), *b = rhs ? mem.at<EF>(ob) : nullptr;
+    double *T0 = mem.at<double>(oT0), *T1 = mem.at<double>(oT1);
     double *bT = rhs ? mem.at<double>(obT) : nullptr, *stage = mem.at<double>(ost);
+    P6* P = mem.at<P6>(oP);
     Sig2<double>* sg = mem.at<Sig2<double>>(osg);
 
     // caller planes -> device layout
@@ -700,27 +779,12 @@ extern "C" m1_status m1_op_level3(const m1_grid3_desc* d, double dt, const doubl
     double* curT = T0;
     EF* nxt = u1;
     double* nxtT = T1;
-    const int passes = jac ? sweeps : 1;
+    const int passes = mode == M1_OP3_JACOBI ? sweeps : 1;
     const int kmode = mode == M1_OP3_APPLY ? m1::OP3K_APPLY
                     : mode == M1_OP3_RESIDUAL ? m1::OP3K_RESID : m1::OP3K_JACOBI;
-    const int xmode = mode == M1_OP3_APPLY ? m1::OPX3_APPLY
-                    : mode == M1_OP3_RESIDUAL ? m1::OPX3_RESID : m1::OPX3_JACOBI;
-    if (fx) {
-        m1::launchx3_block(g, cur, m1::blocks3_at(mem.at<void>(oB[0]), n), n, nullptr, s);
-        if (jac) m1::launchx3_coef(g, sg, mem.at<m1::Coef>(oQ), n, s);
-    }
     for (int it = 0; it < passes; ++it) {
-        if (fx) {
-            m1::Blocks3 next{ nullptr, nullptr };
-            if (it + 1 < passes) next = m1::blocks3_at(mem.at<void>(oB[(it + 1) & 1]), n);
-            m1::launchx3_op(xmode, g, cur, curT, m1::blocks3_at(mem.at<void>(oB[it & 1]), n),
-                            mem.at<m1::Coef>(oQ), sg, b, bT, nullptr, nullptr, nxt, nxtT, next, n,
-                            nullptr, nullptr, s);
-        } else {
-            m1::launch3_closure(g, cur, mem.at<P6>(oP), n, nullptr, s);
-            m1::launch3_op(kmode, g, cur, curT, mem.at<P6>(oP), sg, b, bT, nxt, nxtT, n, nullptr,
-                           nullptr, s);
-        }
+        m1::launch3_closure(g, cur, P, n, nullptr, s);
+        m1::launch3_op(kmode, g, cur, curT, P, sg, b, bT, nxt, nxtT, n, nullptr, nullptr, s);
         M1_CK3(cudaGetLastError());
         EF* t = cur; cur = nxt; nxt = t;
         double* tt = curT; curT = nxtT; nxtT = tt;

@@ -315,6 +315,13 @@ void launchx3_coef(const G3& g, const Sig2<double>* sig, Coef* Q, size_t n, cuda
 void launchx3_op(int mode, const G3& g, const EF* u, const double* uT, const Blocks3& B, Coef* Q,
                  const Sig2<double>* sig, const EF* b, const double* bT, EF* f, double* fT, EF* out,
                  double* outT, const Blocks3& Bo, size_t n, Ctl* ctl, double* part, cudaStream_t s);
+// APPLY, RESID and JACOBI on a caller's planes ([5][n] states, [2][n] opacities);
+// JACOBI may write blocks alone (out null).  Sets *irregular where a stencil holds a
+// cell no block can hold (its results are then not formed).
+void launchx3_planar(int mode, const G3& g, const double* u, const Blocks3& B, const double* sig,
+                     const double* b, double* out, const Blocks3& Bo, size_t n, int* irregular,
+                     cudaStream_t s);
+void launchx3_block_planar(const G3& g, const double* u, const Blocks3& B, size_t n, cudaStream_t s);
 void launchx3_restrict(const G3& gf, const G3& gc, const EF* u, const double* uT, const EF* r,
                        const double* rT, EF* vc, double* vcT, EF* rc, double* rcT, const Blocks3& Bo,
                        const Ctl* ctl, cudaStream_t s);

@@ -82,8 +82,47 @@ __device__ __forceinline__ void solvex3(const Coef& q, double A, double C, doubl
     oT = r.T;
 }
 
-template <int MODE>
-__global__ void __launch_bounds__(kThreadsX3, 4) k_opx3(G3 g, const EF* __restrict__ u,
+// A cell of a state: EF and T arrays, or (PLANAR) the five planes of a caller's array.
+template <bool PLANAR>
+__device__ __forceinline__ EF load3(const EF* __restrict__ x, size_t n, size_t q)
+{
+    if (!PLANAR) return x[q];
+    const double* p = reinterpret_cast<const double*>(x);
+    return EF{ p[q], { p[n + q], p[2 * n + q], p[3 * n + q] } };
+}
+
+template <bool PLANAR>
+__device__ __forceinline__ void store3(EF* __restrict__ x, size_t n, size_t q, const EF& v)
+{
+    if (!PLANAR) {
+        x[q] = v;
+        return;
+    }
+    double* p = reinterpret_cast<double*>(x);
+    p[q] = v.E;
+    p[n + q] = v.F[0];
+    p[2 * n + q] = v.F[1];
+    p[3 * n + q] = v.F[2];
+}
+
+template <bool PLANAR>
+__device__ __forceinline__ Sig2<double> opacity3(const Sig2<double>* __restrict__ s, size_t n, size_t q)
+{
+    if (!PLANAR) return s[q];
+    const double* p = reinterpret_cast<const double*>(s);
+    return Sig2<double>{ p[q], p[n + q] };
+}
+
+// PLANAR (m1_op_level3): the states are a caller's planes, of which intermediate
+// sweeps write none (out null: the blocks alone), the coefficients are formed in
+// place (FP64 operations the pass has room for, against a pass over the opacities
+// and 32 bytes a cell), and a cell with an irregular stencil sets *irregular (the
+// caller then takes the FP64 form).
+#ifndef OPX3_BLOCKS
+#define OPX3_BLOCKS 6
+#endif
+template <int MODE, bool PLANAR = false>
+__global__ void __launch_bounds__(kThreadsX3, OPX3_BLOCKS) k_opx3(G3 g, const EF* __restrict__ u,
                                                      const double* __restrict__ T, Blocks3 B,
                                                      Coef* __restrict__ Q,
                                                      const Sig2<double>* __restrict__ sig,
@@ -92,7 +131,8 @@ __global__ void __launch_bounds__(kThreadsX3, 4) k_opx3(G3 g, const EF* __restri
                                                      EF* __restrict__ f, double* __restrict__ fT,
                                                      EF* __restrict__ out, double* __restrict__ outT,
                                                      Blocks3 Bo, size_t n, Ctl* __restrict__ ctl,
-                                                     double* __restrict__ part)
+                                                     double* __restrict__ part,
+                                                     int* __restrict__ irregular)
 {
     constexpr bool STEP = MODE == OPX3_FIRST || MODE == OPX3_PSEUDO;
     constexpr bool JAC = MODE == OPX3_JACOBI || MODE == OPX3_JACOBI_NORM;
@@ -108,21 +148,25 @@ __global__ void __launch_bounds__(kThreadsX3, 4) k_opx3(G3 g, const EF* __restri
         const unsigned row = (unsigned)q / (unsigned)g.n[0];
         const int p[3] = { (int)((unsigned)q - row * (unsigned)g.n[0]), (int)(row % (unsigned)g.n[1]),
                            (int)(row / (unsigned)g.n[1]) };
-        const EF bb = MODE == OPX3_APPLY ? EF{} : b[q];
+        const EF bb = MODE == OPX3_APPLY ? EF{} : load3<PLANAR>(b, n, q);
         const double bbT = MODE == OPX3_APPLY ? 0.0 : bT[q];
         double N[4], fE = g.cb, fF = g.cbF;
         if (!sums3(g, B, n, (unsigned)q, p, N)) {
+            if (PLANAR) {
+                *irregular = 1;
+                continue;
+            }
             general_sums3(g, u, p[0], p[1], p[2], N);
             fE = fF = 1.0;
         }
         EF uc{};
         double Tc = 0.0;
-        if (!(MODE == OPX3_JACOBI)) { uc = u[q]; Tc = T[q]; }
+        if (!(MODE == OPX3_JACOBI)) { uc = load3<PLANAR>(u, n, q); Tc = T[q]; }
         EF a{};
         double aT = 0.0;
         Sig2<double> sg{};
         if (LOCAL) {
-            sg = sig[q];
+            sg = opacity3<PLANAR>(sig, n, q);
             const double ka = g.cdt * sg.sa, dF = g.diag + g.cdt * (sg.sa + sg.ss);
             const double T2 = Tc * Tc, src = ka * fma(-g.a_r, T2 * T2, uc.E);
             a.E = fma(-fE, N[0], fma(g.diag, uc.E, src));
@@ -131,7 +175,7 @@ __global__ void __launch_bounds__(kThreadsX3, 4) k_opx3(G3 g, const EF* __restri
             aT = fma(g.c_v, Tc, -src);
         }
         if (MODE == OPX3_APPLY) {
-            out[q] = a;
+            store3<PLANAR>(out, n, q, a);
             outT[q] = aT;
             continue;
         }
@@ -144,7 +188,7 @@ __global__ void __launch_bounds__(kThreadsX3, 4) k_opx3(G3 g, const EF* __restri
             nrm += fma(fma(r.F[2], r.F[2], fma(r.F[1], r.F[1], r.F[0] * r.F[0])), g.ic2,
                        fma(r.E, r.E, rT * rT));
             if (MODE == OPX3_RESID) {
-                out[q] = r;
+                store3<PLANAR>(out, n, q, r);
                 outT[q] = rT;
                 continue;
             }
@@ -155,7 +199,7 @@ __global__ void __launch_bounds__(kThreadsX3, 4) k_opx3(G3 g, const EF* __restri
         if (JAC) {
 #pragma unroll
             for (int m = 0; m < 3; ++m) rhs[m] = fma(fF, N[1 + m], bb.F[m]);
-            solvex3(Q[q], A, C, g.a_r, fma(fE, N[0], bb.E), rhs, bbT, o, oT, ok);
+            solvex3(PLANAR ? coef3(g, 0.0, 1.0, opacity3<PLANAR>(sig, n, q)) : Q[q], A, C, g.a_r, fma(fE, N[0], bb.E), rhs, bbT, o, oT, ok);
         } else {
             EF ff = bb;
             double ffT = bbT;
@@ -180,8 +224,10 @@ __global__ void __launch_bounds__(kThreadsX3, 4) k_opx3(G3 g, const EF* __restri
                     fma(tau, ffT, Tc), o, oT, ok);
         }
         if (!ok) ++fails;
-        out[q] = o;
-        outT[q] = oT;
+        if (!PLANAR || out) {
+            store3<PLANAR>(out, n, q, o);
+            outT[q] = oT;
+        }
         if (Bo.m) put_block3(g, o, Bo, n, q);
     }
     if (fails && ctl) atomicAdd(&ctl->newton_fail, fails);
@@ -197,13 +243,14 @@ __global__ void __launch_bounds__(kThreadsX3, 4) k_opx3(G3 g, const EF* __restri
     }
 }
 
+template <bool PLANAR>
 __global__ void __launch_bounds__(kThreadsX3) k_blockx3(G3 g, const EF* __restrict__ u, Blocks3 B,
                                                         size_t n, const Ctl* __restrict__ ctl)
 {
     if (skipx3(ctl)) return;
     for (size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
          q += (size_t)gridDim.x * blockDim.x)
-        put_block3(g, u[q], B, n, q);
+        put_block3(g, load3<PLANAR>(u, n, q), B, n, q);
 }
 
 __global__ void __launch_bounds__(kThreadsX3) k_coefx3(G3 g, const Sig2<double>* __restrict__ sig,
@@ -373,7 +420,7 @@ int blocksx3(size_t n) { return gridx3(n, kThreadsX3); }
 void launchx3_block(const G3& g, const EF* u, const Blocks3& B, size_t n, const Ctl* ctl,
                     cudaStream_t s)
 {
-    k_blockx3<<<blocksx3(n), kThreadsX3, 0, s>>>(g, u, B, n, ctl);
+    k_blockx3<false><<<blocksx3(n), kThreadsX3, 0, s>>>(g, u, B, n, ctl);
 }
 
 void launchx3_coef(const G3& g, const Sig2<double>* sig, Coef* Q, size_t n, cudaStream_t s)
@@ -387,7 +434,8 @@ void launchx3_op(int mode, const G3& g, const EF* u, const double* uT, const Blo
 {
     const int nb = blocksx3(n);
     auto go = [&](auto* k) {
-        k<<<nb, kThreadsX3, 0, s>>>(g, u, uT, B, Q, sig, b, bT, f, fT, out, outT, Bo, n, ctl, part);
+        k<<<nb, kThreadsX3, 0, s>>>(g, u, uT, B, Q, sig, b, bT, f, fT, out, outT, Bo, n, ctl, part,
+                                    nullptr);
     };
     switch (mode) {
     case OPX3_APPLY: go(k_opx3<OPX3_APPLY>); break;
@@ -397,6 +445,28 @@ void launchx3_op(int mode, const G3& g, const EF* u, const double* uT, const Blo
     case OPX3_FIRST: go(k_opx3<OPX3_FIRST>); break;
     default: go(k_opx3<OPX3_PSEUDO>); break;
     }
+}
+
+void launchx3_planar(int mode, const G3& g, const double* u, const Blocks3& B, const double* sig,
+                     const double* b, double* out, const Blocks3& Bo, size_t n, int* irregular,
+                     cudaStream_t s)
+{
+    const int nb = blocksx3(n);
+    auto go = [&](auto* k) {
+        k<<<nb, kThreadsX3, 0, s>>>(g, reinterpret_cast<const EF*>(u), u + 4 * n, B, nullptr,
+                                    reinterpret_cast<const Sig2<double>*>(sig),
+                                    reinterpret_cast<const EF*>(b), b ? b + 4 * n : nullptr, nullptr,
+                                    nullptr, reinterpret_cast<EF*>(out), out ? out + 4 * n : nullptr,
+                                    Bo, n, nullptr, nullptr, irregular);
+    };
+    if (mode == OPX3_APPLY) go(k_opx3<OPX3_APPLY, true>);
+    else if (mode == OPX3_RESID) go(k_opx3<OPX3_RESID, true>);
+    else go(k_opx3<OPX3_JACOBI, true>);
+}
+
+void launchx3_block_planar(const G3& g, const double* u, const Blocks3& B, size_t n, cudaStream_t s)
+{
+    k_blockx3<true><<<blocksx3(n), kThreadsX3, 0, s>>>(g, reinterpret_cast<const EF*>(u), B, n, nullptr);
 }
 
 void launchx3_restrict(const G3& gf, const G3& gc, const EF* u, const double* uT, const EF* r,
