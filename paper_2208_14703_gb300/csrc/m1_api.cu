@@ -194,7 +194,7 @@ m1_status Engine<R>::init(int capacity, int levels, bool correction_form, cudaSt
     strips.assign(L, DevList{});
     tails.assign(L, DevList{});
     tail_first.assign(cap, L);
-    if (sizeof(R) == 8) M1_CK(tail_prepare());
+    M1_CK(sizeof(R) == 8 ? tail_prepare() : tail32_prepare());
     M1_TRY(calloc_common((void**)&d, sizeof(Level<R>) * L * cap));
     M1_TRY(calloc_common((void**)&ctl, sizeof(Ctl) * cap));
     M1_TRY(calloc_common((void**)&bctl, sizeof(BatchCtl)));
@@ -289,17 +289,6 @@ m1_status Engine<R>::add_slot(const m1_grid_desc& dsc, int* out)
         nx /= 2; if (g.dim == 2) ny /= 2;
         hx *= 2; if (g.dim == 2) hy *= 2;
     }
-    // the tail: from the first coarse level that is small enough and whose levels
-    // fit a block's shared memory (a rule on the instance alone, so that its result
-    // does not depend on the batch)
-    tail_first[i] = L;
-    for (int l = L - 1; l >= 1 && sizeof(R) == 8; --l) {
-        const int n = h[(size_t)l * cap + i].n;
-        if (L - l > kTailLevels || n > kTailCells ||
-            tail_smem(n, kTailBlocks, g.dim, L - l) > (size_t)kTailSmem)
-            break;
-        tail_first[i] = l;
-    }
     used[i] = 1;
     dt_set[i] = NAN;
     rhs_valid[i] = 0;
@@ -384,6 +373,30 @@ m1_status Engine<R>::upload_list(DevList& l)
 template <typename R>
 m1_status Engine<R>::rebuild()
 {
+    // The tails: from the first coarse level that is small enough and whose levels fit
+    // a block's shared memory.  FP64: a rule on the instance alone, so that its result
+    // does not depend on the batch; FP32 (bitwise the same either way): also on the
+    // number of instances.
+    int count = 0;
+    for (int i = 0; i < cap; ++i) count += used[i] ? 1 : 0;
+    const int blocks = sizeof(R) == 8 ? kTailBlocks : tail32_blocks(count);
+    if (blocks != tail_blocks) { tail_blocks = blocks; graph_dirty = true; }
+    auto tail_mem = [&](int i, int l) {
+        const int n = h[(size_t)l * cap + i].n;
+        return sizeof(R) == 8 ? tail_smem(n, blocks, desc[i].dim, L - l)
+                              : tail32_smem(n, blocks, desc[i].dim, L - l);
+    };
+    for (int i = 0; i < cap; ++i) {
+        tail_first[i] = L;
+        if (!used[i] || (sizeof(R) == 4 && !delta)) continue;
+        for (int l = L - 1; l >= 1; --l) {
+            if (L - l > kTailLevels ||
+                h[(size_t)l * cap + i].n > (sizeof(R) == 8 ? kTailCells : kTail32Cells * blocks) ||
+                tail_mem(i, l) > (size_t)(sizeof(R) == 8 ? kTailSmem : kTail32Smem))
+                break;
+            tail_first[i] = l;
+        }
+    }
     int off = 0;
     for (int i = 0; i < cap; ++i)
         if (used[i]) { h[i].part_off = off; off += h[i].strips; }
@@ -427,8 +440,7 @@ m1_status Engine<R>::rebuild()
             if (used[i] && tail_first[i] == l) {
                 tails[l].host.push_back(make_int2(i, l));
                 tail_all.host.push_back(make_int2(i, l));
-                bytes = std::max(bytes, tail_smem(h[(size_t)l * cap + i].n, kTailBlocks,
-                                                  desc[i].dim, L - l));
+                bytes = std::max(bytes, tail_mem(i, l));
             }
         M1_TRY(upload_list(tails[l]));
     }
@@ -706,9 +718,14 @@ void Engine<R>::corrections(const Params& p, int l, int shape, std::vector<int>&
 template <typename R>
 void Engine<R>::tail(const DevList& list, int shape, cudaStream_t s)
 {
+    if (!list.n) return;
+    const int2* pr = progs + (size_t)shape * L;
     if constexpr (std::is_same<R, double>::value) {
-        if (list.n)
-            launch_tail(d, cap, L, list.view(), ctl, prog, progs + (size_t)shape * L, tail_bytes, s);
+        launch_tail(d, cap, L, list.view(), ctl, prog, pr, tail_bytes, s);
+    } else {
+        unsigned mask = 0;
+        for (int l = 0; l < L; ++l) mask |= ring[l] ? 1u << l : 0u;
+        launch_tail32(d, cap, L, list.view(), ctl, prog, pr, mask, tail_bytes, tail_blocks, s);
     }
 }
 
@@ -716,17 +733,20 @@ namespace {
 
 // The operations of the coarse-grid corrections of level l, as the tail of an
 // instance walks them (levels counted from `first`): the recursion of
-// Engine::corrections and Engine::visit.
-void program(const Params& p, int L, int first, int l, int shape, std::vector<unsigned char>& out)
+// Engine::corrections and Engine::visit.  fas: with the operation of the FAS
+// right-hand side (the correction form).
+void program(const Params& p, int L, int first, int l, int shape, bool fas,
+             std::vector<unsigned char>& out)
 {
     auto put = [&](int op, int level) { out.push_back((unsigned char)(op + 8 * (level - first))); };
     auto visit = [&](int v, bool fresh, int sh) {
         const int steps = v == L - 1 ? p.mc : p.m;
+        if (fas && fresh) put(TAIL_FAS, v);
         for (int k = 0; k < steps; ++k) put(k == 0 && fresh ? TAIL_FIRST : TAIL_PSEUDO, v);
         if (v == L - 1) return;
         put(TAIL_RESID, v);
         put(TAIL_RESTRICT, v + 1);
-        program(p, L, first, v, sh, out);
+        program(p, L, first, v, sh, fas, out);
         put(TAIL_PROLONG, v);
         for (int k = 0; k < p.m; ++k) put(TAIL_PSEUDO, v);
     };
@@ -764,7 +784,7 @@ m1_status Engine<R>::write_programs(const Params& p)
             const bool reached = shape == p.cycle || (p.cycle == M1_CYCLE_F && shape == M1_CYCLE_V);
             if (!reached || tails[f].n == 0) continue;
             const int off = (int)ops.size();
-            program(p, L, f, f - 1, shape, ops);
+            program(p, L, f, f - 1, shape, delta, ops);
             at[(size_t)shape * L + f] = make_int2(off, (int)ops.size() - off);
         }
     M1_CK(cudaStreamSynchronize(stream));

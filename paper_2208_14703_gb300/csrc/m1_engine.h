@@ -119,6 +119,7 @@ struct Engine {
     int2* progs = nullptr;                  // [shape][first level]: (offset, length) in prog
     Params pparams{};                       // the parameters the programs were written for
     size_t tail_bytes = 0;
+    int tail_blocks = 0;                    // blocks of a cluster
     std::vector<char> ring;                 // per level: the sweeps take the cp.async kernel
     std::vector<char> list_sig;             // which work lists were non-empty at capture
     // double-word copies of each slot's level-0 iterate, right-hand side and

@@ -895,7 +895,9 @@ __global__ void __launch_bounds__(kStripWarps * 32) k_norm_state(const Level<R>*
 // coarse FP32 levels are small and this takes the loads' latency off the chain.
 // FP64 keeps one stencil point at a time: its restriction is bound by the FP64
 // pipe, and the registers of the batched loads cost it occupancy (measured: the
-// FP64 step 3.7% slower).  Both forms sum the same values in the same order.
+// FP64 step 3.7% slower).  Both forms sum the same values in the same order; the FP32
+// sums are written as fma, whose product by a power of two rounds only among subnormal
+// numbers, so that the one-launch tail (m1_tail32.cu) can repeat them there too.
 template <typename R, bool DELTA>
 __device__ __forceinline__ void restrict_cell(const Level<R>& Lf, const Level<R>& Lc, int kc,
                                               int fine_buf)
@@ -950,11 +952,14 @@ __device__ __forceinline__ void restrict_cell(const Level<R>& Lf, const Level<R>
             // carries the prescribed state
             const Cell4<R> sv = ghost_apply(Lf, s[a], g[a], DELTA ? KIND_DIFF : KIND_STATE);
             const Cell4<R> rv = ghost_apply(Lf, r[a], g[a], KIND_DIFF);
-            av.E += wt * sv.E; av.Fx += wt * sv.Fx; av.Fy += wt * sv.Fy; av.T += wt * sv.T;
-            ar.E += wt * rv.E; ar.Fx += wt * rv.Fx; ar.Fy += wt * rv.Fy; ar.T += wt * rv.T;
+            av.E = fma(wt, sv.E, av.E); av.Fx = fma(wt, sv.Fx, av.Fx);
+            av.Fy = fma(wt, sv.Fy, av.Fy); av.T = fma(wt, sv.T, av.T);
+            ar.E = fma(wt, rv.E, ar.E); ar.Fx = fma(wt, rv.Fx, ar.Fx);
+            ar.Fy = fma(wt, rv.Fy, ar.Fy); ar.T = fma(wt, rv.T, ar.T);
             if (DELTA) {
                 const Cell4<R> qv = ghost_apply(Lf, q[a], g[a], KIND_STATE);
-                aw.E += wt * qv.E; aw.Fx += wt * qv.Fx; aw.Fy += wt * qv.Fy; aw.T += wt * qv.T;
+                aw.E = fma(wt, qv.E, aw.E); aw.Fx = fma(wt, qv.Fx, aw.Fx);
+                aw.Fy = fma(wt, qv.Fy, aw.Fy); aw.T = fma(wt, qv.T, aw.T);
             }
         }
     }
@@ -1062,8 +1067,8 @@ __device__ __forceinline__ void prolong_block(const Level<R>& Lc, const Level<R>
             Cell4<R> pe = { 0, 0, 0, 0 };
             for (int b = 0; b <= oy; ++b)
                 for (int a = 0; a <= ox; ++a) {
-                    pe.E += wt * dc[b][a].E; pe.Fx += wt * dc[b][a].Fx;
-                    pe.Fy += wt * dc[b][a].Fy; pe.T += wt * dc[b][a].T;
+                    pe.E = fma(wt, dc[b][a].E, pe.E); pe.Fx = fma(wt, dc[b][a].Fx, pe.Fx);
+                    pe.Fy = fma(wt, dc[b][a].Fy, pe.Fy); pe.T = fma(wt, dc[b][a].T, pe.T);
                 }
             const Cell4<R> e = uf[k];
             Cell4<R> u = e;

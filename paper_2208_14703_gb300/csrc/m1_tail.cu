@@ -7,9 +7,7 @@
 // first of at most kTailCells cells down in its shared memory, one thread per cell,
 // and walks the whole sequence of coarse visits (Algorithm 4, V, W or F) with a
 // cluster barrier (0.2 us) between operations.
-//
-// The FP32 levels of the mixed path keep their launches: their roundings would
-// change, and small mixed problems carry FP32 roundings into the ninth digit.
+// (The mixed path's FP32 levels: m1_tail32.cu.)
 //
 // Layout: a level's cells are split into equal ranges of consecutive cells, one
 // range per block (small levels: fewer blocks).  What a cell's neighbours need,

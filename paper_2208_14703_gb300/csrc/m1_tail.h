@@ -19,8 +19,10 @@ constexpr int kTailCells = 8192;
 // counted from the tail's first.  FIRST: the FAS right-hand side and the first
 // pseudo-time step of a fresh visit; PSEUDO: one more step; RESID: the residual;
 // RESTRICT: from the level above into this one; PROLONG: from the level below onto
-// this one.
-enum TailOp { TAIL_FIRST = 0, TAIL_PSEUDO = 1, TAIL_RESID = 2, TAIL_RESTRICT = 3, TAIL_PROLONG = 4 };
+// this one.  The FP32 tail forms the FAS right-hand side in an operation of its own
+// (FAS) before FIRST.
+enum TailOp { TAIL_FIRST = 0, TAIL_PSEUDO = 1, TAIL_RESID = 2, TAIL_RESTRICT = 3, TAIL_PROLONG = 4,
+              TAIL_FAS = 5 };
 
 // Cells per block of a level of n cells over nb blocks: equal shares, but no
 // fewer than make a block's work worth a cluster barrier.
@@ -43,5 +45,33 @@ cudaError_t tail_prepare();
 // in prog.
 cudaError_t launch_tail(const Level<double>* lv, int cap, int nlev, WorkList wl, Ctl* ctls,
                         const unsigned char* prog, const int2* progs, size_t smem, cudaStream_t s);
+
+// ---- the FP32 hierarchy's (m1_tail32.cu) -----------------------------------------
+// Its levels give the same bits in the tail and in launches of their own, so where it
+// begins may depend on the company: with more instances each gets a smaller cluster
+// (all of them then run at once) and a tail of fewer cells.
+constexpr int kTail32Smem = 216 * 1024, kTail32Cells = 1024;   // a block's; cells a block at most
+
+__host__ __device__ inline int tail32_per(int n, int nb)
+{
+    int p = (n + nb - 1) / nb;
+    const int least = 128;
+    const int cap = n < least ? n : least;
+    p = p < cap ? cap : p;
+    return (p + 3) & ~3;
+}
+
+// Blocks of an instance's cluster when `count` instances step together.
+inline int tail32_blocks(int count)
+{
+    return count <= 8 ? 16 : count <= 18 ? 8 : count <= 36 ? 4 : count <= 74 ? 2 : 1;
+}
+
+size_t tail32_smem(int n0, int nb, int dim, int nlev);
+cudaError_t tail32_prepare();
+// ring: bit l set where the sweeps of level l are those of the cp.async strips.
+cudaError_t launch_tail32(const Level<float>* lv, int cap, int nlev, WorkList wl, Ctl* ctls,
+                          const unsigned char* prog, const int2* progs, unsigned ring, size_t smem,
+                          int blocks, cudaStream_t s);
 
 }  // namespace m1
