@@ -274,19 +274,22 @@ __host__ __device__ __forceinline__ bool fx_quartic(double C, double K, double R
         ok = fabsf(dT) <= 3e-4f * T;
     }
     const unsigned bt = bits_of_float(T);
-    const int eT = (int)(bt >> 23) - 127;                      // sign set: out of range below
+    // A significand at its upper end (T just below a power of two, such as a gas at rest
+    // near T = 1) is taken as one below 1 at the next exponent, so that the corrections
+    // (below 2^-18 T) keep it under 2^62.
+    const int up = (bt & 0x7fffffu) >= 0x7fff00u ? 1 : 0;
+    const int eT = (int)(bt >> 23) - 127 + up;                 // sign set: out of range below
     int eC, eK, eR;
     const i64 mC = fx_significand(C, eC), mR = fx_significand(R, eR);
     const Split sC = split62(mC), sK = split62(fx_significand(K, eK));
     const float dg = fmaf(K4, T * T * T, Cf);
-    // 2^(eR - eT) / g' <= 4; the significand of T away from its upper end, so that
-    // the corrections (below 2^-18 T) keep it under 2^62
+    // 2^(eR - eT) / g' <= 4
     ok = ok && eT > -60 && eT < 60 && eR > -120 && eR < 120 && eR - eT > -120 && eR - eT < 120 &&
-         dg > 1e-35f && dg < 1e35f && (bt & 0x7fffffu) < 0x7fff00u;
+         dg > 1e-35f && dg < 1e35f;
     const float q = float_of_bits((unsigned)((ok ? eR - eT : 0) + 127) << 23) * seed_rcp(dg);
     const int nC = eR - eC - eT + 4, nK = eR - eK - 4 * eT + 1;
     ok = ok && nC >= 0 && nK >= 0;
-    i64 m = (i64)((bt & 0x7fffffu) | 0x800000u) << 38, T4 = 0;
+    i64 m = (i64)((bt & 0x7fffffu) | 0x800000u) << (38 - up), T4 = 0;
     float d = 0.0f;
 #ifdef __CUDA_ARCH__
 #pragma unroll
@@ -308,8 +311,8 @@ __host__ __device__ __forceinline__ bool fx_quartic(double C, double K, double R
             d = ok ? d : 0.0f;
         }
     }
-    // T^4 at the corrected root: T4 (1 - 4 d / m), with 4 T4 / m = t^3 / 2, t in [1, 2)
-    const float t = float_of_bits((bt & 0x7fffffu) | 0x3f800000u);
+    // T^4 at the corrected root: T4 (1 - 4 d / m), with 4 T4 / m = t^3 / 2, t = T / 2^eT
+    const float t = float_of_bits((bt & 0x7fffffu) | (0x3f800000u - ((unsigned)up << 23)));
     T4 -= (i64)(int)(d * t * t * t * 0.5f);
     m -= (i64)(int)d;
     T4out = fx_double(T4, ok ? 4 * eT : 0);

@@ -161,3 +161,26 @@ def test_fixed_point_3d_matches_oracle(name, dims, lengths, c, spread, bc, tiny)
     ka, T = c * dt * sa, got[4]
     row = T - ka * (got[0] - T ** 4) - b[4]
     assert np.max(np.abs(row) / (T + ka * (big + T ** 4) + b[4])) <= 1e-12
+
+
+@pytest.mark.parametrize("power", [-2, -1, 0, 1, 3])
+def test_local_solve_near_powers_of_two(power):
+    """A gas at or close to rest at T near a power of two, where the fixed-point root's
+    significand is at either end of its range: one Jacobi sweep against the oracle.
+    A dozen roundings of the row's right-hand side R reach T (R's relative error bounds
+    T's: g' T >= R) and E: 1e-14 of their sizes, taken ten times."""
+    nx, ny = 60, 32
+    rng = np.random.default_rng(20 + power)
+    case = inputs.random_admissible_2d(nx, ny, 1, fmax=0.0, cfl=100, bc=("reflect",) * 4)
+    off = rng.choice([-1.0, 1.0], (ny, nx)) * 10.0 ** rng.uniform(-17, -3, (ny, nx))
+    T = 2.0 ** power * (1.0 + off)
+    case["state"] = np.stack([T ** 4, 0.0 * T, 0.0 * T, T])
+    g = O.Grid.from_case(case)
+    s, dt = case["state"], case["dt"]
+    b = O.rhs_of(g, s)
+    desc = m1.desc_from_case(case, lmax=1)
+    got, fails = m1.m1_op_level(desc, dt, np.stack([case["sa"], case["ss"]]), s, b, mode=m1.OP_JACOBI)
+    ref, it = O.jacobi_sweep(g, dt, case["sa"], case["ss"], b, s)
+    assert it >= 0 and fails == 0
+    assert np.max(np.abs(got[3] / ref[3] - 1.0)) <= 1e-13
+    assert np.max(np.abs(got[0] / ref[0] - 1.0)) <= 1e-13
