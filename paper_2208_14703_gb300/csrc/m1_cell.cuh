@@ -76,4 +76,20 @@ __device__ __forceinline__ void strip_neighbours(const Level<R>& L, const Staged
     }
 }
 
+// The rows or columns c - 1, c, c + 1 (c even) of an axis of n cells under its low
+// wall's rule: indices, and the rule that c - 1 falls under (-1: none, or periodic).
+// n is even where this is asked (a level that is restricted), so c + 1 < n.
+struct StencilAxis {
+    int k[3], rule;
+};
+__device__ __forceinline__ StencilAxis stencil_axis(int c, int n, int bc)
+{
+    StencilAxis a = { { c - 1, c, c + 1 }, -1 };
+    if (c == 0) {
+        a.k[0] = bc == BC_PERIODIC ? n - 1 : 0;
+        if (bc != BC_PERIODIC) a.rule = bc;
+    }
+    return a;
+}
+
 }  // namespace m1

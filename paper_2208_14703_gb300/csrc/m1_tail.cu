@@ -214,6 +214,55 @@ __device__ __forceinline__ void arrive64(const Tail& t, int l, int q, const Cell
     put_block(t, l, 0, q, v);
 }
 
+// One field (0 to 3: E, Fx, Fy, T) of cell (i, j) of level l restricted from level
+// l - 1 (k_restrict): of the iterate, in buffer c there, into v, or of the residual,
+// in the other, into f.  The walls' rules as indices and signs; an inflow wall, rare,
+// by the whole cell's rules.
+__device__ __forceinline__ void restrict_field(const Tail& t, int l, int c, int q, int i, int j,
+                                               bool resid, int field)
+{
+    const Level<double>& Lf = t.L[l - 1];
+    const bool two_d = Lf.dim == 2;
+    const int arr = resid ? ARR_E + 1 - c : ARR_E + c;
+    const StencilAxis x = stencil_axis(2 * i, Lf.nx, Lf.bc[WALL_W]);
+    const StencilAxis y = stencil_axis(2 * j, Lf.ny, Lf.bc[WALL_S]);
+    double v[3][3];
+    if (x.rule == BC_INFLOW || (two_d && y.rule == BC_INFLOW)) {
+        for (int b = 0; b < 3; ++b)
+            for (int a = 0; a < 3; ++a) {
+                if (!two_d && b != 1) { v[b][a] = 0.0; continue; }
+                const Cell4<double> s = t.fetch(l - 1, arr, 2 * i + a - 1, two_d ? 2 * j + b - 1 : 0,
+                                                resid ? KIND_DIFF : KIND_STATE);
+                v[b][a] = field == 0 ? s.E : field == 1 ? s.Fx : field == 2 ? s.Fy : s.T;
+            }
+    } else {
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            if (!two_d && b != 1) continue;
+            const int row = two_d ? y.k[b] * Lf.nx : 0;
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+                v[b][a] = reinterpret_cast<const double*>(
+                    t.at<Cell4<double>>(l - 1, arr, row + x.k[a]))[field];
+        }
+        if (two_d && field == 2 && y.rule == BC_REFLECT)
+#pragma unroll
+            for (int a = 0; a < 3; ++a) v[0][a] = -v[0][a];
+        if (field == 1 && x.rule == BC_REFLECT)
+#pragma unroll
+            for (int b = 0; b < 3; ++b) v[b][0] = -v[b][0];
+    }
+    double s = 0.0;
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        if (!two_d && b != 1) continue;
+        const double wy = two_d ? (b == 1 ? 0.5 : 0.25) : 1.0;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) s = fma(wy * (a == 1 ? 0.5 : 0.25), v[b][a], s);
+    }
+    reinterpret_cast<double*>(t.own<Cell4<double>>(l, resid ? ARR_F : ARR_V, q))[field] = s;
+}
+
 __device__ __forceinline__ void op_cell(const Tail& t, int op, int l, int cur, int ccur,
                                         int k, int q, const Pseudo<double>& ps, double theta_c,
                                         unsigned& fails, unsigned& damped)
@@ -225,13 +274,35 @@ __device__ __forceinline__ void op_cell(const Tail& t, int op, int l, int cur, i
         const int j = two_d ? row_of(t.geo[l], k) : 0, i = k - j * L.nx;
         const int ic = i >> 1, jc = two_d ? j >> 1 : 0, ox = i & 1, oy = two_d ? j & 1 : 0;
         const double wt = pow2_neg<double>(ox + oy);
+        // the coarse cells past the high walls under the rules of differences
+        const Level<double>& Lc = t.L[l + 1];
+        const bool xo = ic + 1 == Lc.nx, yo = two_d && jc + 1 == Lc.ny;
+        const int bx = Lc.bc[WALL_E], by = Lc.bc[WALL_N];
+        const int xk = !xo ? ic + 1 : bx == BC_PERIODIC ? 0 : ic;
+        const int yk = !yo ? jc + 1 : by == BC_PERIODIC ? 0 : jc;
+        const int off = (ARR_V - ARR_E - ccur) * t.geo[l + 1].per;
+        C cu[2][2], cv[2][2];
+#pragma unroll
+        for (int b = 0; b < 2; ++b)
+#pragma unroll
+            for (int a = 0; a < 2; ++a) {
+                if (b > oy || a > ox) continue;
+                const C* p = t.at<C>(l + 1, ARR_E + ccur, (b ? yk : jc) * Lc.nx + (a ? xk : ic));
+                cu[b][a] = p[0];
+                cv[b][a] = p[off];
+            }
         C pe = { 0, 0, 0, 0 };
-        for (int b = 0; b <= oy; ++b)
-            for (int a = 0; a <= ox; ++a) {
-                const C cu = t.fetch(l + 1, ARR_E + ccur, ic + a, jc + b, KIND_DIFF);
-                const C cv = t.fetch(l + 1, ARR_V, ic + a, jc + b, KIND_DIFF);
-                pe.E += wt * (cu.E - cv.E); pe.Fx += wt * (cu.Fx - cv.Fx);
-                pe.Fy += wt * (cu.Fy - cv.Fy); pe.T += wt * (cu.T - cv.T);
+#pragma unroll
+        for (int b = 0; b < 2; ++b)
+#pragma unroll
+            for (int a = 0; a < 2; ++a) {
+                if (b > oy || a > ox) continue;
+                const bool bo = b && yo, ao = a && xo;
+                if ((bo && by == BC_INFLOW) || (ao && bx == BC_INFLOW)) continue;
+                const C &m = cu[b][a], &n = cv[b][a];
+                const double wx = ao && bx == BC_REFLECT ? -wt : wt, wy = bo && by == BC_REFLECT ? -wt : wt;
+                pe.E += wt * (m.E - n.E); pe.Fx += wx * (m.Fx - n.Fx);
+                pe.Fy += wy * (m.Fy - n.Fy); pe.T += wt * (m.T - n.T);
             }
         const C u = *t.own<C>(l, ARR_E + cur, q);
         C tg = { u.E + pe.E, u.Fx + pe.Fx, u.Fy + pe.Fy, u.T + pe.T };
@@ -242,25 +313,6 @@ __device__ __forceinline__ void op_cell(const Tail& t, int op, int l, int cur, i
         }
         *t.own<C>(l, ARR_E + cur, q) = tg;
         put_block(t, l, cur, q, tg);
-        return;
-    }
-    if (op == TAIL_RESTRICT) {             // cell k of level l from level l - 1; ccur: its buffer
-        const int j = two_d ? row_of(t.geo[l], k) : 0, i = k - j * L.nx;
-        C av = { 0, 0, 0, 0 }, ar = { 0, 0, 0, 0 };
-        const int b0 = two_d ? -1 : 0, b1 = two_d ? 1 : 0;
-        for (int b = b0; b <= b1; ++b) {
-            const int eb = two_d ? (b == 0 ? 1 : 2) : 0;
-            for (int a = -1; a <= 1; ++a) {
-                const double wt = pow2_neg<double>(eb + (a == 0 ? 1 : 2));
-                const Ghost g = ghost_map(t.L[l - 1], 2 * i + a, two_d ? 2 * j + b : 0);
-                const C s = ghost_apply(t.L[l - 1], *t.at<C>(l - 1, ARR_E + ccur, (int)g.k), g, KIND_STATE);
-                const C r = ghost_apply(t.L[l - 1], *t.at<C>(l - 1, ARR_E + 1 - ccur, (int)g.k), g,
-                                        KIND_DIFF);
-                av.E += wt * s.E; av.Fx += wt * s.Fx; av.Fy += wt * s.Fy; av.T += wt * s.T;
-                ar.E += wt * r.E; ar.Fx += wt * r.Fx; ar.Fy += wt * r.Fy; ar.T += wt * r.T;
-            }
-        }
-        arrive64(t, l, q, av, ar);
         return;
     }
     double NE, NFx, NFy;
@@ -388,6 +440,18 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const Level<double>* _
             const int ccur = op == TAIL_RESTRICT ? (curs >> (l - 1)) & 1
                            : op == TAIL_PROLONG ? (curs >> (l + 1)) & 1 : 0;
             const int base = rank * geo[l].per, end = min(geo[l].per, geo[l].n - base);
+            if (op == TAIL_RESTRICT) {
+                // eight threads a cell, a field of one of its two arrays each
+                for (int x = threadIdx.x; x < 8 * end; x += kTailThreads) {
+                    const int q = x >> 3, k = base + q;
+                    const int j = Ls[l].dim == 2 ? row_of(geo[l], k) : 0;
+                    restrict_field(t, l, ccur, q, k - j * geo[l].nx, j, x & 4, x & 3);
+                }
+                if (end > 0) __syncthreads();
+                for (int q = threadIdx.x; q < end; q += kTailThreads)
+                    put_block(t, l, 0, q, *t.own<Cell4<double>>(l, ARR_V, q));
+                continue;
+            }
             for (int q = threadIdx.x; q < end; q += kTailThreads)
                 op_cell(t, op, l, cur, ccur, base + q, q, ps, theta_c, fails, damped);
             if (op == TAIL_FIRST) curs |= 1u << l;

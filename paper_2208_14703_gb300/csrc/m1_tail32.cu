@@ -157,23 +157,6 @@ __device__ __forceinline__ void close32(const Tail32& t, int l, int q, int part)
     else *t.own(l, P0 + 1, q) = closure32<true>(L, w, v);
 }
 
-// The rows or columns c - 1, c, c + 1 (c even) of an axis of n cells under its walls'
-// rules: indices, and the rule of the one that may lie outside (c - 1; -1: none).
-// An inflow wall's profile is the caller's matter.
-struct Axis32 {
-    int k[3], rule;
-};
-__device__ __forceinline__ Axis32 axis32(int c, int n, int bc)
-{
-    Axis32 a = { { c - 1, c, c + 1 }, -1 };
-    if (c == 0) {
-        a.k[0] = bc == BC_PERIODIC ? n - 1 : 0;
-        if (bc != BC_PERIODIC) a.rule = bc;
-    }
-    // c + 1 < n: the coarse grids halve even ones (1D's y axis has one row, not asked for)
-    return a;
-}
-
 // The FAS right-hand side (k_fas_aw32): A(w) and f = [A(w + v) - A(w)] + r.
 __device__ __forceinline__ void op_fas(const Tail32& t, int l, int k, int q, int i, int j)
 {
@@ -241,7 +224,7 @@ __device__ __forceinline__ void op_restrict(const Tail32& t, int l, int c, int q
     const bool two_d = Lf.dim == 2;
     const int arr = part == 0 ? E0 + c : part == 1 ? E0 + 1 - c : (int)W;
     const int kind = part == 2 ? KIND_STATE : KIND_DIFF;
-    const Axis32 x = axis32(2 * i, Lf.nx, Lf.bc[WALL_W]), y = axis32(2 * j, Lf.ny, Lf.bc[WALL_S]);
+    const StencilAxis x = stencil_axis(2 * i, Lf.nx, Lf.bc[WALL_W]), y = stencil_axis(2 * j, Lf.ny, Lf.bc[WALL_S]);
     const bool inflow = x.rule == BC_INFLOW || (two_d && y.rule == BC_INFLOW);
     C4 s = { 0, 0, 0, 0 };
 #pragma unroll
