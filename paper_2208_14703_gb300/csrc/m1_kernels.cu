@@ -366,10 +366,11 @@ __device__ __forceinline__ double strip_sweep64(const Level<double>& L, Ctl* ctl
                     b.T = fma(L.c_v, u.T, -src_e) + b.T;
                     L.f[k] = b;
                 } else {
-                    const double rE = b.E - fma(-L.cb, NE, fma(L.diag, u.E, src_e));
-                    const double rFx = b.Fx - fma(-L.cbF, NFx, dF * u.Fx);
-                    const double rFy = b.Fy - fma(-L.cbF, NFy, dF * u.Fy);
-                    const double rT = b.T - fma(L.c_v, u.T, -src_e);
+                    // b + N is the sweep's own right-hand side
+                    const double rE = fma(-L.diag, u.E, fma(cbE, NE, b.E) - src_e);
+                    const double rFx = fma(-dF, u.Fx, fma(cbF, NFx, b.Fx));
+                    const double rFy = fma(-dF, u.Fy, fma(cbF, NFy, b.Fy));
+                    const double rT = fma(-L.c_v, u.T, b.T + src_e);
                     nrm += fma(fma(rFy, rFy, rFx * rFx), L.ic2, fma(rE, rE, rT * rT));
                 }
             }
