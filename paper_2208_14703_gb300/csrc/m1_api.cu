@@ -668,7 +668,12 @@ void Engine<R>::pseudo(int l, int& cur, int m, bool from_v, cudaStream_t s, bool
                                 fas && !delta);
             cur = 0;
         } else {
-            if (go) launch_sweep<R>(dl, strips[l].view(), ctl, true, cur, 1 - cur, s, delta, rg);
+            // the run's first step but the FAS one stores the local solve's coefficients
+            // for the others (FP64; m1_kernels.cu: KEEP)
+            const int at = k - (from_v ? 1 : 0), keep = at > 0 ? 2 : k + 1 < m ? 1 : 0;
+            if (go)
+                launch_sweep<R>(dl, strips[l].view(), ctl, true, cur, 1 - cur, s, delta, rg, nullptr,
+                                false, keep);
             cur = 1 - cur;
         }
     }

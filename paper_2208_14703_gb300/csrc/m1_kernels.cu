@@ -320,8 +320,14 @@ __device__ __noinline__ double strip_general64(const Level<double>& L, Ctl* ctl,
 }
 
 // One fine Jacobi sweep, or one fused pseudo-time step, of an (instance, strip)
-// item: what update_cell does, with N from the fixed-point sums.
-template <bool PSEUDO, bool NORM, bool FAS>
+// item: what update_cell does, with N from the fixed-point sums.  KEEP: the steps of a
+// visit share dtau, hence the local solve's coefficients (sixteen FP64 operations of a
+// step's thirty): the first that follows the FAS right-hand side stores them in the
+// level's residual array, which is free from there to the residual, and the rest of the
+// run loads them.  A step at 512^2: 15.7 us with them loaded, 18.3 formed and stored
+// (a 1024^2 FP64 cycle of six steps a level: 3% less).
+enum { KEEP_NONE = 0, KEEP_STORE = 1, KEEP_LOAD = 2 };
+template <bool PSEUDO, bool NORM, bool FAS, int KEEP>
 __device__ __forceinline__ double strip_sweep64(const Level<double>& L, Ctl* ctl, int2 it, int lane,
                                                 const Cell4<double>* __restrict__ src, int out_buf)
 {
@@ -341,7 +347,9 @@ __device__ __forceinline__ double strip_sweep64(const Level<double>& L, Ctl* ctl
         auto pre = [&](size_t k) {
             Pre p;
             p.b = FAS ? L.r[k] : L.f[k];
-            if (PSEUDO || NORM) { p.sg = L.sig[k]; p.u = src[k]; }
+            if (PSEUDO || NORM) p.u = src[k];
+            if (KEEP == KEEP_LOAD) p.q = reinterpret_cast<const Coef*>(L.r)[k];
+            else if (PSEUDO || NORM) p.sg = L.sig[k];
             if (!PSEUDO) p.q = reinterpret_cast<const Coef*>(L.v)[k];
             return p;
         };
@@ -350,7 +358,7 @@ __device__ __forceinline__ double strip_sweep64(const Level<double>& L, Ctl* ctl
             const double NE = fx_double(s.E, s.e), NFx = fx_double(s.Fx, s.e),
                          NFy = fx_double(s.Fy, s.e);
             double ka = 0.0, kt = 0.0;
-            if (PSEUDO || NORM) { ka = L.cdt * p.sg.sa; kt = L.cdt * (p.sg.sa + p.sg.ss); }
+            if ((PSEUDO || NORM) && KEEP != KEEP_LOAD) { ka = L.cdt * p.sg.sa; kt = L.cdt * (p.sg.sa + p.sg.ss); }
             Cell4<double> b = p.b;
             bool ok;
             Cell4<double> o;
@@ -379,7 +387,10 @@ __device__ __forceinline__ double strip_sweep64(const Level<double>& L, Ctl* ctl
                                   fma(cbF, NFy, b.Fy), b.T, ok);
             } else {
                 const double tau = limited_step64(p.u, b, ps.dtau, ps.theta, ps.s, L.c);
-                o = local_solve64(make_coef(1.0, ps.dtau, L.diag, ka, kt, L.a_r), Ap, Cp, L.a_r,
+                const Coef q = KEEP == KEEP_LOAD ? p.q
+                                                 : make_coef(1.0, ps.dtau, L.diag, ka, kt, L.a_r);
+                if (KEEP == KEEP_STORE) reinterpret_cast<Coef*>(L.r)[k] = q;
+                o = local_solve64(q, Ap, Cp, L.a_r,
                                   fma(cbE, NE, fma(tau, b.E, p.u.E)),
                                   fma(cbF, NFx, fma(tau, b.Fx, p.u.Fx)),
                                   fma(cbF, NFy, fma(tau, b.Fy, p.u.Fy)), fma(tau, b.T, p.u.T), ok);
@@ -425,7 +436,7 @@ __global__ void __launch_bounds__(kThreads) k_coef64(const Level<double>* __rest
 // Persistent FP64 sweep (the item loop of k_sweep), held to 128 registers (8 blocks
 // per SM).  Bound by the FP64 pipe, now at 36 of its operations a fine update and
 // not 109: 0.37 ms a sweep at 2048^2 where the FP64 form took 0.88 ms.
-template <bool PSEUDO, bool NORM = false, bool FAS = false>
+template <bool PSEUDO, bool NORM = false, bool FAS = false, int KEEP = KEEP_NONE>
 __global__ void __launch_bounds__(kStripWarps * 32, 8) k_sweep64(const Level<double>* __restrict__ lv,
                                                                  WorkList wl, Ctl* __restrict__ ctls,
                                                                  int in_buf, int out_buf,
@@ -441,7 +452,7 @@ __global__ void __launch_bounds__(kStripWarps * 32, 8) k_sweep64(const Level<dou
         const int2 it = nx;
         if (!enter_item(L, lv + it.x, ctls, it.x, lane)) continue;
         const Cell4<double>* __restrict__ src = in_buf < 0 ? L.v : L.u[in_buf];
-        const double nrm = strip_sweep64<PSEUDO, NORM, FAS>(L, ctls + it.x, it, lane, src, out_buf);
+        const double nrm = strip_sweep64<PSEUDO, NORM, FAS, KEEP>(L, ctls + it.x, it, lane, src, out_buf);
         if (NORM) {
             const double sum = warp_sum(nrm);
             if (lane == 0) partials[L.part_off + it.y] = sum * L.vol;
@@ -698,7 +709,7 @@ __device__ __noinline__ double apply_general64(const Level<double>& L, int2 it, 
 // FP64 levels carry no base state).
 template <int MODE>
 __device__ __forceinline__ double apply_item64(const Level<double>& L, int2 it, int lane,
-                                               int state_buf, int write_r)
+                                               int state_buf, int write_r, bool norm)
 {
     struct Pre {
         Cell4<double> u, f;
@@ -727,7 +738,7 @@ __device__ __forceinline__ double apply_item64(const Level<double>& L, int2 it, 
             if (MODE == APPLY_RESID) {
                 const Cell4<double> r = { p.f.E - a.E, p.f.Fx - a.Fx, p.f.Fy - a.Fy, p.f.T - a.T };
                 if (write_r) L.r[k] = r;
-                nrm += fma(fma(r.Fy, r.Fy, r.Fx * r.Fx), L.ic2, fma(r.E, r.E, r.T * r.T));
+                if (norm) nrm += fma(fma(r.Fy, r.Fy, r.Fx * r.Fx), L.ic2, fma(r.E, r.E, r.T * r.T));
             } else if (MODE == APPLY_FAS) {
                 L.f[k] = Cell4<double>{ a.E + p.f.E, a.Fx + p.f.Fx, a.Fy + p.f.Fy, a.T + p.f.T };
             } else {
@@ -764,7 +775,7 @@ __global__ void __launch_bounds__(kStripWarps * 32) k_apply(const Level<R>* __re
         if (!enter_item(L, lv + it.x, ctls, it.x, lane)) continue;
         double nrm;
         if constexpr (std::is_same<R, double>::value)
-            nrm = apply_item64<MODE>(L, it, lane, state_buf, write_r);
+            nrm = apply_item64<MODE>(L, it, lane, state_buf, write_r, partials != nullptr);
         else
             nrm = apply_item<R, MODE, DELTA>(L, it, lane, state_buf, write_r);
         if (MODE == APPLY_RESID && partials) {
@@ -1776,12 +1787,17 @@ static inline int pgrid_warps(const WorkList& wl)
 
 template <typename R>
 void launch_sweep(const Level<R>* lv, WorkList wl, Ctl* ctls, bool pseudo, int in_buf,
-                  int out_buf, cudaStream_t s, bool delta, bool ring, double* partials, bool fas)
+                  int out_buf, cudaStream_t s, bool delta, bool ring, double* partials, bool fas,
+                  int keep)
 {
     const int g = pgrid_warps(wl), t = kStripWarps * 32;
     if constexpr (std::is_same<R, double>::value) {
         if (pseudo && fas)
             k_sweep64<true, false, true><<<g, t, 0, s>>>(lv, wl, ctls, in_buf, out_buf, nullptr);
+        else if (pseudo && keep == KEEP_STORE)
+            k_sweep64<true, false, false, KEEP_STORE><<<g, t, 0, s>>>(lv, wl, ctls, in_buf, out_buf, nullptr);
+        else if (pseudo && keep == KEEP_LOAD)
+            k_sweep64<true, false, false, KEEP_LOAD><<<g, t, 0, s>>>(lv, wl, ctls, in_buf, out_buf, nullptr);
         else if (pseudo)
             k_sweep64<true><<<g, t, 0, s>>>(lv, wl, ctls, in_buf, out_buf, nullptr);
         else if (partials)
@@ -1943,7 +1959,7 @@ void launch_accumulate(const Level<double>* lv64, const Level<float>* lv32, Work
 
 #define M1_INSTANTIATE(R)                                                                          \
     template void launch_sweep<R>(const Level<R>*, WorkList, Ctl*, bool, int, int, cudaStream_t,  \
-                                  bool, bool, double*, bool);                                      \
+                                  bool, bool, double*, bool, int);                                      \
     template void launch_apply<R>(const Level<R>*, WorkList, Ctl*, int, int, double*, int,        \
                                   cudaStream_t, bool);                                             \
     template void launch_norm_state<R>(const Level<R>*, WorkList, const Ctl*, double*,            \

@@ -108,3 +108,21 @@ def test_batched_shape_equals_alone(shape_name, shape):
         alone, st, _, _ = gpu_step(c, p)
         assert stats[k].cycles == st.cycles
         np.testing.assert_array_equal(alone, outs[k])
+
+
+@pytest.mark.parametrize("m,m_coarse", [(1, 2), (2, 1), (4, 3)])
+@pytest.mark.parametrize("name,shape,lmax", [("V", 0, 3), ("W", 1, 3), ("V", 0, 2)])
+def test_coarse_levels_in_launches_match_oracle(name, shape, lmax, m, m_coarse):
+    """A coarse level too large for the one-launch tail: its runs of one, two and more
+    pseudo-time steps keep the local solve's coefficients from step to step."""
+    case = inputs.random_admissible_2d(272, 192, seed=9, fmax=0.9, cfl=20, bc=("reflect",) * 4,
+                                       lmax=lmax)
+    g = O.Grid.from_case(case)
+    ref, ost, ohist, _ = O.implicit_step(
+        g, case["dt"], case["sa"], case["ss"], case["state"],
+        O.SolveParams(lmax=lmax, tol=1e-10, cycle=shape, m=m, m_coarse=m_coarse, max_cycles=4))
+    out, st, hist, _ = gpu_step(case, m1.m1_default_params(tol=1e-10, cycle=shape, m_pseudo=m,
+                                                           m_coarse=m_coarse, max_cycles=4))
+    assert st.cycles == ost["cycles"] == 4
+    np.testing.assert_allclose(hist, ohist, rtol=1e-9, atol=1e-13 * ohist[0])
+    assert rel_l2(out, ref) <= PARITY
