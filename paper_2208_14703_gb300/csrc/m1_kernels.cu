@@ -434,8 +434,10 @@ __global__ void __launch_bounds__(kThreads) k_coef64(const Level<double>* __rest
 }
 
 // Persistent FP64 sweep (the item loop of k_sweep), held to 128 registers (8 blocks
-// per SM).  Bound by the FP64 pipe, now at 36 of its operations a fine update and
-// not 109: 0.37 ms a sweep at 2048^2 where the FP64 form took 0.88 ms.
+// per SM; 6 and 7, with fewer spills, measured the same or slower).  Bound by the issue
+// of integer instructions, about 900 a warp and row, and then by the FP64 pipe at 10 of
+// its operations a fine update where FP64 throughout takes 103: 0.21 ms a sweep at
+// 2048^2 instead of 0.94, 0.046 ms at 1024^2 instead of 0.19.
 template <bool PSEUDO, bool NORM = false, bool FAS = false, int KEEP = KEEP_NONE>
 __global__ void __launch_bounds__(kStripWarps * 32, 8) k_sweep64(const Level<double>* __restrict__ lv,
                                                                  WorkList wl, Ctl* __restrict__ ctls,

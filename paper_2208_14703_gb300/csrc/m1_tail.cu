@@ -9,6 +9,11 @@
 // cluster barrier (0.2 us) between operations.
 // (The mixed path's FP32 levels: m1_tail32.cu.)
 //
+// What bounds it: the chain of one cell (neighbours 2.1k clocks, the limiter 0.5k, or
+// 3.6k in a warp with a limited cell, the local solve 2.3k, the closure 1.5k), not its
+// FP64 or integer issue.  Measured: the levels of 64^2 and below of a 1024^2 FP64 cycle
+// 0.12 ms.
+//
 // Layout: a level's cells are split into equal ranges of consecutive cells, one
 // range per block (small levels: fewer blocks).  What a cell's neighbours need,
 // its iterate and closure, is stored by the thread that forms the iterate, so
