@@ -12,7 +12,11 @@ namespace m1 {
 // a block may take.
 constexpr int kTailBlocks = 16, kTailClusters = 36, kTailLevels = 20;
 constexpr int kTailSmem = 216 * 1024;
-// The tail begins at the first coarse FP64 level of at most this many cells.
+// The tail begins at the first coarse FP64 level of at most this many cells, which is
+// about what 16 blocks hold with the levels below.  With the line at 2048 cells a step of
+// 320 x 208 (a level of 4160) took 112.8 ms, at 8192 106.2; the paper's beam at 512^2
+// (64^2) 23.4 and 23.6; ten small instances, whose clusters no longer all run at once,
+// 85.1 and 89.5.
 constexpr int kTailCells = 8192;
 
 // Operations of a tail's program, one byte each: the operation + 8 x the level
@@ -50,6 +54,8 @@ cudaError_t launch_tail(const Level<double>* lv, int cap, int nlev, WorkList wl,
 // Its levels give the same bits in the tail and in launches of their own, so where it
 // begins may depend on the company: with more instances each gets a smaller cluster
 // (all of them then run at once) and a tail of fewer cells.
+// A 1024^2 mixed step took 263.0 ms with at most 1024 cells a block (128^2 in 16), 269.5
+// with 256 (64^2).
 constexpr int kTail32Smem = 216 * 1024, kTail32Cells = 1024;   // a block's; cells a block at most
 
 __host__ __device__ inline int tail32_per(int n, int nb)
