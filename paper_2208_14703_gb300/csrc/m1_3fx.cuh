@@ -177,9 +177,11 @@ __device__ __forceinline__ void add_face3(const G3& g, const Blocks3& B, size_t 
 #pragma unroll
         for (int a = 0; a < 3; ++a) m[1 + a] = side < 0 ? F[a] + P[a] : F[a] - P[a];
     }
-    const int sh = em - f.e + 3;
+    // rounded down, or up on the high sides, as fx_to does
+    const int sh = min(em - f.e + 3, 62);
+    const i64 h = side < 0 ? 0 : (1ll << sh) - 1;
 #pragma unroll
-    for (int a = 0; a < 4; ++a) sum[a] += fx_sar(m[a], sh);
+    for (int a = 0; a < 4; ++a) sum[a] += (m[a] + h) >> sh;
 }
 
 template <int d>

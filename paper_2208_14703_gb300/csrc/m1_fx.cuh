@@ -206,8 +206,9 @@ __host__ __device__ __forceinline__ bool fx_stage(double E, double Fx, double Fy
     return ok;
 }
 
-// The double nearest s 2^(e - 58) up to one unit in its last place (rounded half
-// up in magnitude); e within the blocks' exponents, |s| < 2^63.
+// The double nearest s 2^(e - 58), ties to even; e within the blocks' exponents, |s| < 2^63.
+// (Sums of blocks whose low bits are mostly zero tie often: rounding those up gave the
+// total energy a drift of 2^-58 a sweep.)
 __host__ __device__ __forceinline__ double fx_double(i64 s, int e)
 {
     const u64 sign = (u64)s & 0x8000000000000000ull;
@@ -219,7 +220,8 @@ __host__ __device__ __forceinline__ double fx_double(i64 s, int e)
     const int z = __builtin_clzll(m);
 #endif
     m <<= z;                                                   // bit 63 set: value m 2^(e - 58 - z)
-    m = (m >> 11) + ((m >> 10) & 1);                           // 53 bits (2^53 carries into the exponent)
+    const u64 q = m >> 11;                                     // 53 bits (2^53 carries into the exponent)
+    m = q + ((((unsigned)m & 0x7ffu) + ((unsigned)q & 1u) + 0x3ffu) >> 11);
     return double_of_bits(sign | (m + ((u64)(1023 + 63 - 58 - 1 - z + e) << 52)));
 }
 

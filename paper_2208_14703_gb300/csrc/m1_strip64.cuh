@@ -29,11 +29,14 @@ __device__ __forceinline__ FxFlux shfl_flux(const FxFlux& v, int from)
 }
 
 // A flux at scale 2^(e - 58) of the exponent e >= v.e (two bits of headroom for
-// the sum of four).
+// the sum of four), rounded down, or up (UP: the east and north faces): together the
+// faces carry no bias, which a total over many sweeps would gather.
+template <bool UP>
 __device__ __forceinline__ FxFlux fx_to(const FxFlux& v, int e)
 {
-    const int n = e - v.e + 2;
-    return FxFlux{ e, fx_sar(v.E, n), fx_sar(v.Fx, n), fx_sar(v.Fy, n) };
+    const int n = min(e - v.e + 2, 62);
+    const i64 h = UP ? (1ll << n) - 1 : 0;
+    return FxFlux{ e, (v.E + h) >> n, (v.Fx + h) >> n, (v.Fy + h) >> n };
 }
 
 __device__ __forceinline__ FxFlux fx_add(const FxFlux& a, const FxFlux& b)
@@ -43,7 +46,9 @@ __device__ __forceinline__ FxFlux fx_add(const FxFlux& a, const FxFlux& b)
 
 __device__ __forceinline__ FxFlux fx_scale(const FxFlux& a, Split r)
 {
-    return FxFlux{ a.e, mul62(split62(a.E), r), mul62(split62(a.Fx), r), mul62(split62(a.Fy), r) };
+    // + 1: a product falls short by 3/4 of a unit on average
+    return FxFlux{ a.e, mul62(split62(a.E), r, 1), mul62(split62(a.Fx), r, 1),
+                   mul62(split62(a.Fy), r, 1) };
 }
 
 // What a cell gives across its faces: to the east and west, and (2D) to the north
@@ -124,8 +129,8 @@ __device__ __forceinline__ bool strip_march_fx(const Level<double>& L, int2 it, 
         if (two_d) {
             const FxFlux n = fx_south(next);
             em = max(em, max(below.e, n.e));
-            s = fx_add(fx_to(w, em), fx_to(e, em));
-            FxFlux sy = fx_add(fx_to(below, em), fx_to(n, em));
+            s = fx_add(fx_to<false>(w, em), fx_to<true>(e, em));
+            FxFlux sy = fx_add(fx_to<false>(below, em), fx_to<true>(n, em));
             if (L.fx == 2) s = fx_scale(s, rho);
             if (L.fx == 3) sy = fx_scale(sy, rho);
             s = fx_add(s, sy);
@@ -133,7 +138,7 @@ __device__ __forceinline__ bool strip_march_fx(const Level<double>& L, int2 it, 
             if (own) cell(k, p, s);
             cur = next;
         } else {
-            s = fx_add(fx_to(w, em), fx_to(e, em));
+            s = fx_add(fx_to<false>(w, em), fx_to<true>(e, em));
             if (own) cell(k, p, s);
         }
     }
@@ -204,9 +209,8 @@ __device__ __forceinline__ double quotient(double x, double y)
     return fma(fma(-y, q, x), r, q);
 }
 
-// max_admissible_step in two (the bound that binds alone) to thirty FP64 operations
-// where the IEEE divisions and square root took sixty-five; the same bounds, each
-// within an ulp or two.  
+// max_admissible_step in thirty FP64 operations at most where the IEEE divisions and
+// square root took sixty-five; the same bounds, each within an ulp or two.
 __device__ __forceinline__ double cone_step(double a, double b, double c0)
 {
     c0 = c0 > 0.0 ? 0.0 : c0;

@@ -192,13 +192,13 @@ __device__ __forceinline__ void sums64(const Tail& t, int l, int arr, int buf, i
     if (two_d) {
         const FxFlux b = side64(t, l, buf, nb.z, WALL_S, k), n = side64(t, l, buf, nb.w, WALL_N, k);
         em = max(em, max(b.e, n.e));
-        s = fx_add(fx_to(w, em), fx_to(e, em));
-        FxFlux sy = fx_add(fx_to(b, em), fx_to(n, em));
+        s = fx_add(fx_to<false>(w, em), fx_to<true>(e, em));
+        FxFlux sy = fx_add(fx_to<false>(b, em), fx_to<true>(n, em));
         if (L.fx == 2) s = fx_scale(s, split62(L.rho));
         if (L.fx == 3) sy = fx_scale(sy, split62(L.rho));
         s = fx_add(s, sy);
     } else {
-        s = fx_add(fx_to(w, em), fx_to(e, em));
+        s = fx_add(fx_to<false>(w, em), fx_to<true>(e, em));
     }
     if (em == kIrregular) {
         general_sums64(t, l, arr, k, two_d, NE, NFx, NFy);
