@@ -45,15 +45,13 @@ __device__ __noinline__ void general_sums3(const G3& g, const EF* __restrict__ u
 }
 
 __device__ __forceinline__ double limited_step3(const EF& u, double T, const EF& f, double fT,
-                                                double dtau, double theta, double s, double c)
+                                                double dtau, double theta, double c,
+                                                const ConeScale& cone)
 {
-    const float s32 = (float)s;
-    FluxSum F;
+    FluxSum F(cone);
 #pragma unroll
-    for (int a = 0; a < 3; ++a) F.add(narrow_rz(u.F[a]), s32 * narrow_rz(f.F[a]));
-    if (admissible_sure(narrow_rz(u.E), s32 * narrow_rz(f.E), narrow_rz(T), s32 * narrow_rz(fT),
-                        (float)c, F) > 0)
-        return dtau;
+    for (int a = 0; a < 3; ++a) F.add(u.F[a], f.F[a]);
+    if (admissible_sure(u.E, T, f.E, fT, F) > 0) return dtau;
     const double cd = c * c * f.E, cu = c * c * u.E;
     double a = -cd * f.E, b = -cu * f.E, c0 = -cu * u.E;
 #pragma unroll
@@ -138,8 +136,9 @@ __global__ void __launch_bounds__(kThreadsX3, OPX3_BLOCKS) k_opx3(G3 g, const EF
     constexpr bool JAC = MODE == OPX3_JACOBI || MODE == OPX3_JACOBI_NORM;
     constexpr bool LOCAL = MODE != OPX3_JACOBI && MODE != OPX3_PSEUDO;   // forms D(u)
     if (skipx3(ctl)) return;
-    double dtau = 0.0, theta = 0.0, s = 0.0;
-    if (STEP) { dtau = ctl->dtau; theta = ctl->theta_ex; s = dtau / theta; }
+    double dtau = 0.0, theta = 0.0;
+    if (STEP) { dtau = ctl->dtau; theta = ctl->theta_ex; }
+    const ConeScale cone = STEP ? cone_scale(dtau / theta, g.ic) : ConeScale{};
     const double A = STEP ? fma(dtau, g.diag, 1.0) : g.diag, C = STEP ? fma(dtau, g.c_v, 1.0) : g.c_v;
     double nrm = 0.0;
     unsigned int fails = 0;
@@ -216,7 +215,7 @@ __global__ void __launch_bounds__(kThreadsX3, OPX3_BLOCKS) k_opx3(G3 g, const EF
             } else {
                 co = Q[q];
             }
-            const double tau = limited_step3(uc, Tc, ff, ffT, dtau, theta, s, g.c);
+            const double tau = limited_step3(uc, Tc, ff, ffT, dtau, theta, g.c, cone);
 #pragma unroll
             for (int m = 0; m < 3; ++m)
                 rhs[m] = fma(dtau * fF, N[1 + m], fma(tau, ff.F[m], uc.F[m]));
@@ -337,6 +336,7 @@ __global__ void __launch_bounds__(kThreadsX3) k_prolongx3(G3 gc, G3 gf, const EF
 {
     if (skipx3(ctl)) return;
     const double theta = ctl->theta_c, c = gf.c;
+    const ConeScale cone = cone_scale(1.0, gf.ic);
     const size_t nf = (size_t)gf.n[0] * gf.n[1] * gf.n[2];
     const int lane = threadIdx.x & 31;
     const unsigned chunks = (unsigned)(gc.n[0] + 30) / 31u;
@@ -384,10 +384,10 @@ __global__ void __launch_bounds__(kThreadsX3) k_prolongx3(G3 gc, G3 gf, const EF
 #pragma unroll
             for (int m = 0; m < 3; ++m) t.F[m] = fma(wt, pe[1 + m], u.F[m]);
             double tT = fma(wt, pe[4], uT);
-            FluxSum F;
+            FluxSum F(cone);
 #pragma unroll
-            for (int m = 0; m < 3; ++m) F.add(narrow_rz(t.F[m]), 0.f);
-            const int sure = admissible_sure(narrow_rz(t.E), 0.f, narrow_rz(tT), 0.f, (float)c, F);
+            for (int m = 0; m < 3; ++m) F.add(t.F[m], 0.0);
+            const int sure = admissible_sure(t.E, tT, 0.0, 0.0, F);
             if (sure < 0 || (sure == 0 && !admissible3(t, tT, c))) {
                 EF d;
                 d.E = wt * pe[0];

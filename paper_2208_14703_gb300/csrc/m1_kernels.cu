@@ -344,6 +344,7 @@ __device__ __forceinline__ double strip_sweep64(const Level<double>& L, Ctl* ctl
         // the pseudo-time step's A and C
         const double Ap = PSEUDO ? fma(ps.dtau, L.diag, 1.0) : 0.0;
         const double Cp = PSEUDO ? fma(ps.dtau, L.c_v, 1.0) : 0.0;
+        const ConeScale cone = PSEUDO ? cone_scale(ps.s, L.ic) : ConeScale{};
         auto pre = [&](size_t k) {
             Pre p;
             p.b = FAS ? L.r[k] : L.f[k];
@@ -386,7 +387,7 @@ __device__ __forceinline__ double strip_sweep64(const Level<double>& L, Ctl* ctl
                 o = local_solve64(p.q, L.diag, L.c_v, L.a_r, fma(cbE, NE, b.E), fma(cbF, NFx, b.Fx),
                                   fma(cbF, NFy, b.Fy), b.T, ok);
             } else {
-                const double tau = limited_step64(p.u, b, ps.dtau, ps.theta, ps.s, L.c);
+                const double tau = limited_step64(p.u, b, ps.dtau, ps.theta, ps.s, L.c, cone);
                 const Coef q = KEEP == KEEP_LOAD ? p.q
                                                  : make_coef(1.0, ps.dtau, L.diag, ka, kt, L.a_r);
                 if (KEEP == KEEP_STORE) reinterpret_cast<Coef*>(L.r)[k] = q;
@@ -1058,18 +1059,14 @@ __device__ __forceinline__ void prolong_cells64(const Level<double>& Lf, const C
 {
     typedef Cell4<double> C;
     auto add = [](const C& a, const C& b) { return C{ a.E + b.E, a.Fx + b.Fx, a.Fy + b.Fy, a.T + b.T }; };
-    const float c32 = (float)Lf.c;
     auto put = [&](int ox, int oy, double wt, const C& s) {
         const size_t k = (size_t)(2 * jc + oy) * Lf.nx + 2 * ic + ox;
         const C u = uf[k];
         C o = { fma(wt, s.E, u.E), fma(wt, s.Fx, u.Fx), fma(wt, s.Fy, u.Fy), fma(wt, s.T, u.T) };
-        const float w32 = (float)wt;
-        FluxSum F;
-        F.add(narrow_rz(u.Fx), w32 * narrow_rz(s.Fx));
-        F.add(narrow_rz(u.Fy), w32 * narrow_rz(s.Fy));
-        if (admissible_sure(narrow_rz(u.E), w32 * narrow_rz(s.E), narrow_rz(u.T),
-                            w32 * narrow_rz(s.T), c32, F) <= 0 &&
-            !admissible(o, Lf.c)) {
+        FluxSum F(cone_scale(wt, Lf.ic));
+        F.add(u.Fx, s.Fx);
+        F.add(u.Fy, s.Fy);
+        if (admissible_sure(u.E, u.T, s.E, s.T, F) <= 0 && !admissible(o, Lf.c)) {
             const C pe = { wt * s.E, wt * s.Fx, wt * s.Fy, wt * s.T };
             const double th = ctl->theta_c * fmin(1.0, max_admissible_step64(u, pe, Lf.c));
             o = C{ fma(th, pe.E, u.E), fma(th, pe.Fx, u.Fx), fma(th, pe.Fy, u.Fy), fma(th, pe.T, u.T) };

@@ -239,42 +239,64 @@ __device__ __forceinline__ double max_admissible_step64(const Cell4<double>& u,
 
 // Whether u + s f is admissible, decided in FP32 where that is beyond doubt (values
 // rounded toward zero, a margin of 1e-6 of the terms' sizes where the roundings
-// leave at most 5e-7): 1 yes, -1 no, 0 unknown.  c, s in FP32; F2 the squared length
-// of u_F + s f_F and its margin are the caller's (two or three components).
+// leave at most 6e-7): 1 yes, -1 no, 0 unknown.
+//
+// The question is put to E, T and F / c, so that light speeds of any unit system leave
+// squares of the size of E^2 (with |F| against c E, CGS light speeds passed FP32's range
+// at E = 6e8).  It is answered inside these bounds, where nothing that FP32 flushes to
+// zero or overflows can reach a margin: s and 1 / c within 1e-30 .. 1e15, their product
+// at most 1e15 (what narrow_rz drops, 1.2e-38, stays below 1e-22), E and T above 1e-15,
+// E below 1e15, the sum of squares within 1e-30 .. 1e37 of an answer that rests on it.
+struct ConeScale {
+    float s, ic;                   // s and 1 / c; s NaN where they are out of range
+};
+
+__host__ __device__ __forceinline__ ConeScale cone_scale(double s, double ic)
+{
+    const float s32 = (float)s, i32 = (float)ic;
+    const bool ok = s32 >= 1e-30f && s32 <= 1e15f && i32 >= 1e-30f && i32 <= 1e15f &&
+                    s32 * i32 <= 1e15f;
+    return ConeScale{ ok ? s32 : float_of_bits(0x7fc00000u), i32 };
+}
+
 struct FluxSum {
-    float hi = 0.f, lo = 0.f;      // squared length with the margins added, taken off
-    __device__ __forceinline__ void add(float u, float f)
+    ConeScale q;
+    float hi = 0.f, lo = 0.f;      // squared length of (u + s f) / c, margins added, taken off
+    __host__ __device__ __forceinline__ explicit FluxSum(const ConeScale& scale) : q(scale) {}
+    __host__ __device__ __forceinline__ void add(double u64, double f64)
     {
+        const float u = q.ic * narrow_rz(u64), f = q.ic * (q.s * narrow_rz(f64));
         const float p = fabsf(u + f), m = 1e-6f * (fabsf(u) + fabsf(f));
         hi = fmaf(p + m, p + m, hi);
         lo = fmaf(fmaxf(p - m, 0.f), fmaxf(p - m, 0.f), lo);
     }
 };
 
-__device__ __forceinline__ int admissible_sure(float uE, float fE, float uT, float fT, float c,
-                                               const FluxSum& F)
+__host__ __device__ __forceinline__ int admissible_sure(double E, double T, double dE, double dT,
+                                                        const FluxSum& F)
 {
     const float m = 1e-6f;
-    if (!(uE > 1e-15f && uT > 1e-30f && uE < 1e15f)) return 0;
+    const float uE = narrow_rz(E), uT = narrow_rz(T);
+    if (!(uE > 1e-15f && uT > 1e-15f && uE < 1e15f)) return 0;
+    const float fE = F.q.s * narrow_rz(dE), fT = F.q.s * narrow_rz(dT);
     const float mE = m * (uE + fabsf(fE)), mT = m * (uT + fabsf(fT));
     const float pE = uE + fE, pT = uT + fT;
     if (pE < -mE || pT < -mT) return -1;
-    const float lo = c * (pE - mE), hi = c * (pE + mE);
-    if (pT > mT && lo > 1e-15f * c && F.hi <= 0.99999f * lo * lo) return 1;
-    if (F.lo >= 1.00001f * hi * hi && F.lo < 1e30f) return -1;
+    const float lo = pE - mE, hi = pE + mE;
+    if (pT > mT && lo > 1e-15f && F.hi <= 0.99999f * lo * lo && F.hi < 1e37f) return 1;
+    if (F.lo >= 1.00001f * hi * hi && F.lo > 1e-30f && F.lo < 1e37f) return -1;
     return 0;
 }
 
 // limited_step with the question whether it binds put in FP32 first.
 __device__ __forceinline__ double limited_step64(const Cell4<double>& u, const Cell4<double>& f,
-                                                 double dtau, double theta, double s, double c)
+                                                 double dtau, double theta, double s, double c,
+                                                 const ConeScale& q)
 {
-    const float s32 = (float)s;
-    FluxSum F;
-    F.add(narrow_rz(u.Fx), s32 * narrow_rz(f.Fx));
-    F.add(narrow_rz(u.Fy), s32 * narrow_rz(f.Fy));
-    const int sure = admissible_sure(narrow_rz(u.E), s32 * narrow_rz(f.E), narrow_rz(u.T),
-                                     s32 * narrow_rz(f.T), (float)c, F);
+    FluxSum F(q);
+    F.add(u.Fx, f.Fx);
+    F.add(u.Fy, f.Fy);
+    const int sure = admissible_sure(u.E, u.T, f.E, f.T, F);
     if (sure > 0) return dtau;
     if (sure == 0) {
         const Cell4<double> p = { fma(s, f.E, u.E), fma(s, f.Fx, u.Fx), fma(s, f.Fy, u.Fy),

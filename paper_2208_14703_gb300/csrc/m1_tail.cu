@@ -59,9 +59,10 @@ __device__ __forceinline__ int arr_at(int a, int per)
 }
 
 // What a level's pseudo-time steps share: dtau c b, dtau c^2 b (the sums' factors),
-// A = 1 + dtau diag, C = 1 + dtau C_v.
+// A = 1 + dtau diag, C = 1 + dtau C_v, the limiter's scale.
 struct TailStep {
     double cbE, cbF, A, C;
+    ConeScale cone;
 };
 
 // A cell's block that could not be formed (m1_fx.cuh: not regular): its
@@ -347,7 +348,7 @@ __device__ __forceinline__ void op_cell(const Tail& t, int op, int l, int cur, i
     }
     const TailStep& ts = t.step[l];
     const double cbE = fx ? ts.cbE : ps.dtau, cbF = fx ? ts.cbF : ps.dtau;
-    const double tau = limited_step64(u, b, ps.dtau, ps.theta, ps.s, L.c);
+    const double tau = limited_step64(u, b, ps.dtau, ps.theta, ps.s, L.c, ts.cone);
     bool ok;
     const C o = local_solve64(co, ts.A, ts.C, L.a_r, fma(cbE, NE, fma(tau, b.E, u.E)),
                               fma(cbF, NFx, fma(tau, b.Fx, u.Fx)),
@@ -408,7 +409,7 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const Level<double>* _
         if (threadIdx.x < nl) {
             const Level<double>& L = Ls[threadIdx.x];
             steps[threadIdx.x] = TailStep{ ps.dtau * L.cb, ps.dtau * L.cbF, fma(ps.dtau, L.diag, 1.0),
-                                           fma(ps.dtau, L.c_v, 1.0) };
+                                           fma(ps.dtau, L.c_v, 1.0), cone_scale(ps.s, L.ic) };
         }
         const double theta_c = ctl->theta_c;
         unsigned fails = 0, damped = 0;

@@ -1,0 +1,51 @@
+"""The fixed-point and FP32-first arithmetic of the FP64 kernels on the host
+(tests/fx_host.py), without a GPU."""
+import ctypes
+
+import numpy as np
+import pytest
+
+from tests import fx_host
+
+D = ctypes.c_double
+
+
+@pytest.fixture(scope="module")
+def host(tmp_path_factory):
+    return fx_host.load(tmp_path_factory.mktemp("fx_host"))
+
+
+def truth(u, f, s, c):
+    """+1 inside, -1 outside the cone, by the exact sign of c E - |F| of u + s f in 80
+    bits; values scaled to E first, so that no square leaves the range."""
+    u, f = u.astype(np.longdouble), f.astype(np.longdouble)
+    p = u + np.longdouble(s) * f
+    E, T = p[:, 0], p[:, 3]
+    x, y = p[:, 1] / np.longdouble(c), p[:, 2] / np.longdouble(c)
+    size = np.maximum(np.maximum(np.abs(E), np.abs(x)), np.maximum(np.abs(y), np.longdouble(1e-4000)))
+    inside = (E > 0) & (T > 0) & ((x / size) ** 2 + (y / size) ** 2 <= (E / size) ** 2)
+    return np.where(inside, 1, -1)
+
+
+@pytest.mark.parametrize("s", [0.25, 1.0, 2e6, 2e-12, 1e-36, 1e20])
+@pytest.mark.parametrize("c", [1.0, 2.99792458e10, 1e-11, 2.99792458e3, 1e-18, 1e30])
+def test_sure_answers_are_right(host, c, s):
+    """Whatever the units, an answer given without doubt is the exact one: states of
+    E from 1e-40 to 1e40 (single sizes and spread), fluxes from deep inside the cone to ten
+    times its length, right-hand sides from nothing to a thousand times the state."""
+    rng = np.random.default_rng(7)
+    n = 4000
+    for lo, hi in ((-1, 1), (5, 12), (-16, -11), (-40, 40)):
+        u, f = np.zeros((n, 4)), np.zeros((n, 4))
+        E = 10.0 ** rng.uniform(lo, hi, n)
+        for a, amp in ((u, 1.0), (f, 10.0 ** rng.uniform(-20, 3, n) / s)):
+            a[:, 0] = E * amp * (1.0 if a is u else rng.uniform(-1, 1, n))
+            a[:, 3] = E * amp * (1.0 if a is u else rng.uniform(-1, 1, n))
+            phi, r = rng.uniform(0, 2 * np.pi, n), 10.0 ** rng.uniform(-2, 1, n)
+            a[:, 1], a[:, 2] = (c * E * amp * r * g(phi) for g in (np.cos, np.sin))
+        out = np.zeros(n, np.int32)
+        host.host_admissible_sure(n, fx_host.ptr(u), fx_host.ptr(f), D(s), D(c), fx_host.ptr(out))
+        t = truth(u, f, s, c)
+        assert np.all((out == 0) | (out == t)), (lo, hi, np.flatnonzero((out != 0) & (out != t))[:5])
+        if 1e-12 <= s <= 2e6 and 1e-11 <= c <= 1e11 and s <= 1e15 * c and lo >= -12 and hi < 15:
+            assert np.mean(out == 0) < 0.01        # ... and it is given
