@@ -60,6 +60,27 @@ m1_status run_until_done(cudaGraphExec_t graph, int graph_cycles, int max_cycles
     return M1_OK;
 }
 
+m1_status end_capture(cudaStream_t s, cudaGraphExec_t* graph, long long* nodes)
+{
+    // the launches leave their refusal in the runtime's last error
+    const cudaError_t launches = cudaGetLastError();
+    cudaGraph_t g = nullptr;
+    cudaError_t e = cudaStreamEndCapture(s, &g);
+    if (e == cudaSuccess && launches == cudaSuccess) {
+        size_t n = 0;
+        if (nodes) *nodes = cudaGraphGetNodes(g, nullptr, &n) == cudaSuccess ? (long long)n : 0;
+        e = cudaGraphInstantiate(graph, g, 0);
+        if (e != cudaSuccess) *graph = nullptr;
+    }
+    if (g) cudaGraphDestroy(g);
+    if (e == cudaSuccess) e = launches;
+    if (e != cudaSuccess) {
+        set_err(e, "recording a cycle");
+        return M1_ERR_CUDA;
+    }
+    return M1_OK;
+}
+
 // Full-weighting restriction of an inflow profile along its wall (1/4, 1/2,
 // 1/4; ends copied), giving the coarse level's prescribed ghost states.
 void restrict_profile(const double* fine, int nf, double* coarse, int nc)
@@ -766,13 +787,6 @@ void program(const Params& p, int L, int first, int l, int shape, bool fas,
     }
 }
 
-// Kernel nodes of a graph.
-long long graph_nodes(cudaGraph_t g)
-{
-    size_t n = 0;
-    return cudaGraphGetNodes(g, nullptr, &n) == cudaSuccess ? (long long)n : 0;
-}
-
 }  // namespace
 
 // The tails' programs for the parameters, on the device: a shape's for every first
@@ -888,17 +902,11 @@ m1_status Engine<R>::build_graph(const Params& p)
     // a captured graph must return the fine iterate to buffer 0
     const int per_cycle = L == 1 ? p.nu0 : 2 * p.nu0;
     graph_cycles = (per_cycle % 2) ? 2 : 1;
-    cudaGraph_t g = nullptr;
     M1_CK(cudaStreamBeginCapture(cap_stream, cudaStreamCaptureModeThreadLocal));
     int cur0 = 0;
     for (int c = 0; c < graph_cycles; ++c) record_cycle(p, cur0, cap_stream);
-    cudaError_t e = cudaStreamEndCapture(cap_stream, &g);
-    if (e != cudaSuccess) { set_err(e, "cudaStreamEndCapture"); return M1_ERR_CUDA; }
-    if (cur0 != 0) { cudaGraphDestroy(g); return M1_ERR_INVALID_ARG; }
-    kernels_per_launch = graph_nodes(g);
-    e = cudaGraphInstantiate(&graph, g, 0);
-    cudaGraphDestroy(g);
-    if (e != cudaSuccess) { set_err(e, "cudaGraphInstantiate"); graph = nullptr; return M1_ERR_CUDA; }
+    M1_TRY(end_capture(cap_stream, &graph, &kernels_per_launch));
+    if (cur0 != 0) { cudaGraphExecDestroy(graph); graph = nullptr; return M1_ERR_INVALID_ARG; }
     gparams = p;
     graph_dirty = false;
     return M1_OK;
@@ -1471,15 +1479,9 @@ m1_status MixedModel::build_graph(const Params& p)
     if (graph && gparams == p && !hi.graph_dirty && !lo.graph_dirty) return M1_OK;
     if (graph) { cudaGraphExecDestroy(graph); graph = nullptr; }
     M1_TRY(lo.write_programs(p));
-    cudaGraph_t g = nullptr;
     M1_CK(cudaStreamBeginCapture(lo.cap_stream, cudaStreamCaptureModeThreadLocal));
     record_cycle(p, lo.cap_stream);
-    cudaError_t e = cudaStreamEndCapture(lo.cap_stream, &g);
-    if (e != cudaSuccess) { set_err(e, "cudaStreamEndCapture"); return M1_ERR_CUDA; }
-    kernels_per_launch = graph_nodes(g);
-    e = cudaGraphInstantiate(&graph, g, 0);
-    cudaGraphDestroy(g);
-    if (e != cudaSuccess) { set_err(e, "cudaGraphInstantiate"); graph = nullptr; return M1_ERR_CUDA; }
+    M1_TRY(end_capture(lo.cap_stream, &graph, &kernels_per_launch));
     gparams = p;
     hi.graph_dirty = lo.graph_dirty = false;
     return M1_OK;

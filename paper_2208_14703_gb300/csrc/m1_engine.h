@@ -65,6 +65,9 @@ Ctl make_ctl(const m1_solve_params& sp, double diag0);
 m1_status run_until_done(cudaGraphExec_t graph, int graph_cycles, int max_cycles,
                          cudaStream_t stream, BatchCtl* bctl, int* done_h, cudaEvent_t* poll,
                          long long* launched_out);
+// Ends the capture of a cycle on s and makes its graph; an error where a launch of the
+// cycle was refused (the graph would lack it).  nodes (may be null): the graph's kernels.
+m1_status end_capture(cudaStream_t s, cudaGraphExec_t* graph, long long* nodes);
 void restrict_profile(const double* fine, int nf, double* coarse, int nc);
 
 template <typename R>

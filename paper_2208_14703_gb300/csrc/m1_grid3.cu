@@ -405,15 +405,10 @@ m1_status Grid3::build_graph(const Params& p, double dt)
 {
     if (graph && gparams == p && graph_dt == dt) return M1_OK;
     if (graph) { cudaGraphExecDestroy(graph); graph = nullptr; }
-    cudaGraph_t g = nullptr;
     kernels_per_cycle = 0;
     M1_CK(cudaStreamBeginCapture(cap_stream, cudaStreamCaptureModeThreadLocal));
     emit_cycle(p, cap_stream);
-    cudaError_t e = cudaStreamEndCapture(cap_stream, &g);
-    if (e != cudaSuccess) { set_err(e, "cudaStreamEndCapture"); return M1_ERR_CUDA; }
-    e = cudaGraphInstantiate(&graph, g, 0);
-    cudaGraphDestroy(g);
-    if (e != cudaSuccess) { set_err(e, "cudaGraphInstantiate"); graph = nullptr; return M1_ERR_CUDA; }
+    M1_TRY(end_capture(cap_stream, &graph, nullptr));
     gparams = p;
     graph_dt = dt;
     return M1_OK;
