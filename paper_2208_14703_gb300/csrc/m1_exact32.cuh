@@ -1,14 +1,15 @@
-// The FP32 correction-form arithmetic with every rounding written out.
+// The FP32 correction-form arithmetic of the coarse levels with every rounding written
+// out, one cell at a time.
 //
-// closure_delta, local_solve_delta, limited_step and the operator's rows
-// (m1_device.cuh, m1_cell.cuh, m1_kernels.cu) leave the choice of fused
-// multiply-adds to the compiler, whose choices differ between kernels; a small mixed
-// problem carries such last-bit differences into the ninth digit of its result.
-// These forms spell out the choices the strip kernels are compiled with (whole steps are
-// compared bit for bit in tests/test_gpu_tail32.py), so that another kernel can take
-// over a level without changing a result.
+// A coarse level of a mixed instance is walked by the strip kernels (m1_kernels.cu) or
+// by the one-launch tail (m1_tail32.cu), as the number of instances beside it decides, and
+// a small mixed problem carries last-bit differences into the ninth digit of its result.
+// Left to the compiler, fused multiply-adds are chosen kernel by kernel.  Both call these
+// functions, so that a level gives the same bits in either whatever the constants and the
+// compiler.  Where a choice is stated below it is the one that the strip kernels were
+// compiled with when the forms were fixed.
 #pragma once
-#include "m1_device.cuh"
+#include "m1_cell.cuh"
 
 namespace m1 {
 
@@ -120,25 +121,39 @@ __device__ __forceinline__ float max_admissible_step_x(const Cell4<float>& u, co
     return fminf(tau, t);
 }
 
+// admissible_c2 (SLACK as there).
+template <bool SLACK>
+__device__ __forceinline__ bool admissible_x(const Cell4<float>& s, float c2)
+{
+    float lim = X_MUL(X_MUL(c2, s.E), s.E);
+    if (SLACK) lim = X_MUL(lim, 1.f + Slack<float>::v);
+    return s.E > 0.f && s.T > 0.f && X_FMA(s.Fx, s.Fx, X_MUL(s.Fy, s.Fy)) <= lim;
+}
+
+__device__ __forceinline__ Cell4<float> add_x(const Cell4<float>& a, const Cell4<float>& b)
+{
+    return Cell4<float>{ X_ADD(a.E, b.E), X_ADD(a.Fx, b.Fx), X_ADD(a.Fy, b.Fy), X_ADD(a.T, b.T) };
+}
+
+// fma by one factor: a + s b.
+__device__ __forceinline__ Cell4<float> axpy_x(const Cell4<float>& a, float s, const Cell4<float>& b)
+{
+    return Cell4<float>{ X_FMA(s, b.E, a.E), X_FMA(s, b.Fx, a.Fx), X_FMA(s, b.Fy, a.Fy),
+                         X_FMA(s, b.T, a.T) };
+}
+
 __device__ __forceinline__ float limited_step_x(const Cell4<float>& u, const Cell4<float>& f,
                                                 float dtau, float theta, float s, float c)
 {
-    const Cell4<float> p = { X_FMA(s, f.E, u.E), X_FMA(s, f.Fx, u.Fx), X_FMA(s, f.Fy, u.Fy),
-                             X_FMA(s, f.T, u.T) };
-    if (admissible_c2<float, false>(p, X_MUL(c, c))) return dtau;
+    if (admissible_x<false>(axpy_x(u, s, f), X_MUL(c, c))) return dtau;
     return fminf(dtau, X_MUL(theta, max_admissible_step_x<false>(u, f, c)));
 }
-
-// What a cell's neighbour holds for its sums.
-struct Near32 {
-    float E, Fx, Fy, Pxx, Pxy, Pyy;
-};
 
 // The neighbour sums N of Eq. (9): the y pair's term fused onto the x pair's product,
 // or (xfused: the strips that stage their rows by cp.async) the other way round.
 __device__ __forceinline__ void sums_x(float c, float bx, float by, bool two_d, bool xfused,
-                                       const Near32& w, const Near32& e, const Near32& s,
-                                       const Near32& n, float& NE, float& NFx, float& NFy)
+                                       const Staged<float>& w, const Staged<float>& e,
+                                       const Staged<float>& s, const Staged<float>& n, float& NE, float& NFx, float& NFy)
 {
     const float cbx = X_MUL(c, bx), cby = X_MUL(c, by);
     const float xE = X_FMA(c, X_ADD(w.E, e.E), X_SUB(w.Fx, e.Fx));
@@ -160,6 +175,73 @@ __device__ __forceinline__ void sums_x(float c, float bx, float by, bool two_d, 
         NFx = X_FMA(cby, yF, X_MUL(cbx, xF));
         NFy = X_FMA(cby, yG, X_MUL(cbx, xG));
     }
+}
+
+// The neighbour sums of a cell.
+struct Sums32 {
+    float E, Fx, Fy;
+};
+
+// One pseudo-time step of a cell (update_cell's correction form): its base w, A(w), iterate
+// e and right-hand side b.
+__device__ __forceinline__ Cell4<float> pseudo_x(const Level<float>& L, const Sig2<float>& sg,
+                                                 const Cell4<float>& w, const Cell4<float>& aw,
+                                                 const Cell4<float>& e, const Cell4<float>& b,
+                                                 const Sums32& N, const Pseudo<float>& ps, bool& ok)
+{
+    const float ka = X_MUL(L.cdt, sg.sa), dk = X_ADD(L.diag, X_MUL(L.cdt, X_ADD(sg.sa, sg.ss)));
+    const float tau = limited_step_x(add_x(w, e), add_x(aw, b), ps.dtau, ps.theta, ps.s, L.c);
+    const float lim = X_SUB(tau, ps.dtau);
+    const Cell4<float> rhs = axpy_x(axpy_x(e, tau, b), lim, aw);
+    return local_solve_delta_x(ps.dtau, L.diag, ka, dk, L.c_v, L.a_r, w.T, X_FMA(ps.dtau, N.E, rhs.E),
+                               X_FMA(ps.dtau, N.Fx, rhs.Fx), X_FMA(ps.dtau, N.Fy, rhs.Fy), rhs.T, ok);
+}
+
+// A(w + e) - A(w) of a cell of base temperature T.
+__device__ __forceinline__ Cell4<float> rows_x(const Level<float>& L, const Sig2<float>& sg, float T,
+                                               const Cell4<float>& e, const Sums32& N)
+{
+    const float ka = X_MUL(L.cdt, sg.sa), dk = X_FMA(L.cdt, X_ADD(sg.sa, sg.ss), L.diag);
+    const float se = X_MUL(ka, X_FMA(-L.a_r, quartic_delta_x<false>(T, e.T), e.E));
+    return Cell4<float>{ X_SUB(X_FMA(L.diag, e.E, se), N.E), X_FMA(dk, e.Fx, -N.Fx),
+                         X_FMA(dk, e.Fy, -N.Fy), X_FMA(L.c_v, e.T, -se) };
+}
+
+__device__ __forceinline__ Cell4<float> sub_x(const Cell4<float>& a, const Cell4<float>& b)
+{
+    return Cell4<float>{ X_SUB(a.E, b.E), X_SUB(a.Fx, b.Fx), X_SUB(a.Fy, b.Fy), X_SUB(a.T, b.T) };
+}
+
+// The right-hand side of a fresh visit: A(w), from the sums of w, and
+// f = [A(w + v) - A(w)] + r, from those of v.
+__device__ __forceinline__ Cell4<float> base_rows_x(const Level<float>& L, const Sig2<float>& sg,
+                                                    const Cell4<float>& w, const Sums32& N)
+{
+    const float ka = X_MUL(L.cdt, sg.sa), dk = X_ADD(L.diag, X_MUL(L.cdt, X_ADD(sg.sa, sg.ss)));
+    const float T2 = X_MUL(w.T, w.T), sw = X_MUL(ka, X_FMA(-X_MUL(L.a_r, T2), T2, w.E));
+    return Cell4<float>{ X_SUB(X_FMA(L.diag, w.E, sw), N.E), X_FMA(dk, w.Fx, -N.Fx),
+                         X_FMA(dk, w.Fy, -N.Fy), X_FMA(L.c_v, w.T, -sw) };
+}
+__device__ __forceinline__ Cell4<float> fas_rhs_x(const Level<float>& L, const Sig2<float>& sg, float T,
+                                                  const Cell4<float>& v, const Cell4<float>& r,
+                                                  const Sums32& N)
+{
+    const float ka = X_MUL(L.cdt, sg.sa), dk = X_ADD(L.diag, X_MUL(L.cdt, X_ADD(sg.sa, sg.ss)));
+    const float sd = X_MUL(ka, X_FMA(-L.a_r, quartic_delta_x<false>(T, v.T), v.E));
+    return add_x(Cell4<float>{ X_SUB(X_FMA(L.diag, v.E, sd), N.E), X_FMA(dk, v.Fx, -N.Fx),
+                               X_FMA(dk, v.Fy, -N.Fy), X_FMA(L.c_v, v.T, -sd) }, r);
+}
+
+// The correction e of a fine cell of base w with the prolongated correction pe added,
+// damped (Eq. (34)) where the target is not admissible.
+__device__ __forceinline__ Cell4<float> prolong_x(const Cell4<float>& e, const Cell4<float>& w,
+                                                  const Cell4<float>& pe, float theta_c, float c,
+                                                  bool& damped)
+{
+    const Cell4<float> u = add_x(e, w);
+    damped = !admissible_x<true>(add_x(u, pe), X_MUL(c, c));
+    const float th = damped ? X_MUL(theta_c, fminf(1.f, max_admissible_step_x<true>(u, pe, c))) : 1.f;
+    return axpy_x(e, th, pe);
 }
 
 }  // namespace m1

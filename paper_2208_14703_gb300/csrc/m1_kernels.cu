@@ -22,6 +22,7 @@
 
 #include "m1_cell.cuh"
 #include "m1_dw.cuh"
+#include "m1_exact32.cuh"
 #include "m1_kernels.cuh"
 #include "m1_strip64.cuh"
 
@@ -91,7 +92,10 @@ __device__ __forceinline__ Raw<R> load_raw(const Level<R>& L, const Cell4<R>* __
     return r;
 }
 
-template <typename R, bool DELTA>
+// FORM (correction form): the compiler's choice of fused operations (the fine level's
+// sweeps), or one of m1_exact32.cuh's, for what the one-launch tail evaluates too.
+enum StageForm { FORM_FREE = 0, FORM_STEP = 1, FORM_FAS = 2 };
+template <typename R, bool DELTA, int FORM = FORM_FREE>
 __device__ __forceinline__ Staged<R> stage_raw(const Level<R>& L, const Raw<R>& r)
 {
     Staged<R> o;
@@ -100,7 +104,11 @@ __device__ __forceinline__ Staged<R> stage_raw(const Level<R>& L, const Raw<R>& 
         closure(r.c.E, r.c.Fx, r.c.Fy, L.ic2, o.Pxx, o.Pxy, o.Pyy);
         o.T = r.c.T;
     } else {
-        closure_delta(r.w.E, r.w.Fx, r.w.Fy, r.c.E, r.c.Fx, r.c.Fy, L.ic2, o.Pxx, o.Pxy, o.Pyy);
+        if constexpr (FORM != FORM_FREE)
+            closure_delta_x<FORM == FORM_FAS>(r.w.E, r.w.Fx, r.w.Fy, r.c.E, r.c.Fx, r.c.Fy, L.ic2,
+                                              o.Pxx, o.Pxy, o.Pyy);
+        else
+            closure_delta(r.w.E, r.w.Fx, r.w.Fy, r.c.E, r.c.Fx, r.c.Fy, L.ic2, o.Pxx, o.Pxy, o.Pyy);
         o.T = r.w.T;
     }
     return o;
@@ -122,7 +130,8 @@ __device__ __forceinline__ Staged<R> stage_raw(const Level<R>& L, const Raw<R>& 
 // step first forms the FAS right-hand side f = A(v) + r (Eq. (24)) from its own
 // neighbour terms, as the FAS kernel writes it, stores it for the later steps
 // and uses it.
-template <typename R, bool PSEUDO, bool DELTA, bool NORM = false, bool FAS = false>
+// RING: from the cp.async strips (which of the two pairs' products is fused).
+template <typename R, bool PSEUDO, bool DELTA, bool NORM = false, bool FAS = false, bool RING = false>
 __device__ __forceinline__ void update_cell(const Level<R>& L, Ctl* ctl, const Staged<R>& wv,
                                             const Staged<R>& ev, const Staged<R>& prev,
                                             const Staged<R>& next, const Staged<R>& cur,
@@ -131,6 +140,19 @@ __device__ __forceinline__ void update_cell(const Level<R>& L, Ctl* ctl, const S
                                             const Cell4<R>& wb, const Pseudo<R>& ps,
                                             double* nrm = nullptr)
 {
+    if constexpr (DELTA && PSEUDO) {
+        // u = w + e and f = A(w) + g: the full-form step u' + dtau A(u') = u + tau f
+        // reads, for the correction,
+        // e' + dtau (A(w+e') - A(w)) = e + tau g + (tau - dtau) A(w);
+        // the last term is zero wherever the step is not limited
+        Sums32 N;
+        sums_x(L.c, L.bx, L.by, two_d, RING, wv, ev, prev, next, N.E, N.Fx, N.Fy);
+        bool ok;
+        const Cell4<R> o = pseudo_x(L, sg, wb, L.aw[k], u, b_in, N, ps, ok);
+        if (!ok) atomicAdd(&ctl->newton_fail, 1u);
+        L.u[out_buf][k] = o;
+        return;
+    } else {
     Cell4<R> b = b_in;
     const R c = L.c, bx = L.bx, by = L.by;
     R NE = bx * (c * (wv.E + ev.E) + (wv.Fx - ev.Fx));
@@ -172,30 +194,14 @@ __device__ __forceinline__ void update_cell(const Level<R>& L, Ctl* ctl, const S
         // explicit half: u~ = u + tau f, tau = min(dtau, theta tau*); implicit half:
         // one Jacobi sweep of u + dtau A(u) = u~ from the old iterate.
         const R dtau = ps.dtau, theta = ps.theta, dts = ps.s;
-        if (!DELTA) {
-            const R tau = limited_step(u, b, dtau, theta, dts, c);
-            out = local_solve<R>(R(1), dtau, L.diag, ka, kt, L.c_v, L.a_r,
-                                 u.E + tau * b.E + dtau * NE, u.Fx + tau * b.Fx + dtau * NFx,
-                                 u.Fy + tau * b.Fy + dtau * NFy, u.T + tau * b.T, ok);
-        } else {
-            // u = w + e and f = A(w) + g: the full-form step u' + dtau A(u') = u + tau f
-            // reads, for the correction,
-            // e' + dtau (A(w+e') - A(w)) = e + tau g + (tau - dtau) A(w);
-            // the last term is zero wherever the step is not limited
-            const Cell4<R> aw = L.aw[k];
-            const Cell4<R> full = { wb.E + u.E, wb.Fx + u.Fx, wb.Fy + u.Fy, wb.T + u.T };
-            const Cell4<R> ff = { aw.E + b.E, aw.Fx + b.Fx, aw.Fy + b.Fy, aw.T + b.T };
-            const R tau = limited_step(full, ff, dtau, theta, dts, c);
-            const R lim = tau - dtau;
-            out = local_solve_delta<R>(R(1), dtau, L.diag, ka, kt, L.c_v, L.a_r, wb.T,
-                                       u.E + tau * b.E + lim * aw.E + dtau * NE,
-                                       u.Fx + tau * b.Fx + lim * aw.Fx + dtau * NFx,
-                                       u.Fy + tau * b.Fy + lim * aw.Fy + dtau * NFy,
-                                       u.T + tau * b.T + lim * aw.T, ok);
-        }
+        const R tau = limited_step(u, b, dtau, theta, dts, c);
+        out = local_solve<R>(R(1), dtau, L.diag, ka, kt, L.c_v, L.a_r,
+                             u.E + tau * b.E + dtau * NE, u.Fx + tau * b.Fx + dtau * NFx,
+                             u.Fy + tau * b.Fy + dtau * NFy, u.T + tau * b.T, ok);
     }
     if (!ok) atomicAdd(&ctl->newton_fail, 1u);
     L.u[out_buf][k] = out;
+    }
 }
 
 // One Jacobi sweep (Algorithm 1) or one fused pseudo-time step (Eq. (30),
@@ -215,6 +221,7 @@ __device__ __forceinline__ double strip_regs(const Level<R>& L, Ctl* ctl, int2 i
 {
     // the cell's right-hand side (FAS: the restricted residual)
     auto rhs = [&](size_t q) { return FAS ? L.r[q] : L.f[q]; };
+    constexpr int FORM = DELTA && PSEUDO ? FORM_STEP : FORM_FREE;
     double nrm = 0.0;
     const int nx = L.nx, ny = L.ny, two_d = L.dim == 2;
     const int x0 = (it.y % L.sx) * kStripW, y0 = (it.y / L.sx) * L.sh;
@@ -226,10 +233,10 @@ __device__ __forceinline__ double strip_regs(const Level<R>& L, Ctl* ctl, int2 i
     Staged<R> prev{}, cur, next{};
     Raw<R> rn{};
     if (two_d) {
-        prev = stage_raw<R, DELTA>(L, load_raw<R, DELTA>(L, src, i, y0 - 1, colfast && y0 >= 1));
+        prev = stage_raw<R, DELTA, FORM>(L, load_raw<R, DELTA>(L, src, i, y0 - 1, colfast && y0 >= 1));
         rn = load_raw<R, DELTA>(L, src, i, y0 + 1, colfast && y0 + 1 < ny);
     }
-    cur = stage_raw<R, DELTA>(L, load_raw<R, DELTA>(L, src, i, y0, colfast));
+    cur = stage_raw<R, DELTA, FORM>(L, load_raw<R, DELTA>(L, src, i, y0, colfast));
     size_t k = (size_t)y0 * nx + i;
     Cell4<R> bn{};
     Sig2<R> sn{};
@@ -237,7 +244,7 @@ __device__ __forceinline__ double strip_regs(const Level<R>& L, Ctl* ctl, int2 i
     for (int r = 0; r < rows; ++r, k += nx) {
         const int j = y0 + r;
         if (two_d) {
-            next = stage_raw<R, DELTA>(L, rn);
+            next = stage_raw<R, DELTA, FORM>(L, rn);
             if (r + 1 < rows) rn = load_raw<R, DELTA>(L, src, i, j + 2, colfast && j + 2 < ny);
         }
         const Cell4<R> b = bn;
@@ -536,7 +543,7 @@ __device__ __forceinline__ void row_1d32(const Level<float>& L, Ctl* ctl, int2 i
     const bool own = lane >= 1 && lane <= kStripW && i < nx;
     const bool fast = x0 >= 1 && x0 + kStripW + 1 <= nx;
     const Pseudo<float> ps = PSEUDO ? pseudo_of<float>(ctl) : Pseudo<float>{};
-    const Staged<float> cur = stage_raw<float, true>(L, load_raw<float, true>(L, src, i, 0, fast));
+    const Staged<float> cur = stage_raw<float, true, PSEUDO ? FORM_STEP : FORM_FREE>(L, load_raw<float, true>(L, src, i, 0, fast));
     const Staged<float> wv = shfl_staged(cur, (lane + 31) & 31);
     const Staged<float> ev = shfl_staged(cur, (lane + 1) & 31);
     if (own) {
@@ -568,7 +575,7 @@ __device__ __forceinline__ void strip_ring32(const Level<float>& L, Ctl* ctl, in
         Raw<float> r;
         r.w = S.w[lane];
         r.c = S.e[lane];
-        return stage_raw<float, true>(L, r);
+        return stage_raw<float, true, PSEUDO ? FORM_STEP : FORM_FREE>(L, r);
     };
     Staged<float> prev = stage(ring[0]), cur = stage(ring[1]), next{};
     size_t k = (size_t)y0 * nx + i;
@@ -584,7 +591,7 @@ __device__ __forceinline__ void strip_ring32(const Level<float>& L, Ctl* ctl, in
             const Sig2<float> sg = S.sig[lane];
             Cell4<float> u{}, wb{};
             if (PSEUDO) { u = S.e[lane]; wb = S.w[lane]; }
-            update_cell<float, PSEUDO, true>(L, ctl, wv, ev, prev, next, cur, b, sg, k, out_buf,
+            update_cell<float, PSEUDO, true, false, false, true>(L, ctl, wv, ev, prev, next, cur, b, sg, k, out_buf,
                                              true, u, wb, ps);
         }
         prev = cur;
@@ -634,15 +641,15 @@ __device__ __forceinline__ void strip_march(const Level<R>& L, int2 it, int lane
     Staged<R> prev{}, cur, next{};
     Raw<R> rn{};
     if (two_d) {
-        prev = stage_raw<R, DELTA>(L, load_raw<R, DELTA>(L, src, i, y0 - 1, colfast && y0 >= 1));
+        prev = stage_raw<R, DELTA, DELTA ? FORM_STEP : FORM_FREE>(L, load_raw<R, DELTA>(L, src, i, y0 - 1, colfast && y0 >= 1));
         rn = load_raw<R, DELTA>(L, src, i, y0 + 1, colfast && y0 + 1 < ny);
     }
-    cur = stage_raw<R, DELTA>(L, load_raw<R, DELTA>(L, src, i, y0, colfast));
+    cur = stage_raw<R, DELTA, DELTA ? FORM_STEP : FORM_FREE>(L, load_raw<R, DELTA>(L, src, i, y0, colfast));
     size_t k = (size_t)y0 * nx + i;
     for (int r = 0; r < rows; ++r, k += nx) {
         const int j = y0 + r;
         if (two_d) {
-            next = stage_raw<R, DELTA>(L, rn);
+            next = stage_raw<R, DELTA, DELTA ? FORM_STEP : FORM_FREE>(L, rn);
             if (r + 1 < rows) rn = load_raw<R, DELTA>(L, src, i, j + 2, colfast && j + 2 < ny);
         }
         const Staged<R> wv = shfl_staged(cur, (lane + 31) & 31);
@@ -665,24 +672,24 @@ __device__ __forceinline__ double apply_item(const Level<R>& L, int2 it, int lan
     strip_march<R, DELTA>(L, it, lane, src, [&](size_t k, const Staged<R>& wv,
                                                  const Staged<R>& ev, const Staged<R>& prev,
                                                  const Staged<R>& next, const Staged<R>& cur) {
-        R NE, NFx, NFy;
-        strip_neighbours(L, wv, ev, prev, next, two_d, NE, NFx, NFy);
         const Cell4<R> u = src[k];
         const Sig2<R> sg = L.sig[k];
-        const R ka = L.cdt * sg.sa, kt = L.cdt * (sg.sa + sg.ss);
-        R src_e;
-        if (!DELTA) {
-            const R T2 = u.T * u.T;
-            src_e = ka * (u.E - L.a_r * T2 * T2);
-        } else {
-            // A(w + e) - A(w): source difference ka (e_E - a_r ((T + e_T)^4 - T^4))
-            src_e = ka * (u.E - L.a_r * quartic_delta(cur.T, u.T));
-        }
         Cell4<R> a;
-        a.E = L.diag * u.E + src_e - NE;
-        a.Fx = (L.diag + kt) * u.Fx - NFx;
-        a.Fy = (L.diag + kt) * u.Fy - NFy;
-        a.T = L.c_v * u.T - src_e;
+        if constexpr (DELTA) {
+            // A(w + e) - A(w)
+            Sums32 N;
+            sums_x(L.c, L.bx, L.by, two_d, false, wv, ev, prev, next, N.E, N.Fx, N.Fy);
+            a = rows_x(L, sg, cur.T, u, N);
+        } else {
+            R NE, NFx, NFy;
+            strip_neighbours(L, wv, ev, prev, next, two_d, NE, NFx, NFy);
+            const R ka = L.cdt * sg.sa, kt = L.cdt * (sg.sa + sg.ss);
+            const R T2 = u.T * u.T, src_e = ka * (u.E - L.a_r * T2 * T2);
+            a.E = L.diag * u.E + src_e - NE;
+            a.Fx = (L.diag + kt) * u.Fx - NFx;
+            a.Fy = (L.diag + kt) * u.Fy - NFy;
+            a.T = L.c_v * u.T - src_e;
+        }
         if (MODE == APPLY_RESID) {
             const Cell4<R> f = L.f[k];
             const Cell4<R> r = { f.E - a.E, f.Fx - a.Fx, f.Fy - a.Fy, f.T - a.T };
@@ -807,7 +814,7 @@ __device__ __forceinline__ void fas_aw32_item(const Level<float>& L, int2 it, in
         Raw<float> rw;
         rw.c = r.w;
         sw = stage_raw<float, false>(L, rw);
-        sd = stage_raw<float, true>(L, r);
+        sd = stage_raw<float, true, FORM_FAS>(L, r);
     };
     Staged<float> pw{}, cw, nw_{}, pd{}, cd, nd{};
     Raw<float> rn{};
@@ -829,20 +836,12 @@ __device__ __forceinline__ void fas_aw32_item(const Level<float>& L, int2 it, in
         const Staged<float> evd = shfl_staged(cd, (lane + 1) & 31);
         if (own) {
             const Sig2<float> sg = L.sig[k];
-            const float ka = L.cdt * sg.sa, kt = L.cdt * (sg.sa + sg.ss);
             const Cell4<float> wb = L.w[k], v = L.v[k];
-            float NE, NFx, NFy;
-            strip_neighbours(L, wvw, evw, pw, nw_, two_d, NE, NFx, NFy);
-            const float T2 = wb.T * wb.T, sw = ka * (wb.E - L.a_r * T2 * T2);
-            L.aw[k] = Cell4<float>{ L.diag * wb.E + sw - NE, (L.diag + kt) * wb.Fx - NFx,
-                                    (L.diag + kt) * wb.Fy - NFy, L.c_v * wb.T - sw };
-            strip_neighbours(L, wvd, evd, pd, nd, two_d, NE, NFx, NFy);
-            const float sd = ka * (v.E - L.a_r * quartic_delta(wb.T, v.T));
-            const Cell4<float> rr = L.r[k];
-            L.f[k] = Cell4<float>{ (L.diag * v.E + sd - NE) + rr.E,
-                                   ((L.diag + kt) * v.Fx - NFx) + rr.Fx,
-                                   ((L.diag + kt) * v.Fy - NFy) + rr.Fy,
-                                   (L.c_v * v.T - sd) + rr.T };
+            Sums32 N;
+            sums_x(L.c, L.bx, L.by, two_d, false, wvw, evw, pw, nw_, N.E, N.Fx, N.Fy);
+            L.aw[k] = base_rows_x(L, sg, wb, N);
+            sums_x(L.c, L.bx, L.by, two_d, false, wvd, evd, pd, nd, N.E, N.Fx, N.Fy);
+            L.f[k] = fas_rhs_x(L, sg, wb.T, v, L.r[k], N);
         }
         pw = cw; cw = nw_;
         pd = cd; cd = nd;
@@ -1125,19 +1124,20 @@ __device__ __forceinline__ void prolong_block(const Level<R>& Lc, const Level<R>
                     pe.Fy = fma(wt, dc[b][a].Fy, pe.Fy); pe.T = fma(wt, dc[b][a].T, pe.T);
                 }
             const Cell4<R> e = uf[k];
-            Cell4<R> u = e;
-            if (DELTA) {   // correction form: the admissible set constrains w + e
-                const Cell4<R> wb = Lf.w[k];
-                u.E += wb.E; u.Fx += wb.Fx; u.Fy += wb.Fy; u.T += wb.T;
+            if constexpr (DELTA) {   // correction form: the admissible set constrains w + e
+                bool damped;
+                uf[k] = prolong_x(e, Lf.w[k], pe, (float)ctl->theta_c, Lf.c, damped);
+                if (damped) atomicAdd(&ctl->damped, 1u);
+            } else {
+                const Cell4<R> tg = { e.E + pe.E, e.Fx + pe.Fx, e.Fy + pe.Fy, e.T + pe.T };
+                R th = R(1);
+                if (!admissible(tg, Lf.c)) {
+                    th = (R)ctl->theta_c * fmin(R(1), max_admissible_step(e, pe, Lf.c));
+                    atomicAdd(&ctl->damped, 1u);
+                }
+                uf[k] = Cell4<R>{ e.E + th * pe.E, e.Fx + th * pe.Fx, e.Fy + th * pe.Fy,
+                                  e.T + th * pe.T };
             }
-            const Cell4<R> tg = { u.E + pe.E, u.Fx + pe.Fx, u.Fy + pe.Fy, u.T + pe.T };
-            R th = R(1);
-            if (!admissible(tg, Lf.c)) {
-                th = (R)ctl->theta_c * fmin(R(1), max_admissible_step(u, pe, Lf.c));
-                atomicAdd(&ctl->damped, 1u);
-            }
-            uf[k] = Cell4<R>{ e.E + th * pe.E, e.Fx + th * pe.Fx, e.Fy + th * pe.Fy,
-                              e.T + th * pe.T };
         }
 }
 
@@ -1860,10 +1860,13 @@ template <typename R>
 void launch_restrict(const Level<R>* lvf, const Level<R>* lvc, WorkList wl, Ctl* ctls,
                      int fine_buf, cudaStream_t s, bool delta)
 {
-    if (delta && std::is_same<R, float>::value)
-        k_restrict<R, true><<<pgrid(wl), kThreads, 0, s>>>(lvf, lvc, wl, ctls, fine_buf);
-    else
-        k_restrict<R><<<pgrid(wl), kThreads, 0, s>>>(lvf, lvc, wl, ctls, fine_buf);
+    if constexpr (std::is_same<R, float>::value) {
+        if (delta) {
+            k_restrict<R, true><<<pgrid(wl), kThreads, 0, s>>>(lvf, lvc, wl, ctls, fine_buf);
+            return;
+        }
+    }
+    k_restrict<R><<<pgrid(wl), kThreads, 0, s>>>(lvf, lvc, wl, ctls, fine_buf);
 }
 
 template <typename R>
@@ -1876,10 +1879,13 @@ template <typename R>
 void launch_prolong(const Level<R>* lvc, const Level<R>* lvf, WorkList wl, Ctl* ctls,
                     int coarse_buf, int fine_buf, cudaStream_t s, bool delta)
 {
-    if (delta && std::is_same<R, float>::value)
-        k_prolong<R, true><<<pgrid(wl), kThreads, 0, s>>>(lvc, lvf, wl, ctls, coarse_buf, fine_buf);
-    else
-        k_prolong<R><<<pgrid(wl), kThreads, 0, s>>>(lvc, lvf, wl, ctls, coarse_buf, fine_buf);
+    if constexpr (std::is_same<R, float>::value) {
+        if (delta) {
+            k_prolong<R, true><<<pgrid(wl), kThreads, 0, s>>>(lvc, lvf, wl, ctls, coarse_buf, fine_buf);
+            return;
+        }
+    }
+    k_prolong<R><<<pgrid(wl), kThreads, 0, s>>>(lvc, lvf, wl, ctls, coarse_buf, fine_buf);
 }
 
 template <typename R>

@@ -1,5 +1,5 @@
 // The coarse end of a mixed cycle in one launch: m1_tail.cu for the FP32 hierarchy in
-// correction form, with the strip kernels' roundings (m1_exact32.cuh), so that a level
+// correction form, on the functions of the strip kernels (m1_exact32.cuh), so that a level
 // gives the same bits here and in launches of its own.
 //
 // A cluster of `blocks` thread blocks per instance, one thread per cell; between
@@ -73,16 +73,16 @@ __device__ __forceinline__ int row32(const Geo32& g, int k)
 }
 
 // A neighbour outside the grid, or w's at an inflow wall: rare, out of line.
-__device__ __noinline__ Near32 wall32(const Tail32& t, int l, int ae, int ap, int wall, bool base,
+__device__ __noinline__ Staged<float> wall32(const Tail32& t, int l, int ae, int ap, int wall, bool base,
                                       int k, int i, int j)
 {
     const Level<float>& L = t.L[l];
     const int bc = L.bc[wall];
     if (bc == BC_INFLOW) {
-        if (!base) return Near32{ 0.f, 0.f, 0.f, 0.f, 0.f, 0.f };
+        if (!base) return Staged<float>{};
         const int q = wall < 2 ? j : i;
         const float* p = L.inflow + (size_t)(wall * 3) * L.prof_len;
-        Near32 s;
+        Staged<float> s;
         s.E = p[q]; s.Fx = p[L.prof_len + q]; s.Fy = p[2 * L.prof_len + q];
         closure(s.E, s.Fx, s.Fy, L.ic2, s.Pxx, s.Pxy, s.Pyy);
         return s;
@@ -91,7 +91,7 @@ __device__ __noinline__ Near32 wall32(const Tail32& t, int l, int ae, int ap, in
         k = wall == WALL_W ? k + L.nx - 1 : wall == WALL_E ? k - L.nx + 1
           : wall == WALL_S ? k + L.n - L.nx : k - L.n + L.nx;
     const C4 e = *t.at(l, ae, k), p = *t.at(l, ap, k);
-    Near32 s = { e.E, e.Fx, e.Fy, p.E, p.Fx, p.Fy };
+    Staged<float> s = { e.E, e.Fx, e.Fy, p.E, p.Fx, p.Fy, 0.f };
     if (bc == BC_REFLECT) {
         if (wall < 2) s.Fx = -s.Fx;
         else s.Fy = -s.Fy;
@@ -101,7 +101,7 @@ __device__ __noinline__ Near32 wall32(const Tail32& t, int l, int ae, int ap, in
 }
 
 template <int WALL>
-__device__ __forceinline__ Near32 side32(const Tail32& t, int l, int ae, int ap, bool base, int k,
+__device__ __forceinline__ Staged<float> side32(const Tail32& t, int l, int ae, int ap, bool base, int k,
                                          int q, int i, int j)
 {
     const Level<float>& L = t.L[l];
@@ -113,21 +113,23 @@ __device__ __forceinline__ Near32 side32(const Tail32& t, int l, int ae, int ap,
     const C4* pe = here ? t.own(l, ae, q + s) : t.at(l, ae, k + s);
     const C4* pp = here ? t.own(l, ap, q + s) : t.at(l, ap, k + s);
     const C4 e = *pe, p = *pp;
-    return Near32{ e.E, e.Fx, e.Fy, p.E, p.Fx, p.Fy };
+    return Staged<float>{ e.E, e.Fx, e.Fy, p.E, p.Fx, p.Fy, 0.f };
 }
 
-__device__ __forceinline__ void sums32(const Tail32& t, int l, int ae, int ap, bool base, bool xfused,
-                                       int k, int q, int i, int j, float& NE, float& NFx, float& NFy)
+__device__ __forceinline__ Sums32 sums32(const Tail32& t, int l, int ae, int ap, bool base, bool xfused,
+                                         int k, int q, int i, int j)
 {
     const Level<float>& L = t.L[l];
-    const Near32 w = side32<WALL_W>(t, l, ae, ap, base, k, q, i, j);
-    const Near32 e = side32<WALL_E>(t, l, ae, ap, base, k, q, i, j);
-    Near32 s{}, n{};
+    const Staged<float> w = side32<WALL_W>(t, l, ae, ap, base, k, q, i, j);
+    const Staged<float> e = side32<WALL_E>(t, l, ae, ap, base, k, q, i, j);
+    Staged<float> s{}, n{};
     if (L.dim == 2) {
         s = side32<WALL_S>(t, l, ae, ap, base, k, q, i, j);
         n = side32<WALL_N>(t, l, ae, ap, base, k, q, i, j);
     }
-    sums_x(L.c, L.bx, L.by, L.dim == 2, xfused, w, e, s, n, NE, NFx, NFy);
+    Sums32 N;
+    sums_x(L.c, L.bx, L.by, L.dim == 2, xfused, w, e, s, n, N.E, N.Fx, N.Fy);
+    return N;
 }
 
 template <bool FAS>
@@ -162,17 +164,9 @@ __device__ __forceinline__ void op_fas(const Tail32& t, int l, int k, int q, int
 {
     const Level<float>& L = t.L[l];
     const Sig2<float> sg = *t.sig(l, q);
-    const float ka = X_MUL(L.cdt, sg.sa), dk = X_ADD(L.diag, X_MUL(L.cdt, X_ADD(sg.sa, sg.ss)));
     const C4 w = *t.own(l, W, q), v = *t.own(l, V, q), r = *t.own(l, F, q);
-    float NE, NFx, NFy;
-    sums32(t, l, W, E0, true, false, k, q, i, j, NE, NFx, NFy);
-    const float T2 = X_MUL(w.T, w.T), sw = X_MUL(ka, X_FMA(-X_MUL(L.a_r, T2), T2, w.E));
-    *t.own(l, AW, q) = C4{ X_SUB(X_FMA(L.diag, w.E, sw), NE), X_FMA(dk, w.Fx, -NFx),
-                           X_FMA(dk, w.Fy, -NFy), X_FMA(L.c_v, w.T, -sw) };
-    sums32(t, l, V, P0 + 1, false, false, k, q, i, j, NE, NFx, NFy);
-    const float sd = X_MUL(ka, X_FMA(-L.a_r, quartic_delta_x<false>(w.T, v.T), v.E));
-    *t.own(l, F, q) = C4{ X_ADD(X_SUB(X_FMA(L.diag, v.E, sd), NE), r.E), X_ADD(X_FMA(dk, v.Fx, -NFx), r.Fx),
-                          X_ADD(X_FMA(dk, v.Fy, -NFy), r.Fy), X_ADD(X_FMA(L.c_v, v.T, -sd), r.T) };
+    *t.own(l, AW, q) = base_rows_x(L, sg, w, sums32(t, l, W, E0, true, false, k, q, i, j));
+    *t.own(l, F, q) = fas_rhs_x(L, sg, w.T, v, r, sums32(t, l, V, P0 + 1, false, false, k, q, i, j));
 }
 
 // One pseudo-time step (the strips' update_cell) from the iterate in array ae with
@@ -181,20 +175,10 @@ __device__ __forceinline__ void op_step(const Tail32& t, int l, int ae, int ap, 
                                         int i, int j, const Pseudo<float>& ps, unsigned& fails)
 {
     const Level<float>& L = t.L[l];
-    float NE, NFx, NFy;
-    sums32(t, l, ae, ap, false, (t.ring >> l) & 1u, k, q, i, j, NE, NFx, NFy);
-    const Sig2<float> sg = *t.sig(l, q);
-    const float ka = X_MUL(L.cdt, sg.sa), dk = X_ADD(L.diag, X_MUL(L.cdt, X_ADD(sg.sa, sg.ss)));
+    const Sums32 N = sums32(t, l, ae, ap, false, (t.ring >> l) & 1u, k, q, i, j);
     const C4 u = *t.own(l, ae, q), b = *t.own(l, F, q), w = *t.own(l, W, q), a = *t.own(l, AW, q);
-    const C4 full = { X_ADD(w.E, u.E), X_ADD(w.Fx, u.Fx), X_ADD(w.Fy, u.Fy), X_ADD(w.T, u.T) };
-    const C4 ff = { X_ADD(a.E, b.E), X_ADD(a.Fx, b.Fx), X_ADD(a.Fy, b.Fy), X_ADD(a.T, b.T) };
-    const float tau = limited_step_x(full, ff, ps.dtau, ps.theta, ps.s, L.c), lim = X_SUB(tau, ps.dtau);
     bool ok;
-    const C4 o = local_solve_delta_x(ps.dtau, L.diag, ka, dk, L.c_v, L.a_r, w.T,
-                                     X_FMA(ps.dtau, NE, X_FMA(lim, a.E, X_FMA(tau, b.E, u.E))),
-                                     X_FMA(ps.dtau, NFx, X_FMA(lim, a.Fx, X_FMA(tau, b.Fx, u.Fx))),
-                                     X_FMA(ps.dtau, NFy, X_FMA(lim, a.Fy, X_FMA(tau, b.Fy, u.Fy))),
-                                     X_FMA(lim, a.T, X_FMA(tau, b.T, u.T)), ok);
+    const C4 o = pseudo_x(L, *t.sig(l, q), w, a, u, b, N, ps, ok);
     if (!ok) ++fails;
     *t.own(l, E0 + out, q) = o;
     *t.own(l, P0 + out, q) = closure32<false>(L, w, o);
@@ -203,17 +187,10 @@ __device__ __forceinline__ void op_step(const Tail32& t, int l, int ae, int ap, 
 // r = f - [A(w + e) - A(w)], into the iterate's other buffer.
 __device__ __forceinline__ void op_resid(const Tail32& t, int l, int cur, int k, int q, int i, int j)
 {
-    const Level<float>& L = t.L[l];
-    float NE, NFx, NFy;
-    sums32(t, l, E0 + cur, P0 + cur, false, false, k, q, i, j, NE, NFx, NFy);
-    const Sig2<float> sg = *t.sig(l, q);
-    const float ka = X_MUL(L.cdt, sg.sa), dk = X_FMA(L.cdt, X_ADD(sg.sa, sg.ss), L.diag);
+    const Sums32 N = sums32(t, l, E0 + cur, P0 + cur, false, false, k, q, i, j);
     const C4 u = *t.own(l, E0 + cur, q), b = *t.own(l, F, q);
-    const float T = t.own(l, W, q)->T;
-    const float se = X_MUL(ka, X_FMA(-L.a_r, quartic_delta_x<false>(T, u.T), u.E));
     *t.own(l, E0 + 1 - cur, q) =
-        C4{ X_SUB(b.E, X_SUB(X_FMA(L.diag, u.E, se), NE)), X_SUB(b.Fx, X_FMA(dk, u.Fx, -NFx)),
-            X_SUB(b.Fy, X_FMA(dk, u.Fy, -NFy)), X_SUB(b.T, X_FMA(L.c_v, u.T, -se)) };
+        sub_x(b, rows_x(t.L[l], *t.sig(l, q), t.own(l, W, q)->T, u, N));
 }
 
 // One of three arrays (0: v from the iterate, 1: f from the residual, 2: w) of cell
@@ -249,8 +226,7 @@ __device__ __forceinline__ void op_restrict(const Tail32& t, int l, int c, int q
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             const float wt = wy * (a == 1 ? 0.5f : 0.25f);
-            s.E = X_FMA(wt, v[a].E, s.E); s.Fx = X_FMA(wt, v[a].Fx, s.Fx);
-            s.Fy = X_FMA(wt, v[a].Fy, s.Fy); s.T = X_FMA(wt, v[a].T, s.T);
+            s = axpy_x(s, wt, v[a]);
         }
     }
     *t.own(l, part == 0 ? (int)V : part == 1 ? (int)F : (int)W, q) = s;
@@ -279,7 +255,7 @@ __device__ __forceinline__ void op_prolong(const Tail32& t, int l, int cur, int 
             const int per = t.geo[l + 1].per;          // the arrays lie 16 per bytes apart
             const C4 cu = p[c * per], cv = p[(V - E0) * per];
             C4& x = d[b][a];
-            x = C4{ X_SUB(cu.E, cv.E), X_SUB(cu.Fx, cv.Fx), X_SUB(cu.Fy, cv.Fy), X_SUB(cu.T, cv.T) };
+            x = sub_x(cu, cv);
             if (b && yo && by == BC_REFLECT) x.Fy = -x.Fy;
             if (a && xo && bx == BC_REFLECT) x.Fx = -x.Fx;
             if ((b && yo && by == BC_INFLOW) || (a && xo && bx == BC_INFLOW)) x = C4{ 0, 0, 0, 0 };
@@ -290,20 +266,12 @@ __device__ __forceinline__ void op_prolong(const Tail32& t, int l, int cur, int 
 #pragma unroll
         for (int a = 0; a < 2; ++a) {
             if (b > oy || a > ox) continue;
-            const C4& x = d[b][a];
-            pe.E = X_FMA(wt, x.E, pe.E); pe.Fx = X_FMA(wt, x.Fx, pe.Fx);
-            pe.Fy = X_FMA(wt, x.Fy, pe.Fy); pe.T = X_FMA(wt, x.T, pe.T);
+            pe = axpy_x(pe, wt, d[b][a]);
         }
-    const C4 e = *t.own(l, E0 + cur, q), w = *t.own(l, W, q);
-    const C4 u = { X_ADD(e.E, w.E), X_ADD(e.Fx, w.Fx), X_ADD(e.Fy, w.Fy), X_ADD(e.T, w.T) };
-    const C4 tg = { X_ADD(u.E, pe.E), X_ADD(u.Fx, pe.Fx), X_ADD(u.Fy, pe.Fy), X_ADD(u.T, pe.T) };
-    float th = 1.f;
-    if (!admissible(tg, L.c)) {
-        th = X_MUL(theta_c, fminf(1.f, max_admissible_step_x<true>(u, pe, L.c)));
-        ++damped;
-    }
-    const C4 o = { X_FMA(th, pe.E, e.E), X_FMA(th, pe.Fx, e.Fx), X_FMA(th, pe.Fy, e.Fy),
-                   X_FMA(th, pe.T, e.T) };
+    const C4 w = *t.own(l, W, q);
+    bool limited;
+    const C4 o = prolong_x(*t.own(l, E0 + cur, q), w, pe, theta_c, L.c, limited);
+    if (limited) ++damped;
     *t.own(l, E0 + cur, q) = o;
     *t.own(l, P0 + cur, q) = closure32<false>(L, w, o);
 }
