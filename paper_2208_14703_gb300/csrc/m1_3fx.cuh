@@ -196,7 +196,7 @@ __device__ __forceinline__ void add_axis3(const G3& g, const Blocks3& B, size_t 
         add_face3<d, -1>(g, B, n, lo, p, em, x);
         add_face3<d, 1>(g, B, n, hi, p, em, x);
 #pragma unroll
-        for (int a = 0; a < 4; ++a) sum[a] += mul62(split62(x[a]), split62(g.rho[d]));
+        for (int a = 0; a < 4; ++a) sum[a] += fx_product(x[a], split62(g.rho[d]));
     }
 }
 

@@ -112,6 +112,19 @@ __host__ __device__ __forceinline__ i64 sqr62(Split a)
     return madw(a.h, a.h, mid >> 30);
 }
 
+// a b / 2^62 to the nearest, ties to even, |a| < 2^61, 0 <= b < 2^62: odd in a and exact at
+// zero, so that a scaled pair of neighbours (unequal cell sides) keeps the signs and the zeros
+// of the sums it scales and adds no bias to a total.
+__host__ __device__ __forceinline__ i64 fx_product(i64 a, Split b)
+{
+    const i64 s = a >> 63;
+    const Split m = split62((a ^ s) - s);
+    const i64 mid = madw(m.h, b.l, madw(m.l, b.h, madw(m.l, b.l, 0) >> 31));
+    i64 v = madw(m.h, b.h, mid >> 31);
+    v += (((unsigned)mid & 0x7fffffffu) + 0x3fffffffu + ((unsigned)v & 1u)) >> 31;
+    return (v ^ s) - s;
+}
+
 // a cell's block: values v = m 2^(e - 60), F over c
 struct FxCell {
     int e;

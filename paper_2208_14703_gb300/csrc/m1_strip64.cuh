@@ -46,9 +46,7 @@ __device__ __forceinline__ FxFlux fx_add(const FxFlux& a, const FxFlux& b)
 
 __device__ __forceinline__ FxFlux fx_scale(const FxFlux& a, Split r)
 {
-    // + 1: a product falls short by 3/4 of a unit on average
-    return FxFlux{ a.e, mul62(split62(a.E), r, 1), mul62(split62(a.Fx), r, 1),
-                   mul62(split62(a.Fy), r, 1) };
+    return FxFlux{ a.e, fx_product(a.E, r), fx_product(a.Fx, r), fx_product(a.Fy, r) };
 }
 
 // What a cell gives across its faces: to the east and west, and (2D) to the north

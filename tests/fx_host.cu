@@ -17,3 +17,8 @@ extern "C" void host_admissible_sure(int n, const double* u, const double* f, do
         out[k] = admissible_sure(a[0], a[3], b[0], b[3], F);
     }
 }
+
+extern "C" void host_product(int n, const long long* a, long long b, long long* out)
+{
+    for (int k = 0; k < n; ++k) out[k] = fx_product(a[k], split62(b));
+}

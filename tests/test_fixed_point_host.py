@@ -49,3 +49,20 @@ def test_sure_answers_are_right(host, c, s):
         assert np.all((out == 0) | (out == t)), (lo, hi, np.flatnonzero((out != 0) & (out != t))[:5])
         if 1e-12 <= s <= 2e6 and 1e-11 <= c <= 1e11 and s <= 1e15 * c and lo >= -12 and hi < 15:
             assert np.mean(out == 0) < 0.01        # ... and it is given
+
+
+@pytest.mark.parametrize("ratio", [0.5, 0.25, 0.75, 1 / 3, 0.9999, 0.2501])
+def test_scaled_pair_product_is_the_nearest(host, ratio):
+    """a b / 2^62 rounded to the nearest, ties to even (dyadic ratios tie every other time),
+    odd in a, zero at zero: against exact integers."""
+    rng = np.random.default_rng(3)
+    b = int(ratio * 2 ** 62)
+    a = np.concatenate([[0, 1, -1, 2 ** 61 - 1, 1 - 2 ** 61], rng.integers(-2 ** 61, 2 ** 61, 4000),
+                        rng.integers(-64, 64, 200), rng.integers(0, 2 ** 50, 800) * 1024]).astype(np.int64)
+    out = np.zeros_like(a)
+    host.host_product(len(a), fx_host.ptr(a), ctypes.c_longlong(b), fx_host.ptr(out))
+    for x, y in zip(a.tolist(), out.tolist()):
+        q, r = divmod(abs(x) * b, 2 ** 62)
+        q += r > 2 ** 61 or (r == 2 ** 61 and q & 1)
+        # the product of the low halves is cut at 2^-31 of a unit
+        assert y == (q if x >= 0 else -q) or abs(r - 2 ** 61) < 2 ** 31, (x, y, q)

@@ -214,3 +214,51 @@ def test_sums_carry_no_bias(name):
                                  mode=m1.OP3_JACOBI, sweeps=3000)
         e0, e1 = math.fsum(E.ravel()), math.fsum(np.asarray(out)[0].ravel())
     assert abs(e1 / e0 - 1.0) <= 3e-15
+
+
+@pytest.mark.parametrize("name", ["2d", "3d"])
+def test_scaled_sums_carry_no_bias(name):
+    """test_sums_carry_no_bias with unequal cell sides (ratio 2, so that every coefficient
+    is exact): the pairs of the longer sides are scaled.  20000 sweeps: a bias of half a unit of such a sum adds 5e-15 or more.  Same
+    bound."""
+    rng = np.random.default_rng(4)
+    if name == "2d":
+        nx, ny = 64, 64
+        E = 1.0 + rng.random((ny, nx))
+        F = 0.1 * rng.standard_normal((2, ny, nx)) * E
+        F *= np.minimum(1.0, 0.9 * E / np.linalg.norm(F, axis=0))
+        d = m1.make_desc(2, nx, ny, 1.0, 0.5, ("periodic",) * 4, 1)
+        g = m1.Grid(d)
+        zero = np.zeros((ny, nx))
+        g.set_state(E, F[0], F[1], np.ones((ny, nx)), zero, zero)
+        g.jacobi(3000.0 / nx, 20000)
+        e1 = math.fsum(np.asarray(g.get_state()[0]).ravel())
+        g.close()
+    else:
+        nx, ny, nz = 32, 32, 32
+        E = 1.0 + rng.random((nz, ny, nx))
+        F = 0.1 * rng.standard_normal((3, nz, ny, nx)) * E
+        F *= np.minimum(1.0, 0.9 * E / np.linalg.norm(F, axis=0))
+        s = np.concatenate([E[None], F, np.ones((1, nz, ny, nx))])
+        d = m1.make_desc3(nx, ny, nz, 1.0, 0.5, 1.0, ("periodic",) * 6)
+        out, _ = m1.m1_op_level3(d, 3000.0 / nx, np.zeros((2, nz, ny, nx)), s, rhs=s,
+                                 mode=m1.OP3_JACOBI, sweeps=20000)
+        e1 = math.fsum(np.asarray(out)[0].ravel())
+    assert abs(e1 / math.fsum(E.ravel()) - 1.0) <= 3e-15
+
+
+@pytest.mark.parametrize("ly", [0.4, 1.3])
+def test_scaled_pairs_keep_zero(ly):
+    """Unequal sides and a state uniform along one axis without flux in that direction: that
+    flux stays exactly zero, as sums of zeros do."""
+    nx = ny = 48
+    rng = np.random.default_rng(6)
+    desc = m1.make_desc(2, nx, ny, 1.0, ly, ("reflect",) * 4, 1)
+    for axis in (0, 1):                               # uniform along y, then along x
+        line = lambda lo, hi: np.broadcast_to((lambda v: v if axis == 0 else v[:, None])(
+            rng.uniform(lo, hi, nx)), (ny, nx)).copy()
+        E, f, T = line(0.5, 2), line(-0.9, 0.9), line(0.5, 2)
+        s = np.stack([E, f * E if axis == 0 else 0 * E, f * E if axis else 0 * E, T])
+        got, _ = m1.m1_op_level(desc, 10.0 / nx, np.stack([line(0.1, 1), line(0.1, 1)]), s, s,
+                                mode=m1.OP_JACOBI)
+        assert np.all(got[2 - axis] == 0.0)
