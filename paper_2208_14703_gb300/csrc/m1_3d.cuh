@@ -48,7 +48,7 @@ inline void set_fx3(G3& g)
     g.cb = g.c * b;
     g.cbF = g.c * g.c * b;
     g.ic = 1.0 / g.c;
-    g.fx = g.c > 1e-60 && g.c < 1e60 && s > 1e-60 && b < 1e60;
+    g.fx = g.c > 1e-60 && g.c < 1e60 && s > 1e-60 && b < 1e60 && s >= kFxAspect * b;
     for (int a = 0; a < 3; ++a)
         g.rho[a] = g.fx && g.beta[a] < b ? (long long)(g.beta[a] / b * 4611686018427387904.0) : 0;
 }

@@ -496,8 +496,8 @@ m1_status Engine<R>::rebuild()
 
 // Constants of the fixed-point form of the FP64 strips (m1_fx.cuh), and whether
 // a level may take it: its blocks hold E in 2^-500 .. 2^500, so c and b = dt / (2 h)
-// of ordinary size keep every product inside FP64's range.  Unequal cell sides
-// scale one axis' pair of neighbours by the ratio of the two b.
+// of ordinary size keep every product inside FP64's range.  Unequal cell sides (up to
+// kFxAspect) scale one axis' pair of neighbours by the ratio of the two b.
 template <typename R>
 static void set_fx(Level<R>& q, double c, double bx, double by)
 {
@@ -506,7 +506,7 @@ static void set_fx(Level<R>& q, double c, double bx, double by)
     q.cbF = c * c * b;
     q.ic = 1.0 / c;
     q.rho = 0;
-    const bool ok = c > 1e-60 && c < 1e60 && s > 1e-60 && b < 1e60;
+    const bool ok = c > 1e-60 && c < 1e60 && s > 1e-60 && b < 1e60 && s >= kFxAspect * b;
     q.fx = !ok ? 0 : (s == b ? 1 : (bx < by ? 2 : 3));
     if (q.fx > 1) q.rho = std::llrint(std::ldexp(s / b, 62));
 }

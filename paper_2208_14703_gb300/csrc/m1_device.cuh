@@ -39,6 +39,13 @@ constexpr int kStripW = 30, kStripH = 16, kStripWarps = 2;
 // Blocks of a persistent strip launch: up to 16 resident 2-warp blocks per SM.
 constexpr int kStripBlocks = 152 * 16;
 
+// Cells of the fixed-point form (m1_fx.cuh): the shortest side at least this part of the
+// longest.  The sums carry 57 bits of the largest E of the stencil times the largest
+// dt / (2 h).  The flux along a long side gets its pressures, which FP64 holds to about
+// 2^-54 E, through that side's smaller dt / (2 h): below an eighth of the largest the sums
+// would be the coarser of the two (and below 2^-62 the ratio itself has no bits).
+constexpr double kFxAspect = 0.25;
+
 // One grid level as the kernels see it.  Constants that depend on the time
 // step (ax, bx, diag, cdt) are rewritten before every implicit step.
 template <typename R>

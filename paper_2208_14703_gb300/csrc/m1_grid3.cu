@@ -58,7 +58,8 @@ size_t face_max3(const int n[3])
 struct Grid3 {
     m1_grid3_desc desc{};
     int L = 0;
-    bool fx = true;                         // the fixed-point passes; false: their arrays did not fit
+    bool fx = true;                         // the fixed-point passes; false: cells too long for them
+                                            // (kFxAspect), or their arrays did not fit
     cudaStream_t stream = nullptr, cap_stream = nullptr;
     bool own_stream = false;
     std::vector<Lev3> lv;
@@ -153,8 +154,10 @@ m1_status Grid3::init(const m1_grid3_desc& d, int lmax, cudaStream_t s)
         q.g.vol = q.h[0] * q.h[1] * q.h[2];
         q.n = (size_t)q.g.n[0] * q.g.n[1] * q.g.n[2];
     }
+    const double* h = lv[0].h;
+    fx = std::min(h[0], std::min(h[1], h[2])) >= kFxAspect * std::max(h[0], std::max(h[1], h[2]));
     m1_status st = alloc_levels();
-    if (st == M1_ERR_OOM) {                 // without the blocks (the FP64 form)
+    if (st == M1_ERR_OOM && fx) {                 // without the blocks (the FP64 form)
         for (void* p : mem) cudaFree(p);
         mem.clear();
         cudaGetLastError();

@@ -262,3 +262,62 @@ def test_scaled_pairs_keep_zero(ly):
         got, _ = m1.m1_op_level(desc, 10.0 / nx, np.stack([line(0.1, 1), line(0.1, 1)]), s, s,
                                 mode=m1.OP_JACOBI)
         assert np.all(got[2 - axis] == 0.0)
+
+
+def rows_exact(s, sig, dt, h, c):
+    """A(u) on periodic walls (c_v = a_r = 1) in 80 bits and, for each value, the sum of the
+    sizes of its terms.  Axes as in s: [E, F of the last axis, ..., T] over (.., y, x)."""
+    L = np.longdouble
+    d = s.ndim - 1
+    s, sig = s.astype(L), sig.astype(L)
+    E, F, T = s[0], s[1:1 + d], s[-1]
+    f2 = sum(x * x for x in F) / (L(c) * E) ** 2
+    root = np.sqrt(4 - 3 * f2)
+    iso, q = (root - 1) / 3 * E, 3 / (2 + root) / (L(c) ** 2 * E)
+    P = [[q * F[a] * F[b] + (iso if a == b else 0) for b in range(d)] for a in range(d)]
+    beta = [L(dt) / (2 * L(x)) for x in h]
+    diag = 1 + 2 * L(c) * sum(beta)
+    ka, kt = L(c) * L(dt) * sig[0], L(c) * L(dt) * (sig[0] + sig[1])
+    src = ka * (E - T ** 4)
+    out = [diag * E + src] + [(diag + kt) * F[a] for a in range(d)] + [T - src]
+    size = [np.abs(diag * E) + ka * (E + T ** 4)] + [np.abs((diag + kt) * F[a]) for a in range(d)] + [
+        T + ka * (E + T ** 4)]
+    for a in range(d):
+        ax = d - 1 - a
+        for side in (1, -1):                          # the low neighbour, then the high one
+            n = lambda x: np.roll(x, side, axis=ax)
+            out[0] = out[0] - beta[a] * (L(c) * n(E) + side * n(F[a]))
+            size[0] = size[0] + beta[a] * (L(c) * n(E) + np.abs(n(F[a])))
+            for b in range(d):
+                out[1 + b] = out[1 + b] - L(c) * beta[a] * (n(F[b]) + side * L(c) * n(P[a][b]))
+                size[1 + b] = size[1 + b] + L(c) * beta[a] * (np.abs(n(F[b])) + L(c) * np.abs(n(P[a][b])))
+    return np.stack(out), np.stack(size)
+
+
+@pytest.mark.parametrize("flux", [0.9, 1e-6, 1e-13])
+@pytest.mark.parametrize("sides", [(1, 1), (1, 2.5), (5, 1), (1, 300), (3e4, 1), (1, 1e9), (1, 1, 3),
+                                   (2, 1, 300), (1, 1e9, 1e3), (1, 1e21, 1)])
+def test_rows_to_the_roundings_of_their_own_terms(sides, flux):
+    """Each row of A(u), flux rows among them, to a few roundings (16) of its own terms, as
+    FP64 arithmetic gives it, whatever the ratio of the cell sides and however small the
+    fluxes beside E."""
+    d = len(sides)
+    shape = (24, 40) if d == 2 else (7, 9, 16)
+    rng = np.random.default_rng(12)
+    E = 10.0 ** rng.uniform(-1, 1, shape)
+    F = rng.standard_normal((d,) + shape)
+    F *= flux * rng.uniform(0, 1, shape) * E / np.linalg.norm(F, axis=0)
+    s = np.concatenate([E[None], F, 10.0 ** rng.uniform(-0.3, 0.3, (1,) + shape)])
+    sig = 10.0 ** rng.uniform(-2, 1, (2,) + shape)
+    n = shape[::-1]
+    h = [sides[a] / n[0] for a in range(d)]
+    dt = 3.0 * min(h)
+    if d == 2:
+        desc = m1.make_desc(2, *n, h[0] * n[0], h[1] * n[1], ("periodic",) * 4, 1)
+        got, _ = m1.m1_op_level(desc, dt, sig, s, mode=m1.OP_APPLY)
+    else:
+        desc = m1.make_desc3(*n, *(h[a] * n[a] for a in range(3)), ("periodic",) * 6)
+        got, _ = m1.m1_op_level3(desc, dt, sig, s, mode=m1.OP3_APPLY)
+    ref, size = rows_exact(s, sig, dt, h, 1.0)
+    err = np.max(np.abs(got - ref) / size, axis=tuple(range(1, d + 1)))
+    assert np.all(err <= 16 * 2.0 ** -53), err * 2.0 ** 53
