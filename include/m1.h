@@ -382,7 +382,7 @@ m1_status m1_op_level(const m1_grid_desc* desc, const double* inflow, double dt,
  *                    (Algorithm 1)
  * on_device = 0: host arrays (copied in and out; the call returns when done);
  * 1: device arrays, stream-ordered on cuda_stream (the call still waits for its
- * own work).  Each call allocates its own device buffers (84 to 168 bytes a cell in
+ * own work).  Each call allocates its own device buffers (96 to 192 bytes a cell in
  * one allocation; device arrays are read and written where they lie).  ms (may be
  * NULL): device time of the operator passes alone.
  * INVALID_ARG: a size < 1 or above 2^31 cells, a non-positive length, dt or

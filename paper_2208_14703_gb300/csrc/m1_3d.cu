@@ -610,7 +610,7 @@ bool overlap(const double* a, size_t na, const double* b, size_t nb)
 }
 
 // m1_op_level3 in fixed point, on the caller's planes themselves (host callers':
-// staged): blocks of the state, then one pass a sweep, 84 or 168 bytes a cell of
+// staged): blocks of the state, then one pass a sweep, 96 or 192 bytes a cell of
 // device memory where packed copies and closures took 250 to 290 (the allocation is a
 // good part of such a call).  done is left false where the FP64 form has to take the
 // call: the output shares memory with an input, the blocks do not fit, or a cell has

@@ -2,8 +2,8 @@
 // result's blocks for the next one.
 //
 // What bounds them: instruction issue and, on grids over L2, the planes' traffic
-// (a Jacobi sweep reads about 84 bytes of blocks, 40 of b, 32 of coefficients and
-// writes 124 a cell).  The FP64 form (m1_3d.cu), a closure pass and an operator
+// (a Jacobi sweep reads about 96 bytes of blocks, 40 of b, 32 of coefficients and
+// writes 136 a cell).  The FP64 form (m1_3d.cu), a closure pass and an operator
 // pass, is bound by the FP64 pipe at about 150 operations a cell; it stays for
 // grids whose blocks do not fit the device and for cells no block can hold.
 #include "m1_3fx.cuh"
@@ -116,11 +116,10 @@ __device__ __forceinline__ Sig2<double> opacity3(const Sig2<double>* __restrict_
 // place (FP64 operations the pass has room for, against a pass over the opacities
 // and 32 bytes a cell), and a cell with an irregular stencil sets *irregular (the
 // caller then takes the FP64 form).
-#ifndef OPX3_BLOCKS
-#define OPX3_BLOCKS 6
-#endif
+// Blocks per SM: a step of 64^3 took 202 ms at 5 of the first form's and 210 at 6; four
+// PLANAR sweeps of 192^3 4.40 ms at 6 and 4.80 at 5.
 template <int MODE, bool PLANAR = false>
-__global__ void __launch_bounds__(kThreadsX3, OPX3_BLOCKS) k_opx3(G3 g, const EF* __restrict__ u,
+__global__ void __launch_bounds__(kThreadsX3, PLANAR ? 6 : 5) k_opx3(G3 g, const EF* __restrict__ u,
                                                      const double* __restrict__ T, Blocks3 B,
                                                      Coef* __restrict__ Q,
                                                      const Sig2<double>* __restrict__ sig,

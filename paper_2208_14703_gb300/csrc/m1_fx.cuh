@@ -4,16 +4,20 @@
 // GB300 issues one FP64 warp instruction per 64 clocks and SM partition, a
 // 32 x 32 + 64-bit multiply-add per 2.6 and a 64-bit add per 4 (measured).  The
 // stencil kernels were bound by the FP64 pipe with nearly 90% of their issue
-// slots idle.  A cell's closure and its contribution to its neighbours need no
-// exponents of their own: with |F| <= c E every quantity (F / c, the tensor
-// P) is at most E in size, so the six numbers of a cell fit one block: an
-// exponent, E's, and 64-bit significands relative to it.  Products keep 62 bits,
-// sums are exact, so the results carry 57 bits or more relative to E where FP64
-// carried 53 with a rounding per operation: no precision is lost.
+// slots idle.  A cell is held as a block: E, F_x / c and F_y / c as 64-bit significands,
+// each with its own exponent, and the anisotropic part of the closure relative to them.
+// With x = E, sigma = sqrt(x^2 - 3/4 |F/c|^2) and A = 3/2 (F/c)(F/c)^T / (x + sigma),
+//   P = A + S/3 I,  S = x - tr A,
+// so the flux of F_x across an x face is F_x +- A_xx +- S/3.  The sums of F and A are formed
+// relative to the largest flux component of the stencil, the differences of S apart, in
+// which like cells cancel exactly: a flux far below E (ahead of a front, across a grid
+// uniform in that direction, transverse to a 1D grid) keeps its 53 bits, as it does in FP64.
+// Products keep 62 bits, significands 58 (S: 61), sums are exact: each row of the sums carries
+// its terms to 2^-56 or so where FP64 carried 2^-53 with a rounding per operation.
 //
-// Blocks are formed for regular cells only (fx_regular below: E a normal number
-// of ordinary size, |F| <= c E up to a slack); a warp that meets another cell
-// takes the FP64 form of its strip instead, which is the one that handles
+// Blocks are formed for regular cells only (fx_stage: E a normal number of ordinary size,
+// |F| <= c E up to a slack, no flux component but zero below 2^-923); a warp that meets another
+// cell takes the FP64 form of its strip instead, which is the one that handles
 // infinities, NaN and inadmissible states.
 //
 // The functions are host code too, so that their arithmetic can be checked
@@ -125,28 +129,49 @@ __host__ __device__ __forceinline__ i64 fx_product(i64 a, Split b)
     return (v ^ s) - s;
 }
 
-// a cell's block: values v = m 2^(e - 60), F over c
-struct FxCell {
-    int e;
-    i64 E, Fx, Fy, Pxx, Pxy, Pyy;
-};
-
-// exponents (biased) of the E a block can hold: 2^-500 .. 2^500
-constexpr unsigned kFxMinExp = 1023 - 500, kFxMaxExp = 1023 + 500;
-
-// The significand of x relative to 2^(be - 1023) at scale 2^61, truncated; the
-// biased exponent of x is at most be (d >= 0), subnormals and zero give 0.
-__host__ __device__ __forceinline__ i64 fx_align(u64 bits, int d)
+// v / 2^d rounded down, d a difference of exponents: any d >= 64, and any d < 0, which a
+// regular cell excludes, leave the sign (the PTX shift's own rule).
+__host__ __device__ __forceinline__ i64 fx_down(i64 v, int d)
 {
-    const u64 m = ((bits & 0xfffffffffffffull) | 0x10000000000000ull) << 9;
-    const i64 v = (i64)(d > 63 ? 0 : m >> d);
-    const i64 s = (i64)bits >> 63;
-    return (v ^ s) - s;
+#ifdef __CUDA_ARCH__
+    i64 r;
+    asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(d));
+    return r;
+#else
+    return v >> ((unsigned)d < 63u ? d : 63);
+#endif
 }
 
-// sigma = sqrt(xi) (scale 2^60; xi at 2^60, in [x^2/4, x^2]) and, returned, 3/2 D =
-// 3/2 / (x + sigma) at scale 2^62, x at 2^61.
-__host__ __device__ __forceinline__ i64 fx_sigma_d(i64 xE, i64 xi, i64& sg)
+// A cell's block, F over c.  Exponents are FP64's biased ones, e of E and ex, ey of the
+// flux (in the halves of ef); the values are E = m 2^(e - 58), F_x = m 2^(ex - 58) and so
+// on, less the bias, A_xx = m 2^(2 ex - e - 58), A_xy = m 2^(ex + ey - e - 58) and A_yy
+// likewise.
+struct FxCell {
+    int e;
+    unsigned ef;
+    i64 E, Fx, Fy, Axx, Axy, Ayy;
+};
+
+// Exponents (biased) of the E a block can hold: 2^-500 .. 2^500; and the least of a flux
+// component (2^-923, so that sums stay normal numbers), which zero is given too.
+constexpr unsigned kFxMinExp = 1023 - 500, kFxMaxExp = 1023 + 500;
+constexpr int kFxMinFlux = 100;
+
+// A flux component's biased exponent and the size of its significand, scale 2^61; ok cleared
+// where it is too small to hold.
+__host__ __device__ __forceinline__ i64 fx_flux(u64 bits, int& t, bool& ok)
+{
+    t = (int)(bits >> 52) & 0x7ff;
+    const i64 m = (i64)(((bits & 0xfffffffffffffull) | 0x10000000000000ull) << 9);
+    if (t >= kFxMinFlux) return m;
+    ok = ok && (bits << 1) == 0;
+    t = kFxMinFlux;
+    return 0;
+}
+
+// 3/2 D = 3/2 / (x + sigma) at scale 2^62, sigma = sqrt(xi); x at scale 2^61, xi at 2^60 and
+// in [x^2/4, x^2].
+__host__ __device__ __forceinline__ i64 fx_d15(i64 xE, i64 xi)
 {
     // sigma = sqrt(xi): a 30-bit start s0 from the seed y of 1/sqrt(xi), then two
     // Newton corrections sigma += (xi - sigma^2) y / 2, exact residuals
@@ -157,7 +182,7 @@ __host__ __device__ __forceinline__ i64 fx_sigma_d(i64 xE, i64 xi, i64& sg)
     const int s0 = (int)(sf * 0x1.fffffcp29f);                  // < 2^31 (sigma < 2 up to rounding)
     const i64 t0 = xi - madw(s0, s0, 0);                       // scale 2^60, |t0| < 2^42
     const i64 d0 = madw((int)(t0 >> 12), Y, 0) >> 18;          // t0 y / 2, scale 2^60
-    sg = ((i64)s0 << 30) + d0;
+    i64 sg = ((i64)s0 << 30) + d0;
     const i64 t1 = xi - sqr62(split62(sg << 1));
     sg += madw((int)t1, Y, 0) >> 30;
     const i64 hx = xE >> 2;                                    // x / 2 at scale 2^60
@@ -176,46 +201,41 @@ __host__ __device__ __forceinline__ i64 fx_sigma_d(i64 xE, i64 xi, i64& sg)
     return D + (D >> 1);
 }
 
-// The closure of Eq. (5) and the cell's block, from E and F / c.  With x = E and
-// sigma = sqrt(x^2 - 3/4 |F/c|^2) >= x/2 it reads
-//   P = (2 sigma - x)/3 I + 3/2 (F/c)(F/c)^T / (x + sigma),
-// the form of closure() multiplied through by E: one square root and one
-// reciprocal, no division by E, smooth at F = 0.  Returns false when the cell is
-// not regular (the block is then meaningless).
+// The closure of Eq. (5) and the cell's block, from E and F / c: one square root and one
+// reciprocal, no division by E, smooth at F = 0, odd and even in the flux components as the
+// closure is.  Returns false when the cell is not regular (the block is then meaningless).
 __host__ __device__ __forceinline__ bool fx_stage(double E, double Fx, double Fy, FxCell& o)
 {
     const u64 be = bits_of_double(E), bx = bits_of_double(Fx), by = bits_of_double(Fy);
     const unsigned te = (unsigned)(be >> 52);                  // sign included
-    const int dx = (int)te - (int)((unsigned)(bx >> 52) & 0x7ffu);
-    const int dy = (int)te - (int)((unsigned)(by >> 52) & 0x7ffu);
-    bool ok = te - kFxMinExp <= kFxMaxExp - kFxMinExp && dx >= 0 && dy >= 0;
-    // scale 2^61: x in [1, 2), |F / c| < 2
+    bool ok = te - kFxMinExp <= kFxMaxExp - kFxMinExp;
+    int tx, ty;
+    // scale 2^61: x in [1, 2), the sizes of the flux components too, each to its exponent
     const i64 xE = (i64)(((be & 0xfffffffffffffull) | 0x10000000000000ull) << 9);
-    const i64 xF = fx_align(bx, dx), yF = fx_align(by, dy);
-    const Split sE = split62(xE), sX = split62(xF), sY = split62(yF);
+    const i64 mX = fx_flux(bx, tx, ok), mY = fx_flux(by, ty, ok);
+    const int dx = (int)te - tx, dy = (int)te - ty;
+    ok = ok && dx >= 0 && dy >= 0;
+    const Split sE = split62(xE), sX = split62(mX), sY = split62(mY);
     // scale 2^60: x^2 and |F/c|^2
     const i64 E2 = sqr62(sE);
-    const i64 midF = madw(sX.h, sX.l, madw(sY.h, sY.l, 0));
-    const i64 F2 = madw(sX.h, sX.h, madw(sY.h, sY.h, midF >> 30));
+    const i64 F2 = fx_down(sqr62(sX), 2 * dx) + fx_down(sqr62(sY), 2 * dy);
     ok = ok && F2 <= E2 + (E2 >> 10);
     // xi = x^2 - 3/4 |F/c|^2 in [x^2/4, x^2], scale 2^60
     i64 xi = E2 - F2 + (F2 >> 2);
     const i64 q2 = E2 >> 2;
     xi = xi > q2 ? xi : q2;
-    i64 sg;
-    const Split sD = split62(fx_sigma_d(xE, xi, sg));          // 3/2 D, scale 2^62
-    // (2 sigma - x) / 3, scale 2^60: the factor is 2^61 / 3
-    constexpr i64 third = 768614336404564651ll;
-    const i64 iso = mul62(split62((sg << 2) - xE), split62(third));
-    // 3/2 D F/c at scale 2^61, the tensor at scale 2^60
+    const Split sD = split62(fx_d15(xE, xi));                  // 3/2 D, scale 2^62
+    // 3/2 D F/c at scale 2^61, A at scale 2^60, then 2^58 to the nearest
     const Split gx = split62(mul62(sX, sD)), gy = split62(mul62(sY, sD));
-    o.Pxx = mul62(gx, sX, iso);
-    o.Pxy = mul62(gx, sY);
-    o.Pyy = mul62(gy, sY, iso);
-    o.E = xE >> 1;
-    o.Fx = xF >> 1;
-    o.Fy = yF >> 1;
-    o.e = (int)te - 1023;
+    const i64 nx = (i64)bx >> 63, ny = (i64)by >> 63, nxy = nx ^ ny;
+    o.Axx = mul62(gx, sX, 2) >> 2;
+    o.Axy = ((mul62(gx, sY, 2) >> 2) ^ nxy) - nxy;
+    o.Ayy = mul62(gy, sY, 2) >> 2;
+    o.E = xE >> 3;
+    o.Fx = ((mX >> 3) ^ nx) - nx;
+    o.Fy = ((mY >> 3) ^ ny) - ny;
+    o.e = (int)te;
+    o.ef = (unsigned)tx | (unsigned)ty << 16;
     return ok;
 }
 
@@ -338,11 +358,133 @@ __host__ __device__ __forceinline__ bool fx_quartic(double C, double K, double R
     return ok;
 }
 
-// What a cell adds to its neighbour's sums across one face (Eq. (9) with F over
-// c and a common factor c dt / (2 h) taken out): E +- F_d, F_x +- P_xd, F_y +- P_yd.
+// S = E - tr A at E's exponent, scale 2^61.
+__host__ __device__ __forceinline__ i64 fx_iso(const FxCell& c)
+{
+    const int dx = c.e - (int)(c.ef & 0xffffu), dy = c.e - (int)(c.ef >> 16);
+    return (c.E << 3) - fx_down(c.Axx << 3, 2 * dx) - fx_down(c.Ayy << 3, 2 * dy);
+}
+
+// What a cell adds to its neighbour's sums across one face (Eq. (9) with F over c and a
+// common factor c dt / (2 h) taken out): E +- F_d, F_x +- A_xd and F_y +- A_yd, each at its own
+// exponent, and S.  A cell gives to the east and north what it has there; what it gives to the
+// west and south is held with the sign changed (-E + F_d, ...), so that rounding down, where a
+// sum brings it to a larger exponent, rounds it up: the two faces of an axis together carry no
+// bias, which a total over many sweeps would gather.
 struct FxFlux {
     int e;
-    i64 E, Fx, Fy;
+    unsigned ef;
+    i64 E, I, X, Y;
 };
+
+// A cell's part of its x or y faces: F_d at E's exponent, A_xd and A_yd at those of the flux.
+struct FxSide {
+    i64 g, X, Y;
+};
+__host__ __device__ __forceinline__ FxSide fx_side_x(const FxCell& c)
+{
+    const int d = c.e - (int)(c.ef & 0xffffu);
+    return FxSide{ fx_down(c.Fx, d), fx_down(c.Axx, d), fx_down(c.Axy, d) };
+}
+__host__ __device__ __forceinline__ FxSide fx_side_y(const FxCell& c)
+{
+    const int d = c.e - (int)(c.ef >> 16);
+    return FxSide{ fx_down(c.Fy, d), fx_down(c.Axy, d), fx_down(c.Ayy, d) };
+}
+
+// Across the east or north faces, and (HIGH) the west or south ones.
+template <bool HIGH>
+__host__ __device__ __forceinline__ FxFlux fx_flux_of(const FxCell& c, const FxSide& s, i64 iso)
+{
+    return HIGH ? FxFlux{ c.e, c.ef, s.g - c.E, iso, s.X - c.Fx, s.Y - c.Fy }
+                : FxFlux{ c.e, c.ef, s.g + c.E, iso, s.X + c.Fx, s.Y + c.Fy };
+}
+
+// The larger of each half of two pairs of flux exponents.
+__host__ __device__ __forceinline__ unsigned fx_max2(unsigned a, unsigned b)
+{
+#ifdef __CUDA_ARCH__
+    return __vmaxu2(a, b);
+#else
+    const unsigned lo = (a & 0xffffu) > (b & 0xffffu) ? a & 0xffffu : b & 0xffffu;
+    return ((a >> 16) > (b >> 16) ? a >> 16 : b >> 16) << 16 | lo;
+#endif
+}
+
+// A cell's neighbour sums: E, X and Y as in FxFlux at their exponents, and the differences
+// of S that X and Y get, at the larger exponent of their pair (ex, ey).
+struct FxSum {
+    int e, ex, ey;
+    unsigned ef;
+    i64 E, X, Y, Ix, Iy;
+};
+
+// The two faces of an axis, the low one's neighbour and the high one's, at the exponents of
+// the sum (I: of the pair, ep).
+struct FxPair {
+    i64 E, I, X, Y;
+};
+__host__ __device__ __forceinline__ FxPair fx_pair(const FxFlux& lo, const FxFlux& hi, int ep, int e,
+                                                   unsigned ef)
+{
+    const unsigned dl = ef - lo.ef, dh = ef - hi.ef;
+    const int xl = (int)(dl & 0xffffu), xh = (int)(dh & 0xffffu), yl = (int)(dl >> 16), yh = (int)(dh >> 16);
+    return FxPair{ fx_down(lo.E, e - lo.e) - fx_down(hi.E, e - hi.e),
+                   fx_down(lo.I, ep - lo.e) - fx_down(hi.I, ep - hi.e),
+                   fx_down(lo.X, xl) - fx_down(hi.X, xh), fx_down(lo.Y, yl) - fx_down(hi.Y, yh) };
+}
+
+__host__ __device__ __forceinline__ FxPair fx_scale(const FxPair& p, Split r)
+{
+    return FxPair{ fx_product(p.E, r), fx_product(p.I, r), fx_product(p.X, r), fx_product(p.Y, r) };
+}
+
+// West and east.
+__host__ __device__ __forceinline__ FxSum fx_sum1(const FxFlux& w, const FxFlux& e)
+{
+    FxSum s;
+    s.e = s.ex = s.ey = w.e > e.e ? w.e : e.e;
+    s.ef = fx_max2(w.ef, e.ef);
+    const FxPair x = fx_pair(w, e, s.ex, s.e, s.ef);
+    s.E = x.E; s.X = x.X; s.Y = x.Y; s.Ix = x.I; s.Iy = 0;
+    return s;
+}
+
+// West and east, south and north.  fx: Level::fx, 2 and 3 scale the x and the y pair by rho.
+__host__ __device__ __forceinline__ FxSum fx_sum2(const FxFlux& w, const FxFlux& e, const FxFlux& b,
+                                                  const FxFlux& n, int fx, Split rho)
+{
+    FxSum s;
+    s.ex = w.e > e.e ? w.e : e.e;
+    s.ey = b.e > n.e ? b.e : n.e;
+    s.e = s.ex > s.ey ? s.ex : s.ey;
+    s.ef = fx_max2(fx_max2(w.ef, e.ef), fx_max2(b.ef, n.ef));
+    FxPair x = fx_pair(w, e, s.ex, s.e, s.ef), y = fx_pair(b, n, s.ey, s.e, s.ef);
+    if (fx == 2) x = fx_scale(x, rho);
+    if (fx == 3) y = fx_scale(y, rho);
+    s.E = x.E + y.E; s.X = x.X + y.X; s.Y = x.Y + y.Y; s.Ix = x.I; s.Iy = y.I;
+    return s;
+}
+
+// v 2^(t - 58) + (i / 3) 2^(e - 61) (biased exponents) in FP64, in units of the larger of the
+// two where both are there.
+__host__ __device__ __forceinline__ double fx_joined(i64 v, int t, i64 i, int e)
+{
+    constexpr i64 third = 1537228672809129301ll;               // 2^62 / 3
+    const i64 i3 = mul62(split62(i), split62(third));
+    const int ei = i == 0 ? 0 : e - 3, m = ei > t ? ei : t;
+    return fx_double(fx_down(v, m - t) + fx_down(i3, m - ei), m - 1023);
+}
+
+// The sums in FP64: N_E / cb, N_F / cbF.
+__host__ __device__ __forceinline__ double fx_value_E(const FxSum& s) { return fx_double(s.E, s.e - 1023); }
+__host__ __device__ __forceinline__ double fx_value_X(const FxSum& s)
+{
+    return fx_joined(s.X, (int)(s.ef & 0xffffu), s.Ix, s.ex);
+}
+__host__ __device__ __forceinline__ double fx_value_Y(const FxSum& s)
+{
+    return fx_joined(s.Y, (int)(s.ef >> 16), s.Iy, s.ey);
+}
 
 }  // namespace m1

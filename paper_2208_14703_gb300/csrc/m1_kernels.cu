@@ -362,9 +362,8 @@ __device__ __forceinline__ double strip_sweep64(const Level<double>& L, Ctl* ctl
             return p;
         };
         const bool regular = strip_march_fx(L, it, lane, src, pre, [&](size_t k, const Pre& p,
-                                                                       const FxFlux& s) {
-            const double NE = fx_double(s.E, s.e), NFx = fx_double(s.Fx, s.e),
-                         NFy = fx_double(s.Fy, s.e);
+                                                                       const FxSum& s) {
+            const double NE = fx_value_E(s), NFx = fx_value_X(s), NFy = fx_value_Y(s);
             double ka = 0.0, kt = 0.0;
             if ((PSEUDO || NORM) && KEEP != KEEP_LOAD) { ka = L.cdt * p.sg.sa; kt = L.cdt * (p.sg.sa + p.sg.ss); }
             Cell4<double> b = p.b;
@@ -441,13 +440,13 @@ __global__ void __launch_bounds__(kThreads) k_coef64(const Level<double>* __rest
     }
 }
 
-// Persistent FP64 sweep (the item loop of k_sweep), held to 128 registers (8 blocks
-// per SM; 6 and 7, with fewer spills, measured the same or slower).  Bound by the issue
-// of integer instructions, about 900 a warp and row, and then by the FP64 pipe at 10 of
-// its operations a fine update where FP64 throughout takes 103: 0.21 ms a sweep at
-// 2048^2 instead of 0.94, 0.046 ms at 1024^2 instead of 0.19.
+// Persistent FP64 sweep (the item loop of k_sweep), 7 blocks per SM (twenty sweeps at
+// 2048^2, 5.37 ms; 8 blocks 5.46, 6 blocks 5.81).  Bound by the issue of integer
+// instructions, and then by the FP64 pipe at 10 of its operations a fine update where FP64
+// throughout takes 103: 0.27 ms a sweep at 2048^2 instead of 0.89.  (With one exponent for
+// the whole cell, which loses the bits of fluxes far below E, 0.25.)
 template <bool PSEUDO, bool NORM = false, bool FAS = false, int KEEP = KEEP_NONE>
-__global__ void __launch_bounds__(kStripWarps * 32, 8) k_sweep64(const Level<double>* __restrict__ lv,
+__global__ void __launch_bounds__(kStripWarps * 32, 7) k_sweep64(const Level<double>* __restrict__ lv,
                                                                  WorkList wl, Ctl* __restrict__ ctls,
                                                                  int in_buf, int out_buf,
                                                                  double* __restrict__ partials)
@@ -737,14 +736,14 @@ __device__ __forceinline__ double apply_item64(const Level<double>& L, int2 it, 
             return p;
         };
         const bool regular = strip_march_fx(L, it, lane, src, pre, [&](size_t k, const Pre& p,
-                                                                       const FxFlux& s) {
+                                                                       const FxSum& s) {
             const double ka = L.cdt * p.sg.sa, dF = L.diag + L.cdt * (p.sg.sa + p.sg.ss);
             const Cell4<double>& u = p.u;
             const double T2 = u.T * u.T, src_e = ka * fma(-L.a_r, T2 * T2, u.E);
             const Cell4<double> a = {
-                fma(-L.cb, fx_double(s.E, s.e), fma(L.diag, u.E, src_e)),
-                fma(-L.cbF, fx_double(s.Fx, s.e), dF * u.Fx),
-                fma(-L.cbF, fx_double(s.Fy, s.e), dF * u.Fy), fma(L.c_v, u.T, -src_e) };
+                fma(-L.cb, fx_value_E(s), fma(L.diag, u.E, src_e)),
+                fma(-L.cbF, fx_value_X(s), dF * u.Fx),
+                fma(-L.cbF, fx_value_Y(s), dF * u.Fy), fma(L.c_v, u.T, -src_e) };
             if (MODE == APPLY_RESID) {
                 const Cell4<double> r = { p.f.E - a.E, p.f.Fx - a.Fx, p.f.Fy - a.Fy, p.f.T - a.T };
                 if (write_r) L.r[k] = r;

@@ -22,50 +22,12 @@ __device__ __forceinline__ FxFlux shfl_flux(const FxFlux& v, int from)
 {
     FxFlux o;
     o.e = __shfl_sync(0xffffffffu, v.e, from);
+    o.ef = __shfl_sync(0xffffffffu, v.ef, from);
     o.E = shfl_i64(v.E, from);
-    o.Fx = shfl_i64(v.Fx, from);
-    o.Fy = shfl_i64(v.Fy, from);
+    o.I = shfl_i64(v.I, from);
+    o.X = shfl_i64(v.X, from);
+    o.Y = shfl_i64(v.Y, from);
     return o;
-}
-
-// A flux at scale 2^(e - 58) of the exponent e >= v.e (two bits of headroom for
-// the sum of four), rounded down, or up (UP: the east and north faces): together the
-// faces carry no bias, which a total over many sweeps would gather.
-template <bool UP>
-__device__ __forceinline__ FxFlux fx_to(const FxFlux& v, int e)
-{
-    const int n = min(e - v.e + 2, 62);
-    const i64 h = UP ? (1ll << n) - 1 : 0;
-    return FxFlux{ e, (v.E + h) >> n, (v.Fx + h) >> n, (v.Fy + h) >> n };
-}
-
-__device__ __forceinline__ FxFlux fx_add(const FxFlux& a, const FxFlux& b)
-{
-    return FxFlux{ a.e, a.E + b.E, a.Fx + b.Fx, a.Fy + b.Fy };
-}
-
-__device__ __forceinline__ FxFlux fx_scale(const FxFlux& a, Split r)
-{
-    return FxFlux{ a.e, fx_product(a.E, r), fx_product(a.Fx, r), fx_product(a.Fy, r) };
-}
-
-// What a cell gives across its faces: to the east and west, and (2D) to the north
-// and south.
-__device__ __forceinline__ FxFlux fx_east(const FxCell& c)
-{
-    return FxFlux{ c.e, c.E + c.Fx, c.Fx + c.Pxx, c.Fy + c.Pxy };
-}
-__device__ __forceinline__ FxFlux fx_west(const FxCell& c)
-{
-    return FxFlux{ c.e, c.E - c.Fx, c.Fx - c.Pxx, c.Fy - c.Pxy };
-}
-__device__ __forceinline__ FxFlux fx_north(const FxCell& c)
-{
-    return FxFlux{ c.e, c.E + c.Fy, c.Fx + c.Pxy, c.Fy + c.Pyy };
-}
-__device__ __forceinline__ FxFlux fx_south(const FxCell& c)
-{
-    return FxFlux{ c.e, c.E - c.Fy, c.Fx - c.Pxy, c.Fy - c.Pyy };
 }
 
 __device__ __forceinline__ bool fx_stage_cell(const Level<double>& L, const Cell4<double>& c,
@@ -77,8 +39,8 @@ __device__ __forceinline__ bool fx_stage_cell(const Level<double>& L, const Cell
 }
 
 // The strip march of strip_march in fixed point: calls cell(k, p, s) for each own
-// cell, s the sum of its neighbours' fluxes (N_E = cb s.E 2^(s.e - 58), N_F with
-// cbF) and p = pre(k), loaded one row ahead.  Returns false, for the whole warp,
+// cell, s the sum of its neighbours' fluxes (N_E = cb fx_value_E(s), N_F with cbF)
+// and p = pre(k), loaded one row ahead.  Returns false, for the whole warp,
 // when some staged cell was not regular: every result of the strip is then to be
 // formed again by the FP64 form.
 template <typename Pre, typename Cell>
@@ -99,6 +61,7 @@ __device__ __forceinline__ bool strip_march_fx(const Level<double>& L, int2 it, 
     bool ok = true;
     Cell4<double> rn{};
     FxCell cur, next;
+    i64 isoc = 0, ison = 0;                      // S of cur and next
     FxFlux below{};                              // what row j - 1 gives to row j
     size_t k = (size_t)y0 * nx + i;
     decltype(pre(k)) pn{};
@@ -108,35 +71,32 @@ __device__ __forceinline__ bool strip_march_fx(const Level<double>& L, int2 it, 
         const Cell4<double> rb = load(y0 - 1);
         rn = load(y0 + 1);
         ok = fx_stage_cell(L, rb, next) && ok;
-        below = fx_north(next);
+        below = fx_flux_of<false>(next, fx_side_y(next), fx_iso(next));
     }
     ok = fx_stage_cell(L, r0, cur) && ok;
+    isoc = fx_iso(cur);
     const Split rho = split62(L.rho);
 #pragma unroll 1
     for (int r = 0; r < rows; ++r, k += nx) {
         if (two_d) {
             ok = fx_stage_cell(L, rn, next) && ok;
+            ison = fx_iso(next);
             if (r + 1 < rows) rn = load(y0 + r + 2);
         }
         const auto p = pn;
         if (own && r + 1 < rows) pn = pre(k + nx);
-        const FxFlux w = shfl_flux(fx_east(cur), (lane + 31) & 31);
-        const FxFlux e = shfl_flux(fx_west(cur), (lane + 1) & 31);
-        int em = max(w.e, e.e);
-        FxFlux s;
+        const FxSide side = fx_side_x(cur);
+        const FxFlux w = shfl_flux(fx_flux_of<false>(cur, side, isoc), (lane + 31) & 31);
+        const FxFlux e = shfl_flux(fx_flux_of<true>(cur, side, isoc), (lane + 1) & 31);
         if (two_d) {
-            const FxFlux n = fx_south(next);
-            em = max(em, max(below.e, n.e));
-            s = fx_add(fx_to<false>(w, em), fx_to<true>(e, em));
-            FxFlux sy = fx_add(fx_to<false>(below, em), fx_to<true>(n, em));
-            if (L.fx == 2) s = fx_scale(s, rho);
-            if (L.fx == 3) sy = fx_scale(sy, rho);
-            s = fx_add(s, sy);
-            below = fx_north(cur);
+            const FxFlux n = fx_flux_of<true>(next, fx_side_y(next), ison);
+            const FxSum s = fx_sum2(w, e, below, n, L.fx, rho);
+            below = fx_flux_of<false>(cur, fx_side_y(cur), isoc);
             if (own) cell(k, p, s);
             cur = next;
+            isoc = ison;
         } else {
-            s = fx_add(fx_to<false>(w, em), fx_to<true>(e, em));
+            const FxSum s = fx_sum1(w, e);
             if (own) cell(k, p, s);
         }
     }

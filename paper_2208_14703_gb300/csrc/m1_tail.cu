@@ -131,7 +131,7 @@ __device__ __forceinline__ unsigned side_code(const Tail& t, int l, int k, int i
 __device__ __forceinline__ void put_block(const Tail& t, int l, int buf, int q,
                                           const Cell4<double>& u)
 {
-    FxCell c;
+    FxCell c{};
     if (!(t.L[l].fx && fx_stage_cell(t.L[l], u, c))) c.e = kIrregular;
     *t.own<FxCell>(l, ARR_P + buf, q) = c;
 }
@@ -156,11 +156,12 @@ __device__ __forceinline__ FxFlux side64(const Tail& t, int l, int buf, unsigned
         if (rule == BC_REFLECT) {
             if (wall < 2) c.Fx = -c.Fx;
             else c.Fy = -c.Fy;
-            c.Pxy = -c.Pxy;
+            c.Axy = -c.Axy;
         }
     }
-    return wall == WALL_W ? fx_east(c) : wall == WALL_E ? fx_west(c)
-         : wall == WALL_S ? fx_north(c) : fx_south(c);
+    const FxSide side = wall < 2 ? fx_side_x(c) : fx_side_y(c);
+    return wall == WALL_W || wall == WALL_S ? fx_flux_of<false>(c, side, fx_iso(c))
+                                            : fx_flux_of<true>(c, side, fx_iso(c));
 }
 
 // The cell's neighbour sums in FP64 throughout (a block nearby is irregular).
@@ -188,28 +189,22 @@ __device__ __forceinline__ void sums64(const Tail& t, int l, int arr, int buf, i
     const Level<double>& L = t.L[l];
     const uint4 nb = *t.own<uint4>(l, ARR_NB, q);
     const FxFlux w = side64(t, l, buf, nb.x, WALL_W, k), e = side64(t, l, buf, nb.y, WALL_E, k);
-    int em = max(w.e, e.e);
-    FxFlux s;
+    FxSum s;
     if (two_d) {
         const FxFlux b = side64(t, l, buf, nb.z, WALL_S, k), n = side64(t, l, buf, nb.w, WALL_N, k);
-        em = max(em, max(b.e, n.e));
-        s = fx_add(fx_to<false>(w, em), fx_to<true>(e, em));
-        FxFlux sy = fx_add(fx_to<false>(b, em), fx_to<true>(n, em));
-        if (L.fx == 2) s = fx_scale(s, split62(L.rho));
-        if (L.fx == 3) sy = fx_scale(sy, split62(L.rho));
-        s = fx_add(s, sy);
+        s = fx_sum2(w, e, b, n, L.fx, split62(L.rho));
     } else {
-        s = fx_add(fx_to<false>(w, em), fx_to<true>(e, em));
+        s = fx_sum1(w, e);
     }
-    if (em == kIrregular) {
+    if (s.e == kIrregular) {
         general_sums64(t, l, arr, k, two_d, NE, NFx, NFy);
         fx = false;
         return;
     }
     fx = true;
-    NE = fx_double(s.E, s.e);
-    NFx = fx_double(s.Fx, s.e);
-    NFy = fx_double(s.Fy, s.e);
+    NE = fx_value_E(s);
+    NFx = fx_value_X(s);
+    NFy = fx_value_Y(s);
 }
 
 __device__ __forceinline__ void arrive64(const Tail& t, int l, int q, const Cell4<double>& v,

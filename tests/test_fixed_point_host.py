@@ -66,3 +66,57 @@ def test_scaled_pair_product_is_the_nearest(host, ratio):
         q += r > 2 ** 61 or (r == 2 ** 61 and q & 1)
         # the product of the low halves is cut at 2^-31 of a unit
         assert y == (q if x >= 0 else -q) or abs(r - 2 ** 61) < 2 ** 31, (x, y, q)
+
+
+def neighbours(n, kind, size, seed):
+    """[west, east, south, north][E, Fx, Fy] of n cells.  free: four unrelated cells, the flux
+    components of sizes of their own, down to `size`; ahead: E equal everywhere, the fluxes at
+    `size`; along: cells south and north alike, fluxes along y at `size`."""
+    rng = np.random.default_rng(seed)
+    E = np.repeat(10.0 ** rng.uniform(-2, 2, (n, 1)), 4, 1)
+    F = rng.uniform(-1, 1, (n, 4, 2)) / 1.5
+    if kind == "free":
+        E = 10.0 ** rng.uniform(-2, 2, (n, 4))
+        F *= size ** rng.uniform(0, 1, (n, 4, 2))
+    elif kind == "ahead":
+        F *= size
+    else:
+        E[:, :2] = 10.0 ** rng.uniform(-2, 2, (n, 2))
+        F[:, :, 1] *= size
+        F[:, 3] = F[:, 2]
+    return np.concatenate([E[:, :, None], F * E[:, :, None]], 2)
+
+
+@pytest.mark.parametrize("dim", [1, 2])
+@pytest.mark.parametrize("size", [1.0, 1e-3, 1e-9, 1e-15, 1e-20, 1e-60, 1e-200])
+@pytest.mark.parametrize("kind", ["free", "ahead", "along"])
+def test_sums_keep_small_fluxes(host, kind, size, dim):
+    """The sums N_E and N_F / (c b) to a few roundings (16) of their own terms: fluxes, the part
+    A of the pressure that goes with them, and of the isotropic rest S / 3 what FP64 leaves.
+    FP64 holds that to 2^-54 E, so a pair's difference is in error by as much where E differs;
+    where E is equal it drops what is below, f^2 E at most; where the cells are alike it
+    cancels.  Reference: 80 bits, with S taken apart, so that it cancels there too."""
+    n = 3000
+    cells = neighbours(n, kind, size, 9)
+    out = np.zeros((n, 3))
+    assert host.host_sums(n, dim, fx_host.ptr(cells), fx_host.ptr(out)) == n
+    L = np.longdouble
+    E, F = cells[:, :, 0].astype(L), [cells[:, :, 1].astype(L), cells[:, :, 2].astype(L)]
+    f2 = (F[0] ** 2 + F[1] ** 2) / E ** 2
+    sigma = np.sqrt(E * E - 0.75 * (F[0] ** 2 + F[1] ** 2))
+    A = [[1.5 * F[a] * F[b] / (E + sigma) for b in range(2)] for a in range(2)]
+    tr = A[0][0] + A[1][1]
+    ref, terms = np.zeros((3, n), L), np.zeros((3, n), L)
+    for a in range(dim):
+        lo, hi = 2 * a, 2 * a + 1
+        ref[0] += (E[:, lo] + F[a][:, lo]) + (E[:, hi] - F[a][:, hi])
+        terms[0] += E[:, lo] + E[:, hi]
+        for b in range(2):
+            ref[1 + b] += (F[b][:, lo] + A[a][b][:, lo]) + (F[b][:, hi] - A[a][b][:, hi])
+            terms[1 + b] += sum(np.abs(x[:, q]) for x in (F[b], A[a][b]) for q in (lo, hi))
+        ref[1 + a] += (E[:, lo] - E[:, hi]) / 3 - (tr[:, lo] - tr[:, hi]) / 3
+        rest = np.where(E[:, lo] != E[:, hi], E[:, lo] + E[:, hi],
+                        E[:, lo] * np.minimum(1, 2.0 ** 53 * np.maximum(f2[:, lo], f2[:, hi])))
+        terms[1 + a] += np.where(np.all(cells[:, lo] == cells[:, hi], axis=1), 0, rest) / 3
+    err = np.max(np.abs(out.T.astype(L) - ref) / terms, axis=1)
+    assert np.all(err <= 16 * 2.0 ** -53), err * 2.0 ** 53

@@ -321,3 +321,46 @@ def test_rows_to_the_roundings_of_their_own_terms(sides, flux):
     ref, size = rows_exact(s, sig, dt, h, 1.0)
     err = np.max(np.abs(got - ref) / size, axis=tuple(range(1, d + 1)))
     assert np.all(err <= 16 * 2.0 ** -53), err * 2.0 ** 53
+
+
+@pytest.mark.parametrize("size", [1.0, 1e-9, 1e-20, 1e-200])
+@pytest.mark.parametrize("shape", [(96,), (20, 70), (6, 10, 40)])
+def test_small_fluxes_keep_their_bits(shape, size):
+    """E varies along x only; the fluxes along x are of its size, those across it (Fy of a 1D
+    grid too) far below.  The pressures of the pairs across x cancel exactly, so a row of A(u)
+    across x holds fluxes and what goes with them alone: to a few roundings (16) of those terms,
+    as in FP64 throughout.  Periodic walls, 80-bit reference with P split into E / 3 and the
+    rest."""
+    L, d = np.longdouble, len(shape)
+    k = 2 if d == 1 else d                            # flux components
+    rng = np.random.default_rng(13)
+    E = np.broadcast_to(10.0 ** rng.uniform(-1, 1, shape[-1]), shape).copy()
+    F = np.stack([E * rng.uniform(0.2, 0.5, shape) * (1 if a == 0 else size) for a in range(k)])
+    for a in range(k):                                # the same on every line along x
+        F[a] = F[a][(0,) * (d - 1)]
+    T, sig = np.ones(shape), 10.0 ** rng.uniform(-2, 1, (2,) + shape)
+    h, n = 1.0 / shape[-1], shape[::-1]
+    dt = 3.0 * h
+    if d < 3:
+        desc = m1.make_desc(d, n[0], n[1] if d == 2 else 1, 1.0, n[1] * h if d == 2 else 1.0,
+                            ("periodic",) * 4, 1)
+        full = (n[1] if d == 2 else 1, n[0])
+        s = np.concatenate([E[None], F, T[None]]).reshape((4,) + full)
+        got, _ = m1.m1_op_level(desc, dt, sig.reshape((2,) + full), s, mode=m1.OP_APPLY)
+        got = got.reshape((4,) + shape)
+    else:
+        desc = m1.make_desc3(*n, *(h * x for x in n), ("periodic",) * 6)
+        got, _ = m1.m1_op_level3(desc, dt, sig, np.concatenate([E[None], F, T[None]]), mode=m1.OP3_APPLY)
+    E, F = E.astype(L), F.astype(L)
+    A = [1.5 * F[a] * F / (E + np.sqrt(E * E - 0.75 * (F * F).sum(0))) for a in range(k)]
+    beta = L(dt) / (2 * L(h))
+    dF = 1 + 2 * d * beta + L(dt) * (sig[0].astype(L) + sig[1].astype(L))
+    for b in range(1, k):                             # the rows across x
+        ref, terms = dF * F[b], dF * np.abs(F[b])
+        for a in range(d):
+            for side in (1, -1):
+                near = lambda x: np.roll(x, side, axis=d - 1 - a)
+                rest = 0 * E if a == b else A[a][b]   # its own pair's pressures cancel
+                ref = ref - beta * (near(F[b]) + side * near(rest))
+                terms = terms + beta * (np.abs(near(F[b])) + np.abs(near(rest)))
+        assert np.max(np.abs(got[1 + b] - ref) / terms) <= 16 * 2.0 ** -53
