@@ -163,6 +163,11 @@ Engine<R>::~Engine()
     if (ev1) cudaEventDestroy(ev1);
     for (auto& e : poll)
         if (e) cudaEventDestroy(e);
+    for (int z = 0; z < kTailSizes; ++z) {
+        if (tail_join[z]) cudaEventDestroy(tail_join[z]);
+        if (tail_side[z]) cudaStreamDestroy(tail_side[z]);
+    }
+    if (tail_fork) cudaEventDestroy(tail_fork);
     if (cap_stream) cudaStreamDestroy(cap_stream);
     if (own_stream && stream) cudaStreamDestroy(stream);
 }
@@ -174,7 +179,7 @@ std::vector<DevList*> Engine<R>::all_lists()
     for (auto& l : chunks) v.push_back(&l);
     for (auto& l : strips) v.push_back(&l);
     for (auto& l : tails) v.push_back(&l);
-    v.push_back(&tail_all);
+    for (auto& l : tail_all) v.push_back(&l);
     v.push_back(&init_strips);
     v.push_back(&init_chunks);
     return v;
@@ -213,8 +218,9 @@ m1_status Engine<R>::init(int capacity, int levels, bool correction_form, cudaSt
     last_cycles.assign(cap, 0);
     chunks.assign(L, DevList{});
     strips.assign(L, DevList{});
-    tails.assign(L, DevList{});
+    tails.assign((size_t)L * kTailSizes, DevList{});
     tail_first.assign(cap, L);
+    tail_size.assign(cap, 0);
     M1_CK(sizeof(R) == 8 ? tail_prepare() : tail32_prepare());
     M1_TRY(calloc_common((void**)&d, sizeof(Level<R>) * L * cap));
     M1_TRY(calloc_common((void**)&ctl, sizeof(Ctl) * cap));
@@ -395,17 +401,17 @@ template <typename R>
 m1_status Engine<R>::rebuild()
 {
     // The tails: from the first coarse level that is small enough and whose levels fit
-    // a block's shared memory.  FP64: a rule on the instance alone, so that its result
-    // does not depend on the batch; FP32 (bitwise the same either way): also on the
-    // number of instances.
+    // a block's shared memory.  FP64: where they begin is a rule on the instance alone, so
+    // that its result does not depend on the batch; the cluster, which no result depends on,
+    // shrinks with the number of instances as far as it still holds the levels.  FP32 (bitwise
+    // the same either way): both depend on the number of instances.
     int count = 0;
     for (int i = 0; i < cap; ++i) count += used[i] ? 1 : 0;
     const int blocks = sizeof(R) == 8 ? kTailBlocks : tail32_blocks(count);
-    if (blocks != tail_blocks) { tail_blocks = blocks; graph_dirty = true; }
-    auto tail_mem = [&](int i, int l) {
+    auto tail_mem = [&](int i, int l, int nb) {
         const int n = h[(size_t)l * cap + i].n;
-        return sizeof(R) == 8 ? tail_smem(n, blocks, desc[i].dim, L - l)
-                              : tail32_smem(n, blocks, desc[i].dim, L - l);
+        return sizeof(R) == 8 ? tail_smem(n, nb, desc[i].dim, L - l)
+                              : tail32_smem(n, nb, desc[i].dim, L - l);
     };
     for (int i = 0; i < cap; ++i) {
         tail_first[i] = L;
@@ -413,10 +419,15 @@ m1_status Engine<R>::rebuild()
         for (int l = L - 1; l >= 1; --l) {
             if (L - l > kTailLevels ||
                 h[(size_t)l * cap + i].n > (sizeof(R) == 8 ? kTailCells : kTail32Cells * blocks) ||
-                tail_mem(i, l) > (size_t)(sizeof(R) == 8 ? kTailSmem : kTail32Smem))
+                tail_mem(i, l, blocks) > (size_t)(sizeof(R) == 8 ? kTailSmem : kTail32Smem))
                 break;
             tail_first[i] = l;
         }
+        int nb = blocks;
+        if (sizeof(R) == 8 && tail_first[i] < L)
+            while (nb > tail_blocks_for(count) && tail_mem(i, tail_first[i], nb / 2) <= (size_t)kTailSmem)
+                nb /= 2;
+        for (tail_size[i] = 0; kTailBlocks >> tail_size[i] > nb;) ++tail_size[i];
     }
     int off = 0;
     for (int i = 0; i < cap; ++i)
@@ -453,27 +464,33 @@ m1_status Engine<R>::rebuild()
         M1_TRY(upload_list(strips[l]));
         M1_TRY(upload_list(chunks[l]));
     }
-    tail_all.host.clear();
-    size_t bytes = 0;
-    for (int l = 0; l < L; ++l) {
-        tails[l].host.clear();
-        for (int i = 0; i < cap; ++i)
-            if (used[i] && tail_first[i] == l) {
-                tails[l].host.push_back(make_int2(i, l));
-                tail_all.host.push_back(make_int2(i, l));
-                bytes = std::max(bytes, tail_mem(i, l));
-            }
-        M1_TRY(upload_list(tails[l]));
+    int sizes = 0;
+    for (int z = 0; z < kTailSizes; ++z) {
+        tail_all[z].host.clear();
+        size_t bytes = 0;
+        for (int l = 0; l < L; ++l) {
+            DevList& list = tails[(size_t)l * kTailSizes + z];
+            list.host.clear();
+            for (int i = 0; i < cap; ++i)
+                if (used[i] && tail_first[i] == l && tail_size[i] == z) {
+                    list.host.push_back(make_int2(i, l));
+                    tail_all[z].host.push_back(make_int2(i, l));
+                    bytes = std::max(bytes, tail_mem(i, l, kTailBlocks >> z));
+                }
+            M1_TRY(upload_list(list));
+        }
+        M1_TRY(upload_list(tail_all[z]));
+        if (bytes != tail_bytes[z]) { tail_bytes[z] = bytes; graph_dirty = true; }
+        sizes += tail_all[z].n > 0 ? 1 : 0;
     }
-    M1_TRY(upload_list(tail_all));
-    if (bytes != tail_bytes) { tail_bytes = bytes; graph_dirty = true; }
+    if (sizes > 1) M1_TRY(tail_streams());
     // a captured cycle launches nothing for an empty list: re-capture when a
     // list becomes empty or stops being empty
     std::vector<char> sig;
     for (int l = 0; l < L; ++l) {
         sig.push_back(strips[l].n > 0);
         sig.push_back(chunks[l].n > 0);
-        sig.push_back(tails[l].n > 0);
+        for (int z = 0; z < kTailSizes; ++z) sig.push_back(tails[(size_t)l * kTailSizes + z].n > 0);
     }
     if (sig != list_sig) { list_sig = sig; graph_dirty = true; }
     // the sweeps of a level share one launch for all slots: the cp.async kernel
@@ -727,7 +744,7 @@ void Engine<R>::corrections(const Params& p, int l, int shape, std::vector<int>&
 {
     // the instances whose tail begins at level l + 1 take all of it in one launch; in a
     // V-cycle one launch at the bottom serves the tails of every level
-    if (p.cycle != M1_CYCLE_V) tail(tails[l + 1], shape, s);
+    if (p.cycle != M1_CYCLE_V) tail(&tails[(size_t)(l + 1) * kTailSizes], shape, s);
     else if (strips[l + 1].n == 0 || l + 1 == L - 1) tail(tail_all, shape, s);
     if (strips[l + 1].n == 0) return;
     if (l + 1 == L - 1 || shape == M1_CYCLE_V) {
@@ -741,18 +758,50 @@ void Engine<R>::corrections(const Params& p, int l, int shape, std::vector<int>&
     }
 }
 
+// The tails of the listed instances (by cluster size), one launch a size; those after the
+// first beside it on streams of their own.
 template <typename R>
-void Engine<R>::tail(const DevList& list, int shape, cudaStream_t s)
+void Engine<R>::tail(const DevList* lists, int shape, cudaStream_t s)
 {
-    if (!list.n) return;
     const int2* pr = progs + (size_t)shape * L;
-    if constexpr (std::is_same<R, double>::value) {
-        launch_tail(d, cap, L, list.view(), ctl, prog, pr, tail_bytes, s);
-    } else {
-        unsigned mask = 0;
-        for (int l = 0; l < L; ++l) mask |= ring[l] ? 1u << l : 0u;
-        launch_tail32(d, cap, L, list.view(), ctl, prog, pr, mask, tail_bytes, tail_blocks, s);
+    unsigned mask = 0;
+    for (int l = 0; l < L; ++l) mask |= ring[l] ? 1u << l : 0u;
+    int first = kTailSizes, last = -1;
+    for (int z = 0; z < kTailSizes; ++z)
+        if (lists[z].n) {
+            first = std::min(first, z);
+            last = z;
+        }
+    if (last > first) cudaEventRecord(tail_fork, s);
+    for (int z = first; z <= last; ++z) {
+        if (!lists[z].n) continue;
+        cudaStream_t t = s;
+        if (z > first) {
+            t = tail_side[z];
+            cudaStreamWaitEvent(t, tail_fork, 0);
+        }
+        const WorkList wl = lists[z].view();
+        if constexpr (std::is_same<R, double>::value)
+            launch_tail(d, cap, L, wl, ctl, prog, pr, tail_bytes[z], kTailBlocks >> z, t);
+        else
+            launch_tail32(d, cap, L, wl, ctl, prog, pr, mask, tail_bytes[z], kTailBlocks >> z, t);
+        if (z > first) {
+            cudaEventRecord(tail_join[z], t);
+            cudaStreamWaitEvent(s, tail_join[z], 0);
+        }
     }
+}
+
+template <typename R>
+m1_status Engine<R>::tail_streams()
+{
+    if (tail_fork) return M1_OK;
+    for (int z = 1; z < kTailSizes; ++z) {
+        if (!tail_side[z]) M1_CK(cudaStreamCreateWithFlags(&tail_side[z], cudaStreamNonBlocking));
+        if (!tail_join[z]) M1_CK(cudaEventCreateWithFlags(&tail_join[z], cudaEventDisableTiming));
+    }
+    M1_CK(cudaEventCreateWithFlags(&tail_fork, cudaEventDisableTiming));
+    return M1_OK;
 }
 
 namespace {
@@ -801,7 +850,9 @@ m1_status Engine<R>::write_programs(const Params& p)
         for (int f = 1; f < L; ++f) {
             // shapes a cycle reaches: its own, and V below an F-cycle
             const bool reached = shape == p.cycle || (p.cycle == M1_CYCLE_F && shape == M1_CYCLE_V);
-            if (!reached || tails[f].n == 0) continue;
+            bool any = false;
+            for (int z = 0; z < kTailSizes; ++z) any = any || tails[(size_t)f * kTailSizes + z].n > 0;
+            if (!reached || !any) continue;
             const int off = (int)ops.size();
             program(p, L, f, f - 1, shape, delta, ops);
             at[(size_t)shape * L + f] = make_int2(off, (int)ops.size() - off);

@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "m1_kernels.cuh"
+#include "m1_tail.h"
 
 namespace m1 {
 
@@ -112,17 +113,20 @@ struct Engine {
     Params gparams{};
     int graph_cycles = 1;
     bool graph_dirty = true;
-    // the coarse end in one launch per cycle (m1_tail.h): each slot's first tail
-    // level (L: none), the lists of (slot, first level) by first level and of all
-    // slots, the programs by cycle shape and first level, the largest slot's memory
-    std::vector<int> tail_first;
-    std::vector<DevList> tails;
-    DevList tail_all;
+    // the coarse end in one launch per cycle and cluster size (m1_tail.h): each slot's first
+    // tail level (L: none) and cluster size (0: 16 blocks .. 4: 1), the lists of (slot, first
+    // level) by first level and size and of all slots by size, the programs by cycle shape
+    // and first level, the largest slot's memory by size
+    std::vector<int> tail_first, tail_size;
+    std::vector<DevList> tails;             // [first level][size]
+    DevList tail_all[kTailSizes];
     unsigned char* prog = nullptr;
     int2* progs = nullptr;                  // [shape][first level]: (offset, length) in prog
     Params pparams{};                       // the parameters the programs were written for
-    size_t tail_bytes = 0;
-    int tail_blocks = 0;                    // blocks of a cluster
+    size_t tail_bytes[kTailSizes] = {};
+    // launches of several sizes run side by side
+    cudaStream_t tail_side[kTailSizes] = {};
+    cudaEvent_t tail_fork = nullptr, tail_join[kTailSizes] = {};
     std::vector<char> ring;                 // per level: the sweeps take the cp.async kernel
     std::vector<char> list_sig;             // which work lists were non-empty at capture
     // double-word copies of each slot's level-0 iterate, right-hand side and
@@ -162,7 +166,8 @@ struct Engine {
                       bool first_done = false);
     void visit(const Params& p, int l, bool fresh, int shape, std::vector<int>& cur, cudaStream_t s);
     void corrections(const Params& p, int l, int shape, std::vector<int>& cur, cudaStream_t s);
-    void tail(const DevList& list, int shape, cudaStream_t s);
+    void tail(const DevList* lists, int shape, cudaStream_t s);
+    m1_status tail_streams();
     m1_status write_programs(const Params& p);
     long long kernels_per_launch = 0;       // kernel nodes of the captured graph
     m1_status build_graph(const Params& p);

@@ -495,18 +495,19 @@ cudaError_t tail_prepare()
 }
 
 cudaError_t launch_tail(const Level<double>* lv, int cap, int nlev, WorkList wl, Ctl* ctls,
-                        const unsigned char* prog, const int2* progs, size_t smem, cudaStream_t s)
+                        const unsigned char* prog, const int2* progs, size_t smem, int blocks,
+                        cudaStream_t s)
 {
-    const int clusters = wl.capacity < kTailClusters ? (wl.capacity > 0 ? wl.capacity : 1)
-                                                     : kTailClusters;
+    const int most = kTailClusters * kTailBlocks / blocks;
+    const int clusters = wl.capacity < most ? (wl.capacity > 0 ? wl.capacity : 1) : most;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(clusters * kTailBlocks);
+    cfg.gridDim = dim3(clusters * blocks);
     cfg.blockDim = dim3(kTailThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute at = {};
     at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = kTailBlocks;
+    at.val.clusterDim.x = blocks;
     at.val.clusterDim.y = 1;
     at.val.clusterDim.z = 1;
     cfg.attrs = &at;

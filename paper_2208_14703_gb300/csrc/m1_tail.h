@@ -8,9 +8,9 @@
 
 namespace m1 {
 
-// Blocks of a cluster, clusters of a launch, levels, and the dynamic shared memory
-// a block may take.
-constexpr int kTailBlocks = 16, kTailClusters = 36, kTailLevels = 20;
+// Blocks of the largest cluster, clusters of that size in a launch, cluster sizes (16, 8,
+// 4, 2, 1), levels, and the dynamic shared memory a block may take.
+constexpr int kTailBlocks = 16, kTailClusters = 36, kTailSizes = 5, kTailLevels = 20;
 constexpr int kTailSmem = 216 * 1024;
 // The tail begins at the first coarse FP64 level of at most this many cells, which is
 // about what 16 blocks hold with the levels below.  With the line at 2048 cells a step of
@@ -39,6 +39,16 @@ __host__ __device__ inline int tail_per(int n, int nb)
     return (p + 3) & ~3;
 }
 
+// Blocks an instance's cluster should have when `count` instances step together, so that
+// all of them run at once (the device holds 9 clusters of 16 of these blocks, 18 of 8).
+// V-cycles of 64^2 instances, ms a cycle, always 16 blocks and by this rule: 10 instances
+// 0.393 and 0.253, 32 0.92 and 0.36, 128 3.59 and 1.05 (a launch per coarse operation: 0.53,
+// 0.89, 2.73); 128^2, whose tails need 8 blocks: 32 1.36 and 1.39 (2.26).
+inline int tail_blocks_for(int count)
+{
+    return count <= 9 ? 16 : count <= 18 ? 8 : count <= 36 ? 4 : count <= 74 ? 2 : 1;
+}
+
 // Dynamic shared memory of a block for a tail of nlev levels, the first of n0 cells.
 size_t tail_smem(int n0, int nb, int dim, int nlev);
 
@@ -46,9 +56,10 @@ size_t tail_smem(int n0, int nb, int dim, int nlev);
 cudaError_t tail_prepare();
 
 // items of wl: (instance, first tail level); progs[first level]: (offset, length)
-// in prog.
+// in prog; a cluster of `blocks` each.
 cudaError_t launch_tail(const Level<double>* lv, int cap, int nlev, WorkList wl, Ctl* ctls,
-                        const unsigned char* prog, const int2* progs, size_t smem, cudaStream_t s);
+                        const unsigned char* prog, const int2* progs, size_t smem, int blocks,
+                        cudaStream_t s);
 
 // ---- the FP32 hierarchy's (m1_tail32.cu) -----------------------------------------
 // Its levels give the same bits in the tail and in launches of their own, so where it

@@ -1,6 +1,7 @@
 // Host entries to the kernels' arithmetic that is host code too (m1_fx.cuh,
 // m1_strip64.cuh), for tests that need no GPU (tests/fx_host.py compiles this file).
 #include "m1_strip64.cuh"
+#include "m1_tail.h"
 
 using namespace m1;
 
@@ -50,3 +51,5 @@ extern "C" int host_sums(int n, int dim, const double* cells, double* out)
     }
     return regular;
 }
+
+extern "C" int host_tail_blocks(int count) { return tail_blocks_for(count); }

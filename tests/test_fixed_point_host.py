@@ -120,3 +120,13 @@ def test_sums_keep_small_fluxes(host, kind, size, dim):
         terms[1 + a] += np.where(np.all(cells[:, lo] == cells[:, hi], axis=1), 0, rest) / 3
     err = np.max(np.abs(out.T.astype(L) - ref) / terms, axis=1)
     assert np.all(err <= 16 * 2.0 ** -53), err * 2.0 ** 53
+
+
+def test_tail_clusters_run_at_once(host):
+    """Up to 152 instances: one cluster each on the device's 152 SMs (16 blocks leave room for
+    nine, not more), none smaller than that asks for."""
+    for count in range(1, 153):
+        blocks = host.host_tail_blocks(count)
+        assert blocks in (1, 2, 4, 8, 16)
+        assert count * blocks <= 152
+        assert blocks == 16 or 2 * blocks * count > 128
