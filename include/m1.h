@@ -382,9 +382,12 @@ m1_status m1_op_level(const m1_grid_desc* desc, const double* inflow, double dt,
  *                    (Algorithm 1)
  * on_device = 0: host arrays (copied in and out; the call returns when done);
  * 1: device arrays, stream-ordered on cuda_stream (the call still waits for its
- * own work).  Each call allocates its own device buffers (96 to 192 bytes a cell in
- * one allocation; device arrays are read and written where they lie).  ms (may be
- * NULL): device time of the operator passes alone.
+ * own work).  Each call allocates its own device buffers in one allocation: for device
+ * arrays, which are read and written where they lie, 96 bytes a cell, several sweeps 192; for
+ * host arrays 96 more, with rhs 136.  A call whose out shares memory with an input or that
+ * holds a cell outside the fixed-point form's range, or a grid with sides of a ratio above 4,
+ * takes 144 bytes a cell, with rhs 184, and for host arrays 40 more.  ms (may be NULL): device
+ * time of the operator passes alone.
  * INVALID_ARG: a size < 1 or above 2^31 cells, a non-positive length, dt or
  * constant, an inflow or unknown wall, an unknown mode, sweeps < 1 for JACOBI,
  * a NULL array the mode needs.  The state must be admissible. */
@@ -411,6 +414,8 @@ m1_status m1_op_level3(const m1_grid3_desc* desc, double dt, const double* sig,
  *   (in pairs), reflecting, Neumann or inflow; cuda_stream NULL: a stream of its
  *   own.  INVALID_ARG: sizes, lengths or constants out of range, an unknown or
  *   unpaired periodic wall, more than 2^31 cells; OOM.
+ *   Device memory: 440 bytes a cell of every level; where that does not fit, or with sides of a
+ *   ratio above 4, 304 on level 0 and 264 below it, and the slower passes of FP64 throughout.
  * m1_grid3_set_state: v^n from planar [5][nz*ny*nx] doubles (E, Fx, Fy, Fz, T;
  *   index (k*ny + j)*nx + i) and opacities [2][nz*ny*nx] (sigma_a, sigma_s),
  *   host arrays (on_device = 0) or device arrays on the grid's stream (1); both

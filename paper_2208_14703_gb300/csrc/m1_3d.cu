@@ -609,12 +609,20 @@ bool overlap(const double* a, size_t na, const double* b, size_t nb)
     return a && b && a < b + nb && b < a + na;
 }
 
+// The FP64 form's device memory: two states, the closures, the opacities and the right-hand
+// side in its own layout; for host arrays a staging of one state's planes.
+size_t fp64_bytes(size_t n, const double* rhs, int on_device)
+{
+    return n * (2 * (sizeof(EF) + sizeof(double)) + sizeof(P6) + sizeof(Sig2<double>) +
+                (rhs ? sizeof(EF) + sizeof(double) : 0) + (on_device ? 0 : 5 * sizeof(double)));
+}
+
 // m1_op_level3 in fixed point, on the caller's planes themselves (host callers':
 // staged): blocks of the state, then one pass a sweep, 96 or 192 bytes a cell of
 // device memory where packed copies and closures took 250 to 290 (the allocation is a
 // good part of such a call).  done is left false where the FP64 form has to take the
-// call: the output shares memory with an input, the blocks do not fit, or a cell has
-// no block.
+// call: the output shares memory with an input, a cell has no block, or the blocks do not
+// fit where that form takes less (host arrays, several sweeps).
 m1_status op3_fx(const G3& g, size_t n, const double* sig, const double* state, const double* rhs,
                  int mode, int sweeps, double* out, int on_device, cudaStream_t s, double* ms, bool& done)
 {
@@ -631,7 +639,7 @@ m1_status op3_fx(const G3& g, size_t n, const double* sig, const double* state, 
     const size_t ob = on_device || !rhs ? 0 : mem.take(5 * n * sizeof(double));
     const size_t oo = on_device ? 0 : mem.take(5 * n * sizeof(double));
     const cudaError_t e = mem.get();
-    if (e == cudaErrorMemoryAllocation) {
+    if (e == cudaErrorMemoryAllocation && mem.size > fp64_bytes(n, rhs, on_device)) {
         mem.base = nullptr;
         cudaGetLastError();
         return M1_OK;
