@@ -376,6 +376,7 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_tail(const Level<double>* _
         Ctl* ctl = ctls + it.x;
         const int first = it.y, nl = nlev - first;
         const Level<double>* src = lv + (size_t)first * cap + it.x;
+        static_assert(sizeof(Level<double>) % 8 == 0 && sizeof(Level<double>) <= 32 * 8, "one word per lane");
         for (int l = threadIdx.x / 32; l < nl; l += kTailThreads / 32) {
             const unsigned long long* s =
                 reinterpret_cast<const unsigned long long*>(src + (size_t)l * cap);

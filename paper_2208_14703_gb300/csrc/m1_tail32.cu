@@ -298,6 +298,7 @@ __global__ void __launch_bounds__(kThreads32, 1) k_tail32(const Level<float>* __
         const int first = it.y, nl = nlev - first;
         Tail32 t{ Ls, geo, smem, rank, ring >> first, cl };
         const Level<float>* src = lv + (size_t)first * cap + it.x;
+        static_assert(sizeof(Level<float>) % 8 == 0 && sizeof(Level<float>) <= 32 * 8, "one word per lane");
         for (int l = threadIdx.x / 32; l < nl; l += kThreads32 / 32) {
             const unsigned long long* s =
                 reinterpret_cast<const unsigned long long*>(src + (size_t)l * cap);
