@@ -129,3 +129,64 @@ def test_step3_matches_oracle(units):
     assert st.damped == ost["damped"] > 0
     np.testing.assert_allclose(hist, ohist, rtol=1e-8, atol=1e-12 * ohist[0])
     assert rel(out, ref, d["c"]) <= 1e-10
+
+
+def fallback(case, kind):
+    """The case where no block holds a cell (c = 1e61), where the cells are too long for the
+    fixed-point sums, or with a dark region (E = 1e-170) in vacuum, wide enough for coarse cells
+    that are dark too, beside regular ones."""
+    d = case["desc"] = dict(case["desc"])
+    s = case["state"]
+    if kind == "far":
+        return rescale(case, e=1.0, c=1e61)
+    if kind == "long":
+        d["ly"] *= 5.0
+        return case
+    dark = tuple(slice(n // 8, n // 8 + 3 * n // 4) for n in s.shape[1:])
+    s[0][dark] = 1e-170
+    for k in range(1, len(s) - 1):
+        s[k][dark] = 0.0
+    case["sa"][dark] = case["ss"][dark] = 0.0
+    return case
+
+
+@pytest.mark.parametrize("kind", ["far", "long", "dark"])
+@pytest.mark.parametrize("lmax,shape,nx,ny", [(3, 0, 272, 192), (4, 1, 64, 48)])
+def test_step_in_the_fallback_forms(kind, lmax, shape, nx, ny):
+    """Whole 2D steps through the FP64 strips and, in the coarse levels' one launch, the FP64
+    sums.  Bounds of test_step_matches_oracle."""
+    case = fallback(inputs.random_admissible_2d(nx, ny, seed=9, fmax=0.99, cfl=20,
+                                                bc=("reflect",) * 4, lmax=lmax), kind)
+    g = O.Grid.from_case(case)
+    ref, ost, ohist, _ = O.implicit_step(g, case["dt"], case["sa"], case["ss"], case["state"],
+                                         O.SolveParams(lmax=lmax, tol=1e-10, cycle=shape, max_cycles=4))
+    grid = m1.grid_from_case(case)
+    st = grid.implicit_step(case["dt"], m1.m1_default_params(tol=1e-10, cycle=shape, max_cycles=4),
+                            allow_not_converged=True)
+    out = np.stack(grid.get_state())
+    hist, _ = grid.step_history(st.cycles + 1)
+    grid.close()
+    assert (st.cycles, st.damped, st.newton_fail) == (ost["cycles"], ost["damped"], 0)
+    np.testing.assert_allclose(hist, ohist, rtol=1e-9, atol=1e-13 * ohist[0])
+    assert rel(out, ref, case["desc"]["c"]) <= 1e-10
+
+
+@pytest.mark.parametrize("kind", ["far", "long", "dark"])
+def test_step3_in_the_fallback_forms(kind):
+    """Whole 3D steps: the FP64 sums in place of the blocks (far, dark), the FP64 passes (long).
+    Bounds of test_step3_matches_oracle."""
+    case = fallback(mixed_walls_case(), kind)
+    d = case["desc"]
+    g = O3.Grid3(d["nx"], d["ny"], d["nz"], d["lx"] / d["nx"], d["ly"] / d["ny"], d["lz"] / d["nz"],
+                 tuple(d["bc"]), d["c"], d["a_r"], d["c_v"], None)
+    ref, ost, ohist = O3.implicit_step(g, case["dt"], case["sa"], case["ss"], case["state"],
+                                       O3.SolveParams3(lmax=3, tol=1e-10, max_cycles=8))
+    grid = m1.grid3_from_case(case, lmax=3)
+    st = grid.implicit_step(case["dt"], m1.m1_default_params(tol=1e-10, max_cycles=8),
+                            allow_not_converged=True)
+    out = grid.get_state()
+    hist, _ = grid.step_history(st.cycles + 1)
+    grid.close()
+    assert (st.cycles, st.damped, st.newton_fail) == (ost["cycles"], ost["damped"], 0)
+    np.testing.assert_allclose(hist, ohist, rtol=1e-8, atol=1e-12 * ohist[0])
+    assert rel(out, ref, d["c"]) <= 1e-10
