@@ -68,8 +68,7 @@ __device__ __forceinline__ bool fx_stage3(double E, const double F[3], FxCell3& 
     i64 xi = E2 - 3 * F2;                        // x^2 - 3/4 |F|^2
     const i64 q2 = E2 >> 2;
     xi = xi > q2 ? xi : q2;
-    const Split sD = split62(fx_d15(xE, xi));
-    i64 tr = 0;
+    const Split sD = split62(fx_d15(xE, xi, o.S));
     int k = 0;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -78,11 +77,9 @@ __device__ __forceinline__ bool fx_stage3(double E, const double F[3], FxCell3& 
         for (int b = a; b < 3; ++b, ++k) {
             const i64 v = mul62(ga, s[b], 2) >> 2, n = neg[a] ^ neg[b];
             o.A[k] = (v ^ n) - n;
-            if (a == b) tr += fx_down(v << 3, 2 * d[a]);
         }
     }
     o.E = xE >> 3;
-    o.S = (o.E << 3) - tr;
     o.t = make_uint2((te & 0x7ffu) | (unsigned)t[0] << 16, (unsigned)t[1] | (unsigned)t[2] << 16);
     return ok;
 }

@@ -7,8 +7,8 @@
 // slots idle.  A cell is held as a block: E, F_x / c and F_y / c as 64-bit significands,
 // each with its own exponent, and the anisotropic part of the closure relative to them.
 // With x = E, sigma = sqrt(x^2 - 3/4 |F/c|^2) and A = 3/2 (F/c)(F/c)^T / (x + sigma),
-//   P = A + S/3 I,  S = x - tr A,
-// so the flux of F_x across an x face is F_x +- A_xx +- S/3.  The sums of F and A are formed
+//   P = A + S I,  S = (x - tr A)/3 = (2 sigma - x)/3,
+// so the flux of F_x across an x face is F_x +- A_xx +- S.  The sums of F and A are formed
 // relative to the largest flux component of the stencil, the differences of S apart, in
 // which like cells cancel exactly: a flux far below E (ahead of a front, across a grid
 // uniform in that direction, transverse to a 1D grid) keeps its 53 bits, as it does in FP64.
@@ -145,11 +145,11 @@ __host__ __device__ __forceinline__ i64 fx_down(i64 v, int d)
 // A cell's block, F over c.  Exponents are FP64's biased ones, e of E and ex, ey of the
 // flux (in the halves of ef); the values are E = m 2^(e - 58), F_x = m 2^(ex - 58) and so
 // on, less the bias, A_xx = m 2^(2 ex - e - 58), A_xy = m 2^(ex + ey - e - 58) and A_yy
-// likewise.
+// likewise; S = m 2^(e - 61).
 struct FxCell {
     int e;
     unsigned ef;
-    i64 E, Fx, Fy, Axx, Axy, Ayy;
+    i64 E, Fx, Fy, Axx, Axy, Ayy, S;
 };
 
 // Exponents (biased) of the E a block can hold: 2^-500 .. 2^500; and the least of a flux
@@ -169,9 +169,9 @@ __host__ __device__ __forceinline__ i64 fx_flux(u64 bits, int& t, bool& ok)
     return 0;
 }
 
-// 3/2 D = 3/2 / (x + sigma) at scale 2^62, sigma = sqrt(xi); x at scale 2^61, xi at 2^60 and
-// in [x^2/4, x^2].
-__host__ __device__ __forceinline__ i64 fx_d15(i64 xE, i64 xi)
+// 3/2 D = 3/2 / (x + sigma) at scale 2^62, sigma = sqrt(xi), and S = (2 sigma - x)/3 at 2^61;
+// x at scale 2^61, xi at 2^60 and in [x^2/4, x^2].
+__host__ __device__ __forceinline__ i64 fx_d15(i64 xE, i64 xi, i64& S)
 {
     // sigma = sqrt(xi): a 30-bit start s0 from the seed y of 1/sqrt(xi), then two
     // Newton corrections sigma += (xi - sigma^2) y / 2, exact residuals
@@ -187,6 +187,8 @@ __host__ __device__ __forceinline__ i64 fx_d15(i64 xE, i64 xi)
     sg += madw((int)t1, Y, 0) >> 30;
     const i64 hx = xE >> 2;                                    // x / 2 at scale 2^60
     sg = sg > hx ? sg : hx;
+    constexpr i64 third = 1537228672809129301ll;               // 2^62 / 3
+    S = mul62(split62((sg << 2) - xE), split62(third));
     // D = 1 / (x + sigma), scale 2^62, from the seed r: D = r (1 + d + d^2),
     // d = 1 - (x + sigma) r, less 2^-57 so that 3/2 D stays below 2^62
     const i64 w = (xE >> 1) + sg;                              // scale 2^60, in [1.5, 4)
@@ -224,7 +226,7 @@ __host__ __device__ __forceinline__ bool fx_stage(double E, double Fx, double Fy
     i64 xi = E2 - F2 + (F2 >> 2);
     const i64 q2 = E2 >> 2;
     xi = xi > q2 ? xi : q2;
-    const Split sD = split62(fx_d15(xE, xi));                  // 3/2 D, scale 2^62
+    const Split sD = split62(fx_d15(xE, xi, o.S));             // 3/2 D, scale 2^62
     // 3/2 D F/c at scale 2^61, A at scale 2^60, then 2^58 to the nearest
     const Split gx = split62(mul62(sX, sD)), gy = split62(mul62(sY, sD));
     const i64 nx = (i64)bx >> 63, ny = (i64)by >> 63, nxy = nx ^ ny;
@@ -358,13 +360,6 @@ __host__ __device__ __forceinline__ bool fx_quartic(double C, double K, double R
     return ok;
 }
 
-// S = E - tr A at E's exponent, scale 2^61.
-__host__ __device__ __forceinline__ i64 fx_iso(const FxCell& c)
-{
-    const int dx = c.e - (int)(c.ef & 0xffffu), dy = c.e - (int)(c.ef >> 16);
-    return (c.E << 3) - fx_down(c.Axx << 3, 2 * dx) - fx_down(c.Ayy << 3, 2 * dy);
-}
-
 // What a cell adds to its neighbour's sums across one face (Eq. (9) with F over c and a
 // common factor c dt / (2 h) taken out): E +- F_d, F_x +- A_xd and F_y +- A_yd, each at its own
 // exponent, and S.  A cell gives to the east and north what it has there; what it gives to the
@@ -394,10 +389,10 @@ __host__ __device__ __forceinline__ FxSide fx_side_y(const FxCell& c)
 
 // Across the east or north faces, and (HIGH) the west or south ones.
 template <bool HIGH>
-__host__ __device__ __forceinline__ FxFlux fx_flux_of(const FxCell& c, const FxSide& s, i64 iso)
+__host__ __device__ __forceinline__ FxFlux fx_flux_of(const FxCell& c, const FxSide& s)
 {
-    return HIGH ? FxFlux{ c.e, c.ef, s.g - c.E, iso, s.X - c.Fx, s.Y - c.Fy }
-                : FxFlux{ c.e, c.ef, s.g + c.E, iso, s.X + c.Fx, s.Y + c.Fy };
+    return HIGH ? FxFlux{ c.e, c.ef, s.g - c.E, c.S, s.X - c.Fx, s.Y - c.Fy }
+                : FxFlux{ c.e, c.ef, s.g + c.E, c.S, s.X + c.Fx, s.Y + c.Fy };
 }
 
 // The larger of each half of two pairs of flux exponents.
@@ -466,14 +461,12 @@ __host__ __device__ __forceinline__ FxSum fx_sum2(const FxFlux& w, const FxFlux&
     return s;
 }
 
-// v 2^(t - 58) + (i / 3) 2^(e - 61) (biased exponents) in FP64, in units of the larger of the
+// v 2^(t - 58) + i 2^(e - 61) (biased exponents) in FP64, in units of the larger of the
 // two where both are there.
 __host__ __device__ __forceinline__ double fx_joined(i64 v, int t, i64 i, int e)
 {
-    constexpr i64 third = 1537228672809129301ll;               // 2^62 / 3
-    const i64 i3 = mul62(split62(i), split62(third));
     const int ei = i == 0 ? 0 : e - 3, m = ei > t ? ei : t;
-    return fx_double(fx_down(v, m - t) + fx_down(i3, m - ei), m - 1023);
+    return fx_double(fx_down(v, m - t) + fx_down(i, m - ei), m - 1023);
 }
 
 // The sums in FP64: N_E / cb, N_F / cbF.

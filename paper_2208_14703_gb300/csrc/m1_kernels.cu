@@ -441,7 +441,7 @@ __global__ void __launch_bounds__(kThreads) k_coef64(const Level<double>* __rest
 }
 
 // Persistent FP64 sweep (the item loop of k_sweep), 7 blocks per SM (twenty sweeps at
-// 2048^2, 5.37 ms; 8 blocks 5.46, 6 blocks 5.81).  Bound by the issue of integer
+// 2048^2, 5.28 ms; 8 blocks 5.33).  Bound by the issue of integer
 // instructions, and then by the FP64 pipe at 10 of its operations a fine update where FP64
 // throughout takes 103: 0.27 ms a sweep at 2048^2 instead of 0.89.  (With one exponent for
 // the whole cell, which loses the bits of fluxes far below E, 0.25.)

@@ -61,7 +61,6 @@ __device__ __forceinline__ bool strip_march_fx(const Level<double>& L, int2 it, 
     bool ok = true;
     Cell4<double> rn{};
     FxCell cur, next;
-    i64 isoc = 0, ison = 0;                      // S of cur and next
     FxFlux below{};                              // what row j - 1 gives to row j
     size_t k = (size_t)y0 * nx + i;
     decltype(pre(k)) pn{};
@@ -71,30 +70,27 @@ __device__ __forceinline__ bool strip_march_fx(const Level<double>& L, int2 it, 
         const Cell4<double> rb = load(y0 - 1);
         rn = load(y0 + 1);
         ok = fx_stage_cell(L, rb, next) && ok;
-        below = fx_flux_of<false>(next, fx_side_y(next), fx_iso(next));
+        below = fx_flux_of<false>(next, fx_side_y(next));
     }
     ok = fx_stage_cell(L, r0, cur) && ok;
-    isoc = fx_iso(cur);
     const Split rho = split62(L.rho);
 #pragma unroll 1
     for (int r = 0; r < rows; ++r, k += nx) {
         if (two_d) {
             ok = fx_stage_cell(L, rn, next) && ok;
-            ison = fx_iso(next);
             if (r + 1 < rows) rn = load(y0 + r + 2);
         }
         const auto p = pn;
         if (own && r + 1 < rows) pn = pre(k + nx);
         const FxSide side = fx_side_x(cur);
-        const FxFlux w = shfl_flux(fx_flux_of<false>(cur, side, isoc), (lane + 31) & 31);
-        const FxFlux e = shfl_flux(fx_flux_of<true>(cur, side, isoc), (lane + 1) & 31);
+        const FxFlux w = shfl_flux(fx_flux_of<false>(cur, side), (lane + 31) & 31);
+        const FxFlux e = shfl_flux(fx_flux_of<true>(cur, side), (lane + 1) & 31);
         if (two_d) {
-            const FxFlux n = fx_flux_of<true>(next, fx_side_y(next), ison);
+            const FxFlux n = fx_flux_of<true>(next, fx_side_y(next));
             const FxSum s = fx_sum2(w, e, below, n, L.fx, rho);
-            below = fx_flux_of<false>(cur, fx_side_y(cur), isoc);
+            below = fx_flux_of<false>(cur, fx_side_y(cur));
             if (own) cell(k, p, s);
             cur = next;
-            isoc = ison;
         } else {
             const FxSum s = fx_sum1(w, e);
             if (own) cell(k, p, s);

@@ -47,15 +47,24 @@ __device__ __forceinline__ int row_of(const TailGeo& g, int k)
 
 // Arrays of a range of `per` cells: the iterates e0, e1, v and f (which first holds
 // the restricted residual) and the local solve's coefficients (formed by the first
-// step of a fresh visit), 32 bytes a cell each; the blocks of e0 (first of v) and e1,
-// 56 each; sigma; the four neighbours (side_code).
-enum { ARR_E = 0, ARR_V = 2, ARR_F = 3, ARR_Q = 4, ARR_P = 5, ARR_SIG = 7, ARR_NB = 8 };
-constexpr int kTailBytes = 5 * 32 + 2 * 56 + 16 + 16;
+// step of a fresh visit), 32 bytes a cell each; the blocks of e0 (first of v) and e1
+// without S, 56 each (64, with it, would put a warp's cells on a quarter of the banks); sigma;
+// the four neighbours (side_code); the two S.
+enum { ARR_E = 0, ARR_V = 2, ARR_F = 3, ARR_Q = 4, ARR_P = 5, ARR_SIG = 7, ARR_NB = 8, ARR_S = 9 };
+
+// A block without its S.
+struct TailBlock {
+    int e;
+    unsigned ef;
+    i64 E, Fx, Fy, Axx, Axy, Ayy;
+};
+constexpr int kTailBytes = 5 * 32 + 2 * 56 + 16 + 16 + 2 * 8;
 
 __device__ __forceinline__ int arr_at(int a, int per)
 {
     return (a < ARR_P ? a * 32 : a < ARR_SIG ? 5 * 32 + (a - ARR_P) * 56
-                                             : 5 * 32 + 2 * 56 + (a - ARR_SIG) * 16) * per;
+          : a < ARR_S ? 5 * 32 + 2 * 56 + (a - ARR_SIG) * 16
+                      : 5 * 32 + 2 * 56 + 2 * 16 + (a - ARR_S) * 8) * per;
 }
 
 // What a level's pseudo-time steps share: dtau c b, dtau c^2 b (the sums' factors),
@@ -133,7 +142,8 @@ __device__ __forceinline__ void put_block(const Tail& t, int l, int buf, int q,
 {
     FxCell c{};
     if (!(t.L[l].fx && fx_stage_cell(t.L[l], u, c))) c.e = kIrregular;
-    *t.own<FxCell>(l, ARR_P + buf, q) = c;
+    *t.own<TailBlock>(l, ARR_P + buf, q) = TailBlock{ c.e, c.ef, c.E, c.Fx, c.Fy, c.Axx, c.Axy, c.Ayy };
+    *t.own<i64>(l, ARR_S + buf, q) = c.S;
 }
 
 // What the neighbour across `wall` gives (its flux towards this cell).
@@ -149,10 +159,14 @@ __device__ __forceinline__ FxFlux side64(const Tail& t, int l, int buf, unsigned
         const Cell4<double> u = { p[q], p[L.prof_len + q], p[2 * L.prof_len + q], 0.0 };
         if (!fx_stage_cell(L, u, c)) c.e = kIrregular;
     } else {
-        const FxCell* p = t.own<FxCell>(l, ARR_P + buf, (int)(code & 0xffffu));
+        const TailBlock* p = t.own<TailBlock>(l, ARR_P + buf, (int)(code & 0xffffu));
+        const i64* ps = t.own<i64>(l, ARR_S + buf, (int)(code & 0xffffu));
         const int b = (int)(code >> 16) & 0xff;
-        if (b != t.rank) p = t.cl.map_shared_rank(p, b);
-        c = *p;
+        if (b != t.rank) {
+            p = t.cl.map_shared_rank(p, b);
+            ps = t.cl.map_shared_rank(ps, b);
+        }
+        c = FxCell{ p->e, p->ef, p->E, p->Fx, p->Fy, p->Axx, p->Axy, p->Ayy, *ps };
         if (rule == BC_REFLECT) {
             if (wall < 2) c.Fx = -c.Fx;
             else c.Fy = -c.Fy;
@@ -160,8 +174,8 @@ __device__ __forceinline__ FxFlux side64(const Tail& t, int l, int buf, unsigned
         }
     }
     const FxSide side = wall < 2 ? fx_side_x(c) : fx_side_y(c);
-    return wall == WALL_W || wall == WALL_S ? fx_flux_of<false>(c, side, fx_iso(c))
-                                            : fx_flux_of<true>(c, side, fx_iso(c));
+    return wall == WALL_W || wall == WALL_S ? fx_flux_of<false>(c, side)
+                                            : fx_flux_of<true>(c, side);
 }
 
 // The cell's neighbour sums in FP64 throughout (a block nearby is irregular).

@@ -11,7 +11,7 @@ namespace m1 {
 // Blocks of the largest cluster, clusters of that size in a launch, cluster sizes (16, 8,
 // 4, 2, 1), levels, and the dynamic shared memory a block may take.
 constexpr int kTailBlocks = 16, kTailClusters = 36, kTailSizes = 5, kTailLevels = 20;
-constexpr int kTailSmem = 216 * 1024;
+constexpr int kTailSmem = 220 * 1024;
 // The tail begins at the first coarse FP64 level of at most this many cells, which is
 // about what 16 blocks hold with the levels below.  With the line at 2048 cells a step of
 // 320 x 208 (a level of 4160) took 112.8 ms, at 8192 106.2; the paper's beam at 512^2

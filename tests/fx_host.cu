@@ -42,7 +42,7 @@ extern "C" int host_sums(int n, int dim, const double* cells, double* out)
         FxFlux f[4];
         for (int q = 0; q < 2 * dim; ++q) {
             const FxSide side = q < 2 ? fx_side_x(c[q]) : fx_side_y(c[q]);
-            f[q] = q & 1 ? fx_flux_of<true>(c[q], side, fx_iso(c[q])) : fx_flux_of<false>(c[q], side, fx_iso(c[q]));
+            f[q] = q & 1 ? fx_flux_of<true>(c[q], side) : fx_flux_of<false>(c[q], side);
         }
         const FxSum s = dim == 1 ? fx_sum1(f[0], f[1]) : fx_sum2(f[0], f[1], f[2], f[3], 1, Split{});
         out[3 * k] = fx_value_E(s);
