@@ -116,8 +116,8 @@ __device__ __forceinline__ Sig2<double> opacity3(const Sig2<double>* __restrict_
 // place (FP64 operations the pass has room for, against a pass over the opacities
 // and 32 bytes a cell), and a cell with an irregular stencil sets *irregular (the
 // caller then takes the FP64 form).
-// Blocks per SM: a step of 64^3 took 202 ms at 5 of the first form's and 210 at 6; four
-// PLANAR sweeps of 192^3 4.40 ms at 6 and 4.80 at 5.
+// Blocks per SM: a step of 64^3 took 187 ms at 5 of the first form's, 193 at 6 and 216 at 4;
+// four PLANAR sweeps of 192^3 4.27 ms at 6, 4.49 at 7 and 4.61 at 5.
 template <int MODE, bool PLANAR = false>
 __global__ void __launch_bounds__(kThreadsX3, PLANAR ? 6 : 5) k_opx3(G3 g, const EF* __restrict__ u,
                                                      const double* __restrict__ T, Blocks3 B,

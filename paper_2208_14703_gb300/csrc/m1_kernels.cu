@@ -331,7 +331,7 @@ __device__ __noinline__ double strip_general64(const Level<double>& L, Ctl* ctl,
 // visit share dtau, hence the local solve's coefficients (sixteen FP64 operations of a
 // step's thirty): the first that follows the FAS right-hand side stores them in the
 // level's residual array, which is free from there to the residual, and the rest of the
-// run loads them.  A step at 512^2: 15.7 us with them loaded, 18.3 formed and stored
+// run loads them.  A step at 512^2: 15.8 us with them loaded, 17.6 formed and stored
 // (a 1024^2 FP64 cycle of six steps a level: 3% less).
 enum { KEEP_NONE = 0, KEEP_STORE = 1, KEEP_LOAD = 2 };
 template <bool PSEUDO, bool NORM, bool FAS, int KEEP>
@@ -441,12 +441,14 @@ __global__ void __launch_bounds__(kThreads) k_coef64(const Level<double>* __rest
 }
 
 // Persistent FP64 sweep (the item loop of k_sweep), 7 blocks per SM (twenty sweeps at
-// 2048^2, 5.28 ms; 8 blocks 5.33).  Bound by the issue of integer
-// instructions, and then by the FP64 pipe at 10 of its operations a fine update where FP64
-// throughout takes 103: 0.27 ms a sweep at 2048^2 instead of 0.89.  (With one exponent for
-// the whole cell, which loses the bits of fluxes far below E, 0.25.)
+// 2048^2, 5.28 ms; 8 blocks 5.33), with the norm 6 (a 1024^2 step 559 ms, at 7 572; at 2048^2
+// 1703 and 1720; the pseudo-time steps at 6 blocks too 579 and 1658).  Bound by the issue of
+// integer instructions, 1150 a warp and row, and then by the FP64 pipe at 10 of its
+// operations a fine update where FP64 throughout takes 103: 0.236 ms a sweep at 2048^2 instead
+// of 0.89.  (With one exponent for the whole cell, which loses the bits of fluxes far below E,
+// 0.22.)
 template <bool PSEUDO, bool NORM = false, bool FAS = false, int KEEP = KEEP_NONE>
-__global__ void __launch_bounds__(kStripWarps * 32, 7) k_sweep64(const Level<double>* __restrict__ lv,
+__global__ void __launch_bounds__(kStripWarps * 32, NORM ? 6 : 7) k_sweep64(const Level<double>* __restrict__ lv,
                                                                  WorkList wl, Ctl* __restrict__ ctls,
                                                                  int in_buf, int out_buf,
                                                                  double* __restrict__ partials)

@@ -11,8 +11,8 @@
 // (12k to 18k clocks a restriction, now 4k to 12k).
 // Measured: the five coarse levels of a 1024^2 mixed cycle (128^2 down to 8^2, 45
 // operations) 0.115 ms; the cycle 0.685 ms with a launch for each, 0.575 ms so.  Eight
-// served 256^2 to 1024^2 streams: 641 to 529 ms; instances of at most 128^2 in a batch,
-// whose levels below 32^2 alone go this way at 24 instances, 1% faster.
+// served 256^2 to 1024^2 streams: 641 to 529 ms.  A batch of 24 of 64^2 to 512^2 (clusters of
+// 4 blocks, tails from 64^2 down): no difference beyond the noise of 1%.
 #include <cooperative_groups.h>
 
 #include "m1_cell.cuh"
