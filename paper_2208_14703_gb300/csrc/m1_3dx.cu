@@ -116,10 +116,11 @@ __device__ __forceinline__ Sig2<double> opacity3(const Sig2<double>* __restrict_
 // place (FP64 operations the pass has room for, against a pass over the opacities
 // and 32 bytes a cell), and a cell with an irregular stencil sets *irregular (the
 // caller then takes the FP64 form).
-// Blocks per SM: a step of 64^3 took 187 ms at 5 of the first form's, 193 at 6 and 216 at 4;
-// four PLANAR sweeps of 192^3 4.27 ms at 6, 4.49 at 7 and 4.61 at 5.
+// Six blocks per SM: cycles of 64^3, 128^3 and 192^3 take 0.550, 2.64 and 8.12 ms (5 blocks
+// 0.535, 2.81 and 8.82; 7 blocks 0.552, 2.77 and 8.68), four PLANAR sweeps of 192^3 4.27 ms
+// (5 blocks 4.61, 7 blocks 4.49).
 template <int MODE, bool PLANAR = false>
-__global__ void __launch_bounds__(kThreadsX3, PLANAR ? 6 : 5) k_opx3(G3 g, const EF* __restrict__ u,
+__global__ void __launch_bounds__(kThreadsX3, 6) k_opx3(G3 g, const EF* __restrict__ u,
                                                      const double* __restrict__ T, Blocks3 B,
                                                      Coef* __restrict__ Q,
                                                      const Sig2<double>* __restrict__ sig,
