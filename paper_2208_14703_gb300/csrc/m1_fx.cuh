@@ -365,7 +365,8 @@ __host__ __device__ __forceinline__ bool fx_quartic(double C, double K, double R
 // exponent, and S.  A cell gives to the east and north what it has there; what it gives to the
 // west and south is held with the sign changed (-E + F_d, ...), so that rounding down, where a
 // sum brings it to a larger exponent, rounds it up: the two faces of an axis together carry no
-// bias, which a total over many sweeps would gather.
+// bias, which a total over many sweeps would gather.  (A mirror image of a state exchanges the
+// faces, so its sums may differ from the state's by that rounding.)
 struct FxFlux {
     int e;
     unsigned ef;
