@@ -88,7 +88,7 @@ static cudaError_t tail_answer()
     return g_last = cudaErrorInvalidConfiguration;
 }
 cudaError_t launch_tail(const Level<double>*, int, int, WorkList, Ctl*, const unsigned char*, const int2*,
-                        size_t, cudaStream_t)
+                        size_t, int, cudaStream_t)
 {
     return tail_answer();
 }
