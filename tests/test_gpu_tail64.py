@@ -13,13 +13,15 @@ m1 = pytest.importorskip("paper_2208_14703_gb300.m1")
 
 
 def cases():
-    """Tails that need 16, 8, 4, 2 and 1 blocks (first levels of 4160, 4096, 2288, 1024, 64)."""
-    return [inputs.random_admissible_2d(320, 208, seed=4, fmax=0.9, cfl=30, bc=("periodic",) * 4, lmax=4),
-            inputs.hot_square_2d(256, lmax=4),
-            inputs.random_admissible_2d(208, 176, seed=5, fmax=0.9, cfl=30, bc=("reflect",) * 4, lmax=4),
-            inputs.beam_channel_2d(64, lmax=4),
-            inputs.gaussian_1d(4096, lmax=4),
-            inputs.hot_square_2d(16, lmax=4)]
+    """Tails that need 16, 16, 8, 4, 2, 1 and 1 blocks (first levels of 8192, which fill the
+    shared memory, 4160, 4096, 2288, 1024, 2048 and 64)."""
+    return [inputs.random_admissible_2d(512, 256, seed=7, fmax=0.9, cfl=30, bc=("neumann",) * 4, lmax=5),
+            inputs.random_admissible_2d(320, 208, seed=4, fmax=0.9, cfl=30, bc=("periodic",) * 4, lmax=5),
+            inputs.hot_square_2d(256, lmax=5),
+            inputs.random_admissible_2d(208, 176, seed=5, fmax=0.9, cfl=30, bc=("reflect",) * 4, lmax=5),
+            inputs.beam_channel_2d(64, lmax=5),
+            inputs.gaussian_1d(4096, lmax=5),
+            inputs.hot_square_2d(16, lmax=5)]
 
 
 @pytest.mark.parametrize("count", [9, 12, 24, 48, 90])
