@@ -465,6 +465,8 @@ m1_status Engine<R>::rebuild()
         M1_TRY(upload_list(chunks[l]));
     }
     int sizes = 0;
+    // a list without entries is not launched, and most sizes never have any
+    auto upload_tail = [&](DevList& l) { return l.host.empty() && !l.items ? M1_OK : upload_list(l); };
     for (int z = 0; z < kTailSizes; ++z) {
         tail_all[z].host.clear();
         size_t bytes = 0;
@@ -477,9 +479,9 @@ m1_status Engine<R>::rebuild()
                     tail_all[z].host.push_back(make_int2(i, l));
                     bytes = std::max(bytes, tail_mem(i, l, kTailBlocks >> z));
                 }
-            M1_TRY(upload_list(list));
+            M1_TRY(upload_tail(list));
         }
-        M1_TRY(upload_list(tail_all[z]));
+        M1_TRY(upload_tail(tail_all[z]));
         if (bytes != tail_bytes[z]) { tail_bytes[z] = bytes; graph_dirty = true; }
         sizes += tail_all[z].n > 0 ? 1 : 0;
     }
